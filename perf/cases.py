@@ -150,6 +150,26 @@ def _in_state(trainer, host, pitch):
     raise RuntimeError("a layer's master weights are not in the workspace")
 
 
+def _initial(layers, normal):
+    """He-normal weights, small biases, on the host as lp_create takes them."""
+    W0, b0 = [], []
+    for l in layers:
+        shape = inputs.weight_shape(l)
+        w = torch.empty(shape, pin_memory=True)
+        w.copy_(normal(*shape) * math.sqrt(2.0 / np.prod(shape[1:])))
+        W0.append(w.numpy())
+        b0.append((0.05 * normal(l["n_out"])).cpu().numpy())
+    return W0, b0
+
+
+def _minibatches(case, layers, normal, gen):
+    shape = inputs.input_shape(layers, case["batch"])
+    x = [normal(*shape).to(torch.bfloat16 if case["input"] == "bf16" else torch.float32) for _ in range(case["steps"])]
+    y = [torch.randint(0, inputs.n_classes(layers), (case["batch"],), generator=gen, device="cuda", dtype=torch.int32)
+         for _ in range(case["steps"])]
+    return x, y
+
+
 def prepare(case, seed):
     dev = torch.device("cuda")
     gen = torch.Generator(device=dev).manual_seed(seed)
@@ -174,13 +194,7 @@ def prepare(case, seed):
                     delta=torch.zeros(B, (C + 7) // 8 * 8, dtype=torch.bfloat16, device=dev), loss=torch.zeros(1, device=dev))
 
     layers = _layers(case)
-    W0, b0 = [], []
-    for l in layers:                                # He-normal weights, small biases, on the host as lp_create takes them
-        shape = inputs.weight_shape(l)
-        w = torch.empty(shape, pin_memory=True)
-        w.copy_(normal(*shape) * math.sqrt(2.0 / np.prod(shape[1:])))
-        W0.append(w.numpy())
-        b0.append((0.05 * normal(l["n_out"])).cpu().numpy())
+    W0, b0 = _initial(layers, normal)
     bf16 = case["input"] == "bf16"
     tr = binding.Trainer(layers, case["batch"], case["stages"], delays=_ints(case["delays"]) if case["delays"] else None,
                          lr=case["lr"], momentum=case["momentum"], W0=W0, b0=b0,
@@ -196,10 +210,7 @@ def prepare(case, seed):
         w = w if one_row else w.reshape(-1, l["n_in"])
         weights.append(_in_state(tr, w, (w.shape[1] + 7) // 8 * 8))
         weights.append(_in_state(tr, b0[i].reshape(1, -1), l["n_out"]))
-    shape = inputs.input_shape(layers, case["batch"])
-    x = [normal(*shape).to(torch.bfloat16 if bf16 else torch.float32) for _ in range(case["steps"])]
-    y = [torch.randint(0, inputs.n_classes(layers), (case["batch"],), generator=gen, device=dev, dtype=torch.int32)
-         for _ in range(case["steps"])]
+    x, y = _minibatches(case, layers, normal, gen)
     return dict(kind="train", trainer=tr, x=x, y=y, weights=weights, done=0)
 
 
@@ -221,6 +232,66 @@ def run(state):
     tr.flush()
     state["done"] += len(state["x"])
     return dict(weights=state["weights"], loss=tr.get_loss(state["done"] - 1))
+
+
+# ---- the same results in 64 bits --------------------------------------------------------------------------
+def exact(case, seed):
+    """What `run` returns after one pass on a new state, in float64 torch without any rounding of what is stored.  Training runs of
+    fully connected networks whose delays are given (or do not matter, with one step); None for the others: two runs
+    of a convolutional network part after a step, and a planned network's delays are the library's to say."""
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+
+    def normal(*shape):
+        return torch.randn(*shape, generator=gen, device="cuda")
+
+    if case["kind"] == "gemm":
+        s = prepare(case, seed)
+        a, w, d = s["a"][:, :s["I"]].double(), s["w"][:, :s["I"]].double(), s["d"][:, :s["O"]].double()
+        return dict(z=a @ w.T, e=d @ w, g=d.T @ a)
+    if case["kind"] == "xent":
+        s = prepare(case, seed)
+        B, C = s["logits"].shape
+        rows, labels = torch.arange(B, device="cuda"), s["labels"].long()
+        logp = torch.log_softmax(s["logits"].double(), 1)
+        delta = torch.zeros(s["delta"].shape, dtype=torch.float64, device="cuda")
+        delta[:, :C] = logp.exp() / B
+        delta[rows, labels] -= 1.0 / B
+        return dict(delta=delta, loss=-logp[rows, labels].mean().reshape(1))
+    if not case["widths"] or not (case["delays"] or case["steps"] == 1):
+        return None
+    layers = _layers(case)
+    W0, b0 = _initial(layers, normal)
+    xs, ys = _minibatches(case, layers, normal, gen)
+    delays = _ints(case["delays"]) if case["delays"] else [0] * len(layers)
+    W = [[torch.from_numpy(w).cuda().double()] for w in W0]        # per layer: every version so far
+    b = [[torch.from_numpy(v).cuda().double()] for v in b0]
+    mW, mb = [torch.zeros_like(w[0]) for w in W], [torch.zeros_like(v[0]) for v in b]
+    gelu = case["act"] == "gelu"
+    loss = 0.0
+    for n, (x, y) in enumerate(zip(xs, ys)):
+        v = [max(0, n - d) for d in delays]
+        a, z = [x.double()], []
+        for l in range(len(layers)):
+            z.append(a[l] @ W[l][v[l]].T + b[l][v[l]])
+            if l + 1 < len(layers):
+                a.append(torch.nn.functional.gelu(z[l]) if gelu else z[l].clamp_min(0.0))
+        logp = torch.log_softmax(z[-1], 1)
+        rows = torch.arange(len(y), device="cuda")
+        loss = float(-logp[rows, y.long()].mean())
+        d = logp.exp()
+        d[rows, y.long()] -= 1.0
+        d /= len(y)
+        for l in reversed(range(len(layers))):
+            mW[l] = case["momentum"] * mW[l] + d.T @ a[l]
+            mb[l] = case["momentum"] * mb[l] + d.sum(0)
+            if l > 0:
+                below = z[l - 1]
+                slope = (0.5 * (1.0 + torch.erf(below / math.sqrt(2.0))) + below * torch.exp(-0.5 * below * below) / math.sqrt(2.0 * math.pi)
+                         if gelu else (below > 0).double())
+                d = (d @ W[l][v[l]]) * slope
+            W[l].append(W[l][-1] - case["lr"] * mW[l])
+            b[l].append(b[l][-1] - case["lr"] * mb[l])
+    return dict(weights=[t for l in range(len(layers)) for t in (W[l][-1], b[l][-1].reshape(1, -1))], loss=loss)
 
 
 # ---- what a pass cannot do without ------------------------------------------------------------------------
