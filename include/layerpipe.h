@@ -127,12 +127,12 @@ int lp_workspace_size(const lp_layer* layers, int n_layers, int n_stages, const 
  * d_l + 1 bf16 versions.  W0_host[l] (fp32, [out][in]) and b0_host[l] (fp32 [out], may be
  * NULL = zeros or has_bias = 0) are copied before the call returns.  workspace_dev:
  * device, 256-byte aligned, >= lp_workspace_size bytes; zeroed by this call.
- * Uses the current CUDA device; creates its own streams and events: three streams (forward,
- * delta, G + update) per group of stages.  Streams overlap only while each owns a hardware
- * work queue, and a process has CUDA_DEVICE_MAX_CONNECTIONS of those (8 if unset, at most 32),
- * fixed when its CUDA context is created: set the variable to 32 before the first CUDA call.
- * lp_create reads the variable and folds the stages onto (value - 2) / 3 stream triples so that
- * no two of its streams share a queue (LP_STREAM_TRIPLES in the environment overrides the count).
+ * Uses the current CUDA device; creates its own streams and events: up to seven streams, four for the
+ * forward / loss / delta chains of the minibatches in flight and three for the G + update tasks (under
+ * LP_SCHED_FUSED_B seven chains).  Streams overlap only while each owns a hardware work queue; with the
+ * caller's stream these are eight, which is what a process has unless CUDA_DEVICE_MAX_CONNECTIONS was set
+ * before the driver was initialised.  lp_create reads the variable and makes fewer streams where it
+ * is smaller than eight (LP_STREAM_TRIPLES in the environment limits each kind further).
  * Kernel selection: a handle uses one kind of tensor-memory allocation -- a fully connected network
  * whose layers are mostly wide (batch, inputs and outputs all >= 1024) runs every contraction on SM
  * pairs (tcgen05 cta_group::2), every other network runs single-CTA kernels only.  LP_CONV_PAIR=1

@@ -7,10 +7,10 @@ thin ctypes layer over the C-ABI library ``liblayerpipe.so`` (see
 """
 import os as _os
 
-# The stage scheduler runs three streams per pipeline stage.  Streams only overlap while each has
-# a hardware work queue of its own, and a process gets 8 of them unless this variable says
-# otherwise when its CUDA context is created (maximum 32).  Importing the package before the
-# first CUDA call is therefore enough; a value the caller has already chosen is kept.
+# Streams only overlap while each has a hardware work queue of its own: a process gets 8 of them unless this
+# variable says otherwise when the driver is initialised (maximum 32; torch.cuda.is_available() initialises it).  One
+# handle's streams and the caller's fit the 8; the larger number serves several handles at work at the same
+# time.  A value the caller has already chosen is kept.
 _os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")
 
 __all__ = ["inputs", "binding", "build"]

@@ -9,11 +9,15 @@
 // weight version max(0, n - d_l), tasks of consecutive minibatches overlap on the device
 // exactly as far as the delays allow -- the pipelining of Section III-A -- while the
 // results stay those of the minibatch-by-minibatch recursion.
-//   LayerPipe schedule: per stage group three streams -- G+update (highest priority: it
-//   hands buffers back to later minibatches), delta, forward -- so delta_l and G_l of one
-//   layer run concurrently and delta^{l-1} is released as soon as delta_l is done.
-//   Fused-B schedule: delta_l, G_l, U_l run back to back as ONE task on the stage's
-//   backward stream and delta^{l-1} is released only when the whole task has finished.
+//   LayerPipe schedule: the chain cast -> F -> loss -> delta of minibatch n runs on chain stream
+//   n mod P (no event between its tasks), the G + update tasks of layer l on G stream l mod Q, so
+//   delta_l and G_l run concurrently and delta^{l-1} is released as soon as delta_l is done.
+//   Fused-B schedule: delta_l, G_l, U_l run back to back as ONE task on the chain stream and
+//   delta^{l-1} is released only when the whole task has finished.
+// Streams belong to minibatches in flight, not to stages: a process has 8 hardware work queues unless
+// CUDA_DEVICE_MAX_CONNECTIONS said otherwise before the driver was initialised (which
+// torch.cuda.is_available() already does), streams that share a queue serialise in enqueue order, and
+// three streams per stage need up to 30 queues.  With P + Q + the caller's stream = 8 no two share one.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -32,17 +36,14 @@ cudaError_t conv_halo_g_launch(const CUtensorMap& tmX, const CUtensorMap& tmD, c
 constexpr int kDeltaSlots = 4;
 constexpr int kLossRing = 256;
 constexpr int kLogRing = 4096;
-constexpr int kEventPool = 2048;
 constexpr int kExtraStashSlots = 1;   // activation stash = d_l + 1 (retiming) + 1 so F may run one ahead
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 static inline int pad8(int x) { return (x + 7) & ~7; }
 
-struct Ev {
-  cudaEvent_t e = nullptr;
-  cudaStream_t s = nullptr;
-  int si = -1;             // index of the stream it was recorded on (see lp_ctx::stream_index)
-  long long seq = 0;       // position in the handle's sequence of recorded events
+struct Ev {                // "task `pos` of stream `si` is done"
+  int si = -1;             // index into lp_ctx::streams, -1: nothing to wait for
+  long long pos = 0;       // tasks of a stream are numbered from 1 and complete in order
 };
 
 struct Res {                 // one buffer (or ring slot) the tracker protects
@@ -86,6 +87,7 @@ struct Layer {
   float* part_g = nullptr;
   unsigned* cnt_g = nullptr;
   Res rAfull;
+  Res rPartF, rPartD;               // split-K partial tiles and arrival counters of the forward / delta contraction
   // device memory (all inside the workspace)
   float *W = nullptr, *mW = nullptr, *b = nullptr, *mb = nullptr, *dW = nullptr, *db = nullptr, *bring = nullptr;
   __nv_bfloat16 *ring = nullptr, *X = nullptr, *Z = nullptr, *delta = nullptr;
@@ -133,7 +135,7 @@ struct lp_ctx {
   lp_config cfg{};
   int n_stages = 0;
   int stages_used = 0;
-  int n_groups = 1;             // stream triples; stage s runs on triple s % n_groups
+  int n_chain = 1, n_g = 1;     // P chain streams (minibatch n on n % P), Q G streams (layer l on l % Q; none under fused-B)
   int tmem_policy = 0;          // TMEM_*: how pair and single-CTA kernels keep out of each other's tensor memory
   int classes = 0, ld_cls = 0;
   // shared buffers
@@ -145,20 +147,23 @@ struct lp_ctx {
   int* status = nullptr;        // device status word
   std::vector<lp::Res> rZL, rLabels;
   // streams / events
-  std::vector<cudaStream_t> sF, sD, sG;
-  // Events of the hazard tracker.  A handle stored in a Res must stay valid until that buffer's next
-  // write, at most max(x_slots) minibatches later, so the pool holds more events than that many
-  // minibatches can record; joins that nothing stores (lp_flush, the two pieces of a split delta)
-  // take theirs from a small pool of their own.
-  std::vector<cudaEvent_t> pool;
-  size_t pool_next = 0;
-  std::vector<cudaEvent_t> jpool;
-  size_t jpool_next = 0;
-  long long ev_seq = 0;
-  // waited[a][b]: the latest event (by sequence number) of stream b that stream a already waits for.
-  // Events of one stream complete in order, so waiting for an earlier one again is redundant.
-  std::vector<cudaStream_t> streams;          // index 0 = the caller's stream of the current lp_step
-  std::vector<std::vector<long long>> waited;
+  // streams[0] = the caller's stream of the current lp_step, then the P chain streams, then the Q G streams
+  static constexpr int kMaxStreams = 16;
+  std::vector<cudaStream_t> streams;
+  int chain_index(long long n) const { return 1 + int(n % n_chain); }
+  int g_index(int l) const { return 1 + n_chain + l % n_g; }
+  // Recorded events of a stream, oldest overwritten first.  A wait for task `pos` takes the first
+  // record at or after it (or records one), so a record that has been overwritten only makes a later wait coarser,
+  // never wrong.  `vc` = what the stream had waited for by then (per stream, the last task known complete).
+  struct Rec { long long pos = 0; cudaEvent_t e = nullptr; long long vc[kMaxStreams] = {}; };
+  static constexpr int kRecs = 256;
+  struct StreamLog {
+    long long pos = 0;                        // tasks enqueued
+    long long n_rec = 0;                      // records made; record k lives in rec[k % kRecs]
+    std::vector<Rec> rec;
+    long long vc[kMaxStreams] = {};           // waits issued on this stream, transitively
+  };
+  std::vector<StreamLog> log;
   int stream_index(cudaStream_t s) const {
     for (size_t i = 1; i < streams.size(); ++i) if (streams[i] == s) return int(i);
     return 0;
@@ -507,43 +512,77 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
 
 // ---------------------------------------------------------------------------
 // hazard tracker
-static inline void wait_on(lp_ctx* c, cudaStream_t s, int si, const Ev& e, cudaError_t* err) {
-  if (!e.e || e.s == s) return;
-  if (e.si > 0) {                         // (index 0 is whatever stream the caller passes: never pruned)
-    long long& w = c->waited[si][e.si];
-    if (w >= e.seq) return;               // this stream already waits for that event or a later one of its stream
-    w = e.seq;
+static cudaError_t record_tail(lp_ctx* c, int si, lp_ctx::Rec** out) {
+  lp_ctx::StreamLog& g = c->log[si];
+  lp_ctx::Rec& r = g.rec[g.n_rec++ % lp_ctx::kRecs];
+  r.pos = g.pos;
+  memcpy(r.vc, g.vc, sizeof r.vc);
+  r.vc[si] = g.pos;
+  if (out) *out = &r;
+  return cudaEventRecord(r.e, c->streams[si]);
+}
+// The earliest kept record that covers task e.pos of stream e.si; records the stream's tail if there is none.
+static cudaError_t resolve(lp_ctx* c, const Ev& e, lp_ctx::Rec** out) {
+  lp_ctx::StreamLog& g = c->log[e.si];
+  const long long n = g.n_rec;
+  long long lo = std::max<long long>(0, n - lp_ctx::kRecs), hi = n;
+  while (lo < hi) {
+    const long long m = (lo + hi) / 2;
+    if (g.rec[m % lp_ctx::kRecs].pos >= e.pos) hi = m; else lo = m + 1;
   }
-  cudaError_t r = cudaStreamWaitEvent(s, e.e, 0);
-  if (r != cudaSuccess && *err == cudaSuccess) *err = r;
+  if (lo == n) return record_tail(c, e.si, out);
+  *out = &g.rec[lo % lp_ctx::kRecs];
+  return cudaSuccess;
+}
+static inline void wait_on(lp_ctx* c, int si, const Ev& e, cudaError_t* err) {
+  if (e.si < 0 || e.si == si) return;
+  long long* vc = c->log[si].vc;
+  if (vc[e.si] >= e.pos) return;          // this stream already waits, directly or through another one, for that task
+  lp_ctx::Rec* r = nullptr;
+  cudaError_t q = resolve(c, e, &r);
+  if (q == cudaSuccess) q = cudaStreamWaitEvent(c->streams[si], r->e, 0);
+  if (q != cudaSuccess) { if (*err == cudaSuccess) *err = q; return; }
+  for (size_t k = 0; k < c->streams.size(); ++k) vc[k] = std::max(vc[k], r->vc[k]);
 }
 
-static cudaError_t task_begin(lp_ctx* c, cudaStream_t s, std::initializer_list<Res*> reads,
-                              std::initializer_list<Res*> writes) {
+static cudaError_t task_begin(lp_ctx* c, int si, std::initializer_list<Res*> reads, std::initializer_list<Res*> writes) {
   cudaError_t err = cudaSuccess;
-  const int si = c->stream_index(s);
-  for (Res* r : reads) if (r) wait_on(c, s, si, r->last_write, &err);
   for (Res* w : writes) {
     if (!w) continue;
-    wait_on(c, s, si, w->last_write, &err);
-    for (const Ev& e : w->readers) wait_on(c, s, si, e, &err);
+    for (const Ev& e : w->readers) wait_on(c, si, e, &err);
+    wait_on(c, si, w->last_write, &err);
   }
+  for (Res* r : reads) if (r) wait_on(c, si, r->last_write, &err);
   return err;
 }
 
-static cudaError_t task_end(lp_ctx* c, cudaStream_t s, std::initializer_list<Res*> reads,
-                            std::initializer_list<Res*> writes, Ev* out_ev) {
-  cudaEvent_t e = c->pool[c->pool_next++ % c->pool.size()];
-  cudaError_t r = cudaEventRecord(e, s);
-  Ev ev{e, s, c->stream_index(s), ++c->ev_seq};
-  for (Res* x : reads) if (x) x->readers.push_back(ev);
+// record: another stream waits for this task before any later task of its own stream is recorded.  Tasks whose
+// output is only read further down their own chain (most forward tasks) are not: the next record covers them.
+static cudaError_t task_end(lp_ctx* c, int si, std::initializer_list<Res*> reads, std::initializer_list<Res*> writes,
+                            Ev* out_ev, bool record = true) {
+  lp_ctx::StreamLog& g = c->log[si];
+  const Ev ev{si, ++g.pos};
+  for (Res* x : reads) {
+    if (!x) continue;
+    size_t keep = 0;                          // readers that this task already waits for need no wait of their own
+    for (const Ev& r : x->readers) if (r.si != si && g.vc[r.si] < r.pos) x->readers[keep++] = r;
+    x->readers.resize(keep);
+    x->readers.push_back(ev);
+  }
   for (Res* w : writes) {
     if (!w) continue;
     w->last_write = ev;
     w->readers.clear();
   }
   if (out_ev) *out_ev = ev;
-  return r;
+  return record ? record_tail(c, si, nullptr) : cudaSuccess;
+}
+// Host wait for a task (none: returns at once).
+static cudaError_t host_wait(lp_ctx* c, const Ev& e) {
+  if (e.si < 0) return cudaSuccess;
+  lp_ctx::Rec* r = nullptr;
+  cudaError_t q = resolve(c, e, &r);
+  return q == cudaSuccess ? cudaEventSynchronize(r->e) : q;
 }
 
 // ---------------------------------------------------------------------------
@@ -668,16 +707,10 @@ static int build_tensor_maps(lp_ctx* c) {
 
 static void destroy_ctx(lp_ctx* c) {
   if (!c) return;
-  auto kill = [](std::vector<cudaStream_t>& v) {
-    for (cudaStream_t s : v) if (s) cudaStreamDestroy(s);
-    v.clear();
-  };
   cudaDeviceSynchronize();
-  kill(c->sF);
-  kill(c->sD);
-  kill(c->sG);
-  for (cudaEvent_t e : c->pool) if (e) cudaEventDestroy(e);
-  for (cudaEvent_t e : c->jpool) if (e) cudaEventDestroy(e);
+  for (size_t i = 1; i < c->streams.size(); ++i) if (c->streams[i]) cudaStreamDestroy(c->streams[i]);
+  for (auto& g : c->log)
+    for (auto& r : g.rec) if (r.e) cudaEventDestroy(r.e);
   for (cudaEvent_t e : c->tpool) if (e) cudaEventDestroy(e);
   if (c->trace_done) { gemm_set_tmem_table(nullptr); cudaFreeHost(c->trace_done); }
   if (c->peek_host) cudaFreeHost(c->peek_host);
@@ -1049,60 +1082,38 @@ extern "C" int lp_create(lp_handle* out, const lp_layer* layers, int n_layers, i
   LP_CUDA(nullptr, gemm_configure());
   int least = 0, greatest = 0;
   LP_CUDA(nullptr, cudaDeviceGetStreamPriorityRange(&least, &greatest));
-  // Priorities: G + update highest, delta next, forward lowest.  The paper puts delta first because
-  // it carries the critical loop between processors; on one GPU the step time is set by how full
-  // the SMs are kept, and the G + update task is the one that hands buffers back (the delta slot,
-  // the ring slot of the next version), so starving it stalls later minibatches.  Measured per step
-  // with every stream on its own hardware queue and four delta slots, (delta > forward > G) against
-  // this order: 8 x 4096 MLP 589 / 588 us, small VGG 478 / 384 us, VGG-16 9.43 / 9.20 ms, 16 x 8192
-  // MLP 11.11 / 10.89 ms; all priorities equal lies in between.
-  // A network whose kernels are too small to fill the GPU (the 784-256-256-256-10 MLP at batch
-  // 32: 0.110 ms per step with delta first, 0.130 ms with G first) is bound by the latency of the
-  // delta chain instead, and keeps the paper's order.
-  long long step_macs = 0;
-  for (int l = 0; l < n_layers; ++l) {
-    long long m = 0;
-    if (layer_macs(layers[l], cfg->batch, &m) == LP_OK) step_macs += 3 * m;
-  }
-  const bool g_first = step_macs >= 1000000000ll;
-  const int pMid = std::min(least, greatest + 1);
-  const int pG = g_first ? greatest : least, pD = g_first ? pMid : greatest, pF = g_first ? least : pMid;
-  // Streams only run concurrently while each has a hardware work queue of its own; the process
-  // has CUDA_DEVICE_MAX_CONNECTIONS of them (8 unless the variable was set, up to 32, before the
-  // CUDA context was created).  Streams that share a queue serialise in enqueue order, which
-  // stalls tasks behind unrelated event waits (measured on the 8 x 4096 workload: 24 streams on 8
-  // queues 838 us per step, on 32 queues 591 us).  So the stages share as many stream triples as
-  // the queues allow, two queues being left to the caller's stream and the default stream.
+  // P chain streams and Q G streams: together with the caller's stream at most eight, the number of hardware
+  // work queues that a process has by default (fewer if CUDA_DEVICE_MAX_CONNECTIONS says so).  Three streams per
+  // stage on the eight queues that a process gets when the driver was initialised before the variable was set,
+  // against four chains and three G streams, microseconds: 8 steps of the 8 x 4096 MLP 6690 / 4780, 16 of the small
+  // VGG 8190 / 5160 (fused-B at half the batch 8730 / 3660), 4 of VGG-16 35 800 / 32 400, 8 of the sample network
+  // 5550 / 4790.  P / Q = 2 / 5 .. 6 / 1 were swept: fewer chains slow the 8 x 4096 MLP (5480), fewer G streams the small VGG (5340, 7920).
+  // The chains come first, as the paper puts delta first (it carries the critical loop): against G first
+  // 4780 / 5010 for the 8 x 4096 MLP and 3660 / 4120 for fused-B, the rest alike.
   int conn = 8;
-  if (const char* e = getenv("CUDA_DEVICE_MAX_CONNECTIONS")) conn = std::max(1, std::min(32, atoi(e)));
-  c->n_groups = std::max(1, std::min(used, (conn - 2) / 3));
-  // A network whose step is bound by the host's enqueue time gains nothing from many stream
-  // triples: every cross-stream edge costs an event wait on the host, same-stream order is free.
-  // Measured on the 784-256-256-256-10 MLP at batch 32 (samples/s, 1 / 2 / 4 triples): 593 k / 645 k / 582 k.
-  if (!g_first) c->n_groups = std::min(c->n_groups, 2);
-  if (const char* e = getenv("LP_STREAM_TRIPLES")) c->n_groups = std::max(1, std::min(c->n_groups, atoi(e)));   // experiments: fewer triples
-  c->sF.assign(c->n_groups, nullptr);
-  c->sD.assign(c->n_groups, nullptr);
-  c->sG.assign(c->n_groups, nullptr);
-  for (int s = 0; s < c->n_groups; ++s) {
-    LP_CUDA(nullptr, cudaStreamCreateWithPriority(&c->sF[s], cudaStreamNonBlocking, pF));
-    LP_CUDA(nullptr, cudaStreamCreateWithPriority(&c->sD[s], cudaStreamNonBlocking, pD));
-    LP_CUDA(nullptr, cudaStreamCreateWithPriority(&c->sG[s], cudaStreamNonBlocking, pG));
+  if (const char* e = getenv("CUDA_DEVICE_MAX_CONNECTIONS")) conn = std::max(1, std::min(8, atoi(e)));
+  const bool fusedB = cfg->schedule == LP_SCHED_FUSED_B;
+  c->n_chain = fusedB ? std::max(1, conn - 1) : std::max(1, conn / 2);
+  c->n_g = fusedB ? 0 : std::max(1, conn - 1 - c->n_chain);
+  if (const char* e = getenv("LP_STREAM_TRIPLES")) {      // experiments: fewer streams
+    const int most = std::max(1, atoi(e));
+    c->n_chain = std::min(c->n_chain, most);
+    c->n_g = std::min(c->n_g, most);
   }
+  c->streams.assign(size_t(1 + c->n_chain + c->n_g), nullptr);
+  for (int i = 1; i <= c->n_chain + c->n_g; ++i)
+    LP_CUDA(nullptr, cudaStreamCreateWithPriority(&c->streams[i], cudaStreamNonBlocking, i <= c->n_chain ? greatest : least));
   {
     int max_delay = 0;
     for (int d : dl) max_delay = std::max(max_delay, d);
-    const size_t per_step = size_t(5) * n_layers + 8;                  // tasks of one minibatch, with room to spare
-    const size_t want = std::max<size_t>(kEventPool, (size_t(max_delay) + 4) * per_step);
-    if (want > (size_t(1) << 20)) return fail(nullptr, LP_ERR_UNSUPPORTED, "delays x layers need more than 2^20 scheduler events");
-    c->pool.assign(want, nullptr);
+    if ((size_t(max_delay) + 4) * (size_t(5) * n_layers + 8) > (size_t(1) << 20))      // tasks that can be in flight
+      return fail(nullptr, LP_ERR_UNSUPPORTED, "delays x layers need more than 2^20 scheduler events");
   }
-  for (auto& e : c->pool) LP_CUDA(nullptr, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  c->jpool.assign(64, nullptr);
-  for (auto& e : c->jpool) LP_CUDA(nullptr, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  c->streams.assign(1, nullptr);
-  for (int s = 0; s < c->n_groups; ++s) { c->streams.push_back(c->sF[s]); c->streams.push_back(c->sD[s]); c->streams.push_back(c->sG[s]); }
-  c->waited.assign(c->streams.size(), std::vector<long long>(c->streams.size(), 0));
+  c->log.resize(c->streams.size());
+  for (auto& g : c->log) {
+    g.rec.resize(lp_ctx::kRecs);
+    for (auto& r : g.rec) LP_CUDA(nullptr, cudaEventCreateWithFlags(&r.e, cudaEventDisableTiming));
+  }
   if (c->cfg.flags & LP_TRACE_TASKS) {
     const size_t ns = c->streams.size();
     LP_CUDA(nullptr, cudaHostAlloc(reinterpret_cast<void**>(&c->trace_done), 2 * ns * sizeof(unsigned), cudaHostAllocMapped));
@@ -1272,10 +1283,19 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
   const bool fusedB = (c->cfg.schedule == LP_SCHED_FUSED_B);
   const bool serial = (c->cfg.flags & LP_SERIAL_TASKS) != 0;   // every task on the caller's stream
   const int ds = int(n % kDeltaSlots);
-  if (c->streams[0] != user) {            // what the previous caller's stream waited for says nothing about this one
+  if (c->streams[0] != user) {
+    // Another caller's stream takes over: it continues behind the last task of the old one (whose record is kept,
+    // the stream itself may be gone), and knows of other streams what had been waited for by then.
+    lp_ctx::StreamLog& g = c->log[0];
     c->streams[0] = user;
-    std::fill(c->waited[0].begin(), c->waited[0].end(), 0ll);
+    if (g.n_rec > 0) {
+      const lp_ctx::Rec& r = g.rec[(g.n_rec - 1) % lp_ctx::kRecs];
+      LP_CUDA(c, cudaStreamWaitEvent(user, r.e, 0));
+      memcpy(g.vc, r.vc, sizeof g.vc);
+    }
   }
+  const int sc = serial ? 0 : c->chain_index(n);               // this minibatch's chain stream
+  cudaStream_t chain = c->streams[sc];
 
   // version bookkeeping (the integers the parity tests compare bit-exactly)
   std::vector<int> slot(nL);
@@ -1291,7 +1311,7 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
     Layer& y0 = c->L[0];
     Res* rx = &y0.rX[n % y0.x_slots];
     Res* rl = &c->rLabels[ds];
-    LP_CUDA(c, task_begin(c, user, {}, {rx, rl}));
+    LP_CUDA(c, task_begin(c, 0, {}, {rx, rl}));
     ++c->launches;
     TimedScope ts(c, LP_TASK_CAST, user);
     if (y0.patch && y0.gen)
@@ -1306,12 +1326,11 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
       LP_CUDA(c, launch_cast_stash(batch_dev, c->cfg.input_dtype == LP_BF16, labels_dev,
                                    y0.X + size_t(n % y0.x_slots) * y0.x_elems, c->labels + size_t(ds) * B, y0.in_rows, B,
                                    y0.n_in, y0.ld_in, user));
-    LP_CUDA(c, task_end(c, user, {}, {rx, rl}, nullptr));
+    LP_CUDA(c, task_end(c, 0, {}, {rx, rl}, nullptr));
   }
   // ---- forward ---------------------------------------------------------------
   for (int l = 0; l < nL; ++l) {
     Layer& y = c->L[l];
-    cudaStream_t st = (serial ? user : c->sF[y.stage % c->n_groups]);
     Res* rin = &y.rX[xf_slot(y, n)];
     Res* rw = &y.rRing[slot[l]];
     const int xo = (l == nL - 1) ? 0 : xf_slot(c->L[l + 1], n);
@@ -1319,23 +1338,24 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
     Res* rz = y.Z ? &y.rZ[xo] : nullptr;
     Res* rpool = y.pool ? &y.rPidx[xo] : nullptr;
     Res* rfull = y.pool ? &y.rAfull : nullptr;
-    LP_CUDA(c, task_begin(c, st, {rin, rw}, {rout, rz, rpool, rfull}));
-    LP_CUDA(c, launch_forward(c, l, n, slot[l], st));
-    if (y.pool) LP_CUDA(c, launch_pool(c, l, n, st));
-    LP_CUDA(c, task_end(c, st, {rin, rw}, {rout, rz, rpool, rfull}, nullptr));
+    Res* rpart = y.split_f > 1 ? &y.rPartF : nullptr;
+    LP_CUDA(c, task_begin(c, sc, {rin, rw}, {rout, rz, rpool, rfull, rpart}));
+    LP_CUDA(c, launch_forward(c, l, n, slot[l], chain));
+    if (y.pool) LP_CUDA(c, launch_pool(c, l, n, chain));
+    // (scratch that the next minibatch's task of this layer reuses: it waits for this very task)
+    LP_CUDA(c, task_end(c, sc, {rin, rw}, {rout, rz, rpool, rfull, rpart}, nullptr, rfull || rpart));
   }
   // ---- loss and delta^L --------------------------------------------------------
   {
     Layer& yl = c->L[nL - 1];
-    cudaStream_t st = (serial ? user : c->sD[yl.stage % c->n_groups]);
     Res* rd = &yl.rDelta[ds];
-    LP_CUDA(c, task_begin(c, st, {&c->rZL[ds], &c->rLabels[ds]}, {rd}));
+    LP_CUDA(c, task_begin(c, sc, {&c->rZL[ds], &c->rLabels[ds]}, {rd}));
     ++c->launches;
-    TimedScope ts(c, LP_TASK_LOSS, st);
+    TimedScope ts(c, LP_TASK_LOSS, chain);
     LP_CUDA(c, launch_softmax_xent(c->zL + size_t(ds) * B * c->ld_cls, c->ld_cls, c->labels + size_t(ds) * B,
                                    yl.delta + size_t(ds) * yl.delta_elems, yl.ld_out, c->row_loss + size_t(ds) * B,
-                                   c->ticket + ds, c->loss + (n % kLossRing), B, c->classes, c->status, st));
-    LP_CUDA(c, task_end(c, st, {&c->rZL[ds], &c->rLabels[ds]}, {rd}, &c->loss_ev[n % kLossRing]));
+                                   c->ticket + ds, c->loss + (n % kLossRing), B, c->classes, c->status, chain));
+    LP_CUDA(c, task_end(c, sc, {&c->rZL[ds], &c->rLabels[ds]}, {rd}, &c->loss_ev[n % kLossRing]));
   }
   // ---- backward: delta and G are independent tasks; update follows G -----------
   for (int l = nL - 1; l >= 0; --l) {
@@ -1350,7 +1370,6 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
       for (int k = lo + 1; k <= l; ++k) {
         if (!c->L[k].recomp) continue;
         Layer& src = c->L[k - 1];
-        cudaStream_t st = (serial ? user : c->sD[y.stage % c->n_groups]);
         const int xo = xb_slot(c->L[k], n);
         Res* rin = &src.rX[xb_slot(src, n)];
         Res* rwv = &src.rRing[slot[k - 1]];
@@ -1358,10 +1377,11 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
         Res* rz = src.Z ? &src.rZ[xo] : nullptr;
         Res* rpool = src.pool ? &src.rPidx[xo] : nullptr;
         Res* rfull = src.pool ? &src.rAfull : nullptr;
-        LP_CUDA(c, task_begin(c, st, {rin, rwv}, {rout, rz, rpool, rfull}));
-        LP_CUDA(c, launch_forward(c, k - 1, n, slot[k - 1], st, true));
-        if (src.pool) LP_CUDA(c, launch_pool(c, k - 1, n, st, true));
-        LP_CUDA(c, task_end(c, st, {rin, rwv}, {rout, rz, rpool, rfull}, nullptr));
+        Res* rpart = src.split_f > 1 ? &src.rPartF : nullptr;
+        LP_CUDA(c, task_begin(c, sc, {rin, rwv}, {rout, rz, rpool, rfull, rpart}));
+        LP_CUDA(c, launch_forward(c, k - 1, n, slot[k - 1], chain, true));
+        if (src.pool) LP_CUDA(c, launch_pool(c, k - 1, n, chain, true));
+        LP_CUDA(c, task_end(c, sc, {rin, rwv}, {rout, rz, rpool, rfull, rpart}, nullptr));
       }
     }
     Res* rdl = &y.rDelta[ds];
@@ -1377,9 +1397,10 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
       raux = (pv.d.act == LP_ACT_GELU) ? &pv.rZ[xb_slot(y, n)] : rx;
       if (pv.pool) ridx = &pv.rPidx[xb_slot(y, n)];
     }
+    Res* rpart = (l > 0 && y.split_d > 1) ? &y.rPartD : nullptr;
     if (fusedB) {
-      cudaStream_t st = (serial ? user : c->sD[y.stage % c->n_groups]);
-      LP_CUDA(c, task_begin(c, st, {rdl, rw, rx, raux, ridx}, {rdprev, &y.rDW, rnew}));
+      cudaStream_t st = chain;
+      LP_CUDA(c, task_begin(c, sc, {rdl, rw, rx, raux, ridx}, {rdprev, &y.rDW, rnew, rpart}));
       if (l > 0 && y.split_col > 0) {      // (one serial task: the pieces follow one another)
         LP_CUDA(c, launch_delta(c, l, n, slot[l], st, 0));
         LP_CUDA(c, launch_delta(c, l, n, slot[l], st, 1));
@@ -1388,50 +1409,49 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
       }
       LP_CUDA(c, launch_G(c, l, n, st));
       LP_CUDA(c, launch_update(c, l, n, st));
-      LP_CUDA(c, task_end(c, st, {rdl, rw, rx, raux, ridx}, {rdprev, &y.rDW, rnew}, &y.last_update));
+      LP_CUDA(c, task_end(c, sc, {rdl, rw, rx, raux, ridx}, {rdprev, &y.rDW, rnew, rpart}, &y.last_update));
     } else {
       if (l > 0 && y.split_col > 0 && !serial) {
-        // delta'' on the streams of the stage that holds layer l+1, delta' on this layer's own:
-        // two kernels over disjoint column ranges of delta^{l-1}, concurrent; the buffer counts as
-        // written when both are done (the second stream joins the first before the event that
-        // later tasks wait on)
-        cudaStream_t s0 = c->sD[y.piece_stage[0] % c->n_groups], s1 = c->sD[y.piece_stage[1] % c->n_groups];
+        // delta'' on a stream picked by the stage that borrowed it, delta' on the minibatch's chain: two kernels over
+        // disjoint column ranges of delta^{l-1}, concurrent; the buffer counts as written when both are
+        // done (the chain joins the other stream before the event that later tasks wait on)
+        const int s0 = c->g_index(y.piece_stage[0]);
         LP_CUDA(c, task_begin(c, s0, {rdl, rw, raux, ridx}, {rdprev}));
-        LP_CUDA(c, task_begin(c, s1, {rdl, rw, raux, ridx}, {rdprev}));
-        LP_CUDA(c, launch_delta(c, l, n, slot[l], s0, 0));
-        LP_CUDA(c, launch_delta(c, l, n, slot[l], s1, 1));
-        if (s0 != s1) {
-          cudaEvent_t e = c->jpool[c->jpool_next++ % c->jpool.size()];
-          LP_CUDA(c, cudaEventRecord(e, s0));
-          LP_CUDA(c, cudaStreamWaitEvent(s1, e, 0));
-        }
-        LP_CUDA(c, task_end(c, s1, {rdl, rw, raux, ridx}, {rdprev}, nullptr));
+        LP_CUDA(c, task_begin(c, sc, {rdl, rw, raux, ridx}, {rdprev}));
+        LP_CUDA(c, launch_delta(c, l, n, slot[l], c->streams[s0], 0));
+        LP_CUDA(c, launch_delta(c, l, n, slot[l], chain, 1));
+        Ev first;
+        LP_CUDA(c, task_end(c, s0, {}, {}, &first));
+        cudaError_t joined = cudaSuccess;
+        wait_on(c, sc, first, &joined);
+        LP_CUDA(c, joined);
+        LP_CUDA(c, task_end(c, sc, {rdl, rw, raux, ridx}, {rdprev}, nullptr));
       } else if (l > 0) {
-        cudaStream_t st = (serial ? user : c->sD[y.stage % c->n_groups]);
-        LP_CUDA(c, task_begin(c, st, {rdl, rw, raux, ridx}, {rdprev}));
+        LP_CUDA(c, task_begin(c, sc, {rdl, rw, raux, ridx}, {rdprev, rpart}));
         if (y.split_col > 0) {
-          LP_CUDA(c, launch_delta(c, l, n, slot[l], st, 0));
-          LP_CUDA(c, launch_delta(c, l, n, slot[l], st, 1));
+          LP_CUDA(c, launch_delta(c, l, n, slot[l], chain, 0));
+          LP_CUDA(c, launch_delta(c, l, n, slot[l], chain, 1));
         } else {
-          LP_CUDA(c, launch_delta(c, l, n, slot[l], st));
+          LP_CUDA(c, launch_delta(c, l, n, slot[l], chain));
         }
-        LP_CUDA(c, task_end(c, st, {rdl, rw, raux, ridx}, {rdprev}, nullptr));
+        LP_CUDA(c, task_end(c, sc, {rdl, rw, raux, ridx}, {rdprev, rpart}, nullptr));
       }
-      cudaStream_t sg = (serial ? user : c->sG[y.stage % c->n_groups]);
+      const int si = serial ? 0 : c->g_index(l);
+      cudaStream_t sg = c->streams[si];
       if (fused_update(c)) {
         // G + update of W in one kernel, then the bias update: one task that writes the ring
         // slot of version n+1 (the slot delta_l(n) reads, so the tracker orders it after it)
-        LP_CUDA(c, task_begin(c, sg, {rdl, rx}, {&y.rDW, rnew}));
+        LP_CUDA(c, task_begin(c, si, {rdl, rx}, {&y.rDW, rnew}));
         LP_CUDA(c, launch_G(c, l, n, sg));
         LP_CUDA(c, launch_update(c, l, n, sg));
-        LP_CUDA(c, task_end(c, sg, {rdl, rx}, {&y.rDW, rnew}, &y.last_update));
+        LP_CUDA(c, task_end(c, si, {rdl, rx}, {&y.rDW, rnew}, &y.last_update));
       } else {
-        LP_CUDA(c, task_begin(c, sg, {rdl, rx}, {&y.rDW}));
+        LP_CUDA(c, task_begin(c, si, {rdl, rx}, {&y.rDW}));
         LP_CUDA(c, launch_G(c, l, n, sg));
-        LP_CUDA(c, task_end(c, sg, {rdl, rx}, {&y.rDW}, nullptr));
-        LP_CUDA(c, task_begin(c, sg, {&y.rDW, rdl}, {rnew}));
+        LP_CUDA(c, task_end(c, si, {rdl, rx}, {&y.rDW}, nullptr));
+        LP_CUDA(c, task_begin(c, si, {&y.rDW, rdl}, {rnew}));
         LP_CUDA(c, launch_update(c, l, n, sg));
-        LP_CUDA(c, task_end(c, sg, {&y.rDW, rdl}, {rnew}, &y.last_update));
+        LP_CUDA(c, task_end(c, si, {&y.rDW, rdl}, {rnew}, &y.last_update));
       }
     }
   }
@@ -1443,19 +1463,18 @@ extern "C" int lp_flush(lp_handle h, void* stream) {
   if (!h) return LP_ERR_INVALID_ARG;
   if (h->latched) return h->latched;
   cudaStream_t user = static_cast<cudaStream_t>(stream);
-  auto join = [&](std::vector<cudaStream_t>& v) -> cudaError_t {
-    for (cudaStream_t s : v) {
-      cudaEvent_t e = h->jpool[h->jpool_next++ % h->jpool.size()];
-      cudaError_t r = cudaEventRecord(e, s);
-      if (r != cudaSuccess) return r;
-      r = cudaStreamWaitEvent(user, e, 0);
-      if (r != cudaSuccess) return r;
+  cudaError_t err = cudaSuccess;
+  if (user == h->streams[0]) {
+    for (size_t si = 1; si < h->streams.size(); ++si) wait_on(h, 0, Ev{int(si), h->log[si].pos}, &err);
+  } else {
+    for (size_t si = 0; si < h->streams.size(); ++si) {
+      if (h->log[si].pos == 0) continue;
+      lp_ctx::Rec* r = nullptr;
+      LP_CUDA(h, resolve(h, Ev{int(si), h->log[si].pos}, &r));
+      LP_CUDA(h, cudaStreamWaitEvent(user, r->e, 0));
     }
-    return cudaSuccess;
-  };
-  LP_CUDA(h, join(h->sF));
-  LP_CUDA(h, join(h->sD));
-  LP_CUDA(h, join(h->sG));
+  }
+  LP_CUDA(h, err);
   return LP_OK;
 }
 
@@ -1463,7 +1482,7 @@ extern "C" int lp_get_weights(lp_handle h, int layer, float* W_out, float* b_out
   if (!h) return LP_ERR_INVALID_ARG;
   if (layer < 0 || layer >= int(h->L.size())) return fail(h, LP_ERR_INVALID_ARG, "layer index out of range");
   Layer& y = h->L[layer];
-  if (y.last_update.e) LP_CUDA(h, cudaEventSynchronize(y.last_update.e));
+  LP_CUDA(h, host_wait(h, y.last_update));
   if (W_out)
     LP_CUDA(h, cudaMemcpy2D(W_out, size_t(y.n_in) * 4, y.W, size_t(y.ld_in) * 4, size_t(y.n_in) * 4,
                             size_t(y.n_out) * y.taps, cudaMemcpyDeviceToHost));
@@ -1478,7 +1497,7 @@ extern "C" int lp_get_grads(lp_handle h, int layer, long long step, float* dW_ou
   if (step != h->n_steps - 1 || step < 0) return fail(h, LP_ERR_NOT_READY, "only the latest step's gradients are held");
   Layer& y = h->L[layer];
   if (dW_out && !y.dW) return fail(h, LP_ERR_NOT_READY, "G is not kept: create the handle with LP_CAPTURE_GRADS");
-  if (y.last_update.e) LP_CUDA(h, cudaEventSynchronize(y.last_update.e));
+  LP_CUDA(h, host_wait(h, y.last_update));
   if (dW_out)
     LP_CUDA(h, cudaMemcpy2D(dW_out, size_t(y.n_in) * 4, y.dW, size_t(y.ld_in) * 4, size_t(y.n_in) * 4,
                             size_t(y.n_out) * y.taps, cudaMemcpyDeviceToHost));
@@ -1661,7 +1680,7 @@ extern "C" int lp_debug_run_task(lp_handle h, int task, int layer, long long ste
   if (step < 0) return fail(h, LP_ERR_INVALID_ARG, "negative step");
   if (task != LP_TASK_LOSS && (layer < 0 || layer >= nL)) return fail(h, LP_ERR_INVALID_ARG, "layer index out of range");
   LP_CUDA(h, cudaDeviceSynchronize());
-  cudaStream_t st = h->sF[0];
+  cudaStream_t st = h->streams[1];
   const int B = h->cfg.batch;
   const int ds = int(step % kDeltaSlots);
   int slot = 0;
@@ -1727,8 +1746,7 @@ extern "C" int lp_get_loss(lp_handle h, long long step, float* loss) {
   if (!h || !loss) return LP_ERR_INVALID_ARG;
   if (step < 0 || step >= h->n_steps || step < h->n_steps - kLossRing)
     return fail(h, LP_ERR_NOT_READY, "step outside the loss ring");
-  const Ev& e = h->loss_ev[step % kLossRing];
-  if (e.e) LP_CUDA(h, cudaEventSynchronize(e.e));
+  LP_CUDA(h, host_wait(h, h->loss_ev[step % kLossRing]));
   LP_CUDA(h, cudaMemcpy(loss, h->loss + (step % kLossRing), 4, cudaMemcpyDeviceToHost));
   return LP_OK;
 }
@@ -1742,10 +1760,9 @@ extern "C" int lp_task_progress(lp_handle h, char* text, int capacity) {
   for (size_t si = 0; si < h->streams.size(); ++si) {
     const unsigned done = *reinterpret_cast<volatile unsigned*>(h->trace_done + si), enq = h->trace_enq[si];
     if (done == enq) continue;
-    const char* role = si == 0 ? "caller" : ((si - 1) % 3 == 0 ? "F" : (si - 1) % 3 == 1 ? "delta" : "G");
+    const char* role = si == 0 ? "caller" : (int(si) <= h->n_chain ? "chain" : "G");
     const unsigned started = *reinterpret_cast<volatile unsigned*>(h->trace_done + h->streams.size() + si);
-    snprintf(line, sizeof line, "stream %d (%s, triple %d): %u of %u tasks done, %s; unfinished:", int(si), role,
-             si == 0 ? -1 : int((si - 1) / 3), done, enq, started > done ? "the next one has STARTED" : "the next one has not started");
+    snprintf(line, sizeof line, "stream %d (%s): %u of %u tasks done, %s; unfinished:", int(si), role, done, enq, started > done ? "the next one has STARTED" : "the next one has not started");
     out += line;
     for (unsigned q = done + 1; q <= enq && q <= done + 3; ++q) {
       if (enq - q >= unsigned(lp_ctx::kTraceRing)) continue;

@@ -266,3 +266,37 @@ def test_inflight_full_size_bitwise_against_synchronised_run(workload, steps, mo
             assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1]) and a[2] == b[2] == steps, (sched, mode, split, l)
         got.close()
     ref.close()
+
+
+@pytest.mark.parametrize("schedule", ["layerpipe", "fused_b"])
+def test_inflight_steps_and_flush_on_changing_caller_streams(schedule):
+    """Consecutive steps on different caller's streams (each minibatch is copied on the stream it is stepped on) and a
+    flush on yet another one: the caller's streams count as one sequence, so the bits are those of the run on one."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    from paper_2108_06629_b200 import inputs as I
+    layers, B, steps = I.mlp([264, 192, 320, 136, 40], "gelu"), 56, 14
+    sched = lpb.LP_SCHED_FUSED_B if schedule == "fused_b" else lpb.LP_SCHED_LAYERPIPE
+    W0, b0 = I.initial_weights(layers, 0)
+    data = [I.minibatch(layers, B, n) for n in range(steps)]
+
+    def go(n_streams):
+        tr = lpb.Trainer(layers, B, 4, delays=[3, 2, 1, 0], lr=0.02, momentum=0.9, schedule=sched, W0=W0, b0=b0)
+        streams = [torch.cuda.Stream() for _ in range(n_streams)]
+        for n, (x, y) in enumerate(data):
+            with torch.cuda.stream(streams[n % n_streams]):
+                xd, yd = torch.from_numpy(x).cuda(non_blocking=True), torch.from_numpy(y).cuda(non_blocking=True)
+                tr.step(xd, yd)
+                xd.record_stream(streams[n % n_streams])
+        last = torch.cuda.Stream()
+        with torch.cuda.stream(last):
+            tr.flush()
+        last.synchronize()
+        out = [tr.get_loss(n) for n in range(steps)], [tr.get_weights(l)[0] for l in range(len(layers))]
+        assert tr.device_status() == (0, 0)
+        tr.close()
+        return out
+
+    (loss1, W1), (loss3, W3) = go(1), go(3)
+    assert loss1 == loss3
+    assert all(np.array_equal(a, b) for a, b in zip(W1, W3))
