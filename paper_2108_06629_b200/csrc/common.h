@@ -87,9 +87,9 @@ cudaError_t launch_cast_patch_general(const void* batch, int input_is_bf16, cons
 cudaError_t gemm_set_tmem_table(int* table);
 // one thread writes `value` to *flag (mapped host memory): the progress mark after a task
 cudaError_t launch_trace_mark(unsigned* flag, unsigned value, cudaStream_t stream);
-cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __nv_bfloat16* delta, int ldd,
-                                float* row_loss, unsigned* ticket, float* loss_out, int B, int C,
-                                int* status, cudaStream_t stream);
+// ticket: count of finished blocks, zero between launches
+cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __nv_bfloat16* delta, int ldd, float* row_loss,
+                                unsigned* ticket, float* loss_out, int B, int C, int* status, cudaStream_t stream);
 // Value of a device status word that does not come from a bounded wait (those are 1..23).
 constexpr int LP_STATUS_BAD_LABEL = 64;   // a label outside [0, classes) reached the loss kernel
 struct UpdateArgs {

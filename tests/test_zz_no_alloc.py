@@ -101,3 +101,33 @@ def test_static_scratch_loss_never_uses_a_bad_label_as_an_address():
     assert lpb.lp_softmax_xent_static(lg, lb, delta, loss, classes) == lpb.LP_OK
     torch.cuda.synchronize()
     assert abs(float(loss.item()) - np.log(8.0)) < 1e-5
+
+
+@pytest.mark.parametrize("B, C, ld", [(1, 1, 1), (3, 2, 2), (9, 1000, 1000), (7, 1001, 1003), (8, 1024, 1024), (5, 1025, 1026),
+                                      (4, 8192, 8192), (3, 8195, 8195), (300, 33, 40)])
+def test_static_loss_at_the_edges_of_its_row_forms(B, C, ld):
+    """A warp or a block per row, classes beyond what the registers hold, odd pitches (one class per access), a masked
+    class (-inf logit): loss and delta against float64.  One bf16 rounding of delta; fp32 sums over C classes."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    g = torch.Generator().manual_seed(B * 10007 + C)
+    z = torch.full((B, ld), 1e30)
+    z[:, :C] = 3.0 * torch.randn(B, C, generator=g)
+    y = torch.randint(0, C, (B,), generator=g, dtype=torch.int32)
+    if C > 2:
+        z[0, (int(y[0]) + 1) % C] = float("-inf")
+    ldd = (C + 7) // 8 * 8 + (ld % 2)
+    delta = torch.full((B, ldd), 7.0, dtype=torch.bfloat16, device="cuda")
+    loss = torch.zeros(1, device="cuda")
+    for _ in range(2):                            # (the second call meets the counter as the first one left it)
+        assert lpb.lp_softmax_xent_static(z.cuda(), y.cuda(), delta, loss, C) == lpb.LP_OK
+    logp = torch.log_softmax(z[:, :C].double(), 1)
+    rows = torch.arange(B)
+    want = logp.exp()
+    want[rows, y.long()] -= 1.0
+    want /= B
+    ref_loss = float(-logp[rows, y.long()].mean())
+    got = delta.double().cpu()
+    assert torch.all((got[:, :C] - want).abs() <= 2.0 ** -8 * want.abs() + 1e-6 / B)
+    assert torch.all(got[:, C:(C + 7) // 8 * 8] == 0.0)
+    assert abs(float(loss) - ref_loss) <= 2e-6 * max(1.0, abs(ref_loss))
