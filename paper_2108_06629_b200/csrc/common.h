@@ -100,8 +100,6 @@ struct UpdateArgs {
   long long n_elems;    // out * ldw (multiple of 8)
   const __nv_bfloat16* delta;  // [rows][ldd]: bias gradient = column sums (null: no bias)
   int rows, ldd, n_out;
-  const float* col_partial;    // if set: [chunks][n_out] partial column sums to add instead of delta
-  int n_chunks;
   float* b;             // master bias
   float* mb;            // bias momentum or null
   float* db;            // bias gradient out
@@ -113,13 +111,24 @@ cudaError_t launch_sgd_update(const UpdateArgs& a, cudaStream_t stream);
 // maximum in (dh, dw) row-major order.
 cudaError_t launch_maxpool2(const __nv_bfloat16* a, __nv_bfloat16* pooled, unsigned char* idx, int B, int H, int W,
                             int C, cudaStream_t stream);
-// Column sums of a [rows][ld] bf16 matrix in two deterministic passes: partial[chunk][col] over
-// chunks of colsum_chunk_rows(rows) rows, then (inside launch_sgd_update) the chunk sums on four
-// interleaved thread rows.  One pass (a serial loop over rows / 4 per thread) only up to 512 rows.
-inline int colsum_chunk_rows(int rows) { return rows <= 131072 ? 256 : 2048; }
-inline int colsum_chunks(int rows) { return rows > 512 ? (rows + colsum_chunk_rows(rows) - 1) / colsum_chunk_rows(rows) : 0; }
-cudaError_t launch_colsum_partial(const __nv_bfloat16* x, int rows, int ld, int n_cols, float* partial,
-                                  cudaStream_t stream);
+// Bias gradient (column sums of the [rows][ld] bf16 matrix x, ld a multiple of 8, rows 16-byte aligned) and bias update of a
+// layer with more than 512 rows; up to that the single pass inside launch_sgd_update or the G kernel does it.
+// partial: colsum_chunks x 64 floats per 64 columns; counter: one word per 64 columns, zero between launches.
+struct BiasUpdate {
+  float *b, *mb, *db, *bring;   // master, momentum (may be null), gradient out, slot that receives b
+  float lr, mu;
+};
+// About four blocks per SM, but no fewer than 256 rows to a block (its fixed cost is a tail of two block-wide sums).
+inline int colsum_chunk_rows(int rows, int n_cols) {
+  const int want = std::max(1, 592 / ((n_cols + 63) / 64));
+  return std::max(256, ((rows + want - 1) / want + 31) / 32 * 32);
+}
+inline int colsum_chunks(int rows, int n_cols) {
+  const int c = colsum_chunk_rows(rows, n_cols);
+  return rows > 512 ? (rows + c - 1) / c : 0;
+}
+cudaError_t launch_colsum_bias(const __nv_bfloat16* x, int rows, int ld, int n_cols, float* partial, unsigned* counter,
+                               const BiasUpdate& u, cudaStream_t stream);
 cudaError_t launch_round_to_bf16(const float* src, __nv_bfloat16* dst, long long n_elems, cudaStream_t stream);
 
 }  // namespace lp

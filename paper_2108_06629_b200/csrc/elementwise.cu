@@ -192,82 +192,123 @@ cudaError_t launch_cast_patch_general(const void* batch, int input_is_bf16, cons
 }
 
 // ---------------------------------------------------------------------------
-// One block per row: p = softmax(z^L), delta^L = RN((p - onehot)/B), row loss; the last
-// block to finish adds the row losses in row order (deterministic mean).
-__device__ __forceinline__ float block_reduce(float v, float* sh, bool is_max) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// p = softmax(z^L), delta^L = RN((p - onehot)/B), row loss; the last block to finish adds the row losses in a fixed
+// order (deterministic mean).  A row belongs to TPR threads (a warp, or the block for wide rows), which keep its logits and
+// exponentials in registers: the logits are read once, one exponential per element, 4 bytes per class in
+// and 2 out.  Before (a block per row, three passes, two exponentials) and now:
+// 8192 x 1000 56 -> 20 us, 2048 x 8192 77 -> 36 us.  VEC = 2: two consecutive classes per thread where pitches and addresses allow 8- and 4-byte accesses.
+constexpr int XENT_THREADS = 256;
+// N = classes that a thread keeps in registers; wider rows go in several sweeps over memory
+
+template <int TPR>
+__device__ __forceinline__ float row_reduce(float v, float* sh, bool is_max) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float other = __shfl_xor_sync(0xffffffffu, v, o);
     v = is_max ? fmaxf(v, other) : v + other;
   }
+  if (TPR == 32) return v;
   __syncthreads();
-  if (lane == 0) sh[w] = v;
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  const int nw = blockDim.x >> 5;
   float r = sh[0];
-  for (int i = 1; i < nw; ++i) r = is_max ? fmaxf(r, sh[i]) : r + sh[i];
+#pragma unroll
+  for (int i = 1; i < TPR / 32; ++i) r = is_max ? fmaxf(r, sh[i]) : r + sh[i];
   return r;
 }
 
-__global__ void softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict__ labels,
-                                    __nv_bfloat16* __restrict__ delta, int ldd, float* __restrict__ row_loss,
-                                    unsigned* __restrict__ ticket, float* __restrict__ loss_out, int B, int C,
-                                    int* __restrict__ status) {
-  __shared__ float sh[32];
+template <int TPR, int VEC, int N>
+__global__ void __launch_bounds__(XENT_THREADS)
+softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict__ labels, __nv_bfloat16* __restrict__ delta, int ldd,
+                    float* __restrict__ row_loss, unsigned* __restrict__ ticket, float* __restrict__ loss_out, int B, int C, int* __restrict__ status) {
+  constexpr int ROWS = XENT_THREADS / TPR;            // rows of a block
+  __shared__ float sh[XENT_THREADS / 32];
   __shared__ bool last;
-  const int row = blockIdx.x;
-  const float* z = zL + (long long)row * ldz;
-  float mx = -INFINITY;
-  for (int c = threadIdx.x; c < C; c += blockDim.x) mx = fmaxf(mx, z[c]);
-  mx = block_reduce(mx, sh, true);
-  float s = 0.f;
-  for (int c = threadIdx.x; c < C; c += blockDim.x) s += expf(z[c] - mx);
-  s = block_reduce(s, sh, false);
-  // A label outside [0, C) comes from caller memory: it must not become an address.  Such a row
-  // gets no one-hot term, its loss is NaN (so the minibatch loss is NaN) and the status word, where
-  // there is one, records it.
-  const int y = labels[row];
-  const bool y_ok = unsigned(y) < unsigned(C);
+  const int t = int(threadIdx.x) % TPR;
   const float invB = 1.0f / float(B);
-  const float inv_s = 1.0f / s;
-  __nv_bfloat16* d = delta + (long long)row * ldd;
   const int Cpad = (C + 7) & ~7;
-  for (int c = threadIdx.x; c < Cpad; c += blockDim.x) {
-    float v = 0.f;
-    if (c < C) v = (expf(z[c] - mx) * inv_s - (c == y ? 1.f : 0.f)) * invB;
-    d[c] = __float2bfloat16_rn(v);
+  // (uniform over the row's threads)
+  for (int row = blockIdx.x * ROWS + int(threadIdx.x) / TPR; row < B; row += int(gridDim.x) * ROWS) {
+    const float* z = zL + (long long)row * ldz;
+    __nv_bfloat16* d = delta + (long long)row * ldd;
+    float v[N];
+    // position k of thread t is class (k / VEC) * TPR * VEC + t * VEC + k % VEC
+    auto cls = [&](int k) { return (k / VEC) * (TPR * VEC) + t * VEC + k % VEC; };
+    const bool wide = C > TPR * N;
+    float mx = -INFINITY, s = 0.f;
+#pragma unroll
+    for (int k = 0; k < N; k += VEC) {
+      const int c = cls(k);
+      if (VEC == 2 && c + 1 < C) {
+        const float2 w = *reinterpret_cast<const float2*>(z + c);
+        v[k] = w.x; v[k + VEC - 1] = w.y;
+      } else {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) v[k + e] = c + e < C ? z[c + e] : -INFINITY;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) mx = fmaxf(mx, v[k]);
+    if (wide) for (int c = TPR * N + t; c < C; c += TPR) mx = fmaxf(mx, z[c]);
+    mx = row_reduce<TPR>(mx, sh, true);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      v[k] = cls(k) < C ? expf(v[k] - mx) : 0.f;
+      s += v[k];
+    }
+    if (wide) for (int c = TPR * N + t; c < C; c += TPR) s += expf(z[c] - mx);
+    s = row_reduce<TPR>(s, sh, false);
+    // A label outside [0, C) comes from caller memory: it must not become an address.  Such a row
+    // gets no one-hot term, its loss is NaN (so the minibatch loss is NaN) and the status word, where
+    // there is one, records it.
+    const int y = labels[row];
+    const bool y_ok = unsigned(y) < unsigned(C);
+    const float inv_s = 1.0f / s;
+    auto out = [&](int c, float e) { return c < C ? (e * inv_s - (c == y ? 1.f : 0.f)) * invB : 0.f; };
+#pragma unroll
+    for (int k = 0; k < N; k += VEC) {
+      const int c = cls(k);
+      if (c >= Cpad) continue;
+      if (VEC == 2) *reinterpret_cast<__nv_bfloat162*>(d + c) = __floats2bfloat162_rn(out(c, v[k]), out(c + 1, v[k + VEC - 1]));
+      else d[c] = __float2bfloat16_rn(out(c, v[k]));
+    }
+    if (wide) for (int c = TPR * N + t; c < Cpad; c += TPR) d[c] = __float2bfloat16_rn(out(c, c < C ? expf(z[c] - mx) : 0.f));
+    if (t == 0) {
+      row_loss[row] = y_ok ? -((z[y] - mx) - logf(s)) : __int_as_float(0x7fc00000);
+      if (!y_ok && status != nullptr) atomicCAS(status, 0, LP_STATUS_BAD_LABEL);
+    }
   }
+  __threadfence();                                    // this block's row losses before its count
+  __syncthreads();
   if (threadIdx.x == 0) {
-    row_loss[row] = y_ok ? -((z[y] - mx) - logf(s)) : __int_as_float(0x7fc00000);
-    if (!y_ok && status != nullptr) atomicCAS(status, 0, LP_STATUS_BAD_LABEL);
-    __threadfence();
-    const unsigned t = atomicAdd(ticket, 1u);
-    last = (t == unsigned(B) - 1u);
+    last = atomicInc(ticket, gridDim.x - 1u) == gridDim.x - 1u;     // (wraps to zero: ready for the next launch)
   }
   __syncthreads();
   if (last) {
-    // deterministic mean: thread t adds rows t, t + 256, ... in that order, then the 256 partial
-    // sums are added in thread order
+    // deterministic mean: thread t adds rows t, t + 256, ... in that order, then a tree over the threads
     __threadfence();
     float acc = 0.f;
-    for (int i = threadIdx.x; i < B; i += blockDim.x) acc += __ldcg(row_loss + i);
-    __shared__ float part[256];
-    part[threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float tot = 0.f;
-      for (int i = 0; i < int(blockDim.x); ++i) tot += part[i];
-      *loss_out = tot * invB;
-      *ticket = 0u;     // ready for the next launch on this scratch
-    }
+#pragma unroll 8
+    for (int i = threadIdx.x; i < B; i += XENT_THREADS) acc += __ldcg(row_loss + i);
+    acc = row_reduce<XENT_THREADS>(acc, sh, false);
+    if (threadIdx.x == 0) *loss_out = acc * invB;
   }
 }
 
-cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __nv_bfloat16* delta, int ldd,
-                                float* row_loss, unsigned* ticket, float* loss_out, int B, int C,
-                                int* status, cudaStream_t stream) {
-  softmax_xent_kernel<<<B, 256, 0, stream>>>(zL, ldz, labels, delta, ldd, row_loss, ticket, loss_out, B, C, status);
+cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __nv_bfloat16* delta, int ldd, float* row_loss,
+                                unsigned* ticket, float* loss_out, int B, int C, int* status, cudaStream_t stream) {
+  const bool vec2 = ldz % 2 == 0 && ldd % 2 == 0 && (reinterpret_cast<uintptr_t>(zL) & 7) == 0 && (reinterpret_cast<uintptr_t>(delta) & 3) == 0;
+  // Rows of up to 256 classes need 8 registers a lane and leave room for twice as many warps (16384 x 10: 12.7 us, with
+  // 32 registers and a block per 8 rows 25.3).  Blocks beyond what is resident loop over rows: each pays for its fence,
+  // count and barriers once (8192 x 1000 in 1024 blocks 24.1 us, in 444 20.3).
+#define LP_XENT(TPR, VEC, N, PER_SM)                                                                                 \
+  softmax_xent_kernel<TPR, VEC, N><<<std::min((B + XENT_THREADS / TPR - 1) / (XENT_THREADS / TPR), 148 * PER_SM),      \
+                                     XENT_THREADS, 0, stream>>>(zL, ldz, labels, delta, ldd, row_loss, ticket,        \
+                                                                loss_out, B, C, status)
+  if (C <= 256)       { if (vec2) LP_XENT(32, 2, 8, 6); else LP_XENT(32, 1, 8, 6); }
+  else if (C <= 1024) { if (vec2) LP_XENT(32, 2, 32, 3); else LP_XENT(32, 1, 32, 3); }
+  else                { if (vec2) LP_XENT(256, 2, 32, 256); else LP_XENT(256, 1, 32, 256); }     // (a block per row: 2048 x 8192 36 us, looping 44)
+#undef LP_XENT
   return cudaGetLastError();
 }
 
@@ -327,14 +368,7 @@ __global__ void __launch_bounds__(UPD_THREADS) sgd_update_kernel(const UpdateArg
   const int col = cb + tx;
   float acc = 0.f;
   if (col < a.n_out) {
-    if (a.col_partial != nullptr) {
-      // chunk sums of the first pass, interleaved over the four thread rows; the loads of eight
-      // chunks are in flight together (one dependent load per chunk cost 124 us on 1568 chunks)
-#pragma unroll 8
-      for (int ch = ty; ch < a.n_chunks; ch += NY) acc += __ldg(a.col_partial + (long long)ch * a.n_out + col);
-    } else {
-      for (int r = ty; r < a.rows; r += NY) acc += __bfloat162float(a.delta[(long long)r * a.ldd + col]);
-    }
+    for (int r = ty; r < a.rows; r += NY) acc += __bfloat162float(a.delta[(long long)r * a.ldd + col]);
   }
   part[ty][tx] = acc;
   __syncthreads();
@@ -437,26 +471,97 @@ cudaError_t launch_maxpool2(const __nv_bfloat16* a, __nv_bfloat16* pooled, unsig
   return cudaGetLastError();
 }
 
-// partial[chunk][col] = sum over the chunk's rows (in row order, 4-way interleaved like the
-// single-pass bias reduction) of x[row][col]
-__global__ void colsum_partial_kernel(const __nv_bfloat16* __restrict__ x, int rows, int ld, int n_cols, int chunk_rows,
-                                      float* __restrict__ partial) {
-  __shared__ float part[4][64];
-  const int tx = threadIdx.x % 64, ty = threadIdx.x / 64;
-  const int col = blockIdx.x * 64 + tx;
+// Bias gradient of a layer with many rows (convolutions, large minibatches): column sums of delta, then Eq. 6 for the
+// bias, in one launch.  It is a read of delta at HBM or L2 rate: a thread owns eight columns (one 16-byte load per row) and
+// every 32nd row of its block's chunk, four rows in flight; consecutive threads read consecutive
+// addresses.  The block adds its 32 row lanes in order and writes one partial sum per column; the last
+// block of a 64-column group (a counter that it leaves at zero) adds the chunks in a fixed order and applies the update.
+// Device time with cold caches, before (two-byte loads, a second launch for the chunk sums) and now: 802 816 x 128
+// 109 + 6 -> 41 us, 3 211 264 x 64 210 + 46 -> 75 us (5.5 TB/s), 2048 x 8192 17 + 4 -> 12 us.
+constexpr int COLSUM_LANES = 32;
+__global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* __restrict__ x, int rows, int ld, int n_cols, int chunk_rows,
+                                                          float* __restrict__ partial, unsigned* __restrict__ counter,
+                                                          const BiasUpdate u) {
+  __shared__ __align__(16) float part[COLSUM_LANES][64 + 4];
+  __shared__ bool last;
+  const int g = threadIdx.x & 7, lane = threadIdx.x >> 3;
+  const int col0 = blockIdx.x * 64;
+  const int c8 = col0 + g * 8;
   const int r0 = blockIdx.y * chunk_rows, r1 = min(rows, r0 + chunk_rows);
-  float acc = 0.f;
-  if (col < n_cols)
-    for (int r = r0 + ty; r < r1; r += 4) acc += __bfloat162float(x[(long long)r * ld + col]);
-  part[ty][tx] = acc;
+  float acc[8] = {};
+  if (c8 < ld) {
+    const __nv_bfloat16* src = x + c8;
+    int r = r0 + lane;
+    auto add = [&](const uint4& v) {
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        acc[2 * j] += __uint_as_float(w[j] << 16);
+        acc[2 * j + 1] += __uint_as_float(w[j] & 0xFFFF0000u);
+      }
+    };
+    for (; r + 3 * COLSUM_LANES < r1; r += 4 * COLSUM_LANES) {
+      uint4 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const uint4*>(src + (long long)(r + k * COLSUM_LANES) * ld);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) add(v[k]);
+    }
+    for (; r < r1; r += COLSUM_LANES) add(*reinterpret_cast<const uint4*>(src + (long long)r * ld));
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) part[lane][g * 8 + j] = acc[j];
   __syncthreads();
-  if (ty == 0 && col < n_cols) partial[(long long)blockIdx.y * n_cols + col] = part[0][tx] + part[1][tx] + part[2][tx] + part[3][tx];
+  const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;          // four threads a column, eight row lanes each
+  float s = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) s += part[ty * 8 + k][tx];
+  __syncthreads();
+  part[ty][tx] = s;
+  __syncthreads();
+  const int n_chunks = gridDim.y;
+  float* mine = partial + (long long)blockIdx.x * n_chunks * 64;   // [chunk][64]
+  if (ty == 0) {
+    __stcg(mine + blockIdx.y * 64 + tx, part[0][tx] + part[1][tx] + part[2][tx] + part[3][tx]);
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(counter + blockIdx.x, 1u) == unsigned(n_chunks) - 1u;
+  __syncthreads();
+  if (!last) return;
+  if (threadIdx.x == 0) counter[blockIdx.x] = 0u;                  // ready for the next launch
+  __threadfence();
+  const int q = (threadIdx.x & 15) * 4, l16 = threadIdx.x >> 4;    // four columns, every 16th chunk
+  float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+  for (int ch = l16; ch < n_chunks; ch += 16) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(mine + ch * 64 + q));
+    t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+  }
+  __syncthreads();
+  *reinterpret_cast<float4*>(&part[l16][q]) = t;
+  __syncthreads();
+  const int col = col0 + threadIdx.x;
+  if (threadIdx.x < 64 && col < n_cols) {
+    float grad = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) grad += part[k][threadIdx.x];
+    u.db[col] = grad;
+    float m = grad;
+    if (u.mb != nullptr) {
+      m = u.mu * u.mb[col] + grad;
+      u.mb[col] = m;
+    }
+    const float b = u.b[col] - u.lr * m;
+    u.b[col] = b;
+    u.bring[col] = b;
+  }
 }
-cudaError_t launch_colsum_partial(const __nv_bfloat16* x, int rows, int ld, int n_cols, float* partial,
-                                  cudaStream_t stream) {
-  const int chunk = colsum_chunk_rows(rows);
+cudaError_t launch_colsum_bias(const __nv_bfloat16* x, int rows, int ld, int n_cols, float* partial, unsigned* counter,
+                               const BiasUpdate& u, cudaStream_t stream) {
+  const int chunk = colsum_chunk_rows(rows, n_cols);
   dim3 grid((n_cols + 63) / 64, (rows + chunk - 1) / chunk);
-  colsum_partial_kernel<<<grid, 256, 0, stream>>>(x, rows, ld, n_cols, chunk, partial);
+  colsum_bias_kernel<<<grid, 256, 0, stream>>>(x, rows, ld, n_cols, chunk, partial, counter, u);
   return cudaGetLastError();
 }
 }  // namespace lp
@@ -467,9 +572,12 @@ cudaError_t launch_colsum_partial(const __nv_bfloat16* x, int rows, int ld, int 
 // of a workspace.  Host code must not pass `g_xent_scratch` itself to a kernel: in host
 // code that name is only a handle for the runtime.  The device address is looked up once
 // per device with cudaGetSymbolAddress and that pointer is what the kernel receives.
+// Counts of finished blocks, one per call in turn: the last block of a call wraps its count to zero, and one left
+// over by two calls that overlapped on this scratch is not met by the calls that follow.
+constexpr int kXentTickets = 64;
 struct XentScratch {
   float row_loss[LP_XENT_STATIC_MAX_BATCH];
-  unsigned ticket;
+  unsigned ticket[kXentTickets];
 };
 static __device__ __align__(256) unsigned char g_xent_scratch[sizeof(XentScratch)];
 
@@ -509,11 +617,10 @@ extern "C" int lp_softmax_xent_static(const float* logits_dev, int ld_logits, co
     }
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // the counter must start at zero whatever an earlier (possibly failed) call left behind
-  cudaError_t e = cudaMemsetAsync(&s->ticket, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return xent_fail(LP_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
-  e = lp::launch_softmax_xent(logits_dev, ld_logits, labels_dev, static_cast<__nv_bfloat16*>(delta_dev), ld_delta,
-                              s->row_loss, &s->ticket, loss_dev, batch, classes, nullptr, st);
+  static std::atomic<unsigned> calls{0};
+  unsigned* ticket = s->ticket + calls.fetch_add(1, std::memory_order_relaxed) % kXentTickets;
+  cudaError_t e = lp::launch_softmax_xent(logits_dev, ld_logits, labels_dev, static_cast<__nv_bfloat16*>(delta_dev), ld_delta,
+                              s->row_loss, ticket, loss_dev, batch, classes, nullptr, st);
   if (e != cudaSuccess) return xent_fail(LP_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
   return LP_OK;
 }

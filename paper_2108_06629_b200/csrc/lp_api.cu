@@ -82,6 +82,7 @@ struct Layer {
   unsigned char* pidx = nullptr;     // pool layers: argmax per pooled element, one slot per stash slot of the next layer
   size_t pidx_elems = 0;
   float* col_partial = nullptr;      // bias gradient of large layers: partial column sums
+  unsigned* col_counter = nullptr;
   int col_chunks = 0;
   int split_g = 1;
   float* part_g = nullptr;
@@ -345,7 +346,11 @@ static size_t carve(lp_ctx* c, char* base) {
       y.pidx_elems = size_t(B) * y.Hp * y.Wp * y.ld_out;
       y.pidx = reinterpret_cast<unsigned char*>(take(y.pidx_elems * c->L[l + 1].x_slots));
     }
-    if (y.col_chunks > 0) y.col_partial = reinterpret_cast<float*>(take(size_t(y.col_chunks) * y.ld_out * 4));
+    if (y.col_chunks > 0) {
+      const size_t groups = (y.n_out + 63) / 64;
+      y.col_partial = reinterpret_cast<float*>(take(groups * y.col_chunks * 64 * 4));
+      y.col_counter = reinterpret_cast<unsigned*>(take(groups * 4));
+    }
     auto tiles_of = [&](int M, int N, int bn) { return size_t((M + GEMM_BM - 1) / GEMM_BM) * ((N + bn - 1) / bn); };
     if (y.split_f > 1) {
       const size_t t = tiles_of(B, y.n_out, y.bn_f);
@@ -469,7 +474,7 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       y.split_d = gemm_is_pair(y.bn_d) ? 1 : gemm_pick_splits(B, y.n_in, y.n_out, y.bn_d);
       y.split_g = 1;
     }
-    y.col_chunks = colsum_chunks(y.out_rows);
+    y.col_chunks = colsum_chunks(y.out_rows, y.n_out);
   }
   // One kind of tensor-memory allocation per handle.  SM-pair kernels (tcgen05 cta_group::2) and
   // single-CTA kernels (cta_group::1) that alternate on the same SMs ended, about once in 10^6 pair
@@ -1001,23 +1006,21 @@ static cudaError_t launch_update(lp_ctx* c, int l, long long n, cudaStream_t st)
   u.n_elems = fused_update(c) ? 0 : (long long)y.w_elems;   // fused: W was updated by the G kernel
   if (u.n_elems == 0 && !y.d.has_bias) return cudaSuccess;  // nothing left to do
   if (fused_bias(c, y)) return cudaSuccess;                 // the G kernel did the bias as well
-  if (y.d.has_bias) {
+  TimedScope ts(c, LP_TASK_UPDATE, st, l);
+  if (y.d.has_bias && y.col_chunks > 0) {
+    const BiasUpdate bu{y.b, y.mb, y.db, y.bring + size_t(dst_slot) * y.ld_out, c->cfg.lr, c->cfg.momentum};
+    ++c->launches;
+    cudaError_t e = launch_colsum_bias(y.delta + size_t(n % kDeltaSlots) * y.delta_elems, y.out_rows, y.ld_out, y.n_out,
+                                       y.col_partial, y.col_counter, bu, st);
+    if (e != cudaSuccess || u.n_elems == 0) return e;
+  } else if (y.d.has_bias) {
     u.delta = y.delta + size_t(n % kDeltaSlots) * y.delta_elems;
     u.rows = y.out_rows; u.ldd = y.ld_out; u.n_out = y.n_out;
     u.b = y.b; u.mb = y.mb; u.db = y.db;
     u.bring = y.bring + size_t(dst_slot) * y.ld_out;
-    if (y.col_chunks > 0) {
-      // many rows (convolution): column sums in two deterministic passes
-      ++c->launches;
-      cudaError_t e = launch_colsum_partial(u.delta, u.rows, u.ldd, u.n_out, y.col_partial, st);
-      if (e != cudaSuccess) return e;
-      u.col_partial = y.col_partial;
-      u.n_chunks = y.col_chunks;
-    }
   }
   u.lr = c->cfg.lr; u.mu = c->cfg.momentum;
   ++c->launches;
-  TimedScope ts(c, LP_TASK_UPDATE, st, l);
   return launch_sgd_update(u, st);
 }
 

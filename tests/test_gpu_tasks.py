@@ -13,6 +13,7 @@ import numpy as np
 import pytest
 
 from gpu_common import assert_bf16_close, rel_l2
+from oracle.bf16 import rn_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -403,3 +404,28 @@ def test_tasks_sm_pair_persistent_g_update():
         run_teacher_forced(I.mlp([2600, 2200, 75], "gelu"), 300, 2, [1, 0], 0.05, 0.0, 2)
     finally:
         lpb.lp_set_tuning(0, 0, 0)
+
+
+@pytest.mark.parametrize("rows, n_out", [(513, 8), (545, 72), (1000, 130), (2049, 64), (70000, 10), (4133, 1000)])
+def test_tasks_bias_gradient_of_many_rows(rows, n_out):
+    """Column sums over chunks of rows (ragged chunks, columns past a 64-column group, one chunk and many) and the bias
+    update, twice in a row, against float64: fp32 sums of `rows` bf16 values, |error| <= sqrt(rows) ulps of the rms sum."""
+    from paper_2108_06629_b200 import binding as lpb
+    from paper_2108_06629_b200 import inputs as I
+    layers = I.mlp([16, n_out, 8], "relu")
+    W0, b0 = I.initial_weights(layers, 0)
+    b0[0] = np.linspace(-1, 1, n_out).astype(np.float32)
+    tr = lpb.Trainer(layers, rows, 1, lr=0.5, momentum=0.9, W0=W0, b0=b0)
+    rng = np.random.default_rng(rows)
+    b, m = b0[0].astype(np.float64), np.zeros(n_out)
+    for n in range(2):
+        d = rn_bf16(rng.standard_normal((rows, n_out), dtype=np.float32))
+        tr.debug_write("delta", 0, n, d)
+        tr.debug_run_task("update", 0, n)
+        g = d.astype(np.float64).sum(0)
+        m = 0.9 * m + g
+        b = b - 0.5 * m
+        bound = 2.0 ** -23 * np.sqrt(rows) * np.sqrt(rows) * 4
+        assert np.max(np.abs(tr.debug_read("grad_b", 0, 0) - g)) < bound
+        assert np.max(np.abs(tr.debug_read("master_b", 0, 0) - b)) < 2 * bound + 2.0 ** -22 * np.max(np.abs(b))
+    tr.close()
