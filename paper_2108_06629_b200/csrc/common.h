@@ -61,6 +61,8 @@ int conv_halo_g_max_ctas();
 cudaError_t gemm_configure();   // opt in to large dynamic shared memory; call once per process
 void gemm_set_tuning(int bn, int stages, int splits);   // 0 = automatic
 int gemm_pick_splits(int M, int N, int K, int bn);
+// CTAs of a cluster that share one tile's contraction (GemmArgs::cluster) and, where that is not 0, the tile width
+int gemm_pick_cluster(int M, int N, int K, int* bn);
 
 // ---- planner.cpp ------------------------------------------------------------
 struct PlanResult {

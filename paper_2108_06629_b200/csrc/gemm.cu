@@ -1,6 +1,7 @@
 // Host side of the tcgen05 GEMM: tensor-map encoding, tile selection, launch, and the
 // stand-alone lp_gemm_bf16 entry point.
 #include "gemm2q.cuh"
+#include "gemmc.cuh"
 #include "conv_halo.cuh"
 
 #include <algorithm>
@@ -156,6 +157,30 @@ int gemm_pick_splits(int M, int N, int K, int bn) {
   return (num_kb + per - 1) / per;      // no empty split
 }
 
+// Outputs of few tiles: one tile per cluster, the contraction divided over its CTAs (gemmc.cuh).  Sets the tile width and
+// returns the cluster size, or 0 where another form is the better one.  Rule, each side measured alone on the GPU (us):
+// * 64-column tiles while they fit one CTA on every SM (100 x 777 x 1003 6.1 against 7.3 with 128 columns, 700^3 6.9 / 7.9,
+//   512 x 2048 x 2048 12.7 / 13.3; beyond that 128: 512 x 4096 x 4096 24.5 / 25.7);
+// * four CTAs to a tile, else two, while that is at most one CTA per SM -- a few k-blocks each are enough
+//   (32 x 256 x 256, one each: 4.5; undivided 5.6) -- or two per SM if each keeps 16 k-blocks (1000^3 on 128 tiles:
+//   undivided 11.0, halves 11.9; 64 x 4096 x 4096 on 64 tiles 14.7 in quarters, 16.6 in halves, undivided 27.6);
+// * eight for a handful of tiles with a long contraction (128 x 512 x 4096: 8.1, in quarters 9.8, undivided 24.9).
+int gemm_pick_cluster(int M, int N, int K, int* bn) {
+  if (g_force_bn != 0 || g_force_stages != 0 || g_force_splits != 0 || g_force_persistent >= 0) return 0;
+  const long long rows = (M + GEMM_BM - 1) / GEMM_BM;
+  const int width = rows * ((N + 63) / 64) <= sm_count() ? 64 : 128;
+  const long long tiles = rows * ((N + width - 1) / width);
+  const int num_kb = (K + GEMM_BK - 1) / GEMM_BK;
+  auto fits = [&](int c) {
+    return num_kb >= c && (tiles * c <= sm_count() || (tiles * c <= 2 * sm_count() && num_kb >= 16 * c));
+  };
+  const int c = (num_kb >= 64 && tiles * 8 <= sm_count()) ? 8 : fits(4) ? 4 : fits(2) ? 2 : 0;
+  // (one tile over a hundred thousand terms: the split through global memory spreads it wider than a cluster can)
+  if (c == 0 || gemm_pick_splits(M, N, K, width) > 2 * c) return 0;
+  *bn = width;
+  return c;
+}
+
 int gemm_pick_bn(int which, int M, int N, int K, bool allow_pair) {
   if (g_force_bn == 64 || g_force_bn == 128 || g_force_bn == 256 || g_force_bn == GEMM_BN_PAIR) return g_force_bn;
   if (g_force_bn == GEMM_BN_PAIR224) return which == 2 ? GEMM_BN_PAIR : GEMM_BN_PAIR224;
@@ -288,6 +313,33 @@ static cudaError_t launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, G
   const int num_kb = (a.K + GEMM_BK - 1) / GEMM_BK;
   int s = g_force_stages > 0 ? g_force_stages : (a.tmem_policy == TMEM_PAIR_ALONE ? 6 : 3);   // 3 x 32 KiB: two CTAs per SM; 6: alone
   s = std::max(2, std::min(std::min(s, GEMM_MAX_STAGES), std::max(num_kb + (a.upd_tma ? GEMM2_BN / 64 : 0), 2)));
+// ---- contraction divided over a cluster ------------------------------------------------------------
+template <int BN, bool A_MN, bool B_MN, int MODE>
+static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB, GemmArgs a, cudaStream_t st) {
+  if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
+  const int tiles_m = (a.M + GEMM_BM - 1) / GEMM_BM, tiles_n = (a.N - a.n_begin + BN - 1) / BN;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.cluster, tiles_m * tiles_n, 1);
+  cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = gemmc_smem_bytes(BN);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = a.cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, gemmc_kernel<BN, A_MN, B_MN, MODE>, tmA, tmB, a, tiles_m);
+}
+#define LP_FOR_EACH_CLUSTER_VARIANT(X, BN) \
+  X(BN, false, false, EPI_FPROP)           \
+  X(BN, false, false, EPI_STORE_F32)       \
+  X(BN, false, true, EPI_DGRAD)            \
+  X(BN, false, true, EPI_DGRAD_UNPOOL)     \
+  X(BN, false, true, EPI_STORE_F32)        \
+  X(BN, true, true, EPI_STORE_F32)
+
   const size_t tail = 1024 + 256 + (a.upd_tma ? 1024 + UPD_RING_BYTES : 0);   // alignment slack, barriers, bf16 staging tile
   while (s > 2 && size_t(s) * stage_bytes + tail > 227 * 1024) --s;
   a.num_stages = s;
@@ -451,6 +503,13 @@ cudaError_t gemm_launch(int which, int bn, const CUtensorMap& tmA, const CUtenso
   if (!A && b_mn == B && args.mode == M) return launch_pair<A, B, M, 224>(tmA, tmB, args, st, nullptr);
     LP_FOR_EACH_PAIR_VARIANT(LP_TRYP224)
 #undef LP_TRYP224
+#define LP_CFGC(BN, A, B, M)                                                                                   \
+  if ((e = cudaFuncSetAttribute(gemmc_kernel<BN, A, B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
+                                gemmc_smem_bytes(BN))) != cudaSuccess)                                         \
+    return e;
+  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 64)
+  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 128)
+#undef LP_CFGC
     return cudaErrorInvalidValue;
   }
   if (bn == GEMM_BN_PAIR) {
@@ -479,6 +538,14 @@ cudaError_t gemm_set_tmem_table(int* table) {
 }  // namespace lp
 
 // status word for the stand-alone entry point (handles keep theirs in the workspace)
+  if (args.cluster > 0 && args.g.kind == GEOM_PLAIN && args.starve_kb == 0) {
+#define LP_TRYC(BN, A, B, M) \
+  if (bn == BN && a_mn == A && b_mn == B && args.mode == M) return launch_cluster<BN, A, B, M>(tmA, tmB, args, st);
+    LP_FOR_EACH_CLUSTER_VARIANT(LP_TRYC, 64)
+    LP_FOR_EACH_CLUSTER_VARIANT(LP_TRYC, 128)
+#undef LP_TRYC
+    return cudaErrorInvalidValue;
+  }
 __device__ int g_gemm_status = 0;
 
 namespace {
@@ -522,7 +589,8 @@ int gemm_standalone(int which, int M, int N, int K, const void* A, int lda, cons
   int* status_dev = nullptr;
   int rc = gemm_device_setup(&status_dev);
   if (rc != LP_OK) return rc;
-  const int bn = gemm_pick_bn(which, M, N, K);
+  int bn = gemm_pick_bn(which, M, N, K);
+  const int cluster = gemm_is_pair(bn) ? 0 : gemm_pick_cluster(M, N, K, &bn);
   uint32_t boxA[2], boxB[2];
   gemm_box_dims(which, bn, boxA, boxB);
   CUtensorMap tmA, tmB;
@@ -560,6 +628,7 @@ extern "C" int lp_gemm_status(int* detail) {
   if (rc != LP_OK) return rc;
   int st = 0;
   const int zero = 0;
+  a.cluster = cluster;
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(&st, status_dev, 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
       cudaMemcpy(status_dev, &zero, 4, cudaMemcpyHostToDevice) != cudaSuccess) {
     lp::set_global_error("lp_gemm_status: a CUDA call failed");

@@ -109,6 +109,8 @@ struct GemmArgs {
   float* partial;           // [tiles][splits][128][BN]
   unsigned* tile_counter;   // [tiles], zero between launches
   ConvGeom g;
+  int split_reduce;
+  int cluster;              // >= 1: one tile per cluster of that many CTAs, which divide the contraction (gemmc.cuh); 0: other forms
   int persistent;           // CTAs loop over tiles (grid sized to the machine) instead of one tile each
   int l2_ahead;             // plain GEMM: k-blocks of the B operand to pull into L2 ahead of the pipeline (0 = off)
   int upd_tma;              // EPI_WGRAD_UPDATE: master / momentum / ring tiles move by TMA through the stage ring

@@ -95,6 +95,7 @@ struct Layer {
   size_t w_elems = 0, x_elems = 0, z_elems = 0, delta_elems = 0;
   int z_slots = 0;
   int bn_f = 128, bn_d = 128, bn_g = 128;
+  int cl_f = 0, cl_d = 0;                       // CTAs of a cluster that share a tile of the forward / delta contraction
   int split_f = 1, split_d = 1;                 // split-K factors of the forward / delta contractions
   float *part_f = nullptr, *part_d = nullptr;   // fp32 partial tiles [tiles][splits][128][BN]
   unsigned *cnt_f = nullptr, *cnt_d = nullptr;  // per-tile arrival counters
@@ -380,6 +381,21 @@ static size_t carve(lp_ctx* c, char* base) {
   return align_up(off, 256);
 }
 
+// Tile width of a fully connected layer's three contractions, and how its forward and delta contractions are divided.
+static void pick_fc_tiles(Layer* y, int B, bool allow_pair) {
+  y->bn_f = gemm_pick_bn(0, B, y->n_out, y->n_in, allow_pair);
+  y->bn_d = gemm_pick_bn(1, B, y->n_in, y->n_out, allow_pair);
+  y->bn_g = gemm_pick_bn(2, y->n_out, y->n_in, B, allow_pair);
+  // Contractions divided over clusters pay where the step is a chain of short kernels (16 steps of a 1003-777-515-131
+  // network 1050 -> 830 us).  A layer of more than four million weights keeps the GPU busy with its update, under which a
+  // cluster waits for room on several SMs at once: 8 steps of the 8 x 4096 network take 4780 us without, 5240 with them.
+  const bool chain_bound = (long long)y->n_in * y->n_out <= (1ll << 22);
+  y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f) : 0;
+  y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d) : 0;
+  y->split_f = gemm_is_pair(y->bn_f) || y->cl_f > 0 ? 1 : gemm_pick_splits(B, y->n_out, y->n_in, y->bn_f);
+  y->split_d = gemm_is_pair(y->bn_d) || y->cl_d > 0 ? 1 : gemm_pick_splits(B, y->n_in, y->n_out, y->bn_d);
+}
+
 static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::vector<int>& st,
                          const std::vector<int>& dl) {
   c->L.resize(n);
@@ -467,11 +483,7 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
     } else {
       y.in_rows = y.out_rows = y.next_rows = B;
       y.w_rows = y.n_out; y.w_ld = y.ld_in;
-      y.bn_f = gemm_pick_bn(0, B, y.n_out, y.n_in);
-      y.bn_d = gemm_pick_bn(1, B, y.n_in, y.n_out);
-      y.bn_g = gemm_pick_bn(2, y.n_out, y.n_in, B);
-      y.split_f = gemm_is_pair(y.bn_f) ? 1 : gemm_pick_splits(B, y.n_out, y.n_in, y.bn_f);
-      y.split_d = gemm_is_pair(y.bn_d) ? 1 : gemm_pick_splits(B, y.n_in, y.n_out, y.bn_d);
+      pick_fc_tiles(&y, B, true);
       y.split_g = 1;
     }
     y.col_chunks = colsum_chunks(y.out_rows, y.n_out);
@@ -502,11 +514,8 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
         if (!gemm_is_pair(y.bn_g)) y.bn_g = GEMM_BN_PAIR;
         y.split_f = y.split_d = 1;
       } else if (fc_pair > 0) {
-        y.bn_f = gemm_pick_bn(0, B, y.n_out, y.n_in, false);
-        y.bn_d = gemm_pick_bn(1, B, y.n_in, y.n_out, false);
-        y.bn_g = gemm_pick_bn(2, y.n_out, y.n_in, B, false);
-        y.split_f = gemm_is_pair(y.bn_f) ? 1 : gemm_pick_splits(B, y.n_out, y.n_in, y.bn_f);
-        y.split_d = gemm_is_pair(y.bn_d) ? 1 : gemm_pick_splits(B, y.n_in, y.n_out, y.bn_d);
+        y.cl_f = y.cl_d = 0;
+        pick_fc_tiles(&y, B, false);
       }
     }
   }
@@ -833,6 +842,7 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
   }
   a.splits = y.split_f; a.partial = y.part_f; a.tile_counter = y.cnt_f;
   ++c->launches;
+  a.cluster = y.cl_f;
   TimedScope ts(c, LP_TASK_FORWARD, st, l);
   if (y.lean_f) {
     const CUtensorMap& tmo = y.pool ? y.tm_hf_O[0] : y.tm_hf_O[xout];
@@ -903,6 +913,7 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   a.splits = y.split_d; a.partial = y.part_d; a.tile_counter = y.cnt_d;
   ++c->launches;
+  a.cluster = y.cl_d;
   TimedScope ts(c, LP_TASK_DELTA, st, l);
   if (y.halo_d) {
     a.g = halo_geom(y, 1);
