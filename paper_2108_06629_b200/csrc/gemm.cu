@@ -340,6 +340,22 @@ static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB
   X(BN, false, true, EPI_STORE_F32)        \
   X(BN, true, true, EPI_STORE_F32)
 
+// ---- two-CTA (SM pair) kernel ---------------------------------------------------------------
+template <bool A_MN, bool B_MN, int MODE, int BN2 = GEMM2_BN>
+static cudaError_t launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, GemmArgs a, cudaStream_t st, const UpdMaps* um) {
+  a.splits = 1;
+  if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
+  static const UpdMaps no_maps{};
+  a.upd_tma = (MODE == EPI_WGRAD_UPDATE && um != nullptr && a.g.kind == GEOM_PLAIN) ? 1 : 0;
+  if (!a.upd_tma) um = &no_maps;
+  const int stage_bytes = 32 * 1024;
+  const int num_kb = (a.K + GEMM_BK - 1) / GEMM_BK;
+  // 3 x 32 KiB: two CTAs per SM, one's epilogue under the other's main loop; 6 where a CTA has its SM to itself anyway,
+  // the launch having no more tiles than there are SM pairs (1024 x 4096 x 4096: 37.2 -> 29.1 us)
+  const long long all_tiles = (long long)((a.M + 255) / 256) * ((a.N - a.n_begin + BN2 - 1) / BN2);
+  const bool alone = a.tmem_policy == TMEM_PAIR_ALONE || all_tiles <= std::max(1, sm_count() / 2);
+  int s = g_force_stages > 0 ? g_force_stages : (alone ? 6 : 3);
+  s = std::max(2, std::min(std::min(s, GEMM_MAX_STAGES), std::max(num_kb + (a.upd_tma ? GEMM2_BN / 64 : 0), 2)));
   const size_t tail = 1024 + 256 + (a.upd_tma ? 1024 + UPD_RING_BYTES : 0);   // alignment slack, barriers, bf16 staging tile
   while (s > 2 && size_t(s) * stage_bytes + tail > 227 * 1024) --s;
   a.num_stages = s;
@@ -379,7 +395,7 @@ static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB
       return cudaLaunchKernelEx(&cfg, gemm2_tcgen05_kernel<A_MN, B_MN, MODE, true>, tmA, tmB, *um, a);
     }
   }
-  if constexpr (!A_MN && (MODE == EPI_FPROP || MODE == EPI_DGRAD || MODE == EPI_DGRAD_UNPOOL)) {
+  if constexpr (MODE == EPI_STORE_F32 || (!A_MN && (MODE == EPI_FPROP || MODE == EPI_DGRAD || MODE == EPI_DGRAD_UNPOOL))) {
     // A pair CTA that has its SM to itself walks the tiles with two accumulators (see gemm2q.cuh)
     const int tiles_m = (a.M + 255) / 256, tiles_n = (a.N - a.n_begin + BN2 - 1) / BN2;
     const int pairs = std::max(1, sm_count() / 2);
@@ -387,13 +403,15 @@ static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB
     // in a burst, 252 -> 246 us in a 300-step run; the forward contraction measures the same either way)
     const bool long_delta = (MODE == EPI_DGRAD || MODE == EPI_DGRAD_UNPOOL) && a.g.kind == GEOM_PLAIN &&
                             tiles_m * tiles_n >= 2 * pairs && num_kb >= 32;
-    if ((a.tmem_policy == TMEM_PAIR_ALONE || g_force_persistent == 1 || long_delta) && a.starve_kb == 0 && g_force_persistent != 0 &&
+    // and for plain fp32 results of at least two tiles per SM pair (4096 x 4096 x 1024: 39.3 -> 35.7 us, 4096^3: 105 -> 100 us)
+    const bool many_stores = MODE == EPI_STORE_F32 && a.g.kind == GEOM_PLAIN && tiles_m * tiles_n >= 2 * pairs;
+    if ((a.tmem_policy == TMEM_PAIR_ALONE || (g_force_persistent == 1 && MODE != EPI_STORE_F32) || long_delta || many_stores) && a.starve_kb == 0 && g_force_persistent != 0 &&
         g_force_stages == 0) {
       cfg.gridDim = dim3(2 * std::min(tiles_m * tiles_n, pairs), 1, 1);
       cfg.blockDim = dim3(GEMM2Q_THREADS, 1, 1);
       cfg.dynamicSmemBytes = GEMM2Q_SMEM_BYTES;
       a.num_stages = GEMM2Q_STAGES;
-      return cudaLaunchKernelEx(&cfg, gemm2q_kernel<B_MN, MODE, BN2>, tmA, tmB, a, tiles_m, tiles_n);
+      return cudaLaunchKernelEx(&cfg, gemm2q_kernel<A_MN, B_MN, MODE, BN2>, tmA, tmB, a, tiles_m, tiles_n);
     }
   }
   return cudaLaunchKernelEx(&cfg, gemm2_tcgen05_kernel<A_MN, B_MN, MODE, false, BN2>, tmA, tmB, *um, a);
@@ -408,12 +426,12 @@ static cudaError_t configure_pair() {
   } else if constexpr (!A_MN) {      // forward / delta also exist with 224-column tiles
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(gemm2_tcgen05_kernel<A_MN, B_MN, MODE, false, 224>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if constexpr (MODE == EPI_FPROP || MODE == EPI_DGRAD || MODE == EPI_DGRAD_UNPOOL) {
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gemm2q_kernel<B_MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM2Q_SMEM_BYTES);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gemm2q_kernel<B_MN, MODE, 224>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM2Q_SMEM_BYTES);
-    }
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(gemm2q_kernel<A_MN, B_MN, MODE, 224>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM2Q_SMEM_BYTES);
+  }
+  if constexpr (MODE != EPI_WGRAD_UPDATE) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(gemm2q_kernel<A_MN, B_MN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM2Q_SMEM_BYTES);
   }
   return e;
 }

@@ -23,7 +23,7 @@ constexpr int GEMM2Q_STAGES = 5;
 constexpr int GEMM2Q_STAGE = 32 * 1024;
 constexpr int GEMM2Q_SMEM_BYTES = GEMM2Q_STAGES * GEMM2Q_STAGE + EPI_TILE_BYTES + 1024 + 1024;   // 181 KiB: no other allocating kernel fits beside it
 
-template <bool B_MN, int MODE, int BN2 = GEMM2_BN>
+template <bool A_MN, bool B_MN, int MODE, int BN2 = GEMM2_BN>
 __global__ void __launch_bounds__(GEMM2Q_THREADS, 1)
 gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs p,
               const int tiles_m, const int tiles_n) {
@@ -123,7 +123,12 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             }
             if (++c_chunk == p.g.chunks_per_tap) { c_chunk = 0; ++c_tap; }
           } else {
-            tma2_load_2d_addr(sa, &tmA, fb, k0, tm.m0);
+            if (A_MN) {
+#pragma unroll
+              for (int c = 0; c < 2; ++c) tma2_load_2d_addr(sa + c * 8192, &tmA, fb, tm.m0 + c * 64, k0);
+            } else {
+              tma2_load_2d_addr(sa, &tmA, fb, k0, tm.m0);
+            }
             if (B_MN) {
 #pragma unroll
               for (int c = 0; c < 2; ++c) tma2_load_2d_addr(sb + c * 8192, &tmB, fb, nb0 + c * 64, k0);
@@ -145,12 +150,12 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader only)
     if (lane == 0 && rank == 0) {
-      constexpr uint32_t idesc = make_idesc_bf16(256, BN2, false, B_MN);
-      const uint64_t dA = make_smem_desc(smem_u32(smem), 16, 1024);
+      constexpr uint32_t idesc = make_idesc_bf16(256, BN2, A_MN, B_MN);
+      const uint64_t dA = A_MN ? make_smem_desc(smem_u32(smem), 8192, 1024) : make_smem_desc(smem_u32(smem), 16, 1024);
       const uint64_t dB = B_MN ? make_smem_desc(smem_u32(smem) + GEMM_A_BYTES, 8192, 1024)
                                : make_smem_desc(smem_u32(smem) + GEMM_A_BYTES, 16, 1024);
       const uint32_t dA_hi = uint32_t(dA >> 32), dB_hi = uint32_t(dB >> 32);
-      constexpr uint32_t stepA = 32 >> 4, stepB = (B_MN ? 2048 : 32) >> 4;
+      constexpr uint32_t stepA = (A_MN ? 2048 : 32) >> 4, stepB = (B_MN ? 2048 : 32) >> 4;
       const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
       const uint32_t accf0 = smem_u32(accf_bar), acce0 = smem_u32(acce_bar);
       uint32_t s = 0, ph = 0, it = 0;
