@@ -301,18 +301,6 @@ static cudaError_t configure_one() {
   X(BN, true, true, EPI_STORE_F32)           \
   X(BN, true, true, EPI_WGRAD_UPDATE)
 
-// ---- two-CTA (SM pair) kernel ---------------------------------------------------------------
-template <bool A_MN, bool B_MN, int MODE, int BN2 = GEMM2_BN>
-static cudaError_t launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, GemmArgs a, cudaStream_t st, const UpdMaps* um) {
-  a.splits = 1;
-  if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
-  static const UpdMaps no_maps{};
-  a.upd_tma = (MODE == EPI_WGRAD_UPDATE && um != nullptr && a.g.kind == GEOM_PLAIN) ? 1 : 0;
-  if (!a.upd_tma) um = &no_maps;
-  const int stage_bytes = 32 * 1024;
-  const int num_kb = (a.K + GEMM_BK - 1) / GEMM_BK;
-  int s = g_force_stages > 0 ? g_force_stages : (a.tmem_policy == TMEM_PAIR_ALONE ? 6 : 3);   // 3 x 32 KiB: two CTAs per SM; 6: alone
-  s = std::max(2, std::min(std::min(s, GEMM_MAX_STAGES), std::max(num_kb + (a.upd_tma ? GEMM2_BN / 64 : 0), 2)));
 // ---- contraction divided over a cluster ------------------------------------------------------------
 template <int BN, bool A_MN, bool B_MN, int MODE>
 static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB, GemmArgs a, cudaStream_t st) {
@@ -503,6 +491,13 @@ cudaError_t gemm_configure() {
   if ((e = configure_pair<A, B, M>()) != cudaSuccess) return e;
   LP_FOR_EACH_PAIR_VARIANT(LP_CFGP)
 #undef LP_CFGP
+#define LP_CFGC(BN, A, B, M)                                                                                   \
+  if ((e = cudaFuncSetAttribute(gemmc_kernel<BN, A, B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
+                                gemmc_smem_bytes(BN))) != cudaSuccess)                                         \
+    return e;
+  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 64)
+  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 128)
+#undef LP_CFGC
 #define LP_CFG(BN, A, B, M) \
   if ((e = configure_one<BN, A, B, M>()) != cudaSuccess) return e;
   LP_FOR_EACH_VARIANT(LP_CFG, 64)
@@ -521,13 +516,6 @@ cudaError_t gemm_launch(int which, int bn, const CUtensorMap& tmA, const CUtenso
   if (!A && b_mn == B && args.mode == M) return launch_pair<A, B, M, 224>(tmA, tmB, args, st, nullptr);
     LP_FOR_EACH_PAIR_VARIANT(LP_TRYP224)
 #undef LP_TRYP224
-#define LP_CFGC(BN, A, B, M)                                                                                   \
-  if ((e = cudaFuncSetAttribute(gemmc_kernel<BN, A, B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
-                                gemmc_smem_bytes(BN))) != cudaSuccess)                                         \
-    return e;
-  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 64)
-  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 128)
-#undef LP_CFGC
     return cudaErrorInvalidValue;
   }
   if (bn == GEMM_BN_PAIR) {
@@ -536,6 +524,14 @@ cudaError_t gemm_launch(int which, int bn, const CUtensorMap& tmA, const CUtenso
   if (a_mn == A && b_mn == B && args.mode == M) return launch_pair<A, B, M>(tmA, tmB, args, st, um);
     LP_FOR_EACH_PAIR_VARIANT(LP_TRYP)
 #undef LP_TRYP
+    return cudaErrorInvalidValue;
+  }
+  if (args.cluster > 0 && args.g.kind == GEOM_PLAIN && args.starve_kb == 0) {
+#define LP_TRYC(BN, A, B, M) \
+  if (bn == BN && a_mn == A && b_mn == B && args.mode == M) return launch_cluster<BN, A, B, M>(tmA, tmB, args, st);
+    LP_FOR_EACH_CLUSTER_VARIANT(LP_TRYC, 64)
+    LP_FOR_EACH_CLUSTER_VARIANT(LP_TRYC, 128)
+#undef LP_TRYC
     return cudaErrorInvalidValue;
   }
 #define LP_TRY(BN, A, B, M) \
@@ -556,14 +552,6 @@ cudaError_t gemm_set_tmem_table(int* table) {
 }  // namespace lp
 
 // status word for the stand-alone entry point (handles keep theirs in the workspace)
-  if (args.cluster > 0 && args.g.kind == GEOM_PLAIN && args.starve_kb == 0) {
-#define LP_TRYC(BN, A, B, M) \
-  if (bn == BN && a_mn == A && b_mn == B && args.mode == M) return launch_cluster<BN, A, B, M>(tmA, tmB, args, st);
-    LP_FOR_EACH_CLUSTER_VARIANT(LP_TRYC, 64)
-    LP_FOR_EACH_CLUSTER_VARIANT(LP_TRYC, 128)
-#undef LP_TRYC
-    return cudaErrorInvalidValue;
-  }
 __device__ int g_gemm_status = 0;
 
 namespace {
@@ -628,6 +616,7 @@ int gemm_standalone(int which, int M, int N, int K, const void* A, int lda, cons
   a.status = status_dev;
   a.wait_limit = wait_limit;
   a.starve_kb = starve_kb;
+  a.cluster = cluster;
   cudaError_t e = gemm_launch(which, bn, tmA, tmB, a, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) { set_global_error(std::string("lp_gemm_bf16 launch: ") + cudaGetErrorString(e)); return LP_ERR_CUDA; }
   return LP_OK;
@@ -646,7 +635,6 @@ extern "C" int lp_gemm_status(int* detail) {
   if (rc != LP_OK) return rc;
   int st = 0;
   const int zero = 0;
-  a.cluster = cluster;
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(&st, status_dev, 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
       cudaMemcpy(status_dev, &zero, 4, cudaMemcpyHostToDevice) != cudaSuccess) {
     lp::set_global_error("lp_gemm_status: a CUDA call failed");
