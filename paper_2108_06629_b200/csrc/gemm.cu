@@ -266,7 +266,19 @@ static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, Ge
     }
   }
   if (a.splits > 1) { if (a.persistent) LP_LAUNCH(true, true); else LP_LAUNCH(true, false); }
-  else              { if (a.persistent) LP_LAUNCH(false, true); else LP_LAUNCH(false, false); }
+  if constexpr (A_MN && BN <= 128) {
+    if (a.splits > 1 && a.split_reduce) {
+      cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+      constexpr int blocks = GEMM_BM * (BN / 4) / 256;      // per tile with one lane
+      const int tiles = tiles_m * tiles_n;
+      if (a.splits >= 16) gemm_split_finish_kernel<BN, MODE, 8><<<tiles * blocks * 8, 256, 0, st>>>(a, tiles_m, tiles_n);
+      else                gemm_split_finish_kernel<BN, MODE, 1><<<tiles * blocks, 256, 0, st>>>(a, tiles_m, tiles_n);
+      return cudaGetLastError();
+    }
+  }
+  if (a.splits > 1) return cudaGetLastError();
+  if (a.persistent) LP_LAUNCH(false, true); else LP_LAUNCH(false, false);
 #undef LP_LAUNCH
   return cudaGetLastError();
 }

@@ -104,10 +104,12 @@ struct GemmArgs {
   // split-K (splits > 1): blockIdx.z owns k-blocks [z*kb_per_split, (z+1)*kb_per_split); every CTA
   // writes its fp32 partial tile to `partial`, the last CTA of a tile to arrive (tile_counter)
   // adds the partials in split order -- a fixed order, so results do not depend on timing --
-  // and runs the epilogue.
+  // and runs the epilogue.  With split_reduce the sum and the epilogue are a launch of their own
+  // (gemm_split_finish_kernel) on all SMs: for many splits, where the last CTA would add them alone.
   int splits, kb_per_split;
   float* partial;           // [tiles][splits][128][BN]
   unsigned* tile_counter;   // [tiles], zero between launches
+  int split_reduce;
   ConvGeom g;
   int split_reduce;
   int cluster;              // >= 1: one tile per cluster of that many CTAs, which divide the contraction (gemmc.cuh); 0: other forms
@@ -966,6 +968,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
       if constexpr (split) {
+        if (p.split_reduce) continue;
         // all four epilogue warps have written their part of the partial tile: publish it, and
         // let the last CTA of this tile reduce the partials in split order
         volatile uint32_t* is_last = tmem_slot + 1;
@@ -1025,6 +1028,40 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     tmem_dealloc(tmem_base, PERSIST ? 2 * BN : BN);
     if (lane == 0) tmem_note_freed(PERSIST ? TK_GEMM_PERSISTENT : TK_GEMM, PERSIST ? 2 * BN : BN);
   }
+}
+
+// Second launch of a split contraction with split_reduce: adds the partial tiles and runs the epilogue.  A thread owns four
+// consecutive columns of a tile row; with LANES > 1 (many splits of few tiles) LANES threads share them, lane j
+// adding splits j, j + LANES, ... in order and the lane sums following in order.  Reads splits x tile from L2 once.
+template <int BN, int MODE, int LANES>
+__global__ void __launch_bounds__(256) gemm_split_finish_kernel(const GemmArgs p, const int tiles_m, const int tiles_n) {
+  constexpr int GROUPS = 256 / LANES;                       // column groups of a block
+  constexpr int BLOCKS = GEMM_BM * (BN / 4) / GROUPS;       // blocks of a tile
+  __shared__ float4 sums[LANES > 1 ? LANES : 1][GROUPS];
+  const int tile = int(blockIdx.x) / BLOCKS;
+  const TileCtx tc = decode_tile<BN>(p, tile, tiles_m, tiles_n);
+  const int j = int(threadIdx.x) / GROUPS, e = int(threadIdx.x) % GROUPS;
+  const int g = (int(blockIdx.x) % BLOCKS) * GROUPS + e;
+  const int r = g / (BN / 4), c = (g % (BN / 4)) * 4;
+  if (tc.tm.m0 + (int(blockIdx.x) % BLOCKS) * GROUPS / (BN / 4) >= p.M) return;     // the block's first row
+  const float* src = p.partial + (size_t(tile) * p.splits * GEMM_BM + r) * BN + c;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+  for (int z = j; z < p.splits; z += LANES) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(src + size_t(z) * (GEMM_BM * BN)));
+    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+  }
+  if constexpr (LANES > 1) {
+    sums[j][e] = acc;
+    __syncthreads();
+    if (j != 0) return;
+#pragma unroll
+    for (int k = 1; k < LANES; ++k) {
+      const float4 v = sums[k][e];
+      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
+  }
+  if (tc.tm.m0 + r < p.M) epilogue_store4<MODE>(p, tc.tm.m0 + r, tc.tm.n0 + c, tc.tm.nlim, acc);
 }
 
 }  // namespace lp

@@ -469,11 +469,11 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       y.halo_g = y.halo_f;   // (128 output channels in two passes of the G kernel measured slower than the split-K kernel: 182 / 160 us)
       y.lean_f = y.patch && y.n_out <= 64 && y.ld_in <= 64 && l + 1 < n;
       // G contracts over all B*H*W pixels but has only (Cout/128) x 9 x (Cin/BN) tiles: the pixel
-      // range is split.  A split costs the last CTA of the tile one more partial tile to add
-      // (measured about 1.1 us for a 128-wide tile, half that for 64), a k-block about 0.33 us, so
-      // the time kb/s * 0.33 + s * 1.1 is least near s = sqrt(0.3 kb) (0.6 kb for 64-wide tiles);
-      // never more splits than fill two CTAs per SM.  Swept on the small VGG (2 .. 148 splits):
-      // the measured optimum of every layer is the power of two next to this value.
+      // range is split, and a second launch adds the partial tiles on all SMs and applies the update
+      // (128 -> 128 channels at 16 x 16, batch 128: 57 -> 24 + 7 us; the 5x5 patch layer of the sample network 108 ->
+      // 64 + 7).  Few k-blocks a split leave little to hide its start behind and write more partial tiles: near
+      // s = sqrt(0.3 kb) (0.6 kb for 64-wide tiles) the networks ran fastest -- 16 steps of the small VGG 4750 us, with at
+      // least 4 / 8 / 16 / 24 k-blocks a split instead 5090 / 5060 / 4930 / 4800; never more splits than fill two CTAs per SM.
       const int tiles = ((y.n_out + GEMM_BM - 1) / GEMM_BM) * y.taps * ((y.ld_in + y.bn_g - 1) / y.bn_g);
       const int num_kb = y.out_rows / GEMM_BK;
       const int s_opt = int(std::lround(std::sqrt(double(num_kb) * (y.bn_g <= 64 ? 0.6 : 0.3))));
@@ -976,7 +976,11 @@ static cudaError_t launch_G(lp_ctx* c, int l, long long n, cudaStream_t st) {
   a.tmem_policy = c->tmem_policy;
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   if (y.conv && !y.patch) a.g = conv_geom(y, GEOM_PIX_K, y.box64, 0, 0, (y.ld_in + y.bn_g - 1) / y.bn_g);
-  if (y.split_g > 1) { a.splits = y.split_g; a.partial = y.part_g; a.tile_counter = y.cnt_g; }
+  if (y.split_g > 1) {
+    a.splits = y.split_g; a.partial = y.part_g; a.tile_counter = y.cnt_g;
+    a.split_reduce = 1;
+    c->launches += a.split_reduce;
+  }
   if (fused_update(c)) {
     // Eq. 5 and Eq. 6 in one kernel: the accumulator tile is G; the epilogue reads the fp32
     // master (and momentum) tile, applies the update and writes master, momentum and the
