@@ -225,7 +225,7 @@ static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, Ge
   const int tiles_m = (a.M + GEMM_BM - 1) / GEMM_BM;
   int tiles_n = (a.N - a.n_begin + BN - 1) / BN;
   if (a.g.kind == GEOM_PIX_K) tiles_n = a.g.n_per_tap * (a.N / a.g.tap_pitch);   // (tap, channel block)
-  const long long work = (long long)tiles_m * tiles_n * a.splits;
+  const long long work = (long long)tiles_m * tiles_n * (a.g.classes > 1 ? a.g.classes : a.splits);
   // BN <= 128: two CTAs per SM (2 x 2 x BN tensor-memory columns); BN = 256: one.
   // Many short tiles (convolutions over large images: thousands of tiles of 9..72 k-blocks) are
   // run by persistent CTAs -- no per-tile launch, barrier and tensor-memory set-up, epilogue

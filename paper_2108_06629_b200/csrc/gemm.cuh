@@ -65,13 +65,14 @@ struct ConvGeom {
   int n_per_tap;         // PIX_K: column tiles per tap
   // General filters and strides.  stride: the convolution's stride (forward and G fetch the input
   // through a tensor map that steps `stride` pixels; start coordinate = box origin * stride + shift).
-  // Delta of a strided layer runs once per residue class (roff_h, roff_w) of the input pixel
-  // modulo the stride: the tile rows are the pixels (h*rs + roff_h, w*rs + roff_w) of the H x W
-  // tensor, rs = stride, and only the taps r = tap_r0 + tap_step*i, s = tap_s0 + tap_step*j
-  // (j < tap_ns) reach such a pixel, from delta pixel (h + (roff_h + pad - r)/stride, ...).
+  // Delta of a strided layer works class by class: the tile rows of class (roff_h, roff_w) are the pixels
+  // (h*rs + roff_h, w*rs + roff_w) of the H x W tensor, rs = stride, and only the taps r = r0 + stride*i,
+  // s = s0 + stride*j reach such a pixel, from delta pixel (h + (roff_h + pad - r)/stride, ...).  One launch
+  // covers the stride^2 classes (decode_tile numbers their tiles one class after the other).
   int stride;            // >= 1
-  int rs, roff_h, roff_w;
-  int tap_r0, tap_s0, tap_step, tap_ns;   // enumeration of the taps of this launch: k-th tap = (r0 + step*(k / ns), s0 + step*(k % ns))
+  int rs;
+  int classes;           // residue classes of this launch: rs * rs, or 1
+  int R;                 // filter height (classes > 1)
 };
 
 struct GemmArgs {
@@ -153,6 +154,7 @@ struct TileMap {
   int m0, n0;         // first global row / column (plain)
   int nlim;           // columns >= nlim do not exist
   int pn0, ph0, pw0;  // GEOM_PIX_M: first image / row / column of the pixel box
+  int roff_h = 0, roff_w = 0;   // GEOM_PIX_M: residue class of the rows (strided delta)
 };
 // Global row index of tile row `tr` (0..127), or -1 if the row does not exist.
 __device__ __forceinline__ int tile_row(const GemmArgs& p, const TileMap& t, int tr) {
@@ -164,7 +166,7 @@ __device__ __forceinline__ int tile_row(const GemmArgs& p, const TileMap& t, int
   const int w = t.pw0 + (tr & ((1 << p.g.lw) - 1));
   const int h = t.ph0 + ((tr >> p.g.lw) & ((1 << p.g.lh) - 1));
   const int n = t.pn0 + (tr >> (p.g.lw + p.g.lh));
-  return (n * p.g.H + h * p.g.rs + p.g.roff_h) * p.g.W + w * p.g.rs + p.g.roff_w;
+  return (n * p.g.H + h * p.g.rs + t.roff_h) * p.g.W + w * p.g.rs + t.roff_w;
 }
 
 // Bias of four consecutive output columns (zero where there is none).
@@ -424,7 +426,8 @@ struct TileCtx {
   TileMap tm;
   int tap, col0;        // GEOM_PIX_K: filter tap and first input channel of the column tile
   int kb_begin, num_kb; // k-blocks of this work item
-  int tile_id, z;       // output tile index and split index
+  int tile_id, z;       // output tile index and split index (or residue class of a strided delta)
+  int tap_r0, tap_s0, tap_ns;   // GEOM_PIX_M: k-th tap = (r0 + rs*(k / ns), s0 + rs*(k % ns))
 };
 
 template <int BN>
@@ -448,6 +451,18 @@ __device__ __forceinline__ TileCtx decode_tile(const GemmArgs& p, int t, int til
     c.tm.pw0 = tw << p.g.lw;
     c.tm.ph0 = th << p.g.lh;
     c.tm.pn0 = tn * (GEMM_BM >> (p.g.lw + p.g.lh));
+    c.tap_r0 = c.tap_s0 = 0;
+    c.tap_ns = p.g.S;
+    if (p.g.classes > 1) {
+      const int sd = p.g.rs;
+      c.tm.roff_h = c.z / sd;
+      c.tm.roff_w = c.z % sd;
+      c.tap_r0 = (c.tm.roff_h + p.g.pad) % sd;
+      c.tap_s0 = (c.tm.roff_w + p.g.pad) % sd;
+      const int nr = c.tap_r0 < p.g.R ? (p.g.R - c.tap_r0 + sd - 1) / sd : 0, ns = c.tap_s0 < p.g.S ? (p.g.S - c.tap_s0 + sd - 1) / sd : 0;
+      c.tap_ns = max(ns, 1);
+      c.num_kb = nr * ns * p.g.chunks_per_tap;       // (a class without taps stores f'(.) x 0)
+    }
   } else if (p.g.kind == GEOM_PIX_K) {
     c.tap = by / p.g.n_per_tap;
     c.col0 = (by % p.g.n_per_tap) * BN;
@@ -605,12 +620,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             k0 += GEMM_BK;
           } else if (p.g.kind == GEOM_PIX_M) {
             // A: 128 pixels x 64 channels of the activation / delta tensor, shifted by the tap
-            const int r = p.g.tap_r0 + p.g.tap_step * (c_tap / p.g.tap_ns), sft = p.g.tap_s0 + p.g.tap_step * (c_tap % p.g.tap_ns);
+            const int r = tc.tap_r0 + p.g.rs * (c_tap / tc.tap_ns), sft = tc.tap_s0 + p.g.rs * (c_tap % tc.tap_ns);
             const int wtap = r * p.g.S + sft;         // position of this tap in a row of the weight matrix
             int cw, ch;
             if (p.g.flip) {   // delta: output pixel of the layer that reaches this input pixel through tap (r, s)
-              cw = tm.pw0 + (p.g.roff_w + p.g.pad - sft) / p.g.stride;
-              ch = tm.ph0 + (p.g.roff_h + p.g.pad - r) / p.g.stride;
+              cw = tm.pw0 + (tm.roff_w + p.g.pad - sft) / p.g.stride;
+              ch = tm.ph0 + (tm.roff_h + p.g.pad - r) / p.g.stride;
             } else {          // forward: first input pixel of the box (the map steps `stride` pixels per element)
               cw = tm.pw0 * p.g.stride + sft - p.g.pad;
               ch = tm.ph0 * p.g.stride + r - p.g.pad;
