@@ -111,9 +111,8 @@ struct GemmArgs {
   float* partial;           // [tiles][splits][128][BN]
   unsigned* tile_counter;   // [tiles], zero between launches
   int split_reduce;
-  ConvGeom g;
-  int split_reduce;
   int cluster;              // >= 1: one tile per cluster of that many CTAs, which divide the contraction (gemmc.cuh); 0: other forms
+  ConvGeom g;
   int persistent;           // CTAs loop over tiles (grid sized to the machine) instead of one tile each
   int l2_ahead;             // plain GEMM: k-blocks of the B operand to pull into L2 ahead of the pipeline (0 = off)
   int upd_tma;              // EPI_WGRAD_UPDATE: master / momentum / ring tiles move by TMA through the stage ring
@@ -561,12 +560,24 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const TileMap& tm = tc.tm;
         // running position of the contraction
         int k0 = tc.kb_begin * GEMM_BK;                    // plain: element offset along K
-        int c_tap = 0, c_chunk = 0;                        // PIX_M: filter tap, 64-channel chunk
+        // PIX_M: the tap as steps (c_r, c_s) of this tile's enumeration, its weight column and the start of its
+        // shifted box, all kept up to date by additions: the loop below is one thread's, and the divisions of a tap
+        // number (four of them in the delta form) cost more cycles than the tensor cores need for the k-block
+        // (256 -> 256 channels at 56 x 56, batch 64: forward 224 -> 177 us, delta 282 -> 202)
+        int c_chunk = 0, c_s = 0, wcol = 0, wrow = 0, cw = 0, ch = 0, cw_first = 0;
         int bw0 = 0, bh0 = 0, bn0 = 0;                     // PIX_K: pixel box of this k-block
         int dh = 0, dw = 0;                                // PIX_K: pixel shift of this tile's tap
         if (p.g.kind == GEOM_PIX_M) {
-          c_tap = tc.kb_begin / p.g.chunks_per_tap;
-          c_chunk = tc.kb_begin % p.g.chunks_per_tap;
+          // (no split-K in this geometry: every tile starts with its first tap)
+          if (p.g.flip) {   // delta: output pixel of the layer that reaches this input pixel through tap (r, s)
+            cw = tm.pw0 + (tm.roff_w + p.g.pad - tc.tap_s0) / p.g.stride;
+            ch = tm.ph0 + (tm.roff_h + p.g.pad - tc.tap_r0) / p.g.stride;
+          } else {          // forward: first input pixel of the box (the map steps `stride` pixels per element)
+            cw = tm.pw0 * p.g.stride + tc.tap_s0 - p.g.pad;
+            ch = tm.ph0 * p.g.stride + tc.tap_r0 - p.g.pad;
+          }
+          cw_first = cw;
+          wrow = wcol = (tc.tap_r0 * p.g.S + tc.tap_s0) * p.g.tap_pitch;
         } else if (p.g.kind == GEOM_PIX_K) {
           const int tw = tc.kb_begin % p.g.tiles_w, th = (tc.kb_begin / p.g.tiles_w) % p.g.tiles_h;
           bw0 = tw << p.g.lw;
@@ -575,6 +586,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           dh = tc.tap / p.g.S - p.g.pad;
           dw = tc.tap % p.g.S - p.g.pad;
         }
+        const int chunks = p.g.chunks_per_tap, step = p.g.flip ? -1 : 1, wstep = p.g.rs * p.g.tap_pitch, wstep_row = wstep * p.g.S;
         // Weight streaming (small batch): the shared-memory pipeline holds only S k-blocks, not
         // enough to cover an HBM round trip, so the B operand is additionally requested into L2
         // l2_ahead k-blocks early; the pipeline then runs at L2-hit latency.
@@ -620,25 +632,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             k0 += GEMM_BK;
           } else if (p.g.kind == GEOM_PIX_M) {
             // A: 128 pixels x 64 channels of the activation / delta tensor, shifted by the tap
-            const int r = tc.tap_r0 + p.g.rs * (c_tap / tc.tap_ns), sft = tc.tap_s0 + p.g.rs * (c_tap % tc.tap_ns);
-            const int wtap = r * p.g.S + sft;         // position of this tap in a row of the weight matrix
-            int cw, ch;
-            if (p.g.flip) {   // delta: output pixel of the layer that reaches this input pixel through tap (r, s)
-              cw = tm.pw0 + (tm.roff_w + p.g.pad - sft) / p.g.stride;
-              ch = tm.ph0 + (tm.roff_h + p.g.pad - r) / p.g.stride;
-            } else {          // forward: first input pixel of the box (the map steps `stride` pixels per element)
-              cw = tm.pw0 * p.g.stride + sft - p.g.pad;
-              ch = tm.ph0 * p.g.stride + r - p.g.pad;
-            }
             tma_load_4d_addr(sa, &tmA, fb, c_chunk * 64, cw, ch, tm.pn0);
             if (B_MN) {   // delta: B[k = (tap, co)][n = ci]: rows co, columns tap*pitch + ci
 #pragma unroll
               for (int c = 0; c < BN / 64; ++c)
-                tma_load_2d_addr(sb + c * 8192, &tmB, fb, wtap * p.g.tap_pitch + tm.n0 + c * 64, c_chunk * 64);
+                tma_load_2d_addr(sb + c * 8192, &tmB, fb, wcol + tm.n0 + c * 64, c_chunk * 64);
             } else {      // forward: B[n = co][k = (tap, ci)]
-              tma_load_2d_addr(sb, &tmB, fb, wtap * p.g.tap_pitch + c_chunk * 64, tm.n0);
+              tma_load_2d_addr(sb, &tmB, fb, wcol + c_chunk * 64, tm.n0);
             }
-            if (++c_chunk == p.g.chunks_per_tap) { c_chunk = 0; ++c_tap; }
+            if (++c_chunk == chunks) {
+              c_chunk = 0;
+              wcol += wstep;
+              cw += step;
+              if (++c_s == tc.tap_ns) { c_s = 0; wrow += wstep_row; wcol = wrow; cw = cw_first; ch += step; }
+            }
           } else {
             // G: A = delta (64 pixels x 128 output channels), B = activations shifted by the tap
 #pragma unroll

@@ -513,8 +513,8 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
         if (!gemm_is_pair(y.bn_d)) y.bn_d = GEMM_BN_PAIR;
         if (!gemm_is_pair(y.bn_g)) y.bn_g = GEMM_BN_PAIR;
         y.split_f = y.split_d = 1;
-      } else if (fc_pair > 0) {
         y.cl_f = y.cl_d = 0;
+      } else if (fc_pair > 0) {
         pick_fc_tiles(&y, B, false);
       }
     }
@@ -842,8 +842,8 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
     }
   }
   a.splits = y.split_f; a.partial = y.part_f; a.tile_counter = y.cnt_f;
-  ++c->launches;
   a.cluster = y.cl_f;
+  ++c->launches;
   TimedScope ts(c, LP_TASK_FORWARD, st, l);
   if (y.lean_f) {
     const CUtensorMap& tmo = y.pool ? y.tm_hf_O[0] : y.tm_hf_O[xout];
@@ -913,8 +913,8 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
   a.tmem_policy = c->tmem_policy;
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   a.splits = y.split_d; a.partial = y.part_d; a.tile_counter = y.cnt_d;
-  ++c->launches;
   a.cluster = y.cl_d;
+  ++c->launches;
   TimedScope ts(c, LP_TASK_DELTA, st, l);
   if (y.halo_d) {
     a.g = halo_geom(y, 1);
