@@ -60,7 +60,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
-    if (MODE == EPI_FPROP) tma_prefetch_desc(&tmO);
+    if (MODE != EPI_DGRAD_UNPOOL) tma_prefetch_desc(&tmO);
     mbar_init(wfull, 1);
     for (int b = 0; b < HALO_STAGES; ++b) {
       mbar_init(&afull[b], 1);
@@ -188,8 +188,26 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     int tw = tw_begin - 1, th = th_begin, tn = tn_begin;
+    // delta: what f' is evaluated on, this lane's pixel and 32 columns, asked for one tile ahead: an accumulator is
+    // usually complete when these warps reach it, and the round trip would be theirs alone
+    uint4 av[4], av_next[4];
+    auto load_aux = [&](int t, uint4 (&v)[4]) {
+      const int img = t / tiles_per_image, r = t - img * tiles_per_image, rh = r / p.g.tiles_w;
+      const int trow = q * 32 + lane;
+      const size_t pix = (size_t(img) * p.g.H + rh * 16 + (trow >> 3)) * p.g.W + (r - rh * p.g.tiles_w) * 8 + (trow & 7);
+      const __nv_bfloat16* src = p.aux + pix * p.ld_aux + half * 32;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        v[u] = (p.act != ACT_NONE && half * 32 + 8 * u < p.ld_aux) ? *reinterpret_cast<const uint4*>(src + 8 * u) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (MODE == EPI_DGRAD && t_begin < t_end) load_aux(t_begin, av_next);
     for (int t = t_begin; t < t_end; ++t, ++it) {
       const uint32_t buf = it & 1u;
+      if constexpr (MODE == EPI_DGRAD) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) av[u] = av_next[u];
+        if (t + 1 < t_end) load_aux(t + 1, av_next);
+      }
       if (!plain && ++tw == p.g.tiles_w) { tw = 0; if (++th == p.g.tiles_h) { th = 0; ++tn; } }
       TileMap tm;
       tm.m0 = t * GEMM_BM;            // (plain geometry)
@@ -206,14 +224,15 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           dead = true;
         }
       }
-      if (dead && MODE != EPI_FPROP) break;      // only the forward epilogue has CTA-wide barriers
+      if (dead && MODE == EPI_DGRAD_UNPOOL) break;      // the other epilogues have CTA-wide barriers
       tc_fence_after();
       const uint32_t tacc = tmem_base + buf * uint32_t(BN);
-      if constexpr (MODE == EPI_FPROP) {
-        // Forward: a lane keeps its accumulator row (one pixel), adds the bias, applies f, and
-        // writes the 64 bf16 channels as one 128-byte swizzled row of a shared-memory tile that a
+      if constexpr (MODE != EPI_DGRAD_UNPOOL) {
+        // A lane keeps its accumulator row (one pixel), adds the bias and applies f (forward) or multiplies by
+        // f' (delta), and writes the 64 bf16 channels as one 128-byte swizzled row of a shared-memory tile that a
         // TMA store sends to the NHWC output (8 x 16 pixel box) -- no transposition, no address
-        // arithmetic per element, and the global writes are whole lines.
+        // arithmetic per element, and the global writes are whole lines.  (Delta through transposition
+        // tiles and 8-byte accesses: 418 us for 64 channels at 224 x 224, batch 64; this form 314, 428 without the look-ahead.)
         const int trow = q * 32 + lane;
         const uint32_t so = smem_u32(sO) + buf * uint32_t(HALO_OUT_BYTES) + uint32_t(trow) * 128u;
         const uint32_t swz = uint32_t(trow & 7);
@@ -228,12 +247,19 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
           for (int g = 0; g < 8; ++g) {
             const int n = half * 32 + 4 * g;
-            float v[4] = {__uint_as_float(r[4 * g]) + bias4[g].x, __uint_as_float(r[4 * g + 1]) + bias4[g].y,
-                          __uint_as_float(r[4 * g + 2]) + bias4[g].z, __uint_as_float(r[4 * g + 3]) + bias4[g].w};
+            float v[4] = {__uint_as_float(r[4 * g]), __uint_as_float(r[4 * g + 1]), __uint_as_float(r[4 * g + 2]), __uint_as_float(r[4 * g + 3])};
+            if constexpr (MODE == EPI_FPROP) {
+              v[0] += bias4[g].x; v[1] += bias4[g].y; v[2] += bias4[g].z; v[3] += bias4[g].w;
+            }
+            const uint32_t a01 = (g & 1) ? av[g >> 1].z : av[g >> 1].x, a23 = (g & 1) ? av[g >> 1].w : av[g >> 1].y;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               if (n + e >= p.N) v[e] = 0.f;
-              else if (p.act == ACT_RELU) v[e] = fmaxf(v[e], 0.f);
+              else if (MODE == EPI_FPROP) { if (p.act == ACT_RELU) v[e] = fmaxf(v[e], 0.f); }
+              else if (p.act != ACT_NONE) {
+                const float z = (e & 1) ? bf16_hi(e < 2 ? a01 : a23) : bf16_lo(e < 2 ? a01 : a23);
+                v[e] = p.act == ACT_RELU ? (z > 0.f ? v[e] : 0.f) : v[e] * gelu_grad(z);
+              }
             }
             packed[2 * g] = pack_bf16x2(v[0], v[1]);
             packed[2 * g + 1] = pack_bf16x2(v[2], v[3]);
@@ -248,6 +274,30 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(so + ((uint32_t(half * 4 + u) ^ swz) << 4)), "r"(packed[4 * u]),
                          "r"(packed[4 * u + 1]), "r"(packed[4 * u + 2]), "r"(packed[4 * u + 3])
                          : "memory");
+        }
+        if (MODE == EPI_FPROP && p.pool_out_idx != nullptr) {
+          // 2x2 max pool of the staged tile: a thread takes one of its 32 windows and eight channels
+          asm volatile("bar.sync 1, 256;" ::: "memory");
+          const int e = int(threadIdx.x) - 64, pp = e >> 3, cg = e & 7;
+          if (!dead && cg * 8 < p.ld_out) {
+            const int pw = pp & 3, ph = pp >> 2;
+            float best[8];
+            uint32_t idx[2] = {0u, 0u};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t tr = uint32_t((2 * ph + (k >> 1)) * 8 + 2 * pw + (k & 1));
+              uint32_t w[4];
+              asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                           : "r"(smem_u32(sO) + buf * uint32_t(HALO_OUT_BYTES) + tr * 128u + ((uint32_t(cg) ^ (tr & 7u)) << 4)));
+#pragma unroll
+              for (int j = 0; j < 4; ++j) pool_step(w[j], k, best + 4 * (j >> 1), idx[j >> 1], 2 * (j & 1));
+            }
+            const size_t off = (size_t(tm.pn0 * p.pool_Hp + (tm.ph0 >> 1) + ph) * p.pool_Wp + (tm.pw0 >> 1) + pw) * p.ld_out + cg * 8;
+            *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + off) =
+                make_uint4(pool_pack(best), pool_pack(best + 2), pool_pack(best + 4), pool_pack(best + 6));
+            *reinterpret_cast<uint2*>(p.pool_out_idx + off) = make_uint2(idx[0], idx[1]);
+          }
+          continue;
         }
         fence_proxy_async_smem();
         asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -282,7 +332,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
     }
   }
-  if (MODE == EPI_FPROP && threadIdx.x == 64) tma_store_wait_read0();   // shared memory must outlive the stores' reads
+  if (MODE != EPI_DGRAD_UNPOOL && threadIdx.x == 64) tma_store_wait_read0();   // shared memory must outlive the stores' reads
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {

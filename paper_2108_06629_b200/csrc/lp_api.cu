@@ -87,6 +87,7 @@ struct Layer {
   int split_g = 1;
   float* part_g = nullptr;
   unsigned* cnt_g = nullptr;
+  bool pool_fused = false;           // the forward epilogue pools (no a_full)
   Res rAfull;
   Res rPartF, rPartD;               // split-K partial tiles and arrival counters of the forward / delta contraction
   // device memory (all inside the workspace)
@@ -106,6 +107,7 @@ struct Layer {
   std::vector<CUtensorMap> tm_hg_D;             // delta as 8 x 16 pixel boxes (the halo-tile G kernel)
   bool lean_f = false;                          // patch-matrix layer with at most 64 output channels: forward through the same kernel
   std::vector<CUtensorMap> tm_hf_A, tm_hd_A;    // halo boxes over the stash slots / the delta slots
+  std::vector<CUtensorMap> tm_hd_O;             // delta^{l-1} slots as 8 x 16 pixel boxes (halo-tile delta without un-pooling)
   std::vector<CUtensorMap> tm_hf_O;             // forward output (next layer's stash slots, or the pre-pool buffer) as 8 x 16 pixel boxes
   bool upd_maps = false;                        // fused update streamed by TMA (fully connected layers, 128-wide tiles)
   CUtensorMap tm_u_W, tm_u_M;                   // fp32 master / momentum as 32-column boxes
@@ -218,9 +220,9 @@ static int fail(lp_ctx* h, int code, const std::string& msg) {
 
 // Factor `pixels` (128 or 64) into a box bw x bh x bn of powers of two with bw | W, bh | H, bn | B,
 // widest in w first (longest contiguous runs).
-static int pick_box(int W, int H, int B, int pixels, PixBox* out) {
+static int pick_box(int W, int H, int B, int pixels, PixBox* out, int widest = 128) {
   int bw = 1, lw = 0;
-  while (bw * 2 <= pixels && W % (bw * 2) == 0) { bw *= 2; ++lw; }
+  while (bw * 2 <= std::min(pixels, widest) && W % (bw * 2) == 0) { bw *= 2; ++lw; }
   int bh = 1, lh = 0;
   while (bw * bh * 2 <= pixels && H % (bh * 2) == 0) { bh *= 2; ++lh; }
   const int bn = pixels / (bw * bh);
@@ -343,7 +345,7 @@ static size_t carve(lp_ctx* c, char* base) {
       y.Z = reinterpret_cast<__nv_bfloat16*>(take(y.z_elems * 2 * y.z_slots));
     }
     if (y.pool && l + 1 < nL) {
-      y.a_full = reinterpret_cast<__nv_bfloat16*>(take(y.delta_elems * 2));
+      if (!y.pool_fused) y.a_full = reinterpret_cast<__nv_bfloat16*>(take(y.delta_elems * 2));
       y.pidx_elems = size_t(B) * y.Hp * y.Wp * y.ld_out;
       y.pidx = reinterpret_cast<unsigned char*>(take(y.pidx_elems * c->L[l + 1].x_slots));
     }
@@ -435,7 +437,10 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       y.pool = layers[l].pool;
       y.Hp = y.pool ? y.oH / 2 : y.oH; y.Wp = y.pool ? y.oW / 2 : y.oW;
       y.next_rows = (l + 1 < n && layers[l + 1].kind == LP_CONV) ? B * y.Hp * y.Wp : B;
-      pick_box(y.oW, y.oH, B, 128, &y.box128);      // forward: tile rows = output pixels
+      // forward: tile rows = output pixels; at most 16 wide where the epilogue pools (a 2x2 window then lies in one
+      // warp's 32 rows), unless that leaves a number of images that does not divide the batch
+      y.pool_fused = y.pool && !y.patch && pick_box(y.oW, y.oH, B, 128, &y.box128, 16) == LP_OK;
+      if (!y.pool_fused) pick_box(y.oW, y.oH, B, 128, &y.box128);
       pick_box(y.oW, y.oH, B, 64, &y.box64);        // G: the contraction runs over output pixels
       pick_box(y.imW / y.cstride, y.imH / y.cstride, B, 128, &y.boxD);   // delta: tile rows = input pixels of one residue class
       y.bn_f = y.n_out <= 64 ? 64 : 128;
@@ -642,10 +647,10 @@ static int build_tensor_maps(lp_ctx* c) {
       if (y.halo_f) {
         // the layer's output: NHWC [B][H][W][ld_out], one map per destination
         Layer& nx = c->L[l + 1];
-        const int n_dst = y.pool ? 1 : nx.x_slots;
+        const int n_dst = y.pool_fused ? 0 : nx.x_slots;       // (a pooled output is stored by the epilogue's threads)
         y.tm_hf_O.resize(n_dst);
         for (int s = 0; s < n_dst; ++s) {
-          const __nv_bfloat16* dst = y.pool ? y.a_full : nx.X + size_t(s) * nx.x_elems;
+          const __nv_bfloat16* dst = nx.X + size_t(s) * nx.x_elems;
           if ((rc = make_tmap_bf16_nhwc(&y.tm_hf_O[s], dst, y.ld_out, y.imW, y.imH, B, y.ld_out, 8, 16, 1, &err)) != LP_OK)
             return fail(c, rc, err);
         }
@@ -654,6 +659,13 @@ static int build_tensor_maps(lp_ctx* c) {
         y.tm_hg_D.resize(kDeltaSlots);
         for (int s = 0; s < kDeltaSlots; ++s)
           if ((rc = make_tmap_bf16_nhwc(&y.tm_hg_D[s], y.delta + s * y.delta_elems, y.ld_out, y.imW, y.imH, B, y.ld_out, 8, 16, 1,
+                                        &err)) != LP_OK) return fail(c, rc, err);
+      }
+      if (y.halo_d && !c->L[l - 1].pool) {
+        Layer& pv = c->L[l - 1];
+        y.tm_hd_O.resize(kDeltaSlots);
+        for (int s = 0; s < kDeltaSlots; ++s)
+          if ((rc = make_tmap_bf16_nhwc(&y.tm_hd_O[s], pv.delta + s * pv.delta_elems, pv.ld_out, y.imW, y.imH, B, pv.ld_out, 8, 16, 1,
                                         &err)) != LP_OK) return fail(c, rc, err);
       }
       if (y.halo_d) {
@@ -829,6 +841,11 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
     a.out2 = c->zL + size_t(n % kDeltaSlots) * c->cfg.batch * c->ld_cls;
     a.ld_out2 = c->ld_cls;
     a.out2_is_f32 = 1;
+  } else if (y.pool_fused) {
+    a.out = c->L[l + 1].X + size_t(xout) * c->L[l + 1].x_elems;
+    a.ld_out = y.ld_out;
+    a.pool_out_idx = y.pidx + size_t(xout) * y.pidx_elems;
+    a.pool_Hp = y.Hp; a.pool_Wp = y.Wp;
   } else if (y.pool) {
     a.out = y.a_full;                 // pooled into the next layer's stash by launch_pool
     a.ld_out = y.ld_out;
@@ -851,7 +868,7 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
   }
   if (y.halo_f) {
     a.g = halo_geom(y, 0);
-    const CUtensorMap& tmo = y.pool ? y.tm_hf_O[0] : y.tm_hf_O[xout];
+    const CUtensorMap& tmo = y.pool_fused ? y.tm_hf_A[xin] : y.tm_hf_O[xout];
     return conv_halo_launch(0, y.tm_hf_A[xin], y.tm_f_B[ring_slot], tmo, a, st);
   }
   return gemm_launch(0, y.bn_f, y.tm_f_A[xin], y.tm_f_B[ring_slot], a, st);
@@ -918,7 +935,8 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
   TimedScope ts(c, LP_TASK_DELTA, st, l);
   if (y.halo_d) {
     a.g = halo_geom(y, 1);
-    return conv_halo_launch(1, y.tm_hd_A[n % kDeltaSlots], y.tm_d_B[ring_slot], y.tm_hd_A[0], a, st);
+    return conv_halo_launch(1, y.tm_hd_A[n % kDeltaSlots], y.tm_d_B[ring_slot],
+                            pv.pool ? y.tm_hd_A[0] : y.tm_hd_O[n % kDeltaSlots], a, st);
   }
   if (y.conv && y.cstride > 1) {
     // Strided layer: input pixel (h, w) is reached through tap (r, s) only when h + pad - r and
@@ -1348,11 +1366,11 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
     Res* rout = (l == nL - 1) ? &c->rZL[ds] : &c->L[l + 1].rX[xo];
     Res* rz = y.Z ? &y.rZ[xo] : nullptr;
     Res* rpool = y.pool ? &y.rPidx[xo] : nullptr;
-    Res* rfull = y.pool ? &y.rAfull : nullptr;
+    Res* rfull = y.pool && !y.pool_fused ? &y.rAfull : nullptr;
     Res* rpart = y.split_f > 1 ? &y.rPartF : nullptr;
     LP_CUDA(c, task_begin(c, sc, {rin, rw}, {rout, rz, rpool, rfull, rpart}));
     LP_CUDA(c, launch_forward(c, l, n, slot[l], chain));
-    if (y.pool) LP_CUDA(c, launch_pool(c, l, n, chain));
+    if (rfull) LP_CUDA(c, launch_pool(c, l, n, chain));
     // (scratch that the next minibatch's task of this layer reuses: it waits for this very task)
     LP_CUDA(c, task_end(c, sc, {rin, rw}, {rout, rz, rpool, rfull, rpart}, nullptr, rfull || rpart));
   }
@@ -1387,11 +1405,11 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
         Res* rout = &c->L[k].rX[xo];
         Res* rz = src.Z ? &src.rZ[xo] : nullptr;
         Res* rpool = src.pool ? &src.rPidx[xo] : nullptr;
-        Res* rfull = src.pool ? &src.rAfull : nullptr;
+        Res* rfull = src.pool && !src.pool_fused ? &src.rAfull : nullptr;
         Res* rpart = src.split_f > 1 ? &src.rPartF : nullptr;
         LP_CUDA(c, task_begin(c, sc, {rin, rwv}, {rout, rz, rpool, rfull, rpart}));
         LP_CUDA(c, launch_forward(c, k - 1, n, slot[k - 1], chain, true));
-        if (src.pool) LP_CUDA(c, launch_pool(c, k - 1, n, chain, true));
+        if (rfull) LP_CUDA(c, launch_pool(c, k - 1, n, chain, true));
         LP_CUDA(c, task_end(c, sc, {rin, rwv}, {rout, rz, rpool, rfull, rpart}, nullptr));
       }
     }
@@ -1702,7 +1720,7 @@ extern "C" int lp_debug_run_task(lp_handle h, int task, int layer, long long ste
   switch (task) {
     case LP_TASK_FORWARD:
       LP_CUDA(h, launch_forward(h, layer, step, slot, st));
-      if (h->L[layer].pool) LP_CUDA(h, launch_pool(h, layer, step, st));
+      if (h->L[layer].pool && !h->L[layer].pool_fused) LP_CUDA(h, launch_pool(h, layer, step, st));
       break;
     case LP_TASK_LOSS: {
       Layer& yl = h->L[nL - 1];
