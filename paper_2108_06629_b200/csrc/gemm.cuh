@@ -159,6 +159,12 @@ struct TileMap {
   int pn0, ph0, pw0;  // GEOM_PIX_M: first image / row / column of the pixel box
   int roff_h = 0, roff_w = 0;   // GEOM_PIX_M: residue class of the rows (strided delta)
 };
+// GEOM_PIX_M: image, row and column of the pixel that tile row `tr` indexes.
+__device__ __forceinline__ void tile_pixel(const GemmArgs& p, const TileMap& t, int tr, int& n, int& h, int& w) {
+  w = (t.pw0 + (tr & ((1 << p.g.lw) - 1))) * p.g.rs + t.roff_w;
+  h = (t.ph0 + ((tr >> p.g.lw) & ((1 << p.g.lh) - 1))) * p.g.rs + t.roff_h;
+  n = t.pn0 + (tr >> (p.g.lw + p.g.lh));
+}
 // Global row index of tile row `tr` (0..127), or -1 if the row does not exist.
 __device__ __forceinline__ int tile_row(const GemmArgs& p, const TileMap& t, int tr) {
   if (p.g.kind != GEOM_PIX_M) {
@@ -372,13 +378,24 @@ __device__ __forceinline__ void epilogue_rows8(const GemmArgs& p, const TileMap&
     }
   } else if constexpr (MODE == EPI_DGRAD_UNPOOL) {
     if (n >= N) return;
+    // The window of an element without a division per element (unpool_pos takes five; they were two thirds of this
+    // epilogue): of a convolution from the tile's pixel box, of a fully connected layer from the column, once.
+    const bool pix = p.g.kind == GEOM_PIX_M;
     UnpoolPos u[8];
     uint32_t idx[8];
     uint2 av[8];
+    const int px = pix ? 0 : n / p.pool_C, ch = n - px * p.pool_C, col_h = pix ? 0 : px / p.pool_Wp, col_w = px - col_h * p.pool_Wp;
 #pragma unroll
     for (int i8 = 0; i8 < 8; ++i8) {
       if (rows[i8] < 0) continue;
-      u[i8] = unpool_pos(p, rows[i8], n);
+      u[i8].c = ch;
+      if (pix) {
+        tile_pixel(p, tm, q * 32 + i8 * 4 + sub_row, u[i8].pn, u[i8].ph, u[i8].pw);
+        u[i8].pp = rows[i8];
+      } else {
+        u[i8].pn = rows[i8]; u[i8].ph = col_h; u[i8].pw = col_w;
+        u[i8].pp = rows[i8] * p.pool_ppr + px;
+      }
       idx[i8] = *reinterpret_cast<const uint32_t*>(p.pool_idx + size_t(u[i8].pp) * p.pool_C + u[i8].c);
       av[i8] = *reinterpret_cast<const uint2*>(p.aux + size_t(u[i8].pp) * p.ld_aux + u[i8].c);
     }
