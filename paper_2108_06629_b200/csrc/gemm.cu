@@ -2,7 +2,7 @@
 // stand-alone lp_gemm_bf16 entry point.
 #include "gemm2q.cuh"
 #include "gemmc.cuh"
-#include "conv_halo.cuh"
+#include "conv_wide.cuh"
 
 #include <algorithm>
 #include <atomic>
@@ -466,6 +466,25 @@ cudaError_t conv_halo_launch(int which, const CUtensorMap& tmA, const CUtensorMa
   return cudaErrorInvalidValue;
 }
 
+#define LP_FOR_EACH_WIDE_VARIANT(X)                                                                            \
+  X(64, false, EPI_FPROP) X(64, true, EPI_DGRAD) X(64, true, EPI_DGRAD_UNPOOL)                                 \
+  X(128, false, EPI_FPROP) X(128, true, EPI_DGRAD) X(128, true, EPI_DGRAD_UNPOOL)
+cudaError_t conv_wide_launch(int which, int bn, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& args, cudaStream_t st) {
+  const bool b_mn = (which != 0);
+  GemmArgs a = args;
+  if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
+  const int tiles = a.g.tiles_w * a.g.tiles_h * (a.M / (a.g.H * a.g.W)), tiles_n = (a.N - a.n_begin + bn - 1) / bn;
+  const int grid = std::min((tiles + 1) / 2 * tiles_n, sm_count());
+#define LP_TRYW(BN, B, M)                                                                                      \
+  if (bn == BN && b_mn == B && a.mode == M) {                                                                  \
+    conv_wide_kernel<BN, B, M><<<grid, WIDE_THREADS, wide_smem_bytes(BN), st>>>(tmA, tmB, a, tiles, tiles_n);  \
+    return cudaGetLastError();                                                                                 \
+  }
+  LP_FOR_EACH_WIDE_VARIANT(LP_TRYW)
+#undef LP_TRYW
+  return cudaErrorInvalidValue;
+}
+
 // G of a halo-tile layer: accumulate over 8 x 16 pixel tiles, then add the CTAs' partial sums and
 // apply the update (upd.W null: store G only).
 cudaError_t conv_halo_g_launch(const CUtensorMap& tmX, const CUtensorMap& tmD, const ConvGeom& g, int batch, float* partial,
@@ -499,6 +518,12 @@ cudaError_t gemm_configure() {
     return e;
   LP_FOR_EACH_HALO_VARIANT(LP_CFGH)
 #undef LP_CFGH
+#define LP_CFGW(BN, B, M)                                                                                      \
+  if ((e = cudaFuncSetAttribute(conv_wide_kernel<BN, B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
+                                wide_smem_bytes(BN))) != cudaSuccess)                                          \
+    return e;
+  LP_FOR_EACH_WIDE_VARIANT(LP_CFGW)
+#undef LP_CFGW
 #define LP_CFGP(A, B, M) \
   if ((e = configure_pair<A, B, M>()) != cudaSuccess) return e;
   LP_FOR_EACH_PAIR_VARIANT(LP_CFGP)

@@ -104,6 +104,7 @@ struct Layer {
   // 3x3 layers with at most 64 channels on both sides and images tiled by 8 x 16 pixels: the
   // activation / delta box is fetched once per tile with its halo (see conv_halo.cuh)
   bool halo_f = false, halo_d = false, halo_g = false;
+  bool wide_f = false, wide_d = false;          // the same idea with more channels (conv_wide.cuh)
   std::vector<CUtensorMap> tm_hg_D;             // delta as 8 x 16 pixel boxes (the halo-tile G kernel)
   bool lean_f = false;                          // patch-matrix layer with at most 64 output channels: forward through the same kernel
   std::vector<CUtensorMap> tm_hf_A, tm_hd_A;    // halo boxes over the stash slots / the delta slots
@@ -472,6 +473,12 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       y.halo_f = !y.patch && tiles_8x16 && y.ld_in <= 64 && y.n_out <= 64;
       y.halo_d = l > 0 && tiles_8x16 && y.ld_out <= 64 && y.n_in <= 64;
       y.halo_g = y.halo_f;   // (128 output channels in two passes of the G kernel measured slower than the split-K kernel: 182 / 160 us)
+      // more channels on such images: two halo tiles under streamed weight taps, where a tap feeds 128 columns from at
+      // least two 64-channel chunks and every CTA gets at least four items (measured in conv_wide.cuh; with one item each,
+      // 16 x 16 pixels at batch 128, 16 steps of the small VGG took 4520 us against 4390)
+      const long long pairs_of_tiles = (long long)B * (y.imW / 8) * (y.imH / 16) / 2;
+      y.wide_f = !y.patch && tiles_8x16 && y.ld_in > 64 && y.bn_f == 128 && pairs_of_tiles * ((y.n_out + 127) / 128) >= 4 * 148;
+      y.wide_d = l > 0 && tiles_8x16 && y.ld_out > 64 && y.bn_d == 128 && pairs_of_tiles * ((y.n_in + 127) / 128) >= 4 * 148;
       y.lean_f = y.patch && y.n_out <= 64 && y.ld_in <= 64 && l + 1 < n;
       // G contracts over all B*H*W pixels but has only (Cout/128) x 9 x (Cin/BN) tiles: the pixel
       // range is split, and a second launch adds the partial tiles on all SMs and applies the update
@@ -638,7 +645,7 @@ static int build_tensor_maps(lp_ctx* c) {
         if ((rc = make_tmap_bf16_nhwc(&y.tm_g_A[s], y.delta + s * y.delta_elems, y.ld_out, y.oW, y.oH, B, y.ld_out,
                                       y.box64.bw, y.box64.bh, y.box64.bn, &err)) != LP_OK) return fail(c, rc, err);
       }
-      if (y.halo_f || y.halo_g) {      // the halo box over the stashed input (forward and G)
+      if (y.halo_f || y.halo_g || y.wide_f) {      // the halo box over the stashed input (forward and G)
         y.tm_hf_A.resize(y.x_slots);
         for (int s = 0; s < y.x_slots; ++s)
           if ((rc = make_tmap_bf16_nhwc(&y.tm_hf_A[s], y.X + s * y.x_elems, y.ld_in, y.imW, y.imH, B, y.ld_in, HALO_W, HALO_H, 1,
@@ -668,7 +675,7 @@ static int build_tensor_maps(lp_ctx* c) {
           if ((rc = make_tmap_bf16_nhwc(&y.tm_hd_O[s], pv.delta + s * pv.delta_elems, pv.ld_out, y.imW, y.imH, B, pv.ld_out, 8, 16, 1,
                                         &err)) != LP_OK) return fail(c, rc, err);
       }
-      if (y.halo_d) {
+      if (y.halo_d || y.wide_d) {
         y.tm_hd_A.resize(kDeltaSlots);
         for (int s = 0; s < kDeltaSlots; ++s)
           if ((rc = make_tmap_bf16_nhwc(&y.tm_hd_A[s], y.delta + s * y.delta_elems, y.ld_out, y.imW, y.imH, B, y.ld_out, HALO_W,
@@ -871,6 +878,11 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
     const CUtensorMap& tmo = y.pool_fused ? y.tm_hf_A[xin] : y.tm_hf_O[xout];
     return conv_halo_launch(0, y.tm_hf_A[xin], y.tm_f_B[ring_slot], tmo, a, st);
   }
+  if (y.wide_f) {
+    a.g = halo_geom(y, 0);
+    a.g.chunks_per_tap = (y.ld_in + 63) / 64;
+    return conv_wide_launch(0, y.bn_f, y.tm_hf_A[xin], y.tm_f_B[ring_slot], a, st);
+  }
   return gemm_launch(0, y.bn_f, y.tm_f_A[xin], y.tm_f_B[ring_slot], a, st);
 }
 
@@ -937,6 +949,11 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
     a.g = halo_geom(y, 1);
     return conv_halo_launch(1, y.tm_hd_A[n % kDeltaSlots], y.tm_d_B[ring_slot],
                             pv.pool ? y.tm_hd_A[0] : y.tm_hd_O[n % kDeltaSlots], a, st);
+  }
+  if (y.wide_d) {
+    a.g = halo_geom(y, 1);
+    a.g.chunks_per_tap = (y.ld_out + 63) / 64;
+    return conv_wide_launch(1, y.bn_d, y.tm_hd_A[n % kDeltaSlots], y.tm_d_B[ring_slot], a, st);
   }
   if (y.conv && y.cstride > 1) {
     // Strided layer: input pixel (h, w) is reached through tap (r, s) only when h + pad - r and

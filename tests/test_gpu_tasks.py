@@ -429,3 +429,20 @@ def test_tasks_bias_gradient_of_many_rows(rows, n_out):
         assert np.max(np.abs(tr.debug_read("grad_b", 0, 0) - g)) < bound
         assert np.max(np.abs(tr.debug_read("master_b", 0, 0) - b)) < 2 * bound + 2.0 ** -22 * np.max(np.abs(b))
     tr.close()
+
+
+@pytest.mark.parametrize("H, W, B, chans, pools", [(16, 8, 3, [72, 136, 40], [0, 0, 2]), (32, 16, 2, [96, 200, 72], [0, 2, 2]),
+                                                   (16, 16, 8, [64, 128, 128], [0, 2, 0]), (16, 24, 16, [80, 24, 160], [0, 0, 2])])
+def test_tasks_two_halo_tiles_under_streamed_weights(H, W, B, chans, pools):
+    """Convolutions of more than 64 channels on 8 x 16 pixel tiles: an odd number of tiles (the last pair holds one),
+    channel counts that end inside a 64-channel chunk or a column tile, several column tiles, delta onto 64 or fewer
+    channels, pooled in the epilogue or not, and un-pooling."""
+    from paper_2108_06629_b200 import inputs as I
+    layers, c = [], 3
+    for n, pool in zip(chans, pools):
+        layers.append(I.conv(c, n, H, W, pool=pool))
+        c = n
+        if pool:
+            H, W = H // 2, W // 2
+    layers.append(I.fc(c * H * W, 10, "none"))
+    run_teacher_forced(layers, B, 2, None, 0.05, 0.9, 2)
