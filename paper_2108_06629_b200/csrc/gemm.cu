@@ -498,7 +498,7 @@ cudaError_t conv_halo_g_launch(const CUtensorMap& tmX, const CUtensorMap& tmD, c
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     upd.co0 = co0;
-    conv_halo_g_update_kernel<0><<<(HALOG_PART_FLOATS + 255) / 256, 256, 0, st>>>(upd);
+    conv_halo_g_update_kernel<0><<<HALOG_PART_FLOATS / 32, 256, 0, st>>>(upd);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
