@@ -106,6 +106,22 @@ EXPORTS = ["lp_plan", "lp_plan_costs", "lp_workspace_size", "lp_create", "lp_ste
            "lp_gemm_bf16", "lp_gemm_status", "lp_debug_gemm_starved", "lp_softmax_xent_static"]
 
 
+_torch = None
+
+
+def _stream_of(stream, device=None):
+    """The caller's stream as an integer: `stream` itself, or the current stream of `device` (None: of the current device).
+    The raw lookup costs a tenth of building a torch.cuda.Stream object, which took 2 us of a 12 us contraction call."""
+    if stream is not None:
+        return stream
+    global _torch
+    if _torch is None:
+        import torch
+        torch.cuda.init()
+        _torch = torch
+    return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice() if device is None else device)
+
+
 def _check(rc, h=None):
     if rc != LP_OK:
         raise LayerPipeError(rc, (lib().lp_last_error(h) or b"").decode())
@@ -182,6 +198,7 @@ class Trainer:
         self.batch = batch
         self.device = torch.device(device)
         torch.cuda.set_device(self.device)
+        self.device_index = torch.cuda.current_device()
         L = lib()
         n = len(layers)
         arr = _layers_array(layers)
@@ -211,13 +228,10 @@ class Trainer:
 
     # ---- the calls ---------------------------------------------------------
     def step(self, batch_dev, labels_dev, stream=None):
-        s = self.torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream
-        _check(lib().lp_step(self.h, C.c_void_p(batch_dev.data_ptr()), C.c_void_p(labels_dev.data_ptr()),
-                             C.c_void_p(s)), self.h)
+        _check(_lib.lp_step(self.h, batch_dev.data_ptr(), labels_dev.data_ptr(), _stream_of(stream, self.device_index)), self.h)
 
     def flush(self, stream=None):
-        s = self.torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream
-        _check(lib().lp_flush(self.h, C.c_void_p(s)), self.h)
+        _check(_lib.lp_flush(self.h, _stream_of(stream, self.device_index)), self.h)
 
     def get_weights(self, layer):
         l = self.layers[layer]
@@ -358,10 +372,7 @@ class Trainer:
 
 def lp_gemm_bf16(which, M, N, K, A, lda, B, ldb, Cout, ldc, stream=None):
     """A, B: torch bf16 device tensors; Cout: torch fp32 device tensor."""
-    import torch
-    s = torch.cuda.current_stream().cuda_stream if stream is None else stream
-    _check(lib().lp_gemm_bf16(which, M, N, K, C.c_void_p(A.data_ptr()), lda, C.c_void_p(B.data_ptr()), ldb,
-                              C.c_void_p(Cout.data_ptr()), ldc, C.c_void_p(s)))
+    _check(lib().lp_gemm_bf16(which, M, N, K, A.data_ptr(), lda, B.data_ptr(), ldb, Cout.data_ptr(), ldc, _stream_of(stream)))
 
 
 def lp_gemm_status():
@@ -386,9 +397,5 @@ def lp_softmax_xent_static(logits, labels, delta, loss, classes, stream=None):
     """Loss kernel on caller-owned torch tensors, no handle and no allocation inside the
     library: logits fp32 [batch][ld], labels int32 [batch], delta bf16 [batch][ld_delta]
     (output), loss fp32 [1] (output).  Returns the library's status code."""
-    import torch
-    s = torch.cuda.current_stream().cuda_stream if stream is None else stream
-    return lib().lp_softmax_xent_static(C.c_void_p(logits.data_ptr()), logits.stride(0),
-                                        C.c_void_p(labels.data_ptr()), C.c_void_p(delta.data_ptr()),
-                                        delta.stride(0), C.c_void_p(loss.data_ptr()), logits.shape[0], classes,
-                                        C.c_void_p(s))
+    return lib().lp_softmax_xent_static(logits.data_ptr(), logits.stride(0), labels.data_ptr(), delta.data_ptr(),
+                                        delta.stride(0), loss.data_ptr(), logits.shape[0], classes, _stream_of(stream))
