@@ -161,7 +161,7 @@ struct lp_ctx {
   // record at or after it (or records one), so a record that has been overwritten only makes a later wait coarser,
   // never wrong.  `vc` = what the stream had waited for by then (per stream, the last task known complete).
   struct Rec { long long pos = 0; cudaEvent_t e = nullptr; long long vc[kMaxStreams] = {}; };
-  static constexpr int kRecs = 256;
+  static constexpr int kRecs = 128;
   struct StreamLog {
     long long pos = 0;                        // tasks enqueued
     long long n_rec = 0;                      // records made; record k lives in rec[k % kRecs]
