@@ -551,6 +551,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   uint64_t* accf_bar = empty_bar + GEMM_MAX_STAGES;     // [2] accumulator buffer full  (MMA -> epilogue)
   uint64_t* acce_bar = accf_bar + 2;                    // [2] accumulator buffer empty (epilogue -> MMA)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce_bar + 2);
+  uint64_t* ufull_bar = acce_bar + 4;                   // [GEMM_MAX_STAGES] chunk fills of the streamed update (UTMA)
   // Staging tiles of the epilogue.  With one tile per CTA they reuse pipeline stage 0 (by the time
   // the accumulator barrier fires every load has landed and every MMA has read its operands);
   // a CTA that loops over tiles keeps loading while the epilogue runs and needs its own space.
@@ -563,6 +564,11 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   // stage ring: 128 x 32 fp32 of the master and of the momentum).  The epilogue updates a chunk
   // in place in shared memory and a TMA store writes it back, so the HBM stream of Eq. 6 is
   // queued by the copy engine, many chunks deep, instead of by the registers of four warps.
+  // A stage completes its operand fills on full_bar (only the MMA issuer waits there) and its chunk fills on
+  // ufull_bar (only the epilogue), each with a phase count of its own: a parity wait tells adjacent phases apart and no
+  // more, so nobody but a barrier's waiters may let its next phase start.  With one barrier for both kinds a
+  // persistent CTA's issuer had to look at every chunk fill, but the epilogue alone handed the stages back: an issuer
+  // that came late by one chunk's epilogue and one load met the phase after the one it waited for, for ever.
   // (UTMA is a template parameter, not a flag: the register-path update keeps 128 registers of
   // prefetched tiles per thread, and a kernel that contains both forms is allocated for the larger --
   // two resident CTAs then own the whole register file and no other stream's block fits beside them.)
@@ -583,6 +589,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     for (int s = 0; s < S; ++s) {
       mbar_init(&full_bar[s], 1);
       mbar_init(&empty_bar[s], 1);
+      if (UTMA) mbar_init(&ufull_bar[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf_bar[b], 1);
@@ -617,6 +624,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       const uint32_t smem0 = smem_u32(smem);
       const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
       uint32_t s = 0, ph = 0;
+      uint32_t op_ph = 0, ch_ph = 0, is_chunk = 0;   // UTMA, a bit per stage: parity of the next operand / chunk fill, kind of the last fill
       for (int t = blockIdx.x; t < total_work && ok; t += (PERSIST ? int(gridDim.x) : total_work)) {
         const TileCtx tc = decode_tile<BN>(p, t, tiles_m, tiles_n);
         const TileMap& tm = tc.tm;
@@ -723,20 +731,24 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
           }
           ++issued;
+          if (UTMA) { op_ph ^= 1u << s; is_chunk &= ~(1u << s); }
           if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
         }
         if constexpr (kUpdTmaOk) {
           if (upd_tma && ok) {
+            const uint32_t ufull0 = smem_u32(ufull_bar);
             const uint32_t bytes = p.mW != nullptr ? 2u * UPD_CHUNK_BYTES : uint32_t(UPD_CHUNK_BYTES);
             for (int c = 0; c < kChunks; ++c) {
               ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
               if (!ok) break;
               const uint32_t sa = smem0 + s * uint32_t(SM::STAGE_BYTES);
-              const uint32_t fb = full0 + 8u * s;
+              const uint32_t fb = ufull0 + 8u * s;
               mbar_arrive_expect_tx_addr(fb, bytes);
               tma_load_2d_addr(sa, &um.W, fb, tm.n0 + c * 32, tm.m0);
               if (p.mW != nullptr) tma_load_2d_addr(sa + UPD_CHUNK_BYTES, &um.M, fb, tm.n0 + c * 32, tm.m0);
               ++issued;
+              ch_ph ^= 1u << s;
+              is_chunk |= 1u << s;
               if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
             }
           }
@@ -745,7 +757,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       if (!ok) {
         atomicExch(p.status, 1);
         // let copies already in flight land before the CTA's shared memory is released
-        for (long long i = (issued > S ? issued - S : 0); i < issued; ++i) mbar_wait(&full_bar[i % S], uint32_t(i / S) & 1u, p.wait_limit);
+        for (long long i = (issued > S ? issued - S : 0); i < issued; ++i) {
+          const int k = int(i % S);
+          if (UTMA) {
+            const bool ch = (is_chunk >> k) & 1u;
+            mbar_wait(ch ? &ufull_bar[k] : &full_bar[k], (((ch ? ch_ph : op_ph) >> k) & 1u) ^ 1u, p.wait_limit);
+          } else {
+            mbar_wait(&full_bar[k], uint32_t(i / S) & 1u, p.wait_limit);
+          }
+        }
       }
     }
   } else if (warp == 1) {
@@ -777,8 +797,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const uint32_t tacc = tmem_base + buf * uint32_t(BN);
         uint32_t acc = 0;
         for (int kb = 0; kb < tc.num_kb; ++kb) {
-          ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
+          ok = mbar_wait_addr(full0 + 8u * s, UTMA ? (ph >> s) & 1u : ph, p.wait_limit);
           if (!ok) break;
+          if (UTMA) ph ^= 1u << s;             // (a bit per stage: not every turn of the ring brings operands)
           tc_fence_after();
 #pragma unroll
           for (int j = 0; j < GEMM_BK / 16; ++j) {
@@ -790,32 +811,17 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           dB_lo += uint32_t(SM::STAGE_BYTES >> 4);
           if (++s == uint32_t(S)) {
             s = 0;
-            ph ^= 1u;
+            if (!UTMA) ph ^= 1u;
             dA_lo = uint32_t(dA);
             dB_lo = uint32_t(dB);
           }
         }
         umma_commit_addr(accf0 + 8u * buf);    // accumulator complete (also releases the epilogue on error)
-        if constexpr (kUpdTmaOk) {
-          if (upd_tma) {
-            // The tile's chunk fills pass through the ring without this warp.  A CTA that goes on
-            // to another tile still has to SEE each of them complete: a parity wait only tells
-            // adjacent phases apart, and a stage may not run two phases ahead of a waiter.
-            for (int c = 0; c < kChunks; ++c) {
-              if (PERSIST) {
-                ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-                if (!ok) break;
-              }
-              dA_lo += uint32_t(SM::STAGE_BYTES >> 4);
-              dB_lo += uint32_t(SM::STAGE_BYTES >> 4);
-              if (++s == uint32_t(S)) {
-                s = 0;
-                ph ^= 1u;
-                dA_lo = uint32_t(dA);
-                dB_lo = uint32_t(dB);
-              }
-            }
-          }
+        if constexpr (kUpdTmaOk && PERSIST) {
+          // the tile's chunk fills pass through the ring without this warp
+          s = (s + kChunks) % uint32_t(S);
+          dA_lo = uint32_t(dA) + s * uint32_t(SM::STAGE_BYTES >> 4);
+          dB_lo = uint32_t(dB) + s * uint32_t(SM::STAGE_BYTES >> 4);
         }
       }
       if (!ok) atomicExch(p.status, 2);
@@ -837,7 +843,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     bool ok = true;
     uint32_t it = 0;
     // TMA update path: position in the stage ring, and the store whose source has not been released yet
-    uint32_t us = 0, uph = 0, pending_stage = 0;
+    uint32_t us = 0, uph = 0, pending_stage = 0;       // (uph: a bit per stage, the parity of its next chunk fill)
     bool pending = false, good = true;
     for (int t = blockIdx.x; t < total_work && ok; t += (PERSIST ? int(gridDim.x) : total_work), ++it) {
       const TileCtx tc = decode_tile<BN>(p, t, tiles_m, tiles_n);
@@ -849,8 +855,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (upd_tma) {
           // Every one of the 128 epilogue threads runs the same number of named barriers whatever
           // happens: after a wait that ran out, the remaining chunks only keep the barrier count.
-          const uint32_t smem0 = smem_u32(smem), full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
-          const uint32_t ringbuf = full0 + 1024u;
+          const uint32_t smem0 = smem_u32(smem), ufull0 = smem_u32(ufull_bar), empty0 = smem_u32(empty_bar);
+          const uint32_t ringbuf = smem_u32(full_bar) + 1024u;
           const int trow = q * 32 + lane;            // row of the tile this lane owns (tensor-memory lane)
           if (p.bdelta != nullptr && tm.n0 == 0 && tm.m0 + trow < p.M) {
             // Bias of output feature m = column sum of delta over the batch, then Eq. 6 -- while
@@ -885,17 +891,17 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             if (!good && lane == 0) atomicExch(p.status, 3);
           }
           tc_fence_after();
-          for (int kb = 0; kb < tc.num_kb; ++kb)       // the operand fills of this tile
-            if (++us == uint32_t(S)) { us = 0; uph ^= 1u; }
+          us = (us + uint32_t(tc.num_kb)) % uint32_t(S);     // the operand fills of this tile
 #pragma unroll 1
           for (int c = 0; c < kChunks; ++c) {
             const uint32_t sW = smem0 + us * uint32_t(SM::STAGE_BYTES);
             const uint32_t sM = sW + UPD_CHUNK_BYTES;
             if (good) {
-              good = mbar_wait_addr(full0 + 8u * us, uph, p.wait_limit);
+              good = mbar_wait_addr(ufull0 + 8u * us, (uph >> us) & 1u, p.wait_limit);
               good = __all_sync(0xffffffffu, good);
               if (!good && lane == 0) atomicExch(p.status, 4);
             }
+            uph ^= 1u << us;
             uint32_t packed[16];
             if (good) {
               uint32_t r[32];
@@ -984,7 +990,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 mbar_arrive_addr(empty0 + 8u * us);   // keep the producer's bounded waits short
               }
             }
-            if (++us == uint32_t(S)) { us = 0; uph ^= 1u; }
+            if (++us == uint32_t(S)) us = 0;
           }
           continue;
         }
