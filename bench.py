@@ -306,6 +306,13 @@ class Workload:
                            schedule=schedule, flags=flags, W0=self.W0, b0=self.b0, device=self.dev)
 
 
+def check_status(lpb, tr):
+    """Ends the run if a bounded wait ran out in a kernel of this handle, with what the status block says about it."""
+    rc, detail = tr.device_status()
+    if rc != 0:
+        raise SystemExit("device status %d (%d): %s" % (rc, detail, lpb.lib().lp_last_error(tr.h).decode()))
+
+
 def throughput(torch, lpb, w, schedule, steps, warmup, min_seconds, stream, flags=0, before_timing=None):
     """samples/s of one handle: warm-up (fills every ring), then repeated blocks of `steps` steps."""
     tr = w.trainer(lpb, schedule, flags)
@@ -322,9 +329,7 @@ def throughput(torch, lpb, w, schedule, steps, warmup, min_seconds, stream, flag
     launches = (tr.kernel_launches() - l0) // len(ts)
     if TRACE:
         note(tr.task_progress())
-    rc, detail = tr.device_status()
-    if rc != 0:
-        raise SystemExit("device status %d (%d)" % (rc, detail))
+    check_status(lpb, tr)
     return tr, ts, launches, prewarm, (stage, delays, slots)
 
 
@@ -480,12 +485,10 @@ def borrowing_report(torch, lpb, w, args, stream):
             tr.flush()
             torch.cuda.synchronize()
             ts = repeat_blocks(lambda: timed_block(torch, tr, w.xs, w.ys, steps, stream), 0.5)
-            rc, detail = tr.device_status()
+            check_status(lpb, tr)
             tr.close()
             del tr
             torch.cuda.empty_cache()
-            if rc != 0:
-                raise SystemExit("device status %d (%d)" % (rc, detail))
             sm = summarize(ts, steps)
             out["variants"]["%s%s" % (pname, "+split" if split else "")] = {
                 "samples_per_s": w.B / (sm["ms_per_step"] * 1e-3), "ms_per_step": sm["ms_per_step"], "stage": plan["stage"],
@@ -656,12 +659,10 @@ def free_running_selfcheck(torch, lpb, w, sched, steps=6):
         tr.flush()
         torch.cuda.synchronize()
         losses.append([tr.get_loss(k) for k in range(steps)])
-        rc, detail = tr.device_status()
+        check_status(lpb, tr)
         tr.close()
         del tr
         torch.cuda.empty_cache()
-        if rc != 0:
-            raise SystemExit("device status %d (%d)" % (rc, detail))
     same = losses[0] == losses[1]
     out = {"steps": steps, "free_running_losses_equal_serialised": same, "last_loss": losses[0][-1]}
     if not same:      # reported, loudly, with the line: the reader decides what the timing is worth

@@ -238,8 +238,9 @@ int lp_get_version_log(lp_handle h, long long step, int* v_fwd, int* v_bwd, int*
  * until that step's loss kernel has finished. */
 int lp_get_loss(lp_handle h, long long step, float* loss);
 
-/* 0, or the status word written by a kernel: a bounded wait that expired (values 1..26: returns
- * LP_ERR_TIMEOUT), or a label outside [0, classes) met by the loss kernel (value 64: returns
+/* 0, or the status word written by a kernel: a bounded wait that expired (values 1..33: returns
+ * LP_ERR_TIMEOUT; every role of every kernel has a value of its own, listed in csrc/wait_codes.h, the word
+ * keeps the first one, and lp_last_error names it and the CTA, tile and k-block it stood at), or a label outside [0, classes) met by the loss kernel (value 64: returns
  * LP_ERR_INVALID_ARG; that row contributes no one-hot term and the minibatch's loss is NaN --
  * the label is never used as an address).  *detail receives the word.  Blocks until the device
  * is idle. */
@@ -301,8 +302,8 @@ int lp_gemm_bf16(int which, int M, int N, int K, const void* A_dev, int lda,
 
 /* Status word of the lp_gemm_bf16 launches on the current device since the last call: waits for
  * the device, returns LP_OK (word 0) or LP_ERR_TIMEOUT (a bounded wait inside a kernel ran out;
- * *detail, may be NULL, receives the word: 1 producer, 2 MMA issuer, 3 / 4 epilogue, 11..13 the
- * same roles of the SM-pair kernel), and clears the word. */
+ * *detail, may be NULL, receives the word: 1 producer, 2 MMA issuer, 3 / 4 epilogue, 5..7 the same
+ * roles of the form divided over a cluster, 11..13 and 24..26 those of the SM-pair kernels), and clears the word. */
 int lp_gemm_status(int* detail);
 
 /* Verification of the bounded waits (Eq. 1 contraction as lp_gemm_bf16 with which = 0, K > 64).

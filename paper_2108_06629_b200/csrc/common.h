@@ -10,12 +10,20 @@
 #include <vector>
 
 #include "../../include/layerpipe.h"
+#include "wait_codes.h"
 
 namespace lp {
 
 // ---- lp_api.cu --------------------------------------------------------------
 // Error text of calls that have no handle: what lp_last_error(NULL) returns on this thread.
 void set_global_error(const std::string& msg);
+// What a status block says: which role of which kernel gave up first, and where it stood.
+inline std::string expired_text(const int* st) {
+  const int code = st[STATUS_CODE];
+  return std::string("a bounded device-side wait expired: ") + wait_code_role(code) + " of the " + wait_code_name(code) + " kernel (status " +
+         std::to_string(code) + "; CTA " + std::to_string(st[STATUS_CTA]) + ", tile " + std::to_string(st[STATUS_TILE]) + ", step " +
+         std::to_string(st[STATUS_STEP]) + ")";
+}
 
 // ---- gemm.cu ---------------------------------------------------------------
 // Encode a 2-D bf16 tensor map (128-byte swizzle, zero fill out of bounds).
@@ -94,7 +102,7 @@ cudaError_t launch_trace_mark(unsigned* flag, unsigned value, cudaStream_t strea
 // ticket: count of finished blocks, zero between launches
 cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __nv_bfloat16* delta, int ldd, float* row_loss,
                                 unsigned* ticket, float* loss_out, int B, int C, int* status, cudaStream_t stream);
-// Value of a device status word that does not come from a bounded wait (those are 1..23).
+// Value of a device status word that does not come from a bounded wait (those are in wait_codes.h).
 constexpr int LP_STATUS_BAD_LABEL = 64;   // a label outside [0, classes) reached the loss kernel
 struct UpdateArgs {
   const float* dW;      // [out][ldw] fp32 (pad lanes zero)

@@ -94,7 +94,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         pixel_tile(min(2 * tp + 1, tiles_total - 1), t1);   // (an odd last tile is computed twice, stored once)
         for (int c = 0; c < chunks && ok; ++c) {
           ok = mbar_wait_addr(aempty0 + 8u * as, aph ^ 1u, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_WIDE_PRODUCER, it, 9 * c); break; }
           mbar_arrive_expect_tx_addr(afull0 + 8u * as, uint32_t(WIDE_A_BYTES));
           const uint32_t sa = sA0 + as * uint32_t(WIDE_A_BYTES);
           tma_load_4d_addr(sa, &tmA, afull0 + 8u * as, c * 64, t0.pw0 - 1, t0.ph0 - 1, t0.pn0);
@@ -104,7 +104,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           int col = 0;
           for (int tap = 0; tap < 9; ++tap, col += p.g.tap_pitch) {
             ok = mbar_wait_addr(bempty0 + 8u * bs, bph ^ 1u, p.wait_limit);
-            if (!ok) break;
+            if (!ok) { report_expired(p.status, WAIT_WIDE_PRODUCER, it, 9 * c + tap); break; }
             const uint32_t fb = bfull0 + 8u * bs, sb = sB0 + bs * uint32_t(B_BYTES);
             mbar_arrive_expect_tx_addr(fb, uint32_t(B_BYTES));
             if (B_MN) {        // delta: B[k = (tap, co)][n = ci]
@@ -119,7 +119,6 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
       }
       if (!ok) {
-        atomicExch(p.status, 31);
         // let copies already in flight land before the CTA's shared memory is released
         for (int i = max(0, ia - WIDE_A_STAGES); i < ia; ++i) mbar_wait(&afull[i % WIDE_A_STAGES], uint32_t(i / WIDE_A_STAGES) & 1u, p.wait_limit);
         for (int i = max(0, ib - WIDE_B_STAGES); i < ib; ++i) mbar_wait(&bfull[i % WIDE_B_STAGES], uint32_t(i / WIDE_B_STAGES) & 1u, p.wait_limit);
@@ -146,18 +145,18 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       for (int it = blockIdx.x; it < items && ok; it += gridDim.x, ++n_it) {
         const uint32_t buf = n_it & 1u;
         ok = mbar_wait_addr(acce0 + 8u * buf, ((n_it >> 1) & 1u) ^ 1u, p.wait_limit);
-        if (!ok) break;
+        if (!ok) { report_expired(p.status, WAIT_WIDE_MMA, it, -1); break; }
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * 256u;        // accumulators of the two pixel tiles: columns 0 and 128 of the buffer
         uint32_t acc = 0;
         for (int c = 0; c < chunks && ok; ++c) {
           ok = mbar_wait_addr(afull0 + 8u * as, aph, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_WIDE_MMA, it, 9 * c); break; }
           const uint32_t a_lo = uint32_t(dA) + as * uint32_t(WIDE_A_BYTES >> 4);
 #pragma unroll
           for (int tap = 0; tap < 9; ++tap) {
-            if (ok) ok = mbar_wait_addr(bfull0 + 8u * bs, bph, p.wait_limit);
-            if (!ok) break;
+            ok = mbar_wait_addr(bfull0 + 8u * bs, bph, p.wait_limit);
+            if (!ok) { report_expired(p.status, WAIT_WIDE_MMA, it, 9 * c + tap); break; }
             tc_fence_after();
             const uint32_t b_lo = uint32_t(dB) + bs * uint32_t(B_BYTES >> 4);
 #pragma unroll
@@ -175,7 +174,6 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         umma_commit_addr(accf0 + 8u * buf);                  // (also releases the epilogue on error)
       }
-      if (!ok) atomicExch(p.status, 32);
     }
   } else {
     const int q = warp & 3;
@@ -194,7 +192,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       bool ok = mbar_wait_addr(accf0 + 8u * buf, (n_it >> 1) & 1u, p.wait_limit);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) {
-        if (lane == 0) atomicExch(p.status, 33);
+        if (lane == 0) report_expired(p.status, WAIT_WIDE_EPILOGUE, it, -1);
         break;
       }
       tc_fence_after();

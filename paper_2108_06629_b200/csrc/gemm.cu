@@ -588,8 +588,8 @@ cudaError_t gemm_set_tmem_table(int* table) {
 }
 }  // namespace lp
 
-// status word for the stand-alone entry point (handles keep theirs in the workspace)
-__device__ int g_gemm_status = 0;
+// status block of the stand-alone entry point (handles keep theirs in the workspace)
+__device__ int g_gemm_status[lp::STATUS_WORDS] = {};
 
 namespace {
 // Per device: the address of g_gemm_status there, and whether the kernels' shared-memory attributes
@@ -670,16 +670,16 @@ extern "C" int lp_gemm_status(int* detail) {
   int* status_dev = nullptr;
   int rc = gemm_device_setup(&status_dev);
   if (rc != LP_OK) return rc;
-  int st = 0;
-  const int zero = 0;
-  if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(&st, status_dev, 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(status_dev, &zero, 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+  int st[lp::STATUS_WORDS] = {};
+  const int zero[lp::STATUS_WORDS] = {};
+  if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(st, status_dev, sizeof st, cudaMemcpyDeviceToHost) != cudaSuccess ||
+      cudaMemcpy(status_dev, zero, sizeof zero, cudaMemcpyHostToDevice) != cudaSuccess) {
     lp::set_global_error("lp_gemm_status: a CUDA call failed");
     return LP_ERR_CUDA;
   }
-  if (detail) *detail = st;
-  if (st != 0) {
-    lp::set_global_error("lp_gemm_bf16: a bounded device-side wait expired (status " + std::to_string(st) + ")");
+  if (detail) *detail = st[lp::STATUS_CODE];
+  if (st[lp::STATUS_CODE] != 0) {
+    lp::set_global_error("lp_gemm_bf16: " + lp::expired_text(st));
     return LP_ERR_TIMEOUT;
   }
   return LP_OK;

@@ -125,7 +125,7 @@ struct GemmArgs {
   const __nv_bfloat16* bdelta;   // delta^l [brows][bld]
   int bld, brows;
   float *bb, *bmb, *bdb, *bbring;   // bias master, momentum (may be null), gradient, destination ring slot
-  int* status;              // device status word: set non-zero if a bounded wait expires
+  int* status;              // status block (STATUS_WORDS): the first bounded wait that expires writes it
   long long wait_limit;     // SM cycles after which a wait on a barrier gives up (0 at the call = the default, about 2 s)
   int tmem_policy;          // host side only, see TMEM_* below
   int* phase;               // diagnosis of a stall (LP_TRACE_TASKS): eight counters of CTAs past each phase of the pair kernel, or null
@@ -681,7 +681,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
           }
           ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_GEMM_PRODUCER, t, kb); break; }
           const uint32_t sa = smem0 + s * uint32_t(SM::STAGE_BYTES);
           const uint32_t sb = sa + GEMM_A_BYTES;
           const uint32_t fb = full0 + 8u * s;
@@ -740,7 +740,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const uint32_t bytes = p.mW != nullptr ? 2u * UPD_CHUNK_BYTES : uint32_t(UPD_CHUNK_BYTES);
             for (int c = 0; c < kChunks; ++c) {
               ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-              if (!ok) break;
+              if (!ok) { report_expired(p.status, WAIT_GEMM_PRODUCER, t, tc.num_kb + c); break; }
               const uint32_t sa = smem0 + s * uint32_t(SM::STAGE_BYTES);
               const uint32_t fb = ufull0 + 8u * s;
               mbar_arrive_expect_tx_addr(fb, bytes);
@@ -755,7 +755,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
       if (!ok) {
-        atomicExch(p.status, 1);
         // let copies already in flight land before the CTA's shared memory is released
         for (long long i = (issued > S ? issued - S : 0); i < issued; ++i) {
           const int k = int(i % S);
@@ -791,14 +790,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (PERSIST) {
           // the epilogue must have drained this accumulator buffer (tile it - 2)
           ok = mbar_wait_addr(acce0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_GEMM_MMA, t, -1); break; }
           tc_fence_after();
         }
         const uint32_t tacc = tmem_base + buf * uint32_t(BN);
         uint32_t acc = 0;
         for (int kb = 0; kb < tc.num_kb; ++kb) {
           ok = mbar_wait_addr(full0 + 8u * s, UTMA ? (ph >> s) & 1u : ph, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_GEMM_MMA, t, kb); break; }
           if (UTMA) ph ^= 1u << s;             // (a bit per stage: not every turn of the ring brings operands)
           tc_fence_after();
 #pragma unroll
@@ -824,7 +823,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           dB_lo = uint32_t(dB) + s * uint32_t(SM::STAGE_BYTES >> 4);
         }
       }
-      if (!ok) atomicExch(p.status, 2);
     }
   } else {
     // ------------------------------------------------------------ epilogue
@@ -888,7 +886,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           if (good) {
             good = mbar_wait_addr(accf0 + 8u * buf, (it >> 1) & 1u, p.wait_limit);
             good = __all_sync(0xffffffffu, good);
-            if (!good && lane == 0) atomicExch(p.status, 3);
+            if (!good && lane == 0) report_expired(p.status, WAIT_GEMM_EPILOGUE, t, -1);
           }
           tc_fence_after();
           us = (us + uint32_t(tc.num_kb)) % uint32_t(S);     // the operand fills of this tile
@@ -899,7 +897,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             if (good) {
               good = mbar_wait_addr(ufull0 + 8u * us, (uph >> us) & 1u, p.wait_limit);
               good = __all_sync(0xffffffffu, good);
-              if (!good && lane == 0) atomicExch(p.status, 4);
+              if (!good && lane == 0) report_expired(p.status, WAIT_GEMM_CHUNK, t, c);
             }
             uph ^= 1u << us;
             uint32_t packed[16];
@@ -1014,7 +1012,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       ok = mbar_wait_addr(accf0 + 8u * buf, (it >> 1) & 1u, p.wait_limit);
       ok = __all_sync(0xffffffffu, ok);      // warp-uniform: tcgen05.ld below is warp-collective
       if (!ok) {
-        if (lane == 0) atomicExch(p.status, 3);
+        if (lane == 0) report_expired(p.status, WAIT_GEMM_EPILOGUE, t, -1);
         break;
       }
       tc_fence_after();

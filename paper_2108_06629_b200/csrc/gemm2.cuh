@@ -182,7 +182,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       int c_tap = 0, c_chunk = 0;                      // convolution: filter tap and 64-channel chunk of this k-block
       for (int kb = 0; kb < num_kb - p.starve_kb; ++kb, k0 += GEMM_BK) {
         ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-        if (!ok) break;
+        if (!ok) { report_expired(p.status, WAIT_PAIR_PRODUCER, int(blockIdx.y), kb); break; }
         const uint32_t sa = smem0 + s * uint32_t(STAGE_BYTES);
         const uint32_t sb = sa + GEMM_A_BYTES;
         const uint32_t fb = map_to_cta(full0 + 8u * s, 0);          // the leader's barrier
@@ -226,7 +226,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
           const uint32_t ufull0 = smem_u32(ufull_bar);
           for (int f = 0; f < kChunks / per; ++f) {
             ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-            if (!ok) break;
+            if (!ok) { report_expired(p.status, WAIT_PAIR_PRODUCER, int(blockIdx.y), num_kb + f); break; }
             const uint32_t sa = smem0 + s * uint32_t(STAGE_BYTES);
             const uint32_t ub = ufull0 + 8u * s;
             mbar_arrive_expect_tx_addr(ub, 2u * UPD_CHUNK_BYTES);
@@ -240,7 +240,6 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         }
       }
       if (!ok) {
-        atomicExch(p.status, 11);
         // let copies already in flight land before the CTA's shared memory is released
         if (rank == 0)
           for (int kb = max(0, issued - S); kb < issued; ++kb) mbar_wait(&full_bar[kb % S], (kb / S) & 1, p.wait_limit);
@@ -264,7 +263,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       bool ok = true;
       for (int kb = 0; kb < num_kb; ++kb) {
         ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-        if (!ok) break;
+        if (!ok) { report_expired(p.status, WAIT_PAIR_MMA, int(blockIdx.y), kb); break; }
         tc_fence_after();
 #pragma unroll
         for (int j = 0; j < GEMM_BK / 16; ++j) {
@@ -281,7 +280,6 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
           dB_lo = uint32_t(dB);
         }
       }
-      if (!ok) atomicExch(p.status, 12);
       umma2_commit_both(smem_u32(acc_bar));
       phase_mark(p, 4);
     }
@@ -301,7 +299,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const int trow = q * 32 + lane;                           // row of this CTA's half tile = tensor-memory lane
       bool good = mbar_wait(acc_bar, 0, p.wait_limit);
       good = __all_sync(0xffffffffu, good);
-      if (!good && lane == 0) atomicExch(p.status, 13);
+      if (!good && lane == 0) report_expired(p.status, WAIT_PAIR_EPILOGUE, int(blockIdx.y), -1);
       tc_fence_after();
       const int per = p.mW != nullptr ? 1 : 2;                  // 32-column chunks per stage fill
       uint32_t us = uint32_t(num_kb % S), pending_stage = 0;
@@ -314,7 +312,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         if (good && sub == 0) {
           good = mbar_wait_addr(ufull0 + 8u * us, uint32_t(f / S) & 1u, p.wait_limit);
           good = __all_sync(0xffffffffu, good);
-          if (!good && lane == 0) atomicExch(p.status, 14);
+          if (!good && lane == 0) report_expired(p.status, WAIT_PAIR_CHUNK, int(blockIdx.y), c);
         }
         uint32_t packed[16];
         if (good) {
@@ -396,7 +394,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     if constexpr (upd) load_wm(p, row0, tm.n0 + sub_col, tm.nlim, sub_row, cur);
     bool ok = mbar_wait(acc_bar, 0, p.wait_limit);
     ok = __all_sync(0xffffffffu, ok);
-    if (!ok && lane == 0) atomicExch(p.status, 13);
+    if (!ok && lane == 0) report_expired(p.status, WAIT_PAIR_EPILOGUE, int(blockIdx.y), -1);
     tc_fence_after();
     if (ok) {
 #pragma unroll 1

@@ -110,7 +110,7 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         int k0 = 0;
         for (int kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
           ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_PAIR_G_PRODUCER, t, kb); break; }
           const uint32_t sa = smem0 + s * uint32_t(STAGE);
           const uint32_t sb = sa + GEMM_A_BYTES;
           const uint32_t fb = map_to_cta(full0 + 8u * s, 0);          // the leader's barrier
@@ -124,7 +124,6 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
       }
       if (!ok) {
-        atomicExch(p.status, 15);
         // let copies already in flight land before the CTA's shared memory is released
         if (rank == 0)
           for (long long i = (issued > SO ? issued - SO : 0); i < issued; ++i) mbar_wait(&full_bar[i % SO], uint32_t(i / SO) & 1u, p.wait_limit);
@@ -147,13 +146,13 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         const uint32_t buf = it & 1u;
         // both CTAs' epilogues must have read this accumulator out (tile it - 2)
         ok = mbar_wait_addr(acce0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, p.wait_limit);
-        if (!ok) break;
+        if (!ok) { report_expired(p.status, WAIT_PAIR_G_MMA, t, -1); break; }
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * uint32_t(GEMM2_BN);
         uint32_t acc = 0;
         for (int kb = 0; kb < num_kb; ++kb) {
           ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_PAIR_G_MMA, t, kb); break; }
           tc_fence_after();
 #pragma unroll
           for (int j = 0; j < GEMM_BK / 16; ++j) {
@@ -172,7 +171,6 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
         umma2_commit_both(accf0 + 8u * buf);      // accumulator complete in both CTAs (also releases the epilogues on error)
       }
-      if (!ok) atomicExch(p.status, 16);
     }
   } else if (warp == 6) {
     // ------------------------------------------------------------ update-tile producer (both CTAs)
@@ -187,7 +185,7 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         const int n0 = (t / tiles_m) * GEMM2_BN;
         for (int c = 0; c < kChunks; ++c) {
           ok = mbar_wait_addr(uempty0 + 8u * u, uph ^ 1u, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_PAIR_G_UPDATE_PRODUCER, t, c); break; }
           const uint32_t dst = chunk0 + u * slot_bytes;
           const uint32_t ub = ufull0 + 8u * u;
           mbar_arrive_expect_tx_addr(ub, slot_bytes);
@@ -198,7 +196,6 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
       }
       if (!ok) {
-        atomicExch(p.status, 17);
         for (long long i = (issued > SC ? issued - SC : 0); i < issued; ++i) mbar_wait(&ufull_bar[i % SC], uint32_t(i / SC) & 1u, p.wait_limit);
       }
     }
@@ -220,7 +217,7 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       good = mbar_wait_addr(accf0 + 8u * buf, (it >> 1) & 1u, p.wait_limit);
       good = __all_sync(0xffffffffu, good);
       if (!good) {
-        if (lane == 0) atomicExch(p.status, 18);
+        if (lane == 0) report_expired(p.status, WAIT_PAIR_G_EPILOGUE, t, -1);
         break;
       }
       tc_fence_after();
@@ -234,7 +231,7 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         good = mbar_wait_addr(ufull0 + 8u * u, uph, p.wait_limit);
         good = __all_sync(0xffffffffu, good);
         if (!good) {
-          if (lane == 0) atomicExch(p.status, 19);
+          if (lane == 0) report_expired(p.status, WAIT_PAIR_G_CHUNK, t, c);
           break;
         }
         uint32_t r[32];

@@ -104,7 +104,7 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         int k0 = 0, c_tap = 0, c_chunk = 0;
         for (int kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
           ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_PAIR_FD_PRODUCER, t, kb); break; }
           const uint32_t sa = smem0 + s * uint32_t(STAGE);
           const uint32_t sb = sa + GEMM_A_BYTES;
           const uint32_t fb = map_to_cta(full0 + 8u * s, 0);          // the leader's barrier
@@ -141,7 +141,6 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
       }
       if (!ok) {
-        atomicExch(p.status, 24);
         // let copies already in flight land before the CTA's shared memory is released
         if (rank == 0)
           for (long long i = (issued > S ? issued - S : 0); i < issued; ++i) mbar_wait(&full_bar[i % S], uint32_t(i / S) & 1u, p.wait_limit);
@@ -165,13 +164,13 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         const uint32_t buf = it & 1u;
         // both CTAs' epilogues must have read this accumulator out (tile it - 2)
         ok = mbar_wait_addr(acce0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, p.wait_limit);
-        if (!ok) break;
+        if (!ok) { report_expired(p.status, WAIT_PAIR_FD_MMA, t, -1); break; }
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * 256u;
         uint32_t acc = 0;
         for (int kb = 0; kb < num_kb; ++kb) {
           ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-          if (!ok) break;
+          if (!ok) { report_expired(p.status, WAIT_PAIR_FD_MMA, t, kb); break; }
           tc_fence_after();
 #pragma unroll
           for (int j = 0; j < GEMM_BK / 16; ++j) {
@@ -190,7 +189,6 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
         umma2_commit_both(accf0 + 8u * buf);      // accumulator complete in both CTAs (also releases the epilogues on error)
       }
-      if (!ok) atomicExch(p.status, 25);
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2-5 of both CTAs, own 128 rows)
@@ -209,7 +207,7 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       good = mbar_wait_addr(accf0 + 8u * buf, (it >> 1) & 1u, p.wait_limit);
       good = __all_sync(0xffffffffu, good);
       if (!good) {
-        if (lane == 0) atomicExch(p.status, 26);
+        if (lane == 0) report_expired(p.status, WAIT_PAIR_FD_EPILOGUE, t, -1);
         break;
       }
       tc_fence_after();

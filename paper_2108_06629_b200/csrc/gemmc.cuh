@@ -130,7 +130,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       int k0 = kb0 * GEMM_BK;
       for (int kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
         ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-        if (!ok) break;
+        if (!ok) { report_expired(p.status, WAIT_CLUSTER_PRODUCER, int(blockIdx.y), kb); break; }
         const uint32_t sa = smem0 + s * uint32_t(SM::STAGE_BYTES), sb = sa + GEMM_A_BYTES, fb = full0 + 8u * s;
         mbar_arrive_expect_tx_addr(fb, SM::STAGE_BYTES);
         if (B_MN) {
@@ -149,7 +149,6 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
       }
       if (!ok) {
-        atomicExch(p.status, 1);
         for (int i = (issued > S ? issued - S : 0); i < issued; ++i) mbar_wait(&full_bar[i % S], uint32_t(i / S) & 1u, p.wait_limit);
       }
     }
@@ -165,7 +164,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       bool ok = true;
       for (int kb = 0; kb < num_kb; ++kb) {
         ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-        if (!ok) break;
+        if (!ok) { report_expired(p.status, WAIT_CLUSTER_MMA, int(blockIdx.y), kb); break; }
         tc_fence_after();
         const uint32_t off = s * uint32_t(SM::STAGE_BYTES >> 4);
 #pragma unroll
@@ -177,7 +176,6 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
       }
       umma_commit(acc_bar);
-      if (!ok) atomicExch(p.status, 2);
     }
   } else {
     const int q = warp & 3;
@@ -197,7 +195,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     __syncwarp();
     bool ok = mbar_wait(acc_bar, 0, p.wait_limit);
     ok = __all_sync(0xffffffffu, ok);
-    if (!ok && lane == 0) atomicExch(p.status, 3);
+    if (!ok && lane == 0) report_expired(p.status, WAIT_CLUSTER_EPILOGUE, int(blockIdx.y), -1);
     tc_fence_after();
     float* row = reinterpret_cast<float*>(smem) + (q * 32 + lane) * gemmc_part_pitch(BN);
     if (ok && tm.m0 + q * 32 < p.M) {

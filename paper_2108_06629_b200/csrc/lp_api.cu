@@ -1853,11 +1853,12 @@ extern "C" int lp_task_progress(lp_handle h, char* text, int capacity) {
 extern "C" int lp_device_status(lp_handle h, int* detail) {
   if (!h) return LP_ERR_INVALID_ARG;
   LP_CUDA(h, cudaDeviceSynchronize());
-  int st = 0;
-  LP_CUDA(h, cudaMemcpy(&st, h->status, 4, cudaMemcpyDeviceToHost));
+  int block[STATUS_WORDS] = {};
+  LP_CUDA(h, cudaMemcpy(block, h->status, sizeof block, cudaMemcpyDeviceToHost));
+  const int st = block[STATUS_CODE];
   if (detail) *detail = st;
   if (st == LP_STATUS_BAD_LABEL)
     return fail(h, LP_ERR_INVALID_ARG, "a label outside [0, classes) reached the loss kernel (that minibatch's loss is NaN)");
-  if (st != 0) return fail(h, LP_ERR_TIMEOUT, "a bounded device-side wait expired (status " + std::to_string(st) + ")");
+  if (st != 0) return fail(h, LP_ERR_TIMEOUT, expired_text(block));
   return LP_OK;
 }

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "wait_codes.h"
+
 namespace lp {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
