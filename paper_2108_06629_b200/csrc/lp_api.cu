@@ -155,6 +155,8 @@ struct lp_ctx {
   // streams[0] = the caller's stream of the current lp_step, then the P chain streams, then the Q G streams
   static constexpr int kMaxStreams = 16;
   std::vector<cudaStream_t> streams;
+  unsigned long long caller_id = 0;   // cudaStreamGetId of streams[0]: two streams can have the same handle (cudaStreamPerThread
+                                      // in two threads, a stream created after another was destroyed), never the same id
   int chain_index(long long n) const { return 1 + int(n % n_chain); }
   int g_index(int l) const { return 1 + n_chain + l % n_g; }
   // Recorded events of a stream, oldest overwritten first.  A wait for task `pos` takes the first
@@ -1329,11 +1331,14 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
   const bool fusedB = (c->cfg.schedule == LP_SCHED_FUSED_B);
   const bool serial = (c->cfg.flags & LP_SERIAL_TASKS) != 0;   // every task on the caller's stream
   const int ds = int(n % kDeltaSlots);
-  if (c->streams[0] != user) {
+  unsigned long long user_id = 0;
+  LP_CUDA(c, cudaStreamGetId(user, &user_id));
+  if (c->streams[0] != user || c->caller_id != user_id) {
     // Another caller's stream takes over: it continues behind the last task of the old one (whose record is kept,
     // the stream itself may be gone), and knows of other streams what had been waited for by then.
     lp_ctx::StreamLog& g = c->log[0];
     c->streams[0] = user;
+    c->caller_id = user_id;
     if (g.n_rec > 0) {
       const lp_ctx::Rec& r = g.rec[(g.n_rec - 1) % lp_ctx::kRecs];
       LP_CUDA(c, cudaStreamWaitEvent(user, r.e, 0));
@@ -1509,18 +1514,19 @@ extern "C" int lp_flush(lp_handle h, void* stream) {
   if (!h) return LP_ERR_INVALID_ARG;
   if (h->latched) return h->latched;
   cudaStream_t user = static_cast<cudaStream_t>(stream);
-  cudaError_t err = cudaSuccess;
-  if (user == h->streams[0]) {
-    for (size_t si = 1; si < h->streams.size(); ++si) wait_on(h, 0, Ev{int(si), h->log[si].pos}, &err);
-  } else {
-    for (size_t si = 0; si < h->streams.size(); ++si) {
-      if (h->log[si].pos == 0) continue;
-      lp_ctx::Rec* r = nullptr;
-      LP_CUDA(h, resolve(h, Ev{int(si), h->log[si].pos}, &r));
-      LP_CUDA(h, cudaStreamWaitEvent(user, r->e, 0));
-    }
+  unsigned long long user_id = 0;
+  LP_CUDA(h, cudaStreamGetId(user, &user_id));
+  const bool caller = user == h->streams[0] && user_id == h->caller_id;
+  // `stream` waits for the tail of every stream with work, whatever has been waited for before: a flush is what the
+  // caller's own reads rely on (and under a stream capture its waits must be in the capture or be refused).
+  for (size_t si = caller ? 1 : 0; si < h->streams.size(); ++si) {
+    if (h->log[si].pos == 0) continue;
+    lp_ctx::Rec* r = nullptr;
+    LP_CUDA(h, resolve(h, Ev{int(si), h->log[si].pos}, &r));
+    LP_CUDA(h, cudaStreamWaitEvent(user, r->e, 0));
+    if (caller)
+      for (size_t k = 0; k < h->streams.size(); ++k) h->log[0].vc[k] = std::max(h->log[0].vc[k], r->vc[k]);
   }
-  LP_CUDA(h, err);
   return LP_OK;
 }
 

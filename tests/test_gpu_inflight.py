@@ -300,3 +300,48 @@ def test_inflight_steps_and_flush_on_changing_caller_streams(schedule):
     (loss1, W1), (loss3, W3) = go(1), go(3)
     assert loss1 == loss3
     assert all(np.array_equal(a, b) for a, b in zip(W1, W3))
+
+
+@pytest.mark.parametrize("reuse", ["per_thread", "own"])
+def test_flush_orders_a_stream_whose_handle_another_one_has_used(reuse):
+    """cudaStreamPerThread is one handle and a stream for every thread.  Thread A holds its own back by a gate, enqueues
+    steps and a flush behind it; thread B flushes under the same handle and copies the trainer's state on its own
+    stream: the copy must be the finished state.  "own": the caller flushes twice on one stream, which changes nothing."""
+    import threading
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    from paper_2108_06629_b200 import inputs as I
+    per_thread = 2                                    # the handle value of cudaStreamPerThread
+    layers, B, steps = I.mlp([264, 192, 320, 136, 40], "gelu"), 56, 6
+    W0, b0 = I.initial_weights(layers, 0)
+    tr = lpb.Trainer(layers, B, 4, delays=[3, 2, 1, 0], lr=0.02, momentum=0.9, W0=W0, b0=b0)
+    data = [tuple(torch.from_numpy(t).cuda() for t in I.minibatch(layers, B, n)) for n in range(steps)]
+    seen = torch.zeros_like(tr.workspace)
+    torch.cuda.synchronize()
+    handle = per_thread if reuse == "per_thread" else torch.cuda.Stream().cuda_stream
+
+    def enqueue():
+        with torch.cuda.stream(torch.cuda.ExternalStream(handle)):
+            torch.cuda._sleep(GATE_CYCLES)
+            for x, y in data:
+                tr.step(x, y)
+            tr.flush()
+
+    def read():
+        stream = torch.cuda.ExternalStream(handle)
+        with torch.cuda.stream(stream):
+            tr.flush()
+            seen.copy_(tr.workspace, non_blocking=True)
+        stream.synchronize()
+
+    for work in (enqueue, read):
+        if reuse == "per_thread":
+            t = threading.Thread(target=work)
+            t.start()
+            t.join()
+        else:
+            work()
+    torch.cuda.synchronize()
+    assert torch.equal(seen, tr.workspace)
+    assert not np.array_equal(tr.get_weights(0)[0], W0[0]) and tr.device_status() == (0, 0)
+    tr.close()
