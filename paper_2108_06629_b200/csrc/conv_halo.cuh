@@ -101,9 +101,10 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       for (int tap = 0; tap < ntaps; ++tap) tma_load_2d(sB + tap * HALO_TAP_BYTES, &tmB, wfull, tap * p.g.tap_pitch, 0);
       uint32_t st = 0, sph = 0;
       int tw = tw_begin, th = th_begin, n = tn_begin;
-      for (int t = t_begin; t < t_end; ++t) {
+      int t = t_begin;
+      for (; t < t_end; ++t) {
         ok = mbar_wait(&aempty[st], sph ^ 1u);
-        if (!ok) { report_expired(p.status, WAIT_HALO_PRODUCER, t, -1); break; }
+        if (!ok) break;
         if (plain) {
           mbar_arrive_expect_tx(&afull[st], GEMM_A_BYTES);
           tma_load_2d(sA + st * HALO_BYTES, &tmA, &afull[st], 0, t * GEMM_BM);
@@ -117,6 +118,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (++st == uint32_t(HALO_STAGES)) { st = 0; sph ^= 1u; }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_HALO_PRODUCER, t, 0);
         mbar_wait(wfull, 0);
         for (int i = (issued > HALO_STAGES ? issued - HALO_STAGES : 0); i < issued; ++i)
           mbar_wait(&afull[i % HALO_STAGES], uint32_t(i / HALO_STAGES) & 1u);
@@ -140,14 +142,14 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         tap_off[tap] = uint32_t(r * HALO_W + s) * (128u >> 4);
       }
       bool ok = mbar_wait(wfull, 0);
-      if (!ok) report_expired(p.status, WAIT_HALO_MMA, t_begin, -2);       // (the weights)
       uint32_t it = 0, st = 0, sph = 0;
-      for (int t = t_begin; t < t_end && ok; ++t, ++it) {
+      int t = t_begin;
+      for (; t < t_end && ok; ++t, ++it) {
         const uint32_t buf = it & 1u;
         ok = mbar_wait(&acce[buf], ((it >> 1) & 1u) ^ 1u);
-        if (!ok) { report_expired(p.status, WAIT_HALO_MMA, t, -1); break; }
+        if (!ok) break;
         ok = mbar_wait(&afull[st], sph);
-        if (!ok) { report_expired(p.status, WAIT_HALO_MMA, t, 0); break; }
+        if (!ok) break;
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * uint32_t(BN);
         const uint32_t a_lo = dA_lo0 + st * uint32_t(HALO_BYTES >> 4);
@@ -166,6 +168,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         umma_commit(&accf[buf]);
         if (++st == uint32_t(HALO_STAGES)) { st = 0; sph ^= 1u; }
       }
+      if (!ok) report_expired(p.status, WAIT_HALO_MMA, t, 0);
     }
   } else {
     // Eight warps: warp w reads tensor-memory lanes 32 * (w % 4) (the rows of its quarter of the
@@ -407,9 +410,10 @@ conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
       int issued = 0;
       uint32_t st = 0, sph = 0;
       int tw = t_begin % g.tiles_w, th = (t_begin / g.tiles_w) % g.tiles_h, n = t_begin / (g.tiles_w * g.tiles_h);
-      for (int t = t_begin; t < t_end; ++t) {
+      int t = t_begin;
+      for (; t < t_end; ++t) {
         ok = mbar_wait(&empty[st], sph ^ 1u);
-        if (!ok) { report_expired(status, WAIT_HALO_G_PRODUCER, t, -1); break; }
+        if (!ok) break;
         uint8_t* base = smem + st * HALOG_STAGE_BYTES;
         mbar_arrive_expect_tx(&full[st], HALO_BYTES + GEMM_A_BYTES);
         tma_load_4d(base, &tmX, &full[st], 0, tw * 8 - 1, th * 16 - 1, n);
@@ -419,6 +423,7 @@ conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         if (++tw == g.tiles_w) { tw = 0; if (++th == g.tiles_h) { th = 0; ++n; } }
       }
       if (!ok) {
+        report_expired(status, WAIT_HALO_G_PRODUCER, t, 0);
         for (int i = (issued > HALOG_STAGES ? issued - HALOG_STAGES : 0); i < issued; ++i)
           mbar_wait(&full[i % HALOG_STAGES], uint32_t(i / HALOG_STAGES) & 1u);
       }
@@ -440,9 +445,10 @@ conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
       const uint32_t dB_lo0 = uint32_t(dB), dB_hi = uint32_t(dB >> 32);
       bool ok = true;
       uint32_t st = 0, sph = 0, acc = 0;
-      for (int t = t_begin; t < t_end; ++t) {
+      int t = t_begin;
+      for (; t < t_end; ++t) {
         ok = mbar_wait(&full[st], sph);
-        if (!ok) { report_expired(status, WAIT_HALO_G_MMA, t, -1); break; }
+        if (!ok) break;
         tc_fence_after();
         const uint32_t soff = st * uint32_t(HALOG_STAGE_BYTES >> 4);
 #pragma unroll
@@ -456,6 +462,7 @@ conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         umma_commit(&empty[st]);
         if (++st == uint32_t(HALOG_STAGES)) { st = 0; sph ^= 1u; }
       }
+      if (!ok) report_expired(status, WAIT_HALO_G_MMA, t, 0);
       umma_commit(accf);
     }
   } else {

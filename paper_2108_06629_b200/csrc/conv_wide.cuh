@@ -87,14 +87,15 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       uint32_t as = 0, aph = 0, bs = 0, bph = 0;
       const uint32_t sA0 = smem_u32(smem), sB0 = smem_u32(sB);
       const uint32_t afull0 = smem_u32(afull), aempty0 = smem_u32(aempty), bfull0 = smem_u32(bfull), bempty0 = smem_u32(bempty);
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      int it = blockIdx.x;
+      for (; it < items && ok; it += gridDim.x) {
         const int tp = it / tiles_n, n0 = p.n_begin + (it - tp * tiles_n) * BN;
         TileMap t0, t1;
         pixel_tile(2 * tp, t0);
         pixel_tile(min(2 * tp + 1, tiles_total - 1), t1);   // (an odd last tile is computed twice, stored once)
         for (int c = 0; c < chunks && ok; ++c) {
           ok = mbar_wait_addr(aempty0 + 8u * as, aph ^ 1u, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_WIDE_PRODUCER, it, 9 * c); break; }
+          if (!ok) break;
           mbar_arrive_expect_tx_addr(afull0 + 8u * as, uint32_t(WIDE_A_BYTES));
           const uint32_t sa = sA0 + as * uint32_t(WIDE_A_BYTES);
           tma_load_4d_addr(sa, &tmA, afull0 + 8u * as, c * 64, t0.pw0 - 1, t0.ph0 - 1, t0.pn0);
@@ -104,7 +105,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           int col = 0;
           for (int tap = 0; tap < 9; ++tap, col += p.g.tap_pitch) {
             ok = mbar_wait_addr(bempty0 + 8u * bs, bph ^ 1u, p.wait_limit);
-            if (!ok) { report_expired(p.status, WAIT_WIDE_PRODUCER, it, 9 * c + tap); break; }
+            if (!ok) break;
             const uint32_t fb = bfull0 + 8u * bs, sb = sB0 + bs * uint32_t(B_BYTES);
             mbar_arrive_expect_tx_addr(fb, uint32_t(B_BYTES));
             if (B_MN) {        // delta: B[k = (tap, co)][n = ci]
@@ -119,6 +120,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_WIDE_PRODUCER, it - int(gridDim.x), ib);
         // let copies already in flight land before the CTA's shared memory is released
         for (int i = max(0, ia - WIDE_A_STAGES); i < ia; ++i) mbar_wait(&afull[i % WIDE_A_STAGES], uint32_t(i / WIDE_A_STAGES) & 1u, p.wait_limit);
         for (int i = max(0, ib - WIDE_B_STAGES); i < ib; ++i) mbar_wait(&bfull[i % WIDE_B_STAGES], uint32_t(i / WIDE_B_STAGES) & 1u, p.wait_limit);
@@ -142,21 +144,22 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
       uint32_t as = 0, aph = 0, bs = 0, bph = 0, n_it = 0;
       bool ok = true;
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x, ++n_it) {
+      int it = blockIdx.x;
+      for (; it < items && ok; it += gridDim.x, ++n_it) {
         const uint32_t buf = n_it & 1u;
         ok = mbar_wait_addr(acce0 + 8u * buf, ((n_it >> 1) & 1u) ^ 1u, p.wait_limit);
-        if (!ok) { report_expired(p.status, WAIT_WIDE_MMA, it, -1); break; }
+        if (!ok) break;
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * 256u;        // accumulators of the two pixel tiles: columns 0 and 128 of the buffer
         uint32_t acc = 0;
         for (int c = 0; c < chunks && ok; ++c) {
           ok = mbar_wait_addr(afull0 + 8u * as, aph, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_WIDE_MMA, it, 9 * c); break; }
+          if (!ok) break;
           const uint32_t a_lo = uint32_t(dA) + as * uint32_t(WIDE_A_BYTES >> 4);
 #pragma unroll
           for (int tap = 0; tap < 9; ++tap) {
-            ok = mbar_wait_addr(bfull0 + 8u * bs, bph, p.wait_limit);
-            if (!ok) { report_expired(p.status, WAIT_WIDE_MMA, it, 9 * c + tap); break; }
+            if (ok) ok = mbar_wait_addr(bfull0 + 8u * bs, bph, p.wait_limit);
+            if (!ok) break;
             tc_fence_after();
             const uint32_t b_lo = uint32_t(dB) + bs * uint32_t(B_BYTES >> 4);
 #pragma unroll
@@ -174,6 +177,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         umma_commit_addr(accf0 + 8u * buf);                  // (also releases the epilogue on error)
       }
+      if (!ok) report_expired(p.status, WAIT_WIDE_MMA, it - int(gridDim.x), int(bs));
     }
   } else {
     const int q = warp & 3;

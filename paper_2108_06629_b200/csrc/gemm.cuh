@@ -625,7 +625,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
       uint32_t s = 0, ph = 0;
       uint32_t op_ph = 0, ch_ph = 0, is_chunk = 0;   // UTMA, a bit per stage: parity of the next operand / chunk fill, kind of the last fill
-      for (int t = blockIdx.x; t < total_work && ok; t += (PERSIST ? int(gridDim.x) : total_work)) {
+      int t = blockIdx.x, kb = 0;                    // (both outlive their loops: a wait that runs out is reported behind them)
+      for (; t < total_work && ok; t += (PERSIST ? int(gridDim.x) : total_work)) {
         const TileCtx tc = decode_tile<BN>(p, t, tiles_m, tiles_n);
         const TileMap& tm = tc.tm;
         // running position of the contraction
@@ -670,7 +671,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             tma_prefetch_l2_2d(&tmB, kk, tm.n0);
           }
         }
-        for (int kb = 0; kb < tc.num_kb - p.starve_kb; ++kb) {
+        for (kb = 0; kb < tc.num_kb - p.starve_kb; ++kb) {
           if (ahead > 0 && kb + ahead < tc.num_kb) {
             const int kk = k0 + ahead * GEMM_BK;
             if (B_MN) {
@@ -681,7 +682,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
           }
           ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_GEMM_PRODUCER, t, kb); break; }
+          if (!ok) break;
           const uint32_t sa = smem0 + s * uint32_t(SM::STAGE_BYTES);
           const uint32_t sb = sa + GEMM_A_BYTES;
           const uint32_t fb = full0 + 8u * s;
@@ -740,7 +741,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const uint32_t bytes = p.mW != nullptr ? 2u * UPD_CHUNK_BYTES : uint32_t(UPD_CHUNK_BYTES);
             for (int c = 0; c < kChunks; ++c) {
               ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-              if (!ok) { report_expired(p.status, WAIT_GEMM_PRODUCER, t, tc.num_kb + c); break; }
+              if (!ok) break;
               const uint32_t sa = smem0 + s * uint32_t(SM::STAGE_BYTES);
               const uint32_t fb = ufull0 + 8u * s;
               mbar_arrive_expect_tx_addr(fb, bytes);
@@ -755,6 +756,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_GEMM_PRODUCER, t - (PERSIST ? int(gridDim.x) : total_work), kb);
         // let copies already in flight land before the CTA's shared memory is released
         for (long long i = (issued > S ? issued - S : 0); i < issued; ++i) {
           const int k = int(i % S);
@@ -784,20 +786,21 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       uint32_t dA_lo = uint32_t(dA), dB_lo = uint32_t(dB);
       bool ok = true;
       uint32_t it = 0;     // tiles done by this CTA
-      for (int t = blockIdx.x; t < total_work && ok; t += (PERSIST ? int(gridDim.x) : total_work), ++it) {
+      int t = blockIdx.x, kb = 0;
+      for (; t < total_work && ok; t += (PERSIST ? int(gridDim.x) : total_work), ++it) {
         const TileCtx tc = decode_tile<BN>(p, t, tiles_m, tiles_n);
         const uint32_t buf = PERSIST ? (it & 1u) : 0u;
         if (PERSIST) {
           // the epilogue must have drained this accumulator buffer (tile it - 2)
           ok = mbar_wait_addr(acce0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_GEMM_MMA, t, -1); break; }
+          if (!ok) break;
           tc_fence_after();
         }
         const uint32_t tacc = tmem_base + buf * uint32_t(BN);
         uint32_t acc = 0;
-        for (int kb = 0; kb < tc.num_kb; ++kb) {
+        for (kb = 0; kb < tc.num_kb; ++kb) {
           ok = mbar_wait_addr(full0 + 8u * s, UTMA ? (ph >> s) & 1u : ph, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_GEMM_MMA, t, kb); break; }
+          if (!ok) break;
           if (UTMA) ph ^= 1u << s;             // (a bit per stage: not every turn of the ring brings operands)
           tc_fence_after();
 #pragma unroll
@@ -823,6 +826,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           dB_lo = uint32_t(dB) + s * uint32_t(SM::STAGE_BYTES >> 4);
         }
       }
+      // (with an accumulator buffer still in use kb is that of the tile before, which is its last)
+      if (!ok) report_expired(p.status, WAIT_GEMM_MMA, t - (PERSIST ? int(gridDim.x) : total_work), kb);
     }
   } else {
     // ------------------------------------------------------------ epilogue

@@ -178,11 +178,11 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const uint32_t smem0 = smem_u32(smem);
       const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
       uint32_t s = 0, ph = 0;
-      int k0 = 0;
+      int k0 = 0, kb = 0;
       int c_tap = 0, c_chunk = 0;                      // convolution: filter tap and 64-channel chunk of this k-block
-      for (int kb = 0; kb < num_kb - p.starve_kb; ++kb, k0 += GEMM_BK) {
+      for (; kb < num_kb - p.starve_kb; ++kb, k0 += GEMM_BK) {
         ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-        if (!ok) { report_expired(p.status, WAIT_PAIR_PRODUCER, int(blockIdx.y), kb); break; }
+        if (!ok) break;
         const uint32_t sa = smem0 + s * uint32_t(STAGE_BYTES);
         const uint32_t sb = sa + GEMM_A_BYTES;
         const uint32_t fb = map_to_cta(full0 + 8u * s, 0);          // the leader's barrier
@@ -226,7 +226,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
           const uint32_t ufull0 = smem_u32(ufull_bar);
           for (int f = 0; f < kChunks / per; ++f) {
             ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-            if (!ok) { report_expired(p.status, WAIT_PAIR_PRODUCER, int(blockIdx.y), num_kb + f); break; }
+            if (!ok) break;
             const uint32_t sa = smem0 + s * uint32_t(STAGE_BYTES);
             const uint32_t ub = ufull0 + 8u * s;
             mbar_arrive_expect_tx_addr(ub, 2u * UPD_CHUNK_BYTES);
@@ -240,6 +240,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_PAIR_PRODUCER, int(blockIdx.y), kb);
         // let copies already in flight land before the CTA's shared memory is released
         if (rank == 0)
           for (int kb = max(0, issued - S); kb < issued; ++kb) mbar_wait(&full_bar[kb % S], (kb / S) & 1, p.wait_limit);
@@ -261,9 +262,10 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       uint32_t s = 0, ph = 0, acc = 0;
       uint32_t dA_lo = uint32_t(dA), dB_lo = uint32_t(dB);
       bool ok = true;
-      for (int kb = 0; kb < num_kb; ++kb) {
+      int kb = 0;
+      for (; kb < num_kb; ++kb) {
         ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-        if (!ok) { report_expired(p.status, WAIT_PAIR_MMA, int(blockIdx.y), kb); break; }
+        if (!ok) break;
         tc_fence_after();
 #pragma unroll
         for (int j = 0; j < GEMM_BK / 16; ++j) {
@@ -280,6 +282,7 @@ gemm2_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
           dB_lo = uint32_t(dB);
         }
       }
+      if (!ok) report_expired(p.status, WAIT_PAIR_MMA, int(blockIdx.y), kb);
       umma2_commit_both(smem_u32(acc_bar));
       phase_mark(p, 4);
     }

@@ -104,13 +104,14 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const uint32_t smem0 = smem_u32(smem);
       const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
       uint32_t s = 0, ph = 0;
-      for (int t = pair_id; t < total && ok; t += pairs) {
+      int t = pair_id, kb = 0;
+      for (; t < total && ok; t += pairs) {
         const int m0 = (t % tiles_m) * 256 + int(rank) * 128;        // this CTA's 128 rows of A
         const int nb0 = (t / tiles_m) * GEMM2_BN + int(rank) * 128;  // the half of B this CTA stages
         int k0 = 0;
-        for (int kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
+        for (kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
           ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_PAIR_G_PRODUCER, t, kb); break; }
+          if (!ok) break;
           const uint32_t sa = smem0 + s * uint32_t(STAGE);
           const uint32_t sb = sa + GEMM_A_BYTES;
           const uint32_t fb = map_to_cta(full0 + 8u * s, 0);          // the leader's barrier
@@ -124,6 +125,7 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_PAIR_G_PRODUCER, t - pairs, kb);
         // let copies already in flight land before the CTA's shared memory is released
         if (rank == 0)
           for (long long i = (issued > SO ? issued - SO : 0); i < issued; ++i) mbar_wait(&full_bar[i % SO], uint32_t(i / SO) & 1u, p.wait_limit);
@@ -142,17 +144,18 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       uint32_t s = 0, ph = 0, it = 0;
       uint32_t dA_lo = uint32_t(dA), dB_lo = uint32_t(dB);
       bool ok = true;
-      for (int t = pair_id; t < total && ok; t += pairs, ++it) {
+      int t = pair_id, kb = 0;
+      for (; t < total && ok; t += pairs, ++it) {
         const uint32_t buf = it & 1u;
         // both CTAs' epilogues must have read this accumulator out (tile it - 2)
         ok = mbar_wait_addr(acce0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, p.wait_limit);
-        if (!ok) { report_expired(p.status, WAIT_PAIR_G_MMA, t, -1); break; }
+        if (!ok) break;
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * uint32_t(GEMM2_BN);
         uint32_t acc = 0;
-        for (int kb = 0; kb < num_kb; ++kb) {
+        for (kb = 0; kb < num_kb; ++kb) {
           ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_PAIR_G_MMA, t, kb); break; }
+          if (!ok) break;
           tc_fence_after();
 #pragma unroll
           for (int j = 0; j < GEMM_BK / 16; ++j) {
@@ -171,6 +174,7 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
         umma2_commit_both(accf0 + 8u * buf);      // accumulator complete in both CTAs (also releases the epilogues on error)
       }
+      if (!ok) report_expired(p.status, WAIT_PAIR_G_MMA, t - pairs, kb);
     }
   } else if (warp == 6) {
     // ------------------------------------------------------------ update-tile producer (both CTAs)
@@ -180,12 +184,13 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const uint32_t chunk0 = smem_u32(chunk_mem);
       const uint32_t ufull0 = smem_u32(ufull_bar), uempty0 = smem_u32(uempty_bar);
       uint32_t u = 0, uph = 0;
-      for (int t = pair_id; t < total && ok; t += pairs) {
+      int t = pair_id, c = 0;
+      for (; t < total && ok; t += pairs) {
         const int m0 = (t % tiles_m) * 256 + int(rank) * 128;
         const int n0 = (t / tiles_m) * GEMM2_BN;
-        for (int c = 0; c < kChunks; ++c) {
+        for (c = 0; c < kChunks; ++c) {
           ok = mbar_wait_addr(uempty0 + 8u * u, uph ^ 1u, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_PAIR_G_UPDATE_PRODUCER, t, c); break; }
+          if (!ok) break;
           const uint32_t dst = chunk0 + u * slot_bytes;
           const uint32_t ub = ufull0 + 8u * u;
           mbar_arrive_expect_tx_addr(ub, slot_bytes);
@@ -196,6 +201,7 @@ gemm2p_g_update_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_PAIR_G_UPDATE_PRODUCER, t - pairs, c);
         for (long long i = (issued > SC ? issued - SC : 0); i < issued; ++i) mbar_wait(&ufull_bar[i % SC], uint32_t(i / SC) & 1u, p.wait_limit);
       }
     }

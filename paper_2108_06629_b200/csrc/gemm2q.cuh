@@ -98,13 +98,14 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       const uint32_t smem0 = smem_u32(smem);
       const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
       uint32_t s = 0, ph = 0;
-      for (int t = pair_id; t < total && ok; t += pairs) {
+      int t = pair_id, kb = 0;
+      for (; t < total && ok; t += pairs) {
         const TileMap tm = tile_map(t);
         const int nb0 = tm.n0 + int(rank) * (BN2 / 2);        // the half of B this CTA stages
         int k0 = 0, c_tap = 0, c_chunk = 0;
-        for (int kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
+        for (kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
           ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_PAIR_FD_PRODUCER, t, kb); break; }
+          if (!ok) break;
           const uint32_t sa = smem0 + s * uint32_t(STAGE);
           const uint32_t sb = sa + GEMM_A_BYTES;
           const uint32_t fb = map_to_cta(full0 + 8u * s, 0);          // the leader's barrier
@@ -141,6 +142,7 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_PAIR_FD_PRODUCER, t - pairs, kb);
         // let copies already in flight land before the CTA's shared memory is released
         if (rank == 0)
           for (long long i = (issued > S ? issued - S : 0); i < issued; ++i) mbar_wait(&full_bar[i % S], uint32_t(i / S) & 1u, p.wait_limit);
@@ -160,17 +162,18 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       uint32_t s = 0, ph = 0, it = 0;
       uint32_t dA_lo = uint32_t(dA), dB_lo = uint32_t(dB);
       bool ok = true;
-      for (int t = pair_id; t < total && ok; t += pairs, ++it) {
+      int t = pair_id, kb = 0;
+      for (; t < total && ok; t += pairs, ++it) {
         const uint32_t buf = it & 1u;
         // both CTAs' epilogues must have read this accumulator out (tile it - 2)
         ok = mbar_wait_addr(acce0 + 8u * buf, ((it >> 1) & 1u) ^ 1u, p.wait_limit);
-        if (!ok) { report_expired(p.status, WAIT_PAIR_FD_MMA, t, -1); break; }
+        if (!ok) break;
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * 256u;
         uint32_t acc = 0;
-        for (int kb = 0; kb < num_kb; ++kb) {
+        for (kb = 0; kb < num_kb; ++kb) {
           ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-          if (!ok) { report_expired(p.status, WAIT_PAIR_FD_MMA, t, kb); break; }
+          if (!ok) break;
           tc_fence_after();
 #pragma unroll
           for (int j = 0; j < GEMM_BK / 16; ++j) {
@@ -189,6 +192,7 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
         umma2_commit_both(accf0 + 8u * buf);      // accumulator complete in both CTAs (also releases the epilogues on error)
       }
+      if (!ok) report_expired(p.status, WAIT_PAIR_FD_MMA, t - pairs, kb);
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2-5 of both CTAs, own 128 rows)

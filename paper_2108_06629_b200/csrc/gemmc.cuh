@@ -127,10 +127,10 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       int issued = 0;
       const uint32_t smem0 = smem_u32(smem);
       uint32_t s = 0, ph = 0;
-      int k0 = kb0 * GEMM_BK;
-      for (int kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
+      int k0 = kb0 * GEMM_BK, kb = 0;
+      for (; kb < num_kb; ++kb, k0 += GEMM_BK) {
         ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
-        if (!ok) { report_expired(p.status, WAIT_CLUSTER_PRODUCER, int(blockIdx.y), kb); break; }
+        if (!ok) break;
         const uint32_t sa = smem0 + s * uint32_t(SM::STAGE_BYTES), sb = sa + GEMM_A_BYTES, fb = full0 + 8u * s;
         mbar_arrive_expect_tx_addr(fb, SM::STAGE_BYTES);
         if (B_MN) {
@@ -149,6 +149,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
       }
       if (!ok) {
+        report_expired(p.status, WAIT_CLUSTER_PRODUCER, int(blockIdx.y), kb);
         for (int i = (issued > S ? issued - S : 0); i < issued; ++i) mbar_wait(&full_bar[i % S], uint32_t(i / S) & 1u, p.wait_limit);
       }
     }
@@ -162,9 +163,10 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
       constexpr uint32_t stepA = (A_MN ? 2048 : 32) >> 4, stepB = (B_MN ? 2048 : 32) >> 4;
       uint32_t s = 0, ph = 0, acc = 0;
       bool ok = true;
-      for (int kb = 0; kb < num_kb; ++kb) {
+      int kb = 0;
+      for (; kb < num_kb; ++kb) {
         ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-        if (!ok) { report_expired(p.status, WAIT_CLUSTER_MMA, int(blockIdx.y), kb); break; }
+        if (!ok) break;
         tc_fence_after();
         const uint32_t off = s * uint32_t(SM::STAGE_BYTES >> 4);
 #pragma unroll
@@ -176,6 +178,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
       }
       umma_commit(acc_bar);
+      if (!ok) report_expired(p.status, WAIT_CLUSTER_MMA, int(blockIdx.y), kb);
     }
   } else {
     const int q = warp & 3;
