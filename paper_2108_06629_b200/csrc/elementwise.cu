@@ -587,12 +587,9 @@ cudaError_t launch_colsum_bias(const __nv_bfloat16* x, int rows, int ld, int n_c
 // of a workspace.  Host code must not pass `g_xent_scratch` itself to a kernel: in host
 // code that name is only a handle for the runtime.  The device address is looked up once
 // per device with cudaGetSymbolAddress and that pointer is what the kernel receives.
-// Counts of finished blocks, one per call in turn: the last block of a call wraps its count to zero, and one left
-// over by two calls that overlapped on this scratch is not met by the calls that follow.
-constexpr int kXentTickets = 64;
 struct XentScratch {
   float row_loss[LP_XENT_STATIC_MAX_BATCH];
-  unsigned ticket[kXentTickets];
+  unsigned ticket;
 };
 static __device__ __align__(256) unsigned char g_xent_scratch[sizeof(XentScratch)];
 
@@ -632,10 +629,13 @@ extern "C" int lp_softmax_xent_static(const float* logits_dev, int ld_logits, co
     }
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  static std::atomic<unsigned> calls{0};
-  unsigned* ticket = s->ticket + calls.fetch_add(1, std::memory_order_relaxed) % kXentTickets;
-  cudaError_t e = lp::launch_softmax_xent(logits_dev, ld_logits, labels_dev, static_cast<__nv_bfloat16*>(delta_dev), ld_delta,
-                              s->row_loss, ticket, loss_dev, batch, classes, nullptr, st);
+  // The counter must start at zero whatever two calls that overlapped have left in it: the kernel wraps it to zero
+  // only from a right start, and a call that finds a remainder adds up the rows before all of them are written.
+  // (8192 x 1000: 24.4 us with the memset, 22.5 without.)
+  cudaError_t e = cudaMemsetAsync(&s->ticket, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return xent_fail(LP_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+  e = lp::launch_softmax_xent(logits_dev, ld_logits, labels_dev, static_cast<__nv_bfloat16*>(delta_dev), ld_delta, s->row_loss,
+                              &s->ticket, loss_dev, batch, classes, nullptr, st);
   if (e != cudaSuccess) return xent_fail(LP_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
   return LP_OK;
 }

@@ -119,7 +119,7 @@ def test_static_loss_at_the_edges_of_its_row_forms(B, C, ld):
     ldd = (C + 7) // 8 * 8 + (ld % 2)
     delta = torch.full((B, ldd), 7.0, dtype=torch.bfloat16, device="cuda")
     loss = torch.zeros(1, device="cuda")
-    for _ in range(2):                            # (the second call meets the counter as the first one left it)
+    for _ in range(2):
         assert lpb.lp_softmax_xent_static(z.cuda(), y.cuda(), delta, loss, C) == lpb.LP_OK
     logp = torch.log_softmax(z[:, :C].double(), 1)
     rows = torch.arange(B)
@@ -131,3 +131,39 @@ def test_static_loss_at_the_edges_of_its_row_forms(B, C, ld):
     assert torch.all((got[:, :C] - want).abs() <= 2.0 ** -8 * want.abs() + 1e-6 / B)
     assert torch.all(got[:, C:(C + 7) // 8 * 8] == 0.0)
     assert abs(float(loss) - ref_loss) <= 2e-6 * max(1.0, abs(ref_loss))
+
+
+def test_static_loss_after_calls_that_overlapped():
+    """Two calls that overlap on the shared scratch may give wrong losses and leave its counter anywhere; the header
+    promises that ordered calls after them are right again.  16 pairs of calls of many blocks, numbers unequal, run on
+    two streams at the same time; then ordered calls of many batch sizes against float64."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    C, wide, big = 1000, 4000, [3000, 2900]
+    g = torch.Generator().manual_seed(3)
+    z = torch.randn(8192, C, generator=g)
+    y = torch.randint(0, C, (8192,), generator=g, dtype=torch.int32)
+    zd, yd, zw = z.cuda(), y.cuda(), torch.randn(3000, wide, device="cuda")
+    delta, loss = torch.zeros(8192, C, dtype=torch.bfloat16, device="cuda"), torch.zeros(1, device="cuda")
+    scrap = [torch.zeros(3000, wide, dtype=torch.bfloat16, device="cuda") for _ in range(3)]
+    losses = [torch.zeros(1, device="cuda") for _ in range(3)]
+    streams, hold = [torch.cuda.Stream() for _ in range(2)], torch.cuda.Stream()
+    for _ in range(16):
+        torch.cuda.synchronize()
+        with torch.cuda.stream(hold):
+            torch.cuda._sleep(20_000_000)             # (about ten milliseconds: both calls are enqueued before it ends)
+            gate = hold.record_event()
+        for k, s in enumerate(streams):
+            s.wait_event(gate)
+            with torch.cuda.stream(s):
+                assert lpb.lp_softmax_xent_static(zw[:big[k]], yd[:big[k]], scrap[k], losses[k], wide) == lpb.LP_OK
+            for _ in range(63 if k == 0 else 0):      # (counters may be handed out in turn: the pair shares one of 64)
+                assert lpb.lp_softmax_xent_static(zw, yd[:3000], scrap[2], losses[2], wide) == lpb.LP_OK
+    torch.cuda.synchronize()
+    logp = torch.log_softmax(z.double(), 1)
+    for i in range(130):
+        B = 2048 + 47 * i
+        labels = (y[:B] + 7 * i) % C                  # (new row losses: what the scratch holds from the call before is wrong)
+        assert lpb.lp_softmax_xent_static(zd[:B], labels.cuda(), delta, loss, C) == lpb.LP_OK
+        want = float(-logp[torch.arange(B), labels.long()].mean())
+        assert abs(float(loss) - want) <= 2e-6 * max(1.0, abs(want)), (i, B)
