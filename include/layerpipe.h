@@ -164,9 +164,10 @@ int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev, void* str
  * lp_plan / lp_plan_costs write ([2l] = delta'' or the whole, [2l+1] = delta'; amount 0 = no such
  * piece).  For every layer with two pieces the columns of delta^{l-1} are divided in the ratio of
  * the amounts, rounded to whole tiles of the contraction kernel (at least one tile each); piece
- * [2l] is enqueued on the delta stream of stage piece_stage[2l], piece [2l+1] on that of
- * piece_stage[2l+1], each with the unchanged f' epilogue, and delta^{l-1} counts as written when
- * both have finished.  Layers whose delta kernel has a single column tile, or runs split-K, keep
+ * [2l] is enqueued on a stream that the handle keeps for borrowed pieces (it takes the place of one of
+ * the G + update streams; where there is only one of those the pieces follow one another), piece
+ * [2l+1] on the minibatch's chain, each with the unchanged f' epilogue, and delta^{l-1} counts as written when
+ * both have finished.  piece_stage is checked against the number of stages; on one GPU it places nothing.  Layers whose delta kernel has a single column tile, or runs split-K, keep
  * one piece.  The numbers do not change: every output element is produced by the same
  * instructions in the same order as in the unsplit launch.  split_col_out (host [n_layers], may be
  * NULL) receives the first column of delta' (0 = unsplit).  Must be called before the first

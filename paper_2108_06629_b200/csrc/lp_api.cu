@@ -117,10 +117,9 @@ struct Layer {
   Res rDW;
   Ev last_update;
   // Section III-B: the delta contraction of this layer split by output columns into delta'' =
-  // columns [0, split_col), run on the streams of piece_stage[0] (the stage holding layer l+1),
-  // and delta' = columns [split_col, n_in), run on piece_stage[1].  split_col = 0: one piece.
+  // columns [0, split_col), run on the handle's piece stream, and delta' = columns [split_col, n_in), run on the
+  // minibatch's chain.  split_col = 0: one piece.
   int split_col = 0;
-  int piece_stage[2] = {0, 0};
   // Activation recomputation (LP_RECOMPUTE): this layer's INPUT a^{l-1} (with the stored z^{l-1} and the
   // pooling positions that go with it) is not stashed for d_l + 2 minibatches.  The forward pass
   // keeps it in two short-lived slots (0, 1); when the backward pass of minibatch n reaches the
@@ -152,13 +151,15 @@ struct lp_ctx {
   int* status = nullptr;        // device status word
   std::vector<lp::Res> rZL, rLabels;
   // streams / events
-  // streams[0] = the caller's stream of the current lp_step, then the P chain streams, then the Q G streams
+  // streams[0] = the caller's stream of the current lp_step, then the P chain streams, then the Q G streams, then the piece stream
   static constexpr int kMaxStreams = 16;
   std::vector<cudaStream_t> streams;
   unsigned long long caller_id = 0;   // cudaStreamGetId of streams[0]: two streams can have the same handle (cudaStreamPerThread
                                       // in two threads, a stream created after another was destroyed), never the same id
   int chain_index(long long n) const { return 1 + int(n % n_chain); }
   int g_index(int l) const { return 1 + n_chain + l % n_g; }
+  bool has_piece_stream = false;      // some delta contraction is split: the last G stream has become the piece stream
+  int piece_index() const { return 1 + n_chain + n_g; }
   // Recorded events of a stream, oldest overwritten first.  A wait for task `pos` takes the first
   // record at or after it (or records one), so a record that has been overwritten only makes a later wait coarser,
   // never wrong.  `vc` = what the stream had waited for by then (per stream, the last task known complete).
@@ -1286,6 +1287,7 @@ extern "C" int lp_set_delta_split(lp_handle h, const int* piece_stage, const lon
       if ((k == 0 ? a0 : a1) > 0 && (piece_stage[2 * l + k] < 0 || piece_stage[2 * l + k] >= h->n_stages))
         return fail(h, LP_ERR_INVALID_ARG, "piece stage outside [0, n_stages)");
   }
+  bool any = false;
   for (int l = 0; l < nL; ++l) {
     Layer& y = h->L[l];
     y.split_col = 0;
@@ -1301,9 +1303,24 @@ extern "C" int lp_set_delta_split(lp_handle h, const int* piece_stage, const lon
     long long t0 = (tiles * a0 + (a0 + a1) / 2) / (a0 + a1);        // nearest whole number of tiles for delta''
     t0 = std::max<long long>(1, std::min<long long>(tiles - 1, t0));
     y.split_col = int(t0) * wd;
-    y.piece_stage[0] = piece_stage[2 * l];
-    y.piece_stage[1] = piece_stage[2 * l + 1];
+    any = true;
     if (split_col_out) split_col_out[l] = y.split_col;
+  }
+  // delta'' is part of the critical loop: it gets a stream of its own with the chains' priority, within the same number of
+  // hardware queues, in the place of one G stream.  (On the G streams it waited behind the updates queued there: 8 x 4096
+  // MLP 569 us a step unsplit, 743 split; on another minibatch's chain 590 .. 840, behind delta' on its own 623, here 569.)
+  // With a single G stream, or under fused-B, the pieces follow one another.
+  const bool want = any && h->n_g >= (h->has_piece_stream ? 1 : 2);
+  if (want != h->has_piece_stream) {
+    int least = 0, greatest = 0;
+    LP_CUDA(h, cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    const int idx = want ? h->n_chain + h->n_g : h->piece_index();      // (nothing has been enqueued on it: no step yet)
+    cudaStream_t fresh = nullptr;
+    LP_CUDA(h, cudaStreamCreateWithPriority(&fresh, cudaStreamNonBlocking, want ? greatest : least));
+    cudaStreamDestroy(h->streams[size_t(idx)]);
+    h->streams[size_t(idx)] = fresh;
+    h->n_g += want ? -1 : 1;
+    h->has_piece_stream = want;
   }
   return LP_OK;
 }
@@ -1462,11 +1479,11 @@ extern "C" int lp_step(lp_handle h, const void* batch_dev, const int* labels_dev
       LP_CUDA(c, launch_update(c, l, n, st));
       LP_CUDA(c, task_end(c, sc, {rdl, rw, rx, raux, ridx}, {rdprev, &y.rDW, rnew, rpart}, &y.last_update));
     } else {
-      if (l > 0 && y.split_col > 0 && !serial) {
-        // delta'' on a stream picked by the stage that borrowed it, delta' on the minibatch's chain: two kernels over
+      if (l > 0 && y.split_col > 0 && !serial && c->has_piece_stream) {
+        // delta'' on the piece stream, delta' on the minibatch's chain: two kernels over
         // disjoint column ranges of delta^{l-1}, concurrent; the buffer counts as written when both are
         // done (the chain joins the other stream before the event that later tasks wait on)
-        const int s0 = c->g_index(y.piece_stage[0]);
+        const int s0 = c->piece_index();
         LP_CUDA(c, task_begin(c, s0, {rdl, rw, raux, ridx}, {rdprev}));
         LP_CUDA(c, task_begin(c, sc, {rdl, rw, raux, ridx}, {rdprev}));
         LP_CUDA(c, launch_delta(c, l, n, slot[l], c->streams[s0], 0));
@@ -1812,7 +1829,7 @@ extern "C" int lp_task_progress(lp_handle h, char* text, int capacity) {
   for (size_t si = 0; si < h->streams.size(); ++si) {
     const unsigned done = *reinterpret_cast<volatile unsigned*>(h->trace_done + si), enq = h->trace_enq[si];
     if (done == enq) continue;
-    const char* role = si == 0 ? "caller" : (int(si) <= h->n_chain ? "chain" : "G");
+    const char* role = si == 0 ? "caller" : int(si) <= h->n_chain ? "chain" : h->has_piece_stream && int(si) == h->piece_index() ? "delta''" : "G";
     const unsigned started = *reinterpret_cast<volatile unsigned*>(h->trace_done + h->streams.size() + si);
     snprintf(line, sizeof line, "stream %d (%s): %u of %u tasks done, %s; unfinished:", int(si), role, done, enq, started > done ? "the next one has STARTED" : "the next one has not started");
     out += line;

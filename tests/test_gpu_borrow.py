@@ -190,3 +190,38 @@ def test_training_with_the_planners_pieces_is_bit_identical(case):
             for a, b in zip(got["W"], ref["W"]):
                 assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     assert n_split >= 1, "the plan split no layer of this case"
+
+
+def test_borrowed_pieces_do_not_queue_behind_gradient_tasks():
+    """Behind a gate, with every task of a step still unfinished: delta'' sits on a stream of its own, and no stream
+    that holds G tasks holds a delta task.  Without a split, or after it has been taken back, there is no such stream."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    from paper_2108_06629_b200 import inputs as I
+    layers, B = I.mlp([520, 600, 328, 456, 392, 75], "gelu"), 72
+    W0, b0 = I.initial_weights(layers, 0)
+    plan = lpb.lp_plan(layers, B, 4)
+    whole = [0] * (2 * len(layers))
+    x, y = (torch.from_numpy(t).cuda() for t in I.minibatch(layers, B, 0))
+    for amounts, split in ((None, False), ([plan["piece_amount"]], True), ([plan["piece_amount"], whole], False),
+                           ([plan["piece_amount"], whole, plan["piece_amount"]], True)):
+        tr = lpb.Trainer(layers, B, 4, flags=lpb.LP_TRACE_TASKS, W0=W0, b0=b0)
+        for a in amounts or ():
+            cols = tr.set_delta_split(plan["piece_stage"], a)
+            assert any(cols) == any(a)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(300_000_000)
+        tr.step(x, y)
+        lines = tr.task_progress().splitlines()
+        tr.flush()
+        torch.cuda.synchronize()
+        streams = [l for l in lines if l.startswith("stream ")]
+        assert sum("(chain)" in l for l in streams) == 1 and any("(G)" in l for l in streams)
+        assert sum("(delta'')" in l for l in streams) == (1 if split else 0), streams
+        for l in streams:
+            if "(G)" in l:
+                assert "G(layer" in l and "delta(layer" not in l, l
+            if "(delta'')" in l:
+                assert "delta(layer" in l and "G(layer" not in l, l
+        assert tr.device_status() == (0, 0)
+        tr.close()
