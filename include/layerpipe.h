@@ -138,7 +138,8 @@ int lp_workspace_size(const lp_layer* layers, int n_layers, int n_stages, const 
  * pairs (tcgen05 cta_group::2), every other network runs single-CTA kernels only.  LP_CONV_PAIR=1
  * in the environment also puts wide convolution layers on SM pairs: a measurement mode, not for
  * long runs (networks that alternate the two kinds on the same SMs have stalled in tcgen05.alloc
- * after some 10^6 pair CTAs).  Two handles of different kinds should not run concurrently on one GPU.
+ * after some 10^6 pair CTAs).  LP_CONV_WIDE_ITEMS=n in the environment lets the two-tile convolution
+ * kernel of more than 64 channels start at n items a launch instead of 592 (verification).  Two handles of different kinds should not run concurrently on one GPU.
  */
 int lp_create(lp_handle* out, const lp_layer* layers, int n_layers, int n_stages,
               const int* stage, const int* delays, const lp_config* cfg,
@@ -300,6 +301,12 @@ int lp_destroy(lp_handle h);
  */
 int lp_gemm_bf16(int which, int M, int N, int K, const void* A_dev, int lda,
                  const void* B_dev, int ldb, float* C_dev, int ldc, void* stream);
+
+/* Verification: the kernel form that the calling thread's latest contraction launch took (lp_step,
+ * lp_debug_run_task, lp_gemm_bf16), its tile width and, behind an x, the cluster size or the pipeline depth where the
+ * choice includes one: "cluster 64 x4", "pair persistent 256", "wide halo 128".  "" before the first.  Valid
+ * until the thread's next call. */
+const char* lp_debug_last_contraction(void);
 
 /* Status word of the lp_gemm_bf16 launches on the current device since the last call: waits for
  * the device, returns LP_OK (word 0) or LP_ERR_TIMEOUT (a bounded wait inside a kernel ran out;

@@ -96,6 +96,8 @@ def lib():
     L.lp_kernel_launches.restype = C.c_longlong
     L.lp_last_error.argtypes = [vp]
     L.lp_last_error.restype = C.c_char_p
+    L.lp_debug_last_contraction.argtypes = []
+    L.lp_debug_last_contraction.restype = C.c_char_p
     _lib = L
     return L
 
@@ -103,7 +105,7 @@ def lib():
 EXPORTS = ["lp_plan", "lp_plan_costs", "lp_workspace_size", "lp_create", "lp_step", "lp_flush",
            "lp_get_weights", "lp_get_grads", "lp_debug_read", "lp_debug_write", "lp_debug_run_task", "lp_get_schedule", "lp_get_version_log", "lp_get_loss",
            "lp_device_status", "lp_task_progress", "lp_get_task_time", "lp_reset_task_times", "lp_get_layer_task_time", "lp_set_delta_split", "lp_get_task_timeline", "lp_kernel_launches", "lp_set_tuning", "lp_last_error", "lp_destroy",
-           "lp_gemm_bf16", "lp_gemm_status", "lp_debug_gemm_starved", "lp_softmax_xent_static"]
+           "lp_gemm_bf16", "lp_gemm_status", "lp_debug_last_contraction", "lp_debug_gemm_starved", "lp_softmax_xent_static"]
 
 
 _torch = None
@@ -373,6 +375,11 @@ class Trainer:
 def lp_gemm_bf16(which, M, N, K, A, lda, B, ldb, Cout, ldc, stream=None):
     """A, B: torch bf16 device tensors; Cout: torch fp32 device tensor."""
     _check(lib().lp_gemm_bf16(which, M, N, K, A.data_ptr(), lda, B.data_ptr(), ldb, Cout.data_ptr(), ldc, _stream_of(stream)))
+
+
+def lp_debug_last_contraction():
+    """Kernel form of this thread's latest contraction launch, e.g. "cluster 64 x4"."""
+    return lib().lp_debug_last_contraction().decode()
 
 
 def lp_gemm_status():

@@ -68,6 +68,7 @@ struct HaloGUpdate;
 // G (+ fused update) of a halo-tile layer: tmX = the activations with the 64 x 10 x 18 x 1 halo box,
 // tmD = delta with a 64 x 8 x 16 x 1 box; partial: conv_halo_g_max_ctas() x 5 x 128 x 64 floats.
 int conv_halo_g_max_ctas();
+const char* gemm_last_contraction();   // see lp_debug_last_contraction
 cudaError_t gemm_configure();   // opt in to large dynamic shared memory; call once per process
 void gemm_set_tuning(int bn, int stages, int splits);   // 0 = automatic
 int gemm_pick_splits(int M, int N, int K, int bn);

@@ -127,6 +127,21 @@ void gemm_set_tuning(int bn, int stages, int splits) {
   if (g_force_persistent > 1) g_force_persistent = -1;
 }
 
+// What lp_debug_last_contraction tells: the kernel form of this thread's latest contraction launch, its tile width, and
+// the cluster size or pipeline depth where that is part of the choice.
+struct LastContraction {
+  const char* kernel;
+  int tile, detail;
+};
+static thread_local LastContraction t_last = {"", 0, 0};
+static void note_form(const char* kernel, int tile, int detail = 0) { t_last = {kernel, tile, detail}; }
+const char* gemm_last_contraction() {
+  static thread_local char text[96];
+  if (t_last.detail > 0) snprintf(text, sizeof text, "%s %d x%d", t_last.kernel, t_last.tile, t_last.detail);
+  else                   snprintf(text, sizeof text, "%s %d", t_last.kernel, t_last.tile);
+  return t_last.tile == 0 ? "" : text;
+}
+
 static int sm_count() {
   static int n = 0;
   if (n == 0) {
@@ -258,6 +273,7 @@ static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, Ge
   gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, SPL, PER><<<grid, GEMM_THREADS, smem, st>>>(tmA, tmB, *um, a, tiles_m, tiles_n, int(work))
   if constexpr (MODE == EPI_WGRAD_UPDATE && BN >= 128) {
     if (a.upd_tma) {
+      note_form(a.persistent ? "single streamed persistent" : "single streamed", BN);
       if (a.persistent)
         gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, false, true, true><<<grid, GEMM_THREADS, smem, st>>>(tmA, tmB, *um, a, tiles_m, tiles_n, int(work));
       else
@@ -265,6 +281,7 @@ static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, Ge
       return cudaGetLastError();
     }
   }
+  note_form(a.splits > 1 ? (a.persistent ? "single split persistent" : "single split") : (a.persistent ? "single persistent" : "single"), BN);
   if (a.splits > 1) { if (a.persistent) LP_LAUNCH(true, true); else LP_LAUNCH(true, false); }
   if constexpr (A_MN && BN <= 128) {
     if (a.splits > 1 && a.split_reduce) {
@@ -330,6 +347,7 @@ static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  note_form("cluster", BN, a.cluster);
   return cudaLaunchKernelEx(&cfg, gemmc_kernel<BN, A_MN, B_MN, MODE>, tmA, tmB, a, tiles_m);
 }
 #define LP_FOR_EACH_CLUSTER_VARIANT(X, BN) \
@@ -390,8 +408,10 @@ static cudaError_t launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, G
         // 192 KiB of shared memory divided between operand stages and update-chunk slots
         // (chunk slots are 16 KiB, 32 KiB with momentum: four operand stages leave four / two of them, three leave six / three)
         a.num_stages = g_force_stages > 0 ? std::max(2, std::min(g_force_stages, 5)) : (a.mW != nullptr ? 3 : 4);
+        note_form("pair streamed persistent", BN2);
         return cudaLaunchKernelEx(&cfg, gemm2p_g_update_kernel<0>, tmA, tmB, *um, a, tiles_m, tiles_n);
       }
+      note_form("pair streamed", BN2, s);
       return cudaLaunchKernelEx(&cfg, gemm2_tcgen05_kernel<A_MN, B_MN, MODE, true>, tmA, tmB, *um, a);
     }
   }
@@ -411,9 +431,11 @@ static cudaError_t launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, G
       cfg.blockDim = dim3(GEMM2Q_THREADS, 1, 1);
       cfg.dynamicSmemBytes = GEMM2Q_SMEM_BYTES;
       a.num_stages = GEMM2Q_STAGES;
+      note_form("pair persistent", BN2);
       return cudaLaunchKernelEx(&cfg, gemm2q_kernel<A_MN, B_MN, MODE, BN2>, tmA, tmB, a, tiles_m, tiles_n);
     }
   }
+  note_form("pair", BN2, s);
   return cudaLaunchKernelEx(&cfg, gemm2_tcgen05_kernel<A_MN, B_MN, MODE, false, BN2>, tmA, tmB, *um, a);
 }
 template <bool A_MN, bool B_MN, int MODE>
@@ -456,6 +478,7 @@ cudaError_t conv_halo_launch(int which, const CUtensorMap& tmA, const CUtensorMa
   const int tiles = args.g.kind == GEOM_PLAIN ? (args.M + GEMM_BM - 1) / GEMM_BM
                                                : args.g.tiles_w * args.g.tiles_h * (args.M / (args.g.H * args.g.W));
   const int grid = std::min(tiles, sm_count());
+  note_form(args.g.kind == GEOM_PLAIN ? "halo plain" : "halo", 64);
 #define LP_TRYH(B, M)                                                                                          \
   if (b_mn == B && args.mode == M) {                                                                           \
     conv_halo_kernel<B, M><<<grid, HALO_THREADS, HALO_SMEM_BYTES, st>>>(tmA, tmB, tmO, args, tiles);                \
@@ -475,6 +498,7 @@ cudaError_t conv_wide_launch(int which, int bn, const CUtensorMap& tmA, const CU
   if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
   const int tiles = a.g.tiles_w * a.g.tiles_h * (a.M / (a.g.H * a.g.W)), tiles_n = (a.N - a.n_begin + bn - 1) / bn;
   const int grid = std::min((tiles + 1) / 2 * tiles_n, sm_count());
+  note_form("wide halo", bn);
 #define LP_TRYW(BN, B, M)                                                                                      \
   if (bn == BN && b_mn == B && a.mode == M) {                                                                  \
     conv_wide_kernel<BN, B, M><<<grid, WIDE_THREADS, wide_smem_bytes(BN), st>>>(tmA, tmB, a, tiles, tiles_n);  \
@@ -494,6 +518,7 @@ cudaError_t conv_halo_g_launch(const CUtensorMap& tmX, const CUtensorMap& tmD, c
   upd.partial = partial;
   upd.n_ctas = grid;
   for (int co0 = 0; co0 < upd.n_out; co0 += 64) {      // one pass per 64 output channels; the stream orders the reuse of `partial`
+    note_form("halo G", 64);
     conv_halo_g_kernel<0><<<grid, GEMM_THREADS, HALOG_SMEM_BYTES, st>>>(tmX, tmD, g, tiles, co0, partial, status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -665,6 +690,8 @@ extern "C" int lp_gemm_bf16(int which, int M, int N, int K, const void* A, int l
                             float* C, int ldc, void* stream) {
   return gemm_standalone(which, M, N, K, A, lda, B, ldb, C, ldc, stream, 0, 0);
 }
+
+extern "C" const char* lp_debug_last_contraction(void) { return lp::gemm_last_contraction(); }
 
 extern "C" int lp_gemm_status(int* detail) {
   int* status_dev = nullptr;

@@ -480,8 +480,11 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       // least two 64-channel chunks and every CTA gets at least four items (measured in conv_wide.cuh; with one item each,
       // 16 x 16 pixels at batch 128, 16 steps of the small VGG took 4520 us against 4390)
       const long long pairs_of_tiles = (long long)B * (y.imW / 8) * (y.imH / 16) / 2;
-      y.wide_f = !y.patch && tiles_8x16 && y.ld_in > 64 && y.bn_f == 128 && pairs_of_tiles * ((y.n_out + 127) / 128) >= 4 * 148;
-      y.wide_d = l > 0 && tiles_8x16 && y.ld_out > 64 && y.bn_d == 128 && pairs_of_tiles * ((y.n_in + 127) / 128) >= 4 * 148;
+      // (LP_CONV_WIDE_ITEMS in the environment is another least number of items: what the tests force the form with)
+      const char* items = getenv("LP_CONV_WIDE_ITEMS");
+      const long long enough = items != nullptr ? atoll(items) : 4 * 148;
+      y.wide_f = !y.patch && tiles_8x16 && y.ld_in > 64 && y.bn_f == 128 && pairs_of_tiles * ((y.n_out + 127) / 128) >= enough;
+      y.wide_d = l > 0 && tiles_8x16 && y.ld_out > 64 && y.bn_d == 128 && pairs_of_tiles * ((y.n_in + 127) / 128) >= enough;
       y.lean_f = y.patch && y.n_out <= 64 && y.ld_in <= 64 && l + 1 < n;
       // G contracts over all B*H*W pixels but has only (Cout/128) x 9 x (Cin/BN) tiles: the pixel
       // range is split, and a second launch adds the partial tiles on all SMs and applies the update

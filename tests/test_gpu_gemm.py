@@ -123,10 +123,10 @@ def test_bounded_wait_runs_out_reports_and_leaves_the_device_usable():
     assert lib.lp_debug_gemm_starved(M, N, K, Ad.data_ptr(), K, Bd.data_ptr(), K, Cd.data_ptr(), N, 5, None) == lpb.LP_ERR_INVALID_ARG
 
 
-# Outputs of few tiles, where the contraction is divided over a cluster: fewer, as many and more k-blocks than CTAs, a last
-# rank without or with a ragged k-block, clusters of 2, 4 and 8, tiles of 64 and 128 columns with ragged edges, one row.
+# Outputs of few tiles, where the contraction is divided over a cluster: as many and more k-blocks than CTAs, ranks with
+# one k-block more than others, a ragged last k-block, clusters of 2, 4 and 8, tiles of 64 and 128 columns with ragged edges, one row.
 CLUSTER_SHAPES = [(1, 8, 65), (33, 70, 128), (128, 64, 200), (100, 777, 1003), (129, 130, 256), (64, 2050, 4100), (250, 513, 1000),
-                  (40, 300, 4160), (384, 1000, 3000), (300, 4100, 1100)]
+                  (40, 300, 4160), (384, 1000, 3000), (300, 4100, 1100), (300, 4100, 2100)]
 
 
 @pytest.mark.parametrize("which", [0, 1, 2])
@@ -134,14 +134,38 @@ def test_contraction_divided_over_a_cluster(which):
     """Against float64; the partial sums are shorter than the undivided one, so its bound holds."""
     import torch
     from paper_2108_06629_b200 import binding as lpb
+    forms = set()
     for i, (M, N, K) in enumerate(CLUSTER_SHAPES):
         A, B = _operands(which, M, N, K, 900 + 100 * which + i)
         ldc = (N + 3) // 4 * 4
         Cd = torch.full((M, ldc), 7.0, device="cuda")
         Ad, Bd = A.cuda(), B.cuda()
         lpb.lp_gemm_bf16(which, M, N, K, Ad, A.shape[1], Bd, B.shape[1], Cd, ldc)
+        forms.add(lpb.lp_debug_last_contraction())
         torch.cuda.synchronize()
         got = Cd.cpu().numpy()
         assert rel_l2(got[:, :N], _reference(which, M, N, K, A, B)) < 1e-6 + 2e-7 * np.sqrt(K), (which, M, N, K)
         assert np.all(got[:, N:] == 0.0)
         assert lpb.lp_gemm_status() == (lpb.LP_OK, 0)
+    assert {"cluster 64 x2", "cluster 64 x4", "cluster 64 x8", "cluster 128 x2"} <= forms, forms
+
+
+# Plain fp32 results on SM pairs: at least two tiles a pair (persistent, 256 and 224 columns, MN-major A in the G form), and no
+# more tiles than pairs (six stages), with ragged last rows, columns and k-blocks.
+@pytest.mark.parametrize("which, M, N, K, form", [
+    (0, 1024, 9467, 1100, "pair persistent 256"), (1, 1024, 9467, 1100, "pair persistent 256"), (2, 1024, 9467, 1100, "pair persistent 256"),
+    (0, 1100, 7677, 1030, "pair persistent 224"), (1, 1100, 7677, 1030, "pair persistent 224"), (2, 1100, 7677, 1030, "pair persistent 256"),
+    (0, 1030, 1100, 1040, "pair 224 x6"), (1, 1030, 1100, 1040, "pair 224 x6"), (2, 1030, 1100, 1040, "pair 256 x6")])
+def test_contraction_on_sm_pairs(which, M, N, K, form):
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    A, B = _operands(which, M, N, K, 77 + which)
+    ldc = (N + 3) // 4 * 4
+    Cd = torch.full((M, ldc), 7.0, device="cuda")
+    lpb.lp_gemm_bf16(which, M, N, K, A.cuda(), A.shape[1], B.cuda(), B.shape[1], Cd, ldc)
+    assert lpb.lp_debug_last_contraction() == form
+    torch.cuda.synchronize()
+    got = Cd.cpu().numpy()
+    assert rel_l2(got[:, :N], _reference(which, M, N, K, A, B)) < 1e-6 + 2e-7 * np.sqrt(K)
+    assert np.all(got[:, N:] == 0.0)
+    assert lpb.lp_gemm_status() == (lpb.LP_OK, 0)

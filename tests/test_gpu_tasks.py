@@ -431,13 +431,38 @@ def test_tasks_bias_gradient_of_many_rows(rows, n_out):
     tr.close()
 
 
-@pytest.mark.parametrize("H, W, B, chans, pools", [(16, 8, 3, [72, 136, 40], [0, 0, 2]), (32, 16, 2, [96, 200, 72], [0, 2, 2]),
-                                                   (16, 16, 8, [64, 128, 128], [0, 2, 0]), (16, 24, 16, [80, 24, 160], [0, 0, 2])])
-def test_tasks_two_halo_tiles_under_streamed_weights(H, W, B, chans, pools):
-    """Convolutions of more than 64 channels on 8 x 16 pixel tiles: an odd number of tiles (the last pair holds one),
-    channel counts that end inside a 64-channel chunk or a column tile, several column tiles, delta onto 64 or fewer
-    channels, pooled in the epilogue or not, and un-pooling."""
+def _forms(monkeypatch):
+    """Records the kernel form of every contraction that a task runs: {(task, layer): forms}."""
+    from paper_2108_06629_b200 import binding as lpb
+    forms, run = {}, lpb.Trainer.debug_run_task
+
+    def recorded(self, task, layer, step):
+        run(self, task, layer, step)
+        forms.setdefault((task, layer), set()).add(lpb.lp_debug_last_contraction())
+    monkeypatch.setattr(lpb.Trainer, "debug_run_task", recorded)
+    return forms
+
+
+def _wide_layers(forms, task):
+    return [l for (t, l), f in sorted(forms.items()) if t == task and f == {"wide halo 128"}]
+
+
+# wide: the layers whose forward / delta must run on the kernel (layer 0 is the patch-matrix form)
+@pytest.mark.parametrize("H, W, B, chans, pools, wide_f, wide_d", [
+    (16, 8, 3, [72, 136, 80], [0, 0, 2], [1, 2], [1, 2]),            # three tiles: the last pair holds one; two column tiles
+    (32, 16, 2, [96, 200, 72], [0, 2, 2], [1, 2], [1, 2]),           # pooled forward, un-pooling delta over two column tiles
+    (16, 16, 8, [80, 128, 128], [0, 0, 0], [1, 2], [1, 2]),
+    (32, 32, 3, [136, 264], [2, 0], [1], [1]),                       # three column tiles, un-pooling onto a ragged one
+    (16, 24, 16, [80, 72, 160], [0, 0, 2], [1, 2], [1, 2]),
+    (16, 24, 2, [64, 128, 24], [0, 0, 0], [], []),                   # at most 64 channels on the other side: not for this kernel
+])
+def test_tasks_two_halo_tiles_under_streamed_weights(H, W, B, chans, pools, wide_f, wide_d, monkeypatch):
+    """Convolutions of more than 64 channels on 8 x 16 pixel tiles, from one item a launch on: an odd number of tiles,
+    channel counts that end inside a 64-channel chunk or a column tile, several column tiles, pooled in
+    the epilogue or not, and un-pooling."""
     from paper_2108_06629_b200 import inputs as I
+    monkeypatch.setenv("LP_CONV_WIDE_ITEMS", "0")
+    forms = _forms(monkeypatch)
     layers, c = [], 3
     for n, pool in zip(chans, pools):
         layers.append(I.conv(c, n, H, W, pool=pool))
@@ -446,3 +471,13 @@ def test_tasks_two_halo_tiles_under_streamed_weights(H, W, B, chans, pools):
             H, W = H // 2, W // 2
     layers.append(I.fc(c * H * W, 10, "none"))
     run_teacher_forced(layers, B, 2, None, 0.05, 0.9, 2)
+    assert _wide_layers(forms, "forward") == wide_f and _wide_layers(forms, "delta") == wide_d, forms
+
+
+def test_tasks_two_halo_tiles_by_the_automatic_rule(monkeypatch):
+    """600 items (300 pairs of pixel tiles, two column tiles) take the kernel, 300 items do not."""
+    from paper_2108_06629_b200 import inputs as I
+    forms = _forms(monkeypatch)
+    layers = [I.conv(3, 72, 80, 120), I.conv(72, 136, 80, 120), I.conv(136, 72, 80, 120, pool=2), I.fc(72 * 40 * 60, 10, "none")]
+    run_teacher_forced(layers, 8, 2, None, 0.05, 0.0, 1)
+    assert _wide_layers(forms, "forward") == [1] and _wide_layers(forms, "delta") == [2], forms

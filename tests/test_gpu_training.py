@@ -261,10 +261,13 @@ def test_serial_tasks_agree_and_timeline_is_consistent():
     tr.close()
 
 
-def test_fewer_hardware_queues_fold_the_stages_and_change_nothing():
-    """With CUDA_DEVICE_MAX_CONNECTIONS = 8 (the CUDA default) lp_create folds the stages onto two
-    stream triples; the tensors must be bit-identical to the unfolded run.  The variable is read
-    when the CUDA context is created, so the folded run is a child process."""
+@pytest.mark.parametrize("env, layerpipe, fused_b", [
+    ({"CUDA_DEVICE_MAX_CONNECTIONS": "8"}, (4, 3), (7, 0)), ({"CUDA_DEVICE_MAX_CONNECTIONS": "4"}, (2, 1), (3, 0)),
+    ({"CUDA_DEVICE_MAX_CONNECTIONS": "2"}, (1, 1), (1, 0)), ({"CUDA_DEVICE_MAX_CONNECTIONS": "32", "LP_STREAM_TRIPLES": "3"}, (3, 3), (3, 0))])
+def test_fewer_hardware_queues_make_fewer_streams_and_change_nothing(env, layerpipe, fused_b):
+    """lp_create makes as many (chain, G) streams as the process has hardware queues for, and the tensors do not depend
+    on their number.  The variable is read when the driver is initialised, so every arrangement is a child process; it
+    counts the streams that hold unfinished tasks of eight minibatches behind a gate."""
     import json
     import os
     import subprocess
@@ -276,22 +279,38 @@ def test_fewer_hardware_queues_fold_the_stages_and_change_nothing():
     a, _, _ = free_run(layers, 56, 4, [3, 2, 1, 0], 0.02, 0.9, 8, lpb.LP_SCHED_LAYERPIPE)
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     child = (
-        "import sys, json, numpy as np\n"
+        "import sys, json, numpy as np, torch\n"
         "sys.path.insert(0, %r); sys.path.insert(0, %r)\n"
-        "import test_gpu_training as T\n"
         "from paper_2108_06629_b200 import binding as lpb, inputs as I\n"
         "layers = I.mlp([264, 192, 320, 136, 40], 'gelu')\n"
-        "a, _, _ = T.free_run(layers, 56, 4, [3, 2, 1, 0], 0.02, 0.9, 8, lpb.LP_SCHED_LAYERPIPE)\n"
-        "np.savez(sys.argv[1], loss=np.array(a['loss']), **{'W%%d' %% l: a['W'][l][0] for l in range(len(layers))})\n"
+        "W0, b0 = I.initial_weights(layers, 0)\n"
+        "data = [tuple(torch.from_numpy(t).cuda() for t in I.minibatch(layers, 56, n)) for n in range(8)]\n"
+        "counts = []\n"
+        "for sched in (lpb.LP_SCHED_LAYERPIPE, lpb.LP_SCHED_FUSED_B):\n"
+        "    tr = lpb.Trainer(layers, 56, 4, delays=[3, 2, 1, 0], lr=0.02, momentum=0.9, schedule=sched, W0=W0, b0=b0)\n"
+        "    for x, y in data: tr.step(x, y)\n"
+        "    tr.flush(); torch.cuda.synchronize()\n"
+        "    assert tr.device_status() == (0, 0)\n"
+        "    np.savez(sys.argv[1] + '%%d.npz' %% sched, loss=np.array([tr.get_loss(n) for n in range(8)]), **{'W%%d' %% l: tr.get_weights(l)[0] for l in range(len(layers))})\n"
+        "    tr.close()\n"
+        "    tr = lpb.Trainer(layers, 56, 4, delays=[3, 2, 1, 0], schedule=sched, flags=lpb.LP_TRACE_TASKS, W0=W0, b0=b0)\n"
+        "    torch.cuda.synchronize()\n"
+        "    torch.cuda._sleep(300_000_000)\n"
+        "    for x, y in data: tr.step(x, y)\n"
+        "    lines = tr.task_progress().splitlines()\n"
+        "    counts.append([sum(l.startswith('stream') and ('(%%s)' %% k) in l for l in lines) for k in ('chain', 'G')])\n"
+        "    tr.flush(); torch.cuda.synchronize(); tr.close()\n"
+        "print(json.dumps(counts))\n"
     ) % (root, os.path.join(root, "tests"))
     with tempfile.TemporaryDirectory() as d:
-        out = os.path.join(d, "folded.npz")
-        env = dict(os.environ, CUDA_DEVICE_MAX_CONNECTIONS="8")
-        subprocess.run([sys.executable, "-c", child, out], check=True, env=env, timeout=600)
-        z = np.load(out)
-        for l in range(len(layers)):
-            assert np.array_equal(z["W%d" % l], a["W"][l][0])
-        assert np.array_equal(z["loss"], np.array(a["loss"]))
+        out = os.path.join(d, "run")
+        run = subprocess.run([sys.executable, "-c", child, out], check=True, env=dict(os.environ, **env), timeout=600, stdout=subprocess.PIPE)
+        assert json.loads(run.stdout.decode().splitlines()[-1]) == [list(layerpipe), list(fused_b)]
+        for sched in (lpb.LP_SCHED_LAYERPIPE, lpb.LP_SCHED_FUSED_B):
+            z = np.load(out + "%d.npz" % sched)
+            for l in range(len(layers)):
+                assert np.array_equal(z["W%d" % l], a["W"][l][0])
+            assert np.array_equal(z["loss"], np.array(a["loss"]))
 
 
 def test_patch_matrix_of_the_first_convolution_layer():
