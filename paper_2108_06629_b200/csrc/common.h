@@ -61,8 +61,8 @@ cudaError_t gemm_launch(int which, int bn, const CUtensorMap& tmA, const CUtenso
 // call is a forward GEMM with K <= 64 and N <= 64: tmA and tmO are 2-D maps with 64 x 128 boxes.
 cudaError_t conv_halo_launch(int which, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO,
                              const GemmArgs& args, cudaStream_t stream);
-// The same with more than 64 channels on a side (conv_wide.cuh); bn = 64 or 128 output columns, tmB with boxes to match.
-cudaError_t conv_wide_launch(int which, int bn, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& args, cudaStream_t stream);
+// The same with more than 64 channels on a side (conv_wide.cuh); tmB with boxes of 128 output columns.
+cudaError_t conv_wide_launch(int which, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& args, cudaStream_t stream);
 struct ConvGeom;
 struct HaloGUpdate;
 // G (+ fused update) of a halo-tile layer: tmX = the activations with the 64 x 10 x 18 x 1 halo box,

@@ -6,7 +6,7 @@
 // 10 x 18 halo box of a chunk lands in shared memory once and the nine taps are views of it (see conv_halo.cuh), and
 // a CTA works on TWO 8 x 16 pixel tiles at a time, so that each 64 x BN weight tap feeds two accumulators: 16 KiB of
 // weights and 5 KiB of pixels per 512 cycles.  Two accumulators x two buffers x 128 columns are all of tensor memory;
-// with 222 KiB of shared memory no other allocating kernel fits beside a CTA.
+// with 223 KiB of shared memory no other allocating kernel fits beside a CTA.
 //   warp 0     producer: per chunk two halo boxes, then nine weight taps (rings of 2 and 6 stages)
 //   warp 1     MMA issuer: per tap four k-slices into either accumulator
 //   warps 2-9  epilogue, two warps per tensor-memory quarter, under the next item's main loop
@@ -23,22 +23,20 @@ namespace lp {
 constexpr int WIDE_A_STAGES = 2;
 constexpr int WIDE_A_BYTES = 2 * HALO_BYTES;                   // the halo boxes of both pixel tiles, one 64-channel chunk
 constexpr int WIDE_B_STAGES = 6;
-constexpr int wide_b_bytes(int bn) { return bn * GEMM_BK * 2; }
+constexpr int WIDE_BN = 128;                                   // output columns of a tile
+constexpr int WIDE_B_BYTES = WIDE_BN * GEMM_BK * 2;            // one weight tap of a chunk
 constexpr int WIDE_THREADS = 320;
 constexpr int WIDE_B_OFF = WIDE_A_STAGES * WIDE_A_BYTES;       // 92 160 = 90 KiB
 static_assert(WIDE_B_OFF % 1024 == 0, "the weight ring stays 1 KiB aligned");
-constexpr int wide_smem_bytes(int bn) {
-  const int need = WIDE_B_OFF + WIDE_B_STAGES * wide_b_bytes(bn) + 2 * EPI_TILE_BYTES + 256 + 1024;
-  return need < 200 * 1024 ? 200 * 1024 : need;                // (alone on its SM: it holds all of tensor memory)
-}
+constexpr int WIDE_SMEM_BYTES = WIDE_B_OFF + WIDE_B_STAGES * WIDE_B_BYTES + 2 * EPI_TILE_BYTES + 256 + 1024;   // 223 KiB: alone on its SM (it holds all of tensor memory)
 
-template <int BN, bool B_MN, int MODE>
+template <bool B_MN, int MODE>
 __global__ void __launch_bounds__(WIDE_THREADS, 1)
 conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs p,
                  const int tiles_total, const int tiles_n) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr int B_BYTES = wide_b_bytes(BN);
+  constexpr int BN = WIDE_BN, B_BYTES = WIDE_B_BYTES;
   uint8_t* sB = smem + WIDE_B_OFF;
   float* epi_tile = reinterpret_cast<float*>(sB + WIDE_B_STAGES * B_BYTES);
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(epi_tile) + 2 * EPI_TILE_BYTES);

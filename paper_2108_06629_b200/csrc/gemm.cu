@@ -230,10 +230,16 @@ void gemm_box_dims(int which, int bn, uint32_t boxA[2], uint32_t boxB[2]) {
 }
 
 
+// Which contractions exist in a form split over k: forward and delta of a layer (the last CTA of a tile adds), and G of a
+// convolution (a launch of its own adds).
+template <int BN, bool A_MN, int MODE>
+constexpr bool kHasSplit = A_MN ? BN <= 128 : MODE != EPI_STORE_F32;
+
 template <int BN, bool A_MN, bool B_MN, int MODE>
 static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, GemmArgs a, cudaStream_t st,
                               const UpdMaps* um) {
   if (a.splits < 1 || a.partial == nullptr) a.splits = 1;
+  if (a.splits > 1 && !kHasSplit<BN, A_MN, MODE>) return cudaErrorInvalidValue;
   if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
   const int num_kb = (a.K + GEMM_BK - 1) / GEMM_BK;
   a.kb_per_split = (num_kb + a.splits - 1) / a.splits;
@@ -282,19 +288,20 @@ static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, Ge
     }
   }
   note_form(a.splits > 1 ? (a.persistent ? "single split persistent" : "single split") : (a.persistent ? "single persistent" : "single"), BN);
-  if (a.splits > 1) { if (a.persistent) LP_LAUNCH(true, true); else LP_LAUNCH(true, false); }
-  if constexpr (A_MN && BN <= 128) {
-    if (a.splits > 1 && a.split_reduce) {
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-      constexpr int blocks = GEMM_BM * (BN / 4) / 256;      // per tile with one lane
-      const int tiles = tiles_m * tiles_n;
-      if (a.splits >= 16) gemm_split_finish_kernel<BN, MODE, 8><<<tiles * blocks * 8, 256, 0, st>>>(a, tiles_m, tiles_n);
-      else                gemm_split_finish_kernel<BN, MODE, 1><<<tiles * blocks, 256, 0, st>>>(a, tiles_m, tiles_n);
+  if constexpr (kHasSplit<BN, A_MN, MODE>) {
+    if (a.splits > 1) {
+      if (a.persistent) LP_LAUNCH(true, true); else LP_LAUNCH(true, false);
+      if constexpr (A_MN) {
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        constexpr int blocks = GEMM_BM * (BN / 4) / 256;      // per tile with one lane
+        const int tiles = tiles_m * tiles_n;
+        if (a.splits >= 16) gemm_split_finish_kernel<BN, MODE, 8><<<tiles * blocks * 8, 256, 0, st>>>(a, tiles_m, tiles_n);
+        else                gemm_split_finish_kernel<BN, MODE, 1><<<tiles * blocks, 256, 0, st>>>(a, tiles_m, tiles_n);
+      }
       return cudaGetLastError();
     }
   }
-  if (a.splits > 1) return cudaGetLastError();
   if (a.persistent) LP_LAUNCH(false, true); else LP_LAUNCH(false, false);
 #undef LP_LAUNCH
   return cudaGetLastError();
@@ -307,7 +314,8 @@ static cudaError_t configure_one() {
   if ((e = cudaFuncSetAttribute(gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, SPL, PER>,                          \
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)) != cudaSuccess)   \
     return e;
-  LP_ATTR(false, false) LP_ATTR(false, true) LP_ATTR(true, false) LP_ATTR(true, true)
+  LP_ATTR(false, false) LP_ATTR(false, true)
+  if constexpr (kHasSplit<BN, A_MN, MODE>) { LP_ATTR(true, false) LP_ATTR(true, true) }
 #undef LP_ATTR
   if constexpr (MODE == EPI_WGRAD_UPDATE && BN >= 128) {
     if ((e = cudaFuncSetAttribute(gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, false, false, true>,
@@ -489,19 +497,17 @@ cudaError_t conv_halo_launch(int which, const CUtensorMap& tmA, const CUtensorMa
   return cudaErrorInvalidValue;
 }
 
-#define LP_FOR_EACH_WIDE_VARIANT(X)                                                                            \
-  X(64, false, EPI_FPROP) X(64, true, EPI_DGRAD) X(64, true, EPI_DGRAD_UNPOOL)                                 \
-  X(128, false, EPI_FPROP) X(128, true, EPI_DGRAD) X(128, true, EPI_DGRAD_UNPOOL)
-cudaError_t conv_wide_launch(int which, int bn, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& args, cudaStream_t st) {
+#define LP_FOR_EACH_WIDE_VARIANT(X) X(false, EPI_FPROP) X(true, EPI_DGRAD) X(true, EPI_DGRAD_UNPOOL)
+cudaError_t conv_wide_launch(int which, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& args, cudaStream_t st) {
   const bool b_mn = (which != 0);
   GemmArgs a = args;
   if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
-  const int tiles = a.g.tiles_w * a.g.tiles_h * (a.M / (a.g.H * a.g.W)), tiles_n = (a.N - a.n_begin + bn - 1) / bn;
+  const int tiles = a.g.tiles_w * a.g.tiles_h * (a.M / (a.g.H * a.g.W)), tiles_n = (a.N - a.n_begin + WIDE_BN - 1) / WIDE_BN;
   const int grid = std::min((tiles + 1) / 2 * tiles_n, sm_count());
-  note_form("wide halo", bn);
-#define LP_TRYW(BN, B, M)                                                                                      \
-  if (bn == BN && b_mn == B && a.mode == M) {                                                                  \
-    conv_wide_kernel<BN, B, M><<<grid, WIDE_THREADS, wide_smem_bytes(BN), st>>>(tmA, tmB, a, tiles, tiles_n);  \
+  note_form("wide halo", WIDE_BN);
+#define LP_TRYW(B, M)                                                                                          \
+  if (b_mn == B && a.mode == M) {                                                                              \
+    conv_wide_kernel<B, M><<<grid, WIDE_THREADS, WIDE_SMEM_BYTES, st>>>(tmA, tmB, a, tiles, tiles_n);          \
     return cudaGetLastError();                                                                                 \
   }
   LP_FOR_EACH_WIDE_VARIANT(LP_TRYW)
@@ -543,9 +549,9 @@ cudaError_t gemm_configure() {
     return e;
   LP_FOR_EACH_HALO_VARIANT(LP_CFGH)
 #undef LP_CFGH
-#define LP_CFGW(BN, B, M)                                                                                      \
-  if ((e = cudaFuncSetAttribute(conv_wide_kernel<BN, B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
-                                wide_smem_bytes(BN))) != cudaSuccess)                                          \
+#define LP_CFGW(B, M)                                                                                          \
+  if ((e = cudaFuncSetAttribute(conv_wide_kernel<B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
+                                WIDE_SMEM_BYTES)) != cudaSuccess)                                              \
     return e;
   LP_FOR_EACH_WIDE_VARIANT(LP_CFGW)
 #undef LP_CFGW

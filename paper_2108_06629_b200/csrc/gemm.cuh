@@ -109,13 +109,12 @@ struct GemmArgs {
   // split-K (splits > 1): blockIdx.z owns k-blocks [z*kb_per_split, (z+1)*kb_per_split); every CTA
   // writes its fp32 partial tile to `partial`, the last CTA of a tile to arrive (tile_counter)
   // adds the partials in split order -- a fixed order, so results do not depend on timing --
-  // and runs the epilogue.  With split_reduce the sum and the epilogue are a launch of their own
-  // (gemm_split_finish_kernel) on all SMs: for many splits, where the last CTA would add them alone.
+  // and runs the epilogue.  In the G contraction (A_MN), which has many splits, the sum and the epilogue are a
+  // launch of their own on all SMs (gemm_split_finish_kernel).
   int splits, kb_per_split;
   float* partial;           // [tiles][splits][128][BN]
-  unsigned* tile_counter;   // [tiles], zero between launches
-  int split_reduce;
-  int cluster;              // >= 1: one tile per cluster of that many CTAs, which divide the contraction (gemmc.cuh); 0: other forms
+  unsigned* tile_counter;   // [tiles], zero between launches (not in the G contraction)
+  int cluster;              // 2, 4 or 8: one tile per cluster of that many CTAs, which divide the contraction (gemmc.cuh); 0: other forms
   ConvGeom g;
   int persistent;           // CTAs loop over tiles (grid sized to the machine) instead of one tile each
   int l2_ahead;             // plain GEMM: k-blocks of the B operand to pull into L2 ahead of the pipeline (0 = off)
@@ -1060,8 +1059,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           epilogue_rows8<MODE>(p, tm, tile, q, sub_row, sub_col, n);
         }
       }
-      if constexpr (split) {
-        if (p.split_reduce) continue;
+      if constexpr (split && !A_MN) {
         // all four epilogue warps have written their part of the partial tile: publish it, and
         // let the last CTA of this tile reduce the partials in split order
         volatile uint32_t* is_last = tmem_slot + 1;
@@ -1123,7 +1121,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   }
 }
 
-// Second launch of a split contraction with split_reduce: adds the partial tiles and runs the epilogue.  A thread owns four
+// Second launch of a split G contraction: adds the partial tiles and runs the epilogue.  A thread owns four
 // consecutive columns of a tile row; with LANES > 1 (many splits of few tiles) LANES threads share them, lane j
 // adding splits j, j + LANES, ... in order and the lane sums following in order.  Reads splits x tile from L2 once.
 template <int BN, int MODE, int LANES>

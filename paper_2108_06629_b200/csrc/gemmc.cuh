@@ -97,7 +97,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   const int kb_total = (p.K + GEMM_BK - 1) / GEMM_BK;
   const int kb_each = kb_total / C, kb_more = kb_total % C;       // the first kb_more ranks take one more
   const int kb0 = int(rank) * kb_each + min(int(rank), kb_more);
-  const int num_kb = kb_each + (int(rank) < kb_more ? 1 : 0);
+  const int num_kb = kb_each + (int(rank) < kb_more ? 1 : 0);     // (at least one: gemm_pick_cluster)
 
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmA);
@@ -205,13 +205,8 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 #pragma unroll
       for (int c = 0; c < BN / 32; ++c) {
         uint32_t r[32];
-        if (num_kb > 0) {
-          tmem_ld_32x32(tmem_base + (uint32_t(q * 32) << 16) + uint32_t(c * 32), r);
-          tmem_ld_wait();
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) r[j] = 0u;
-        }
+        tmem_ld_32x32(tmem_base + (uint32_t(q * 32) << 16) + uint32_t(c * 32), r);
+        tmem_ld_wait();
 #pragma unroll
         for (int g = 0; g < 8; ++g)
           *reinterpret_cast<uint4*>(row + c * 32 + g * 4) = make_uint4(r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
@@ -228,7 +223,6 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   }
   const uint32_t part = smem_u32(smem);
   switch (C) {
-    case 1: gemmc_reduce_store<BN, MODE, 1>(p, tm, part, rank); break;
     case 2: gemmc_reduce_store<BN, MODE, 2>(p, tm, part, rank); break;
     case 4: gemmc_reduce_store<BN, MODE, 4>(p, tm, part, rank); break;
     default: gemmc_reduce_store<BN, MODE, 8>(p, tm, part, rank); break;

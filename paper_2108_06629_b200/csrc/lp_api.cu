@@ -86,7 +86,6 @@ struct Layer {
   int col_chunks = 0;
   int split_g = 1;
   float* part_g = nullptr;
-  unsigned* cnt_g = nullptr;
   bool pool_fused = false;           // the forward epilogue pools (no a_full)
   Res rAfull;
   Res rPartF, rPartD;               // split-K partial tiles and arrival counters of the forward / delta contraction
@@ -374,7 +373,6 @@ static size_t carve(lp_ctx* c, char* base) {
     } else if (y.split_g > 1) {
       const size_t t = size_t((y.n_out + GEMM_BM - 1) / GEMM_BM) * y.taps * ((y.ld_in + y.bn_g - 1) / y.bn_g);
       y.part_g = reinterpret_cast<float*>(take(t * y.split_g * GEMM_BM * y.bn_g * 4));
-      y.cnt_g = reinterpret_cast<unsigned*>(take(t * 4));
     }
   }
   c->zL = reinterpret_cast<float*>(take(size_t(kDeltaSlots) * B * c->ld_cls * 4));
@@ -887,7 +885,7 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
   if (y.wide_f) {
     a.g = halo_geom(y, 0);
     a.g.chunks_per_tap = (y.ld_in + 63) / 64;
-    return conv_wide_launch(0, y.bn_f, y.tm_hf_A[xin], y.tm_f_B[ring_slot], a, st);
+    return conv_wide_launch(0, y.tm_hf_A[xin], y.tm_f_B[ring_slot], a, st);
   }
   return gemm_launch(0, y.bn_f, y.tm_f_A[xin], y.tm_f_B[ring_slot], a, st);
 }
@@ -959,7 +957,7 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
   if (y.wide_d) {
     a.g = halo_geom(y, 1);
     a.g.chunks_per_tap = (y.ld_out + 63) / 64;
-    return conv_wide_launch(1, y.bn_d, y.tm_hd_A[n % kDeltaSlots], y.tm_d_B[ring_slot], a, st);
+    return conv_wide_launch(1, y.tm_hd_A[n % kDeltaSlots], y.tm_d_B[ring_slot], a, st);
   }
   if (y.conv && y.cstride > 1) {
     // Strided layer: input pixel (h, w) is reached through tap (r, s) only when h + pad - r and
@@ -1011,9 +1009,8 @@ static cudaError_t launch_G(lp_ctx* c, int l, long long n, cudaStream_t st) {
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   if (y.conv && !y.patch) a.g = conv_geom(y, GEOM_PIX_K, y.box64, 0, 0, (y.ld_in + y.bn_g - 1) / y.bn_g);
   if (y.split_g > 1) {
-    a.splits = y.split_g; a.partial = y.part_g; a.tile_counter = y.cnt_g;
-    a.split_reduce = 1;
-    c->launches += a.split_reduce;
+    a.splits = y.split_g; a.partial = y.part_g;
+    ++c->launches;
   }
   if (fused_update(c)) {
     // Eq. 5 and Eq. 6 in one kernel: the accumulator tile is G; the epilogue reads the fp32
