@@ -14,6 +14,10 @@
 
 namespace lp {
 
+// Streaming multiprocessors of a B200.  Sizes and rules that must come out the same with and without a device in the
+// process (workspace, splits, kernel forms of a layer) use this number; grids of launches ask the device.
+constexpr int kSMs = 148;
+
 // ---- lp_api.cu --------------------------------------------------------------
 // Error text of calls that have no handle: what lp_last_error(NULL) returns on this thread.
 void set_global_error(const std::string& msg);
@@ -133,7 +137,7 @@ struct BiasUpdate {
 };
 // About four blocks per SM, but no fewer than 256 rows to a block (its fixed cost is a tail of two block-wide sums).
 inline int colsum_chunk_rows(int rows, int n_cols) {
-  const int want = std::max(1, 592 / ((n_cols + 63) / 64));
+  const int want = std::max(1, 4 * kSMs / ((n_cols + 63) / 64));
   return std::max(256, ((rows + want - 1) / want + 31) / 32 * 32);
 }
 inline int colsum_chunks(int rows, int n_cols) {

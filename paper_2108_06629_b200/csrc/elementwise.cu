@@ -64,7 +64,7 @@ __global__ void cast_stash_kernel(const void* __restrict__ batch, int input_is_b
 cudaError_t launch_cast_stash(const void* batch, int input_is_bf16, const int* labels, __nv_bfloat16* x0,
                               int* labels_copy, int rows, int B, int n_in, int ld, cudaStream_t stream) {
   const long long total = (long long)rows * (ld / 8);
-  int blocks = int(std::min<long long>((total + 255) / 256, 148 * 8));
+  int blocks = int(std::min<long long>((total + 255) / 256, kSMs * 8));
   if (blocks < 1) blocks = 1;
   cast_stash_kernel<<<blocks, 256, 0, stream>>>(batch, input_is_bf16, labels, x0, labels_copy, rows, B, n_in, ld);
   return cudaGetLastError();
@@ -129,7 +129,7 @@ cudaError_t launch_cast_patch3x3(const void* batch, int input_is_bf16, const int
                                  int* labels_copy, int B, int H, int W, int C, int ld, cudaStream_t stream) {
   const long long total = (long long)B * H * W;
   if (C < 1 || C > 7 || ld != (9 * C + 7) / 8 * 8 || total >= (1ll << 31)) return cudaErrorInvalidValue;
-  int blocks = int(std::min<long long>((total + 255) / 256, 148 * 8));
+  int blocks = int(std::min<long long>((total + 255) / 256, kSMs * 8));
   if (blocks < 1) blocks = 1;
 #define LP_PATCH_CASE(c)                                                                                        \
   case c: cast_patch3x3_kernel<c><<<blocks, 256, 0, stream>>>(batch, input_is_bf16, labels, x0, labels_copy, B, H, W); break;
@@ -317,7 +317,7 @@ cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __n
   // 32 registers and a block per 8 rows 25.3).  Blocks beyond what is resident loop over rows: each pays for its fence,
   // count and barriers once (8192 x 1000 in 1024 blocks 24.1 us, in 444 20.3).
 #define LP_XENT(TPR, VEC, N, PER_SM)                                                                                 \
-  softmax_xent_kernel<TPR, VEC, N><<<std::min((B + XENT_THREADS / TPR - 1) / (XENT_THREADS / TPR), 148 * PER_SM),      \
+  softmax_xent_kernel<TPR, VEC, N><<<std::min((B + XENT_THREADS / TPR - 1) / (XENT_THREADS / TPR), kSMs * PER_SM),      \
                                      XENT_THREADS, 0, stream>>>(zL, ldz, labels, delta, ldd, row_loss, ticket,        \
                                                                 loss_out, B, C, status)
   if (C <= 256)       { if (vec2) LP_XENT(32, 2, 8, 6); else LP_XENT(32, 1, 8, 6); }
@@ -430,7 +430,7 @@ __global__ void round_to_bf16_kernel(const float* __restrict__ src, __nv_bfloat1
 }
 cudaError_t launch_round_to_bf16(const float* src, __nv_bfloat16* dst, long long n_elems, cudaStream_t stream) {
   const long long nvec = n_elems >> 3;
-  int blocks = int(std::min<long long>((nvec + 255) / 256, 148 * 16));
+  int blocks = int(std::min<long long>((nvec + 255) / 256, kSMs * 16));
   if (blocks < 1) blocks = 1;
   round_to_bf16_kernel<<<blocks, 256, 0, stream>>>(src, dst, nvec);
   return cudaGetLastError();
@@ -480,7 +480,7 @@ __global__ void maxpool2_kernel(const __nv_bfloat16* __restrict__ a, __nv_bfloat
 cudaError_t launch_maxpool2(const __nv_bfloat16* a, __nv_bfloat16* pooled, unsigned char* idx, int B, int H, int W,
                             int C, cudaStream_t stream) {
   const long long total = (long long)B * (H / 2) * (W / 2) * (C / 8);
-  int blocks = int(std::min<long long>((total + 255) / 256, 148 * 16));
+  int blocks = int(std::min<long long>((total + 255) / 256, kSMs * 16));
   if (blocks < 1) blocks = 1;
   maxpool2_kernel<<<blocks, 256, 0, stream>>>(a, pooled, idx, B, H, W, C);
   return cudaGetLastError();

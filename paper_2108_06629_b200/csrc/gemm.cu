@@ -147,7 +147,7 @@ static int sm_count() {
   if (n == 0) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      n = 148;
+      n = kSMs;
   }
   return n;
 }
@@ -165,7 +165,7 @@ int gemm_pick_splits(int M, int N, int K, int bn) {
   const long long tiles = (long long)((M + GEMM_BM - 1) / GEMM_BM) * ((N + bn - 1) / bn);
   // Fewer tiles with longer contractions take more splits: about one CTA per SM, never fewer than 64 k-blocks per
   // split (a single 10-column tile over 100352 inputs, the classifier behind an unpooled 28 x 28 x 128 image: 24 splits).
-  const int automatic = (tiles <= 48 && num_kb >= 256) ? int(std::max<long long>(1, std::min<long long>(std::min<long long>(148 / tiles, num_kb / 64), 64))) : 1;
+  const int automatic = (tiles <= 48 && num_kb >= 256) ? int(std::max<long long>(1, std::min<long long>(std::min<long long>(kSMs / tiles, num_kb / 64), 64))) : 1;
   int s = g_force_splits > 0 ? g_force_splits : automatic;
   s = std::max(1, std::min(s, num_kb));
   const int per = (num_kb + s - 1) / s;
@@ -216,7 +216,7 @@ int gemm_pick_bn(int which, int M, int N, int K, bool allow_pair) {
   // 1130 TFLOP/s on 2048 x 8192 x 8192; they only pay off when the contraction is long and
   // there are enough tiles to fill two CTAs on every SM
   const long long tiles256 = (long long)((M + GEMM_BM - 1) / GEMM_BM) * ((N + 255) / 256);
-  if (K >= 1024 && tiles256 >= 2 * 148) return 256;
+  if (K >= 1024 && tiles256 >= 2 * kSMs) return 256;
   // (Narrower tiles for small batches were tried: 128 x 64 tiles make a lone forward kernel
   // 35 % faster, but re-read the activations twice as often, and with every stage's kernels
   // sharing L2 and HBM the whole step got 5 % slower.)

@@ -463,8 +463,8 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       // one persistent CTA on every SM): a third less operand traffic per multiply-accumulate than 128 x 128
       const long long row_tiles = y.in_rows / GEMM_BM;
       if (!y.gen) {      // (VGG-16 step 8.40 -> 8.17 ms)
-        if (y.n_out >= 256 && y.taps * y.ld_in >= 1024 && row_tiles * ((y.n_out + 255) / 256) >= 2 * 148) y.bn_f = 256;
-        if (l > 0 && y.ld_in >= 256 && y.taps * y.n_out >= 1024 && row_tiles * ((y.ld_in + 255) / 256) >= 2 * 148) y.bn_d = 256;
+        if (y.n_out >= 256 && y.taps * y.ld_in >= 1024 && row_tiles * ((y.n_out + 255) / 256) >= 2 * kSMs) y.bn_f = 256;
+        if (l > 0 && y.ld_in >= 256 && y.taps * y.n_out >= 1024 && row_tiles * ((y.ld_in + 255) / 256) >= 2 * kSMs) y.bn_d = 256;
       }
       const bool conv_pair = getenv("LP_CONV_PAIR") != nullptr;
       if (conv_pair && !y.gen && even_boxes && y.n_out >= 256 && y.ld_in >= 256) y.bn_f = GEMM_BN_PAIR;
@@ -480,7 +480,7 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       const long long pairs_of_tiles = (long long)B * (y.imW / 8) * (y.imH / 16) / 2;
       // (LP_CONV_WIDE_ITEMS in the environment is another least number of items: what the tests force the form with)
       const char* items = getenv("LP_CONV_WIDE_ITEMS");
-      const long long enough = items != nullptr ? atoll(items) : 4 * 148;
+      const long long enough = items != nullptr ? atoll(items) : 4 * kSMs;
       y.wide_f = !y.patch && tiles_8x16 && y.ld_in > 64 && y.bn_f == 128 && pairs_of_tiles * ((y.n_out + 127) / 128) >= enough;
       y.wide_d = l > 0 && tiles_8x16 && y.ld_out > 64 && y.bn_d == 128 && pairs_of_tiles * ((y.n_in + 127) / 128) >= enough;
       y.lean_f = y.patch && y.n_out <= 64 && y.ld_in <= 64 && l + 1 < n;
@@ -493,7 +493,7 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       const int tiles = ((y.n_out + GEMM_BM - 1) / GEMM_BM) * y.taps * ((y.ld_in + y.bn_g - 1) / y.bn_g);
       const int num_kb = y.out_rows / GEMM_BK;
       const int s_opt = int(std::lround(std::sqrt(double(num_kb) * (y.bn_g <= 64 ? 0.6 : 0.3))));
-      y.split_g = std::max(1, std::min(std::min(296 / std::max(tiles, 1), s_opt), y.patch ? 148 : 64));
+      y.split_g = std::max(1, std::min(std::min(2 * kSMs / std::max(tiles, 1), s_opt), y.patch ? kSMs : 64));
       const int per = (num_kb + y.split_g - 1) / y.split_g;
       y.split_g = (num_kb + per - 1) / per;
     } else {
