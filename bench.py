@@ -12,7 +12,7 @@ import argparse
 import json
 import os
 
-os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")  # one hardware queue per scheduler stream; read when the CUDA context is created
+os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")  # hardware queues for several handles at work at the same time (one needs 8, the default); read when the driver is initialised
 import statistics
 import subprocess
 import sys

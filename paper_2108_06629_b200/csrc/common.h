@@ -59,7 +59,7 @@ void gemm_box_dims(int which, int bn, uint32_t boxA[2], uint32_t boxB[2]);
 cudaError_t gemm_launch(int which, int bn, const CUtensorMap& tmA, const CUtensorMap& tmB,
                         const GemmArgs& args, cudaStream_t stream, const UpdMaps* um = nullptr);
 // 3x3 convolution forward (which = 0) / delta (which = 1) with at most 64 channels on both sides:
-// tmA = NHWC tensor map with a 64 x 16 x 18 x 1 box, tmB = the layer's weight map (64 x 64 boxes);
+// tmA = NHWC tensor map with a 64 x 10 x 18 x 1 box, tmB = the layer's weight map (64 x 64 boxes);
 // args.g describes 8 x 16 pixel tiles (lw = 3, lh = 4).  tmO (forward only; any valid map otherwise): the
 // NHWC output with a 64 x 8 x 16 x 1 box, written by TMA stores.  With plain geometry (which = 0 only) the
 // call is a forward GEMM with K <= 64 and N <= 64: tmA and tmO are 2-D maps with 64 x 128 boxes.

@@ -213,7 +213,6 @@ cudaError_t launch_cast_patch_general(const void* batch, int input_is_bf16, cons
 // and 2 out.  Before (a block per row, three passes, two exponentials) and now:
 // 8192 x 1000 56 -> 20 us, 2048 x 8192 77 -> 36 us.  VEC = 2: two consecutive classes per thread where pitches and addresses allow 8- and 4-byte accesses.
 constexpr int XENT_THREADS = 256;
-// N = classes that a thread keeps in registers; wider rows go in several sweeps over memory
 
 template <int TPR>
 __device__ __forceinline__ float row_reduce(float v, float* sh, bool is_max) {
@@ -232,6 +231,7 @@ __device__ __forceinline__ float row_reduce(float v, float* sh, bool is_max) {
   return r;
 }
 
+// N = classes that a thread keeps in registers; what lies beyond TPR * N goes in several sweeps over memory
 template <int TPR, int VEC, int N>
 __global__ void __launch_bounds__(XENT_THREADS)
 softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict__ labels, __nv_bfloat16* __restrict__ delta, int ldd,

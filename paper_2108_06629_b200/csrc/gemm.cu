@@ -190,7 +190,8 @@ int gemm_pick_cluster(int M, int N, int K, int* bn) {
     return num_kb >= c && (tiles * c <= sm_count() || (tiles * c <= 2 * sm_count() && num_kb >= 16 * c));
   };
   const int c = (num_kb >= 64 && tiles * 8 <= sm_count()) ? 8 : fits(4) ? 4 : fits(2) ? 2 : 0;
-  // (one tile over a hundred thousand terms: the split through global memory spreads it wider than a cluster can)
+  // (one tile over a hundred thousand terms: the split through global memory, which a layer has and lp_gemm_bf16 has not,
+  // spreads it wider than a cluster can)
   if (c == 0 || gemm_pick_splits(M, N, K, width) > 2 * c) return 0;
   *bn = width;
   return c;

@@ -390,9 +390,11 @@ static void pick_fc_tiles(Layer* y, int B, bool allow_pair) {
   y->bn_f = gemm_pick_bn(0, B, y->n_out, y->n_in, allow_pair);
   y->bn_d = gemm_pick_bn(1, B, y->n_in, y->n_out, allow_pair);
   y->bn_g = gemm_pick_bn(2, y->n_out, y->n_in, B, allow_pair);
-  // Contractions divided over clusters pay where the step is a chain of short kernels (16 steps of a 1003-777-515-131
-  // network 1050 -> 830 us).  A layer of more than four million weights keeps the GPU busy with its update, under which a
-  // cluster waits for room on several SMs at once: 8 steps of the 8 x 4096 network take 4780 us without, 5240 with them.
+  // Contractions divided over clusters pay where the step is a chain of short kernels.  A wide layer keeps the GPU busy with
+  // its update, under which a cluster waits for room on several SMs at once.  Eight equal layers with momentum, delays
+  // 7 .. 0, microseconds a step in a run of 60, undivided / over clusters: batch 256, 1024 wide 143 / 102, 2048 227 / 197, 2560
+  // 289 / 280, 3072 357 / 378, 4096 565 / 623; batch 64, 2048 218 / 156, 3072 341 / 291, 4096 520 / 529.  So the line, at
+  // 2048 x 2048, is on the safe side of where clusters begin to cost, which lies between 2560 and 4096 with the batch.
   const bool chain_bound = (long long)y->n_in * y->n_out <= (1ll << 22);
   y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f) : 0;
   y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d) : 0;
