@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/layerpipe.h"
@@ -17,6 +18,38 @@ namespace lp {
 // Streaming multiprocessors of a B200.  Sizes and rules that must come out the same with and without a device in the
 // process (workspace, splits, kernel forms of a layer) use this number; grids of launches ask the device.
 constexpr int kSMs = 148;
+
+// ---- launches -----------------------------------------------------------------
+// Kernels of a stream follow one another at once: the launch carries the programmatic-serialisation attribute, so the
+// next kernel's blocks start (barriers, tensor memory, descriptors) while the tail of the one before still runs, and
+// launch_wait() in front of its first access to global memory holds it until that one has completed and its writes are
+// visible.  Every thread block executes the wait, so completion stays transitive along a stream whatever the launches in between did.
+// Where an event wait stands between two launches the attribute has no effect.  Measured on a chain of one-block kernels: 1.9 us
+// from the end of a kernel to the start of the next one, 0.54 us with the attribute; the launch call itself 2.9 -> 2.4 us.
+template <class... KArgs, class... Args>
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+// Holds until the kernel before this one in the stream has completed (returns at once in a launch without the attribute).
+__device__ __forceinline__ void launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next kernel of the stream may start its blocks once every block of this one has said so or has ended.  Said by the
+// kernels of short chains only (cluster contractions, loss, column sums), once a block has asked for its last operands.  Blocks that
+// wait take room from other streams: with the tile kernels saying it too, 16 steps of the small VGG took 4370 us
+// (4160 without, 4260 with plain launches) and nothing was faster for it.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- lp_api.cu --------------------------------------------------------------
 // Error text of calls that have no handle: what lp_last_error(NULL) returns on this thread.

@@ -82,6 +82,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  launch_wait();
   // CTA b works through the contiguous tile range [t_begin, t_end): neighbouring tiles share halo
   // pixels in L2, and the tile coordinates advance without divisions.
   const bool plain = (p.g.kind == GEOM_PLAIN);          // one tap, 128 consecutive rows per tile
@@ -400,6 +401,7 @@ conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  launch_wait();
   const int per_cta = (tiles_total + int(gridDim.x) - 1) / int(gridDim.x);
   const int t_begin = min(int(blockIdx.x) * per_cta, tiles_total);
   const int t_end = min(t_begin + per_cta, tiles_total);
@@ -523,6 +525,7 @@ __global__ void __launch_bounds__(256) conv_halo_g_update_kernel(const HaloGUpda
   const int e = blockIdx.x * 32 + lane;              // (the partial tile is a whole number of blocks)
   const float* src = a.partial + e;
   float g = 0.f;
+  launch_wait();
 #pragma unroll 8
   for (int c = wrp; c < a.n_ctas; c += 8) g += __ldcg(src + size_t(c) * HALOG_PART_FLOATS);
   sums[wrp][lane] = g;

@@ -67,6 +67,7 @@ conv_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  launch_wait();
   const int items = ((tiles_total + 1) / 2) * tiles_n;
   const int chunks = p.g.chunks_per_tap;
   const int per_image = p.g.tiles_w * p.g.tiles_h;

@@ -23,6 +23,7 @@ cudaError_t launch_trace_mark(unsigned* flag, unsigned value, cudaStream_t strea
 __global__ void cast_stash_kernel(const void* __restrict__ batch, int input_is_bf16,
                                   const int* __restrict__ labels, __nv_bfloat16* __restrict__ x0,
                                   int* __restrict__ labels_copy, int rows, int B, int n_in, int ld) {
+  launch_wait();
   const long long groups_per_row = ld / 8;
   const long long total = (long long)rows * groups_per_row;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
@@ -66,8 +67,7 @@ cudaError_t launch_cast_stash(const void* batch, int input_is_bf16, const int* l
   const long long total = (long long)rows * (ld / 8);
   int blocks = int(std::min<long long>((total + 255) / 256, kSMs * 8));
   if (blocks < 1) blocks = 1;
-  cast_stash_kernel<<<blocks, 256, 0, stream>>>(batch, input_is_bf16, labels, x0, labels_copy, rows, B, n_in, ld);
-  return cudaGetLastError();
+  return launch_chained(cast_stash_kernel, blocks, 256, 0, stream, 1, batch, input_is_bf16, labels, x0, labels_copy, rows, B, n_in, ld);
 }
 
 // ---------------------------------------------------------------------------
@@ -83,6 +83,7 @@ __global__ void cast_patch3x3_kernel(const void* __restrict__ batch, int input_i
                                      const int* __restrict__ labels, __nv_bfloat16* __restrict__ x0,
                                      int* __restrict__ labels_copy, int B, int H, int W) {
   constexpr int LD = (9 * C + 7) / 8 * 8;
+  launch_wait();
   const int total = B * H * W;
   for (int pix = blockIdx.x * blockDim.x + threadIdx.x; pix < total; pix += gridDim.x * blockDim.x) {
     const int w = pix % W;
@@ -132,12 +133,12 @@ cudaError_t launch_cast_patch3x3(const void* batch, int input_is_bf16, const int
   int blocks = int(std::min<long long>((total + 255) / 256, kSMs * 8));
   if (blocks < 1) blocks = 1;
 #define LP_PATCH_CASE(c)                                                                                        \
-  case c: cast_patch3x3_kernel<c><<<blocks, 256, 0, stream>>>(batch, input_is_bf16, labels, x0, labels_copy, B, H, W); break;
+  case c: return launch_chained(cast_patch3x3_kernel<c>, blocks, 256, 0, stream, 1, batch, input_is_bf16, labels, x0, labels_copy, B, H, W);
   switch (C) {
     LP_PATCH_CASE(1) LP_PATCH_CASE(2) LP_PATCH_CASE(3) LP_PATCH_CASE(4) LP_PATCH_CASE(5) LP_PATCH_CASE(6) LP_PATCH_CASE(7)
   }
 #undef LP_PATCH_CASE
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 // General filters / strides.  A block writes the patch rows of PATCH_PIX output pixels of one image row: it stages the R
@@ -162,6 +163,7 @@ cast_patch_general_kernel(const void* __restrict__ batch, int input_is_bf16, con
     col_off[c] = c < R * S * C ? short((tap / S) * span * C + (tap % S) * C + c % C) : short(-1);
   }
   const int w0 = wo0 * stride - pad, row_vals = span * C;
+  launch_wait();
   for (int i = threadIdx.x; i < R * row_vals; i += blockDim.x) {
     const int r = i / row_vals, q = i - r * row_vals;
     const int hh = ho * stride - pad + r, x = w0 * C + q;      // x: position in the image row, in values
@@ -201,9 +203,8 @@ cudaError_t launch_cast_patch_general(const void* batch, int input_is_bf16, cons
   const size_t smem = size_t(R) * span * C * 2;
   // (filters up to 7x7, stride up to 2, at most 8 channels: 15 KiB)
   if (C < 1 || R * S * C > ld || (ld & 7) || ld > PATCH_COLS_MAX || smem > 48 * 1024 || blocks >= (1ll << 31)) return cudaErrorInvalidValue;
-  cast_patch_general_kernel<<<int(blocks), 256, smem, stream>>>(batch, input_is_bf16, labels, x0, labels_copy, B, H, W, C, R, S, stride,
-                                                                pad, Ho, Wo, ld, span, segs);
-  return cudaGetLastError();
+  return launch_chained(cast_patch_general_kernel, int(blocks), 256, smem, stream, 1, batch, input_is_bf16, labels, x0, labels_copy, B, H, W, C,
+                        R, S, stride, pad, Ho, Wo, ld, span, segs);
 }
 
 // ---------------------------------------------------------------------------
@@ -242,6 +243,7 @@ softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict
   const int t = int(threadIdx.x) % TPR;
   const float invB = 1.0f / float(B);
   const int Cpad = (C + 7) & ~7;
+  launch_wait();
   // (uniform over the row's threads)
   for (int row = blockIdx.x * ROWS + int(threadIdx.x) / TPR; row < B; row += int(gridDim.x) * ROWS) {
     const float* z = zL + (long long)row * ldz;
@@ -293,6 +295,7 @@ softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict
       if (!y_ok && status != nullptr) atomicCAS(status, 0, LP_STATUS_BAD_LABEL);
     }
   }
+  launch_next();
   __threadfence();                                    // this block's row losses before its count
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -317,14 +320,12 @@ cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __n
   // 32 registers and a block per 8 rows 25.3).  Blocks beyond what is resident loop over rows: each pays for its fence,
   // count and barriers once (8192 x 1000 in 1024 blocks 24.1 us, in 444 20.3).
 #define LP_XENT(TPR, VEC, N, PER_SM)                                                                                 \
-  softmax_xent_kernel<TPR, VEC, N><<<std::min((B + XENT_THREADS / TPR - 1) / (XENT_THREADS / TPR), kSMs * PER_SM),      \
-                                     XENT_THREADS, 0, stream>>>(zL, ldz, labels, delta, ldd, row_loss, ticket,        \
-                                                                loss_out, B, C, status)
+  return launch_chained(softmax_xent_kernel<TPR, VEC, N>, std::min((B + XENT_THREADS / TPR - 1) / (XENT_THREADS / TPR), kSMs * PER_SM), \
+                        XENT_THREADS, 0, stream, 1, zL, ldz, labels, delta, ldd, row_loss, ticket, loss_out, B, C, status)
   if (C <= 256)       { if (vec2) LP_XENT(32, 2, 8, 6); else LP_XENT(32, 1, 8, 6); }
   else if (C <= 1024) { if (vec2) LP_XENT(32, 2, 32, 3); else LP_XENT(32, 1, 32, 3); }
   else                { if (vec2) LP_XENT(256, 2, 32, 256); else LP_XENT(256, 1, 32, 256); }     // (a block per row: 2048 x 8192 36 us, looping 44)
 #undef LP_XENT
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -337,6 +338,7 @@ constexpr int UPD_VEC_PER_THREAD = 2;     // x 8 elements
 constexpr int BIAS_COLS = 64;
 
 __global__ void __launch_bounds__(UPD_THREADS) sgd_update_kernel(const UpdateArgs a, int w_blocks) {
+  launch_wait();
   if (int(blockIdx.x) < w_blocks) {
     const long long nvec = a.n_elems >> 3;
     const long long base = (long long)blockIdx.x * (UPD_THREADS * UPD_VEC_PER_THREAD) + threadIdx.x;
@@ -408,8 +410,7 @@ cudaError_t launch_sgd_update(const UpdateArgs& a, cudaStream_t stream) {
   const long long per_block = UPD_THREADS * UPD_VEC_PER_THREAD;
   const int w_blocks = int((nvec + per_block - 1) / per_block);
   const int b_blocks = a.delta ? (a.n_out + BIAS_COLS - 1) / BIAS_COLS : 0;
-  sgd_update_kernel<<<w_blocks + b_blocks, UPD_THREADS, 0, stream>>>(a, w_blocks);
-  return cudaGetLastError();
+  return launch_chained(sgd_update_kernel, w_blocks + b_blocks, UPD_THREADS, 0, stream, 1, a, w_blocks);
 }
 
 }  // namespace lp
@@ -444,6 +445,7 @@ __global__ void maxpool2_kernel(const __nv_bfloat16* __restrict__ a, __nv_bfloat
                                 unsigned char* __restrict__ idx, int B, int H, int W, int C) {
   const int Hp = H / 2, Wp = W / 2, cg = C / 8;
   const long long total = (long long)B * Hp * Wp * cg;
+  launch_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
     const int c8 = int(t % cg);
     long long pp = t / cg;
@@ -482,8 +484,7 @@ cudaError_t launch_maxpool2(const __nv_bfloat16* a, __nv_bfloat16* pooled, unsig
   const long long total = (long long)B * (H / 2) * (W / 2) * (C / 8);
   int blocks = int(std::min<long long>((total + 255) / 256, kSMs * 16));
   if (blocks < 1) blocks = 1;
-  maxpool2_kernel<<<blocks, 256, 0, stream>>>(a, pooled, idx, B, H, W, C);
-  return cudaGetLastError();
+  return launch_chained(maxpool2_kernel, blocks, 256, 0, stream, 1, a, pooled, idx, B, H, W, C);
 }
 
 // Bias gradient of a layer with many rows (convolutions, large minibatches): column sums of delta, then Eq. 6 for the
@@ -504,6 +505,7 @@ __global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* _
   const int c8 = col0 + g * 8;
   const int r0 = blockIdx.y * chunk_rows, r1 = min(rows, r0 + chunk_rows);
   float acc[8] = {};
+  launch_wait();
   if (c8 < ld) {
     const __nv_bfloat16* src = x + c8;
     int r = r0 + lane;
@@ -527,6 +529,7 @@ __global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* _
 #pragma unroll
   for (int j = 0; j < 8; ++j) part[lane][g * 8 + j] = acc[j];
   __syncthreads();
+  launch_next();
   const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;          // four threads a column, eight row lanes each
   float s = 0.f;
 #pragma unroll
@@ -576,8 +579,7 @@ cudaError_t launch_colsum_bias(const __nv_bfloat16* x, int rows, int ld, int n_c
                                const BiasUpdate& u, cudaStream_t stream) {
   const int chunk = colsum_chunk_rows(rows, n_cols);
   dim3 grid((n_cols + 63) / 64, (rows + chunk - 1) / chunk);
-  colsum_bias_kernel<<<grid, 256, 0, stream>>>(x, rows, ld, n_cols, chunk, partial, counter, u);
-  return cudaGetLastError();
+  return launch_chained(colsum_bias_kernel, grid, 256, 0, stream, 1, x, rows, ld, n_cols, chunk, partial, counter, u);
 }
 }  // namespace lp
 

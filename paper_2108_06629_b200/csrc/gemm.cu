@@ -277,35 +277,30 @@ static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, Ge
   // single-wave launches stream their weights once: request them into L2 well ahead of the pipeline
   a.l2_ahead = (a.g.kind == GEOM_PLAIN && work <= slots && a.kb_per_split >= 8) ? g_l2_ahead : 0;
 #define LP_LAUNCH(SPL, PER) \
-  gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, SPL, PER><<<grid, GEMM_THREADS, smem, st>>>(tmA, tmB, *um, a, tiles_m, tiles_n, int(work))
+  launch_chained(gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, SPL, PER>, grid, GEMM_THREADS, smem, st, 1, tmA, tmB, *um, a, tiles_m, tiles_n, int(work))
   if constexpr (MODE == EPI_WGRAD_UPDATE && BN >= 128) {
     if (a.upd_tma) {
       note_form(a.persistent ? "single streamed persistent" : "single streamed", BN);
-      if (a.persistent)
-        gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, false, true, true><<<grid, GEMM_THREADS, smem, st>>>(tmA, tmB, *um, a, tiles_m, tiles_n, int(work));
-      else
-        gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, false, false, true><<<grid, GEMM_THREADS, smem, st>>>(tmA, tmB, *um, a, tiles_m, tiles_n, int(work));
-      return cudaGetLastError();
+      return launch_chained(a.persistent ? gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, false, true, true> : gemm_tcgen05_kernel<BN, A_MN, B_MN, MODE, false, false, true>,
+                            grid, GEMM_THREADS, smem, st, 1, tmA, tmB, *um, a, tiles_m, tiles_n, int(work));
     }
   }
   note_form(a.splits > 1 ? (a.persistent ? "single split persistent" : "single split") : (a.persistent ? "single persistent" : "single"), BN);
   if constexpr (kHasSplit<BN, A_MN, MODE>) {
     if (a.splits > 1) {
-      if (a.persistent) LP_LAUNCH(true, true); else LP_LAUNCH(true, false);
+      const cudaError_t e = a.persistent ? LP_LAUNCH(true, true) : LP_LAUNCH(true, false);
       if constexpr (A_MN) {
-        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         constexpr int blocks = GEMM_BM * (BN / 4) / 256;      // per tile with one lane
         const int tiles = tiles_m * tiles_n;
-        if (a.splits >= 16) gemm_split_finish_kernel<BN, MODE, 8><<<tiles * blocks * 8, 256, 0, st>>>(a, tiles_m, tiles_n);
-        else                gemm_split_finish_kernel<BN, MODE, 1><<<tiles * blocks, 256, 0, st>>>(a, tiles_m, tiles_n);
+        if (a.splits >= 16) return launch_chained(gemm_split_finish_kernel<BN, MODE, 8>, tiles * blocks * 8, 256, 0, st, 1, a, tiles_m, tiles_n);
+        return launch_chained(gemm_split_finish_kernel<BN, MODE, 1>, tiles * blocks, 256, 0, st, 1, a, tiles_m, tiles_n);
       }
-      return cudaGetLastError();
+      return e;
     }
   }
-  if (a.persistent) LP_LAUNCH(false, true); else LP_LAUNCH(false, false);
+  return a.persistent ? LP_LAUNCH(false, true) : LP_LAUNCH(false, false);
 #undef LP_LAUNCH
-  return cudaGetLastError();
 }
 
 template <int BN, bool A_MN, bool B_MN, int MODE>
@@ -344,20 +339,9 @@ template <int BN, bool A_MN, bool B_MN, int MODE>
 static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB, GemmArgs a, cudaStream_t st) {
   if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
   const int tiles_m = (a.M + GEMM_BM - 1) / GEMM_BM, tiles_n = (a.N - a.n_begin + BN - 1) / BN;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.cluster, tiles_m * tiles_n, 1);
-  cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = gemmc_smem_bytes(BN);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = a.cluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   note_form("cluster", BN, a.cluster);
-  return cudaLaunchKernelEx(&cfg, gemmc_kernel<BN, A_MN, B_MN, MODE>, tmA, tmB, a, tiles_m);
+  return launch_chained(gemmc_kernel<BN, A_MN, B_MN, MODE>, dim3(a.cluster, tiles_m * tiles_n), GEMM_THREADS, gemmc_smem_bytes(BN), st, a.cluster,
+                        tmA, tmB, a, tiles_m);
 }
 #define LP_FOR_EACH_CLUSTER_VARIANT(X, BN) \
   X(BN, false, false, EPI_FPROP)           \
@@ -489,10 +473,8 @@ cudaError_t conv_halo_launch(int which, const CUtensorMap& tmA, const CUtensorMa
   const int grid = std::min(tiles, sm_count());
   note_form(args.g.kind == GEOM_PLAIN ? "halo plain" : "halo", 64);
 #define LP_TRYH(B, M)                                                                                          \
-  if (b_mn == B && args.mode == M) {                                                                           \
-    conv_halo_kernel<B, M><<<grid, HALO_THREADS, HALO_SMEM_BYTES, st>>>(tmA, tmB, tmO, args, tiles);                \
-    return cudaGetLastError();                                                                                 \
-  }
+  if (b_mn == B && args.mode == M)                                                                             \
+    return launch_chained(conv_halo_kernel<B, M>, grid, HALO_THREADS, HALO_SMEM_BYTES, st, 1, tmA, tmB, tmO, args, tiles);
   LP_FOR_EACH_HALO_VARIANT(LP_TRYH)
 #undef LP_TRYH
   return cudaErrorInvalidValue;
@@ -507,10 +489,8 @@ cudaError_t conv_wide_launch(int which, const CUtensorMap& tmA, const CUtensorMa
   const int grid = std::min((tiles + 1) / 2 * tiles_n, sm_count());
   note_form("wide halo", WIDE_BN);
 #define LP_TRYW(B, M)                                                                                          \
-  if (b_mn == B && a.mode == M) {                                                                              \
-    conv_wide_kernel<B, M><<<grid, WIDE_THREADS, WIDE_SMEM_BYTES, st>>>(tmA, tmB, a, tiles, tiles_n);          \
-    return cudaGetLastError();                                                                                 \
-  }
+  if (b_mn == B && a.mode == M)                                                                                \
+    return launch_chained(conv_wide_kernel<B, M>, grid, WIDE_THREADS, WIDE_SMEM_BYTES, st, 1, tmA, tmB, a, tiles, tiles_n);
   LP_FOR_EACH_WIDE_VARIANT(LP_TRYW)
 #undef LP_TRYW
   return cudaErrorInvalidValue;
@@ -526,12 +506,10 @@ cudaError_t conv_halo_g_launch(const CUtensorMap& tmX, const CUtensorMap& tmD, c
   upd.n_ctas = grid;
   for (int co0 = 0; co0 < upd.n_out; co0 += 64) {      // one pass per 64 output channels; the stream orders the reuse of `partial`
     note_form("halo G", 64);
-    conv_halo_g_kernel<0><<<grid, GEMM_THREADS, HALOG_SMEM_BYTES, st>>>(tmX, tmD, g, tiles, co0, partial, status);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained(conv_halo_g_kernel<0>, grid, GEMM_THREADS, HALOG_SMEM_BYTES, st, 1, tmX, tmD, g, tiles, co0, partial, status);
     if (e != cudaSuccess) return e;
     upd.co0 = co0;
-    conv_halo_g_update_kernel<0><<<HALOG_PART_FLOATS / 32, 256, 0, st>>>(upd);
-    e = cudaGetLastError();
+    e = launch_chained(conv_halo_g_update_kernel<0>, HALOG_PART_FLOATS / 32, 256, 0, st, 1, upd);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -22,6 +22,7 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include "common.h"
 #include "ptx.cuh"
 
 namespace lp {
@@ -611,6 +612,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  launch_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -1136,6 +1138,7 @@ __global__ void __launch_bounds__(256) gemm_split_finish_kernel(const GemmArgs p
   const int r = g / (BN / 4), c = (g % (BN / 4)) * 4;
   if (tc.tm.m0 + (int(blockIdx.x) % BLOCKS) * GROUPS / (BN / 4) >= p.M) return;     // the block's first row
   const float* src = p.partial + (size_t(tile) * p.splits * GEMM_BM + r) * BN + c;
+  launch_wait();
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
   for (int z = j; z < p.splits; z += LANES) {

@@ -119,6 +119,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  launch_wait();
   const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
 
   if (warp == 0) {
@@ -148,6 +149,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         ++issued;
         if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
       }
+      launch_next();
       if (!ok) {
         report_expired(p.status, WAIT_CLUSTER_PRODUCER, int(blockIdx.y), kb);
         for (int i = (issued > S ? issued - S : 0); i < issued; ++i) mbar_wait(&full_bar[i % S], uint32_t(i / S) & 1u, p.wait_limit);

@@ -169,3 +169,56 @@ def test_contraction_on_sm_pairs(which, M, N, K, form):
     assert rel_l2(got[:, :N], _reference(which, M, N, K, A, B)) < 1e-6 + 2e-7 * np.sqrt(K)
     assert np.all(got[:, N:] == 0.0)
     assert lpb.lp_gemm_status() == (lpb.LP_OK, 0)
+
+
+@pytest.mark.parametrize("B, n, classes", [(33, 200, 10), (128, 1000, 513), (300, 64, 1000)])
+def test_kernels_of_a_stream_see_what_the_one_before_wrote(B, n, classes):
+    """Launches of one stream start before the kernel in front of them has ended and wait inside.  A chain in which every
+    call reads what the call before it wrote (loss -> contraction -> loss ...), enqueued at once, against the same with the
+    device idle between the calls, and captured into a graph that is replayed: bit for bit."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    g = torch.Generator().manual_seed(B)
+    ld, ldc = (n + 7) // 8 * 8, (classes + 7) // 8 * 8
+    w = torch.zeros(classes, ld, dtype=torch.bfloat16)
+    w[:, :n] = torch.randn(classes, n, generator=g) * n ** -0.5
+    w = w.cuda()
+    y = torch.randint(0, classes, (B,), generator=g, dtype=torch.int32).cuda()
+    z0 = torch.randn(B, ldc, generator=g).cuda()
+
+    def chain(wait):
+        z, e = z0.clone(), torch.zeros(B, ld, device="cuda")
+        d, loss, dw = torch.zeros(B, ldc, dtype=torch.bfloat16, device="cuda"), torch.zeros(1, device="cuda"), torch.zeros(classes, ld, device="cuda")
+        a = torch.zeros(B, ld, dtype=torch.bfloat16, device="cuda")
+
+        def once():
+            for _ in range(6):
+                assert lpb.lp_softmax_xent_static(z, y, d, loss, classes) == lpb.LP_OK
+                wait()
+                lpb.lp_gemm_bf16(1, B, n, classes, d, ldc, w, ld, e, ld)
+                wait()
+                a.copy_(e * B)
+                wait()
+                lpb.lp_gemm_bf16(2, classes, n, B, d, ldc, a, ld, dw, ld)
+                wait()
+                lpb.lp_gemm_bf16(0, B, classes, n, a, ld, w, ld, z, ldc)
+                wait()
+        return once, (z, e, d, loss, dw)
+
+    once, want = chain(torch.cuda.synchronize)
+    once()
+    for _ in range(3):
+        once, got = chain(lambda: None)
+        once()
+        torch.cuda.synchronize()
+        assert all(torch.equal(p, q) for p, q in zip(want, got))
+    side = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    once, got = chain(lambda: None)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        once()
+    got[0].copy_(z0)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(p, q) for p, q in zip(want, got))
