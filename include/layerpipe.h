@@ -348,13 +348,13 @@ int lp_debug_gemm_starved(int M, int N, int K, const void* A_dev, int lda, const
  * fp32 [1].  All caller-owned.  `stream` is a cudaStream_t (may be 0); the call is
  * asynchronous.
  *
- * The scratch (one fp32 per row plus a counter) is a fixed array inside the library image:
+ * The scratch (one fp32 per row) is a fixed array inside the library image:
  * LP_XENT_STATIC_MAX_BATCH rows, about 64 KiB, resident on every GPU that loads the
  * library for as long as the process lives.  Consequences the caller must know:
  *   - batch > LP_XENT_STATIC_MAX_BATCH (or batch < 1, classes < 1, bad pitches, null
  *     pointers) -> LP_ERR_INVALID_ARG, nothing is launched; lp_last_error(NULL) says which.
- *   - all calls on one GPU share that array.  The call clears the part that must start
- *     at zero, so leftovers of an earlier call are harmless, but two calls that overlap
+ *   - all calls on one GPU share that array.  A call writes every element that it
+ *     reads, so leftovers of an earlier call are harmless, but two calls that overlap
  *     on the device (different streams, no ordering between them) race on it and give
  *     wrong losses.  Order them.
  *   - the first call on each device looks up the array's device address (a host-side

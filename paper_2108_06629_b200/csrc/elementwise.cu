@@ -208,21 +208,26 @@ cudaError_t launch_cast_patch_general(const void* batch, int input_is_bf16, cons
 }
 
 // ---------------------------------------------------------------------------
-// p = softmax(z^L), delta^L = RN((p - onehot)/B), row loss; the last block to finish adds the row losses in a fixed
-// order (deterministic mean).  A row belongs to TPR threads (a warp, or the block for wide rows), which keep its logits and
-// exponentials in registers: the logits are read once, one exponential per element, 4 bytes per class in
-// and 2 out.  Before (a block per row, three passes, two exponentials) and now:
-// 8192 x 1000 56 -> 20 us, 2048 x 8192 77 -> 36 us.  VEC = 2: two consecutive classes per thread where pitches and addresses allow 8- and 4-byte accesses.
+// p = softmax(z^L), delta^L = RN((p - onehot)/B), row loss.  A row belongs to TPR threads (eight, a warp, or the block for
+// wide rows), which keep its logits and exponentials in registers: the logits are read once, one exponential per element, 4
+// bytes per class in and 2 out.  What bounds it beside memory is the instructions of an element, so there is no test per
+// element: lanes past C hold -inf, and the label's owner overwrites its element.  Time of the static call, its
+// inputs in L2 or not as 40 calls in a row leave them, before (a comparison per element, 8-byte loads, three or four rows to a
+// warp of 72 registers, the counter cleared by a launch in front) and now: 8192 x 1000 22.6 -> 13.3 us, 16384 x 1000 35.2 -> 21.5,
+// 16384 x 4000 266 -> 104, 1000 x 1500 20.5 -> 6.0.  (A look-ahead of one row in registers, 128 a thread: 18.4 for the first.)
+// VEC: consecutive classes of a thread, 4 or 2 where pitches and addresses allow accesses of that width.
+// The mean of the row losses, in a fixed order: by the last block to finish where the caller has a counter for that (a
+// trainer), by the block itself where it is the only one, else by a launch of its own (softmax_xent_mean_kernel).
 constexpr int XENT_THREADS = 256;
 
 template <int TPR>
 __device__ __forceinline__ float row_reduce(float v, float* sh, bool is_max) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = TPR < 32 ? TPR / 2 : 16; o > 0; o >>= 1) {
     const float other = __shfl_xor_sync(0xffffffffu, v, o);
     v = is_max ? fmaxf(v, other) : v + other;
   }
-  if (TPR == 32) return v;
+  if (TPR <= 32) return v;
   __syncthreads();
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
@@ -232,9 +237,25 @@ __device__ __forceinline__ float row_reduce(float v, float* sh, bool is_max) {
   return r;
 }
 
+// Mean of B row losses by the block: thread t adds rows t, t + THREADS, ... in that order, then a tree over the threads.
+template <int THREADS>
+__device__ __forceinline__ void row_loss_mean(const float* row_loss, float* loss_out, int B, float* sh) {
+  float acc = 0.f;
+#pragma unroll 8
+  for (int i = threadIdx.x; i < B; i += THREADS) acc += __ldcg(row_loss + i);
+  acc = row_reduce<THREADS>(acc, sh, false);
+  if (threadIdx.x == 0) *loss_out = acc * (1.0f / float(B));
+}
+constexpr int XENT_MEAN_THREADS = 1024;
+__global__ void __launch_bounds__(XENT_MEAN_THREADS) softmax_xent_mean_kernel(const float* row_loss, float* loss_out, int B) {
+  __shared__ float sh[XENT_MEAN_THREADS / 32];
+  launch_wait();
+  row_loss_mean<XENT_MEAN_THREADS>(row_loss, loss_out, B, sh);
+}
+
 // N = classes that a thread keeps in registers; what lies beyond TPR * N goes in several sweeps over memory
 template <int TPR, int VEC, int N>
-__global__ void __launch_bounds__(XENT_THREADS)
+__global__ void __launch_bounds__(XENT_THREADS, 4)
 softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict__ labels, __nv_bfloat16* __restrict__ delta, int ldd,
                     float* __restrict__ row_loss, unsigned* __restrict__ ticket, float* __restrict__ loss_out, int B, int C, int* __restrict__ status) {
   constexpr int ROWS = XENT_THREADS / TPR;            // rows of a block
@@ -243,20 +264,24 @@ softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict
   const int t = int(threadIdx.x) % TPR;
   const float invB = 1.0f / float(B);
   const int Cpad = (C + 7) & ~7;
+  const bool wide = C > TPR * N;
+  // position k of thread t is class (k / VEC) * TPR * VEC + t * VEC + k % VEC
+  auto cls = [&](int k) { return (k / VEC) * (TPR * VEC) + t * VEC + k % VEC; };
   launch_wait();
-  // (uniform over the row's threads)
-  for (int row = blockIdx.x * ROWS + int(threadIdx.x) / TPR; row < B; row += int(gridDim.x) * ROWS) {
+  for (int first = blockIdx.x * ROWS; first < B; first += int(gridDim.x) * ROWS) {
+    const bool mine = first + int(threadIdx.x) / TPR < B;       // (the last rows' warps keep together: they shuffle)
+    const int row = mine ? first + int(threadIdx.x) / TPR : B - 1;
     const float* z = zL + (long long)row * ldz;
     __nv_bfloat16* d = delta + (long long)row * ldd;
     float v[N];
-    // position k of thread t is class (k / VEC) * TPR * VEC + t * VEC + k % VEC
-    auto cls = [&](int k) { return (k / VEC) * (TPR * VEC) + t * VEC + k % VEC; };
-    const bool wide = C > TPR * N;
     float mx = -INFINITY, s = 0.f;
 #pragma unroll
     for (int k = 0; k < N; k += VEC) {
       const int c = cls(k);
-      if (VEC == 2 && c + 1 < C) {
+      if (VEC == 4 && c + 3 < C) {
+        const float4 w = *reinterpret_cast<const float4*>(z + c);
+        v[k] = w.x; v[k + VEC / 4] = w.y; v[k + VEC / 2] = w.z; v[k + VEC - 1] = w.w;
+      } else if (VEC == 2 && c + 1 < C) {
         const float2 w = *reinterpret_cast<const float2*>(z + c);
         v[k] = w.x; v[k + VEC - 1] = w.y;
       } else {
@@ -264,68 +289,92 @@ softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict
         for (int e = 0; e < VEC; ++e) v[k + e] = c + e < C ? z[c + e] : -INFINITY;
       }
     }
+    const int y = labels[row];
 #pragma unroll
     for (int k = 0; k < N; ++k) mx = fmaxf(mx, v[k]);
     if (wide) for (int c = TPR * N + t; c < C; c += TPR) mx = fmaxf(mx, z[c]);
     mx = row_reduce<TPR>(mx, sh, true);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      v[k] = cls(k) < C ? expf(v[k] - mx) : 0.f;
+      v[k] = expf(v[k] - mx);                         // (0 in the lanes past C)
       s += v[k];
     }
     if (wide) for (int c = TPR * N + t; c < C; c += TPR) s += expf(z[c] - mx);
     s = row_reduce<TPR>(s, sh, false);
-    // A label outside [0, C) comes from caller memory: it must not become an address.  Such a row
-    // gets no one-hot term, its loss is NaN (so the minibatch loss is NaN) and the status word, where
-    // there is one, records it.
-    const int y = labels[row];
-    const bool y_ok = unsigned(y) < unsigned(C);
+    // Every class as if it were not the label, whose owner then overwrites its element: no comparison per element.
     const float inv_s = 1.0f / s;
-    auto out = [&](int c, float e) { return c < C ? (e * inv_s - (c == y ? 1.f : 0.f)) * invB : 0.f; };
 #pragma unroll
     for (int k = 0; k < N; k += VEC) {
       const int c = cls(k);
-      if (c >= Cpad) continue;
-      if (VEC == 2) *reinterpret_cast<__nv_bfloat162*>(d + c) = __floats2bfloat162_rn(out(c, v[k]), out(c + 1, v[k + VEC - 1]));
-      else d[c] = __float2bfloat16_rn(out(c, v[k]));
+      if (c >= Cpad || !mine) continue;
+      float o[VEC];
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) o[e] = v[k + e] * inv_s * invB;
+      if (c + VEC > C) {                              // (lanes past C are zeros whatever the row holds)
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) if (c + e >= C) o[e] = 0.f;
+      }
+      if (VEC == 4) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(o[0], o[VEC / 4]), hi = __floats2bfloat162_rn(o[VEC / 2], o[VEC - 1]);
+        *reinterpret_cast<uint2*>(d + c) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+      } else if (VEC == 2) {
+        *reinterpret_cast<__nv_bfloat162*>(d + c) = __floats2bfloat162_rn(o[0], o[VEC - 1]);
+      } else {
+        d[c] = __float2bfloat16_rn(o[0]);
+      }
     }
-    if (wide) for (int c = TPR * N + t; c < Cpad; c += TPR) d[c] = __float2bfloat16_rn(out(c, c < C ? expf(z[c] - mx) : 0.f));
-    if (t == 0) {
-      row_loss[row] = y_ok ? -((z[y] - mx) - logf(s)) : __int_as_float(0x7fc00000);
-      if (!y_ok && status != nullptr) atomicCAS(status, 0, LP_STATUS_BAD_LABEL);
+    if (wide) for (int c = TPR * N + t; c < Cpad; c += TPR) d[c] = __float2bfloat16_rn(c < C ? expf(z[c] - mx) * inv_s * invB : 0.f);
+    // A label outside [0, C) comes from caller memory: it must not become an address.  Such a row
+    // gets no one-hot term, its loss is NaN (so the minibatch loss is NaN) and the status word, where
+    // there is one, records it.
+    if (!mine) continue;
+    if (unsigned(y) < unsigned(C)) {
+      if (t == (y < TPR * N ? y / VEC : y - TPR * N) % TPR) {         // the thread that wrote element y
+        const float zy = z[y] - mx;
+        d[y] = __float2bfloat16_rn((expf(zy) * inv_s - 1.f) * invB);
+        row_loss[row] = -(zy - logf(s));
+      }
+    } else if (t == 0) {
+      row_loss[row] = __int_as_float(0x7fc00000);
+      if (status != nullptr) atomicCAS(status, 0, LP_STATUS_BAD_LABEL);
     }
   }
   launch_next();
+  if (ticket == nullptr && gridDim.x > 1) return;
   __threadfence();                                    // this block's row losses before its count
   __syncthreads();
   if (threadIdx.x == 0) {
-    last = atomicInc(ticket, gridDim.x - 1u) == gridDim.x - 1u;     // (wraps to zero: ready for the next launch)
+    last = gridDim.x == 1 || atomicInc(ticket, gridDim.x - 1u) == gridDim.x - 1u;     // (wraps to zero: ready for the next launch)
   }
   __syncthreads();
   if (last) {
-    // deterministic mean: thread t adds rows t, t + 256, ... in that order, then a tree over the threads
     __threadfence();
-    float acc = 0.f;
-#pragma unroll 8
-    for (int i = threadIdx.x; i < B; i += XENT_THREADS) acc += __ldcg(row_loss + i);
-    acc = row_reduce<XENT_THREADS>(acc, sh, false);
-    if (threadIdx.x == 0) *loss_out = acc * invB;
+    row_loss_mean<XENT_THREADS>(row_loss, loss_out, B, sh);
   }
 }
 
 cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __nv_bfloat16* delta, int ldd, float* row_loss,
                                 unsigned* ticket, float* loss_out, int B, int C, int* status, cudaStream_t stream) {
-  const bool vec2 = ldz % 2 == 0 && ldd % 2 == 0 && (reinterpret_cast<uintptr_t>(zL) & 7) == 0 && (reinterpret_cast<uintptr_t>(delta) & 3) == 0;
-  // Rows of up to 256 classes need 8 registers a lane and leave room for twice as many warps (16384 x 10: 12.7 us, with
-  // 32 registers and a block per 8 rows 25.3).  Blocks beyond what is resident loop over rows: each pays for its fence,
-  // count and barriers once (8192 x 1000 in 1024 blocks 24.1 us, in 444 20.3).
-#define LP_XENT(TPR, VEC, N, PER_SM)                                                                                 \
-  return launch_chained(softmax_xent_kernel<TPR, VEC, N>, std::min((B + XENT_THREADS / TPR - 1) / (XENT_THREADS / TPR), kSMs * PER_SM), \
-                        XENT_THREADS, 0, stream, 1, zL, ldz, labels, delta, ldd, row_loss, ticket, loss_out, B, C, status)
-  if (C <= 256)       { if (vec2) LP_XENT(32, 2, 8, 6); else LP_XENT(32, 1, 8, 6); }
-  else if (C <= 1024) { if (vec2) LP_XENT(32, 2, 32, 3); else LP_XENT(32, 1, 32, 3); }
-  else                { if (vec2) LP_XENT(256, 2, 32, 256); else LP_XENT(256, 1, 32, 256); }     // (a block per row: 2048 x 8192 36 us, looping 44)
+  const uintptr_t z_at = reinterpret_cast<uintptr_t>(zL), d_at = reinterpret_cast<uintptr_t>(delta);
+  const int vec = ldz % 4 == 0 && ldd % 4 == 0 && (z_at & 15) == 0 && (d_at & 7) == 0   ? 4
+                  : ldz % 2 == 0 && ldd % 2 == 0 && (z_at & 7) == 0 && (d_at & 3) == 0 ? 2
+                                                                                       : 1;
+  // Eight threads a row up to 64 classes, a warp up to 1024, a block beyond.  More blocks than are resident at once (four of 64
+  // registers a thread) keep an SM's share even; beyond that a block takes several rows.
+  const int rows = C <= 64 ? XENT_THREADS / 8 : C <= 1024 ? XENT_THREADS / 32 : 1;
+  const int grid = B <= 2 * rows ? 1 : std::min((B + rows - 1) / rows, kSMs * (C <= 1024 ? 8 : 256));
+#define LP_XENT(TPR, VEC, N) \
+  launch_chained(softmax_xent_kernel<TPR, VEC, N>, grid, XENT_THREADS, 0, stream, 1, zL, ldz, labels, delta, ldd, row_loss, ticket, loss_out, B, C, status)
+#define LP_XENT_VEC(TPR, N) (vec == 4 ? LP_XENT(TPR, 4, N) : vec == 2 ? LP_XENT(TPR, 2, N) : LP_XENT(TPR, 1, N))
+  const cudaError_t e = C <= 64     ? LP_XENT_VEC(8, 8)
+                        : C <= 256  ? LP_XENT_VEC(32, 8)
+                        : C <= 1024 ? LP_XENT_VEC(32, 32)
+                        : C <= 2048 ? LP_XENT_VEC(256, 8)
+                                    : LP_XENT_VEC(256, 32);
+#undef LP_XENT_VEC
 #undef LP_XENT
+  if (e != cudaSuccess || ticket != nullptr || grid == 1) return e;
+  return launch_chained(softmax_xent_mean_kernel, 1, XENT_MEAN_THREADS, 0, stream, 1, static_cast<const float*>(row_loss), loss_out, B);
 }
 
 // ---------------------------------------------------------------------------
@@ -585,13 +634,11 @@ cudaError_t launch_colsum_bias(const __nv_bfloat16* x, int rows, int ld, int n_c
 
 // ---------------------------------------------------------------------------
 // lp_softmax_xent_static: the loss kernel for callers that cannot supply scratch memory.
-// The per-row losses and the completion counter live in this fixed device array instead
-// of a workspace.  Host code must not pass `g_xent_scratch` itself to a kernel: in host
+// The per-row losses live in this fixed device array instead of a workspace.  Host code must not pass `g_xent_scratch` itself to a kernel: in host
 // code that name is only a handle for the runtime.  The device address is looked up once
 // per device with cudaGetSymbolAddress and that pointer is what the kernel receives.
 struct XentScratch {
   float row_loss[LP_XENT_STATIC_MAX_BATCH];
-  unsigned ticket;
 };
 static __device__ __align__(256) unsigned char g_xent_scratch[sizeof(XentScratch)];
 
@@ -631,13 +678,10 @@ extern "C" int lp_softmax_xent_static(const float* logits_dev, int ld_logits, co
     }
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // The counter must start at zero whatever two calls that overlapped have left in it: the kernel wraps it to zero
-  // only from a right start, and a call that finds a remainder adds up the rows before all of them are written.
-  // (8192 x 1000: 24.4 us with the memset, 22.5 without.)
-  cudaError_t e = cudaMemsetAsync(&s->ticket, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return xent_fail(LP_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
-  e = lp::launch_softmax_xent(logits_dev, ld_logits, labels_dev, static_cast<__nv_bfloat16*>(delta_dev), ld_delta, s->row_loss,
-                              &s->ticket, loss_dev, batch, classes, nullptr, st);
+  // No counter here: two calls that overlapped could leave anything in it, and clearing it is a launch before the kernel that
+  // nothing overlaps with; the mean is a launch behind it, which is in place when the rows are done.
+  const cudaError_t e = lp::launch_softmax_xent(logits_dev, ld_logits, labels_dev, static_cast<__nv_bfloat16*>(delta_dev), ld_delta, s->row_loss,
+                              nullptr, loss_dev, batch, classes, nullptr, st);
   if (e != cudaSuccess) return xent_fail(LP_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
   return LP_OK;
 }

@@ -104,7 +104,11 @@ def test_static_scratch_loss_never_uses_a_bad_label_as_an_address():
 
 
 @pytest.mark.parametrize("B, C, ld", [(1, 1, 1), (3, 2, 2), (9, 1000, 1000), (7, 1001, 1003), (8, 1024, 1024), (5, 1025, 1026),
-                                      (4, 8192, 8192), (3, 8195, 8195), (300, 33, 40)])
+                                      (4, 8192, 8192), (3, 8195, 8195), (300, 33, 40),
+                                      # eight threads a row: one class, 64 and 65, rows that end inside a warp; four classes an access and a ragged last four;
+                                      # more rows than a pass of the grid; 257, 2048 and 2049 classes
+                                      (67, 1, 4), (133, 64, 64), (70, 65, 68), (131, 61, 64), (16384, 10, 12), (9500, 258, 260),
+                                      (33, 257, 257), (41, 2048, 2048), (40, 2049, 2052), (37, 2047, 2048)])
 def test_static_loss_at_the_edges_of_its_row_forms(B, C, ld):
     """A warp or a block per row, classes beyond what the registers hold, odd pitches (one class per access), a masked
     class (-inf logit): loss and delta against float64.  One bf16 rounding of delta; fp32 sums over C classes."""
