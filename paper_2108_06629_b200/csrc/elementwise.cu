@@ -380,11 +380,11 @@ cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __n
 // ---------------------------------------------------------------------------
 // Fused update (Eq. 6, optional momentum): m <- mu m + G; W <- W - eta m; ring <- RN(W).
 // 8 elements per thread, 128-bit loads and stores throughout.  Blocks past the weight
-// range own 64 bias columns each: bias gradient = column sums of delta (row order),
+// range own BIAS_COLS bias columns each: bias gradient = column sums of delta (row order),
 // then the same update for the bias.
 constexpr int UPD_THREADS = 256;
 constexpr int UPD_VEC_PER_THREAD = 2;     // x 8 elements
-constexpr int BIAS_COLS = 64;
+constexpr int BIAS_COLS = UPD_THREADS / BIAS_LANES;
 
 __global__ void __launch_bounds__(UPD_THREADS) sgd_update_kernel(const UpdateArgs a, int w_blocks) {
   launch_wait();
@@ -427,10 +427,10 @@ __global__ void __launch_bounds__(UPD_THREADS) sgd_update_kernel(const UpdateArg
     return;
   }
   // ---- bias part: this block owns BIAS_COLS columns --------------------------
-  __shared__ float part[UPD_THREADS / BIAS_COLS][BIAS_COLS];
+  __shared__ float part[BIAS_LANES][BIAS_COLS];
   const int cb = (int(blockIdx.x) - w_blocks) * BIAS_COLS;
   const int tx = threadIdx.x % BIAS_COLS, ty = threadIdx.x / BIAS_COLS;
-  constexpr int NY = UPD_THREADS / BIAS_COLS;
+  constexpr int NY = BIAS_LANES;
   const int col = cb + tx;
   float acc = 0.f;
   if (col < a.n_out) {

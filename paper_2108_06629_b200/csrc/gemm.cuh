@@ -862,32 +862,43 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           const uint32_t smem0 = smem_u32(smem), ufull0 = smem_u32(ufull_bar), empty0 = smem_u32(empty_bar);
           const uint32_t ringbuf = smem_u32(full_bar) + 1024u;
           const int trow = q * 32 + lane;            // row of the tile this lane owns (tensor-memory lane)
-          if (p.bdelta != nullptr && tm.n0 == 0 && tm.m0 + trow < p.M) {
+          if (p.bdelta != nullptr && tm.n0 == 0) {
             // Bias of output feature m = column sum of delta over the batch, then Eq. 6 -- while
             // the tile's main loop runs.  Same order of additions as the stand-alone update
-            // kernel (four interleaved partial sums, combined in order), so both give the same bits.
+            // kernel (BIAS_LANES interleaved partial sums, combined in order), so both give the same bits.  A thread takes
+            // eight features (16 bytes a row) of one partial sum; the staging tile holds the partial sums for a moment.
+            if (PERSIST) asm volatile("bar.sync 1, 128;" ::: "memory");     // (the last store of the tile before has read the staging tile)
+            float* sums = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(full_bar) + 1024);   // [BIAS_LANES][128]
+            const int e = q * 32 + lane, c8 = (e & 15) * 8, part = e >> 4;
+            static_assert(BIAS_LANES == 8 && BIAS_LANES * GEMM_BM * 4 <= UPD_RING_BYTES, "128 threads, 16 of them to a row");
+            float acc8[8] = {};
+            if (tm.m0 + c8 < p.bld) {
+              const __nv_bfloat16* src = p.bdelta + tm.m0 + c8;
+#pragma unroll 8
+              for (int r = part; r < p.brows; r += BIAS_LANES) {
+                const uint4 v = *reinterpret_cast<const uint4*>(src + size_t(r) * p.bld);
+                acc8[0] += bf16_lo(v.x); acc8[1] += bf16_hi(v.x); acc8[2] += bf16_lo(v.y); acc8[3] += bf16_hi(v.y);
+                acc8[4] += bf16_lo(v.z); acc8[5] += bf16_hi(v.z); acc8[6] += bf16_lo(v.w); acc8[7] += bf16_hi(v.w);
+              }
+            }
+            *reinterpret_cast<float4*>(sums + part * GEMM_BM + c8) = make_float4(acc8[0], acc8[1], acc8[2], acc8[3]);
+            *reinterpret_cast<float4*>(sums + part * GEMM_BM + c8 + 4) = make_float4(acc8[4], acc8[5], acc8[6], acc8[7]);
+            asm volatile("bar.sync 1, 128;" ::: "memory");
             const int m = tm.m0 + trow;
-            float part[4] = {0.f, 0.f, 0.f, 0.f};
-            const __nv_bfloat16* src = p.bdelta + m;
-            int r = 0;
-#pragma unroll 4
-            for (; r + 4 <= p.brows; r += 4) {
+            if (m < p.M) {
+              float g = 0.f;
 #pragma unroll
-              for (int i = 0; i < 4; ++i) part[i] += __bfloat162float(src[size_t(r + i) * p.bld]);
+              for (int i = 0; i < BIAS_LANES; ++i) g += sums[i * GEMM_BM + trow];
+              p.bdb[m] = g;
+              float mm = g;
+              if (p.bmb != nullptr) {
+                mm = p.mu * p.bmb[m] + g;
+                p.bmb[m] = mm;
+              }
+              const float b = p.bb[m] - p.lr * mm;
+              p.bb[m] = b;
+              p.bbring[m] = b;
             }
-            for (int i = 0; r + i < p.brows; ++i) part[i] += __bfloat162float(src[size_t(r + i) * p.bld]);
-            float g = 0.f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) g += part[i];
-            p.bdb[m] = g;
-            float mm = g;
-            if (p.bmb != nullptr) {
-              mm = p.mu * p.bmb[m] + g;
-              p.bmb[m] = mm;
-            }
-            const float b = p.bb[m] - p.lr * mm;
-            p.bb[m] = b;
-            p.bbring[m] = b;
           }
           if (good) {
             good = mbar_wait_addr(accf0 + 8u * buf, (it >> 1) & 1u, p.wait_limit);
