@@ -21,6 +21,8 @@
 // 2-D map, the output tile stored through a 2-D map.  Such a layer is 25 000 tiles of a single
 // k-block each, and what it needs is this kernel's epilogue.
 #pragma once
+#include <type_traits>
+
 #include "gemm.cuh"
 
 namespace lp {
@@ -127,7 +129,11 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc_bf16(GEMM_BM, BN, false, B_MN);
+      // Narrow layers: only the slices of 16 channels that exist are multiplied, into as many columns as there are (what
+      // lies beyond in the boxes is zero fill).  224 x 224, batch 32, pooled: 16 -> 16 channels 134 -> 95 us; 112 x 112,
+      // 32 -> 32 43 -> 33.  The loop is written out per number of slices: a test in front of each MMA cost more than it saved.
+      const uint32_t idesc = idesc_with_cols(make_idesc_bf16(GEMM_BM, BN, false, B_MN), min(BN, (p.N + 15) & ~15));
+      const int slices = p.g.last_slices;
       constexpr uint32_t stepB = (B_MN ? 2048 : 32) >> 4;
       // One thread issues 36 MMAs per tile, so everything that can be is computed once: the
       // descriptors of box 0 / tap 0, and per tap the start-address offset of its view (the
@@ -154,17 +160,23 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * uint32_t(BN);
         const uint32_t a_lo = dA_lo0 + st * uint32_t(HALO_BYTES >> 4);
-        uint32_t acc = 0;
+        auto taps = [&](auto SLICES) {
+          uint32_t acc = 0;
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          if (tap >= ntaps) break;
+          for (int tap = 0; tap < 9; ++tap) {
+            if (tap >= ntaps) break;
 #pragma unroll
-          for (int j = 0; j < GEMM_BK / 16; ++j) {
-            umma_f16_lohi(tacc, a_lo + tap_off[tap] + uint32_t(j * 2), dA_hi,
-                          dB_lo0 + uint32_t(tap) * uint32_t(HALO_TAP_BYTES >> 4) + uint32_t(j) * stepB, dB_hi, idesc, acc);
-            acc = 1;
+            for (int j = 0; j < int(SLICES); ++j) {
+              umma_f16_lohi(tacc, a_lo + tap_off[tap] + uint32_t(j * 2), dA_hi,
+                            dB_lo0 + uint32_t(tap) * uint32_t(HALO_TAP_BYTES >> 4) + uint32_t(j) * stepB, dB_hi, idesc, acc);
+              acc = 1;
+            }
           }
-        }
+        };
+        if (slices == 4) taps(std::integral_constant<int, 4>{});
+        else if (slices == 3) taps(std::integral_constant<int, 3>{});
+        else if (slices == 2) taps(std::integral_constant<int, 2>{});
+        else taps(std::integral_constant<int, 1>{});
         umma_commit(&aempty[st]);
         umma_commit(&accf[buf]);
         if (++st == uint32_t(HALO_STAGES)) { st = 0; sph ^= 1u; }
@@ -240,15 +252,19 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const uint32_t so = smem_u32(sO) + buf * uint32_t(HALO_OUT_BYTES) + uint32_t(trow) * 128u;
         const uint32_t swz = uint32_t(trow & 7);
         uint32_t packed[16];
+        const bool live = !dead && half * 32 < p.N;       // (at most 32 channels: the second half has none)
         if (!dead) {
           uint32_t r[32];
-          tmem_ld_32x32(tacc + (uint32_t(q * 32) << 16) + uint32_t(half * 32), r);
-          tmem_ld_wait();
+          if (live) {
+            tmem_ld_32x32(tacc + (uint32_t(q * 32) << 16) + uint32_t(half * 32), r);
+            tmem_ld_wait();
+          }
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&acce[buf]);
 #pragma unroll
           for (int g = 0; g < 8; ++g) {
+            if (!live) break;
             const int n = half * 32 + 4 * g;
             float v[4] = {__uint_as_float(r[4 * g]), __uint_as_float(r[4 * g + 1]), __uint_as_float(r[4 * g + 2]), __uint_as_float(r[4 * g + 3])};
             if constexpr (MODE == EPI_FPROP) {
@@ -271,7 +287,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // the staging tile of two tiles ago must have been read by its store
         if (threadIdx.x == 64) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (!dead) {
+        if (live) {
 #pragma unroll
           for (int u = 0; u < 4; ++u)
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(so + ((uint32_t(half * 4 + u) ^ swz) << 4)), "r"(packed[4 * u]),
@@ -371,7 +387,7 @@ constexpr int HALOG_PART_FLOATS = HALOG_GROUPS * GEMM_BM * 64;  // partial sums 
 template <int kInstance = 0>   // (a template only so that the header may be included by several translation units)
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD, const ConvGeom g,
-                   const int tiles_total, const int co0, float* __restrict__ partial, int* __restrict__ status) {
+                   const int tiles_total, const int co0, const int cols, float* __restrict__ partial, int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + HALOG_STAGES * HALOG_STAGE_BYTES);
@@ -432,7 +448,7 @@ conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc_bf16(GEMM_BM, 64, true, true);
+      const uint32_t idesc = idesc_with_cols(make_idesc_bf16(GEMM_BM, 64, true, true), min(64, (cols + 15) & ~15));
       // tap groups: first tap of the group as a halo row offset, and the distance to its partner
       const uint32_t first_row[HALOG_GROUPS] = {0u, 2u, uint32_t(HALO_W + 1), uint32_t(2 * HALO_W), uint32_t(2 * HALO_W + 2)};
       const uint32_t lbo[HALOG_GROUPS] = {128u, uint32_t((HALO_W - 2) * 128), 128u, 128u, 0u};

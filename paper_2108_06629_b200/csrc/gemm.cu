@@ -506,7 +506,8 @@ cudaError_t conv_halo_g_launch(const CUtensorMap& tmX, const CUtensorMap& tmD, c
   upd.n_ctas = grid;
   for (int co0 = 0; co0 < upd.n_out; co0 += 64) {      // one pass per 64 output channels; the stream orders the reuse of `partial`
     note_form("halo G", 64);
-    cudaError_t e = launch_chained(conv_halo_g_kernel<0>, grid, GEMM_THREADS, HALOG_SMEM_BYTES, st, 1, tmX, tmD, g, tiles, co0, partial, status);
+    cudaError_t e = launch_chained(conv_halo_g_kernel<0>, grid, GEMM_THREADS, HALOG_SMEM_BYTES, st, 1, tmX, tmD, g, tiles, co0,
+                                   std::min(64, upd.n_out - co0), partial, status);
     if (e != cudaSuccess) return e;
     upd.co0 = co0;
     e = launch_chained(conv_halo_g_update_kernel<0>, HALOG_PART_FLOATS / 32, 256, 0, st, 1, upd);

@@ -790,6 +790,8 @@ struct TimedScope {
 
 // ---------------------------------------------------------------------------
 // the kernels of one minibatch
+// slices of 16 that the last 64 of `channels` hold
+static int last_slices(int channels) { return ((channels - 1) % 64) / 16 + 1; }
 static ConvGeom conv_geom(const Layer& y, int kind, const PixBox& bx, int flip, int chunks_per_tap, int n_per_tap) {
   ConvGeom g{};
   g.kind = kind;
@@ -801,6 +803,7 @@ static ConvGeom conv_geom(const Layer& y, int kind, const PixBox& bx, int flip, 
   g.S = y.cS; g.pad = y.cpad;
   g.flip = flip;
   g.chunks_per_tap = chunks_per_tap;
+  g.last_slices = last_slices(flip ? y.n_out : y.n_in);
   g.tap_pitch = y.ld_in;
   g.n_per_tap = n_per_tap;
   g.stride = y.cstride;
@@ -820,6 +823,7 @@ static ConvGeom halo_geom(const Layer& y, int flip) {
   g.S = 3; g.pad = 1;
   g.flip = flip;
   g.chunks_per_tap = 1;
+  g.last_slices = last_slices(flip ? y.n_out : y.n_in);
   g.tap_pitch = y.ld_in;
   g.stride = 1;
   g.rs = 1;
@@ -876,6 +880,7 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
   ++c->launches;
   TimedScope ts(c, LP_TASK_FORWARD, st, l);
   if (y.lean_f) {
+    a.g.last_slices = last_slices(y.n_in);      // (plain geometry otherwise)
     const CUtensorMap& tmo = y.pool ? y.tm_hf_O[0] : y.tm_hf_O[xout];
     return conv_halo_launch(0, y.tm_f_A[xin], y.tm_f_B[ring_slot], tmo, a, st);
   }

@@ -266,4 +266,9 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N, bool a_mn, 
          (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
 
+// The same with the number of columns put in at run time (a multiple of 16 with M = 128).
+__device__ __forceinline__ uint32_t idesc_with_cols(uint32_t idesc, int cols) {
+  return (idesc & ~(0x3Fu << 17)) | (uint32_t(cols >> 3) << 17);
+}
+
 }  // namespace lp
