@@ -21,8 +21,6 @@
 // 2-D map, the output tile stored through a 2-D map.  Such a layer is 25 000 tiles of a single
 // k-block each, and what it needs is this kernel's epilogue.
 #pragma once
-#include <type_traits>
-
 #include "gemm.cuh"
 
 namespace lp {
@@ -33,16 +31,25 @@ constexpr int HALO_BYTES = HALO_W * HALO_H * 128;             // 64 bf16 channel
 constexpr int HALO_TAP_BYTES = 64 * 64 * 2;                   // one weight tap: 64 x 64 bf16
 constexpr int HALO_OUT_BYTES = GEMM_BM * 128;                 // forward: one output tile, 128 pixels x 64 bf16 channels
 constexpr int HALO_THREADS = 320;                             // producer warp, MMA warp, eight epilogue warps
-constexpr int HALO_EPI_BYTES = 2 * EPI_TILE_BYTES;            // forward: two output tiles (32 KiB); delta: eight transposition tiles (36 KiB)
+constexpr int HALO_EPI_BYTES = 2 * EPI_TILE_BYTES;            // two output tiles (32 KiB); un-pooling delta: eight transposition tiles (36 KiB)
 static_assert(HALO_EPI_BYTES >= 2 * HALO_OUT_BYTES, "the epilogue area holds two output tiles");
 constexpr int HALO_SMEM_BYTES = 9 * HALO_TAP_BYTES + HALO_STAGES * HALO_BYTES + HALO_EPI_BYTES + 256 + 1024;
 static_assert((HALO_STAGES * HALO_BYTES) % 1024 == 0, "the buffers behind the halo boxes stay 1 KiB aligned");
 
-template <bool B_MN, int MODE>
+// SLICES: 16-channel slices of the contraction that exist; the rest of a 64-channel box is zero fill and not multiplied.  A template
+// parameter: with a test in front of each MMA the one thread that issues them lost more than it saved.
+// TURNS: the epilogue's eight warps are two groups that take the tiles in turn, instead of sharing each tile.  A tile's way from
+// accumulator to store is a chain of waits (tensor memory, staging tile free, barriers), and where the MMAs of a tile are
+// few -- narrow layers, the patch-matrix form -- that chain is what a tile costs, so two tiles are on it at once.  Times of layers at
+// 224 x 224, batch 32, 16 -> 16 channels pooled: forward 134 us with all MMAs, 95 with SLICES, 70 with TURNS; delta 137, 122, 77;
+// patch-matrix forward 76, 74, 52.  Wide layers share: 64 -> 64 delta at batch 64 316 us, in turns 333, and the small VGG 1 % slower.
+template <bool B_MN, int MODE, int SLICES, bool TURNS>
 __global__ void __launch_bounds__(HALO_THREADS, 1)
 conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmO, const GemmArgs p, const int tiles_total) {
   constexpr int BN = 64;
+  constexpr int HALO_ACC = TURNS ? 4 : 2;               // accumulators: two per group
+  constexpr int NGRP = TURNS ? 2 : 1, GW = 8 / NGRP, H = TURNS ? 2 : 1;      // epilogue groups, warps of a group, column halves of a warp
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sB = smem;                                   // [9][64 x 64] weight taps
@@ -53,9 +60,9 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   uint64_t* wfull = bars;          // weights resident
   uint64_t* afull = bars + 1;                       // [HALO_STAGES] halo box landed
   uint64_t* aempty = afull + HALO_STAGES;           // [HALO_STAGES] halo box consumed
-  uint64_t* accf = aempty + HALO_STAGES;            // [2] accumulator complete
-  uint64_t* acce = accf + 2;                        // [2] accumulator drained
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
+  uint64_t* accf = aempty + HALO_STAGES;            // [HALO_ACC] accumulator complete
+  uint64_t* acce = accf + HALO_ACC;                 // [HALO_ACC] accumulator drained
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + HALO_ACC);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -68,16 +75,16 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       mbar_init(&afull[b], 1);
       mbar_init(&aempty[b], 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < HALO_ACC; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], 8);      // one arrival per epilogue warp
+      mbar_init(&acce[b], GW);     // one arrival per warp of the epilogue group
     }
     fence_barrier_init();
   }
   if (warp == 1) {
     if (lane == 0) tmem_note_enter(TK_HALO);
-    tmem_alloc(tmem_slot, 2 * BN);
-    if (lane == 0) tmem_note_got(TK_HALO, 2 * BN);
+    tmem_alloc(tmem_slot, HALO_ACC * BN);
+    if (lane == 0) tmem_note_got(TK_HALO, HALO_ACC * BN);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -129,11 +136,9 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      // Narrow layers: only the slices of 16 channels that exist are multiplied, into as many columns as there are (what
-      // lies beyond in the boxes is zero fill).  224 x 224, batch 32, pooled: 16 -> 16 channels 134 -> 95 us; 112 x 112,
-      // 32 -> 32 43 -> 33.  The loop is written out per number of slices: a test in front of each MMA cost more than it saved.
-      const uint32_t idesc = idesc_with_cols(make_idesc_bf16(GEMM_BM, BN, false, B_MN), min(BN, (p.N + 15) & ~15));
-      const int slices = p.g.last_slices;
+      // (narrow layers: as many accumulator columns as there are channels)
+      const uint32_t idesc = TURNS ? idesc_with_cols(make_idesc_bf16(GEMM_BM, BN, false, B_MN), min(BN, (p.N + 15) & ~15))
+                                   : make_idesc_bf16(GEMM_BM, BN, false, B_MN);
       constexpr uint32_t stepB = (B_MN ? 2048 : 32) >> 4;
       // One thread issues 36 MMAs per tile, so everything that can be is computed once: the
       // descriptors of box 0 / tap 0, and per tap the start-address offset of its view (the
@@ -152,31 +157,25 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       uint32_t it = 0, st = 0, sph = 0;
       int t = t_begin;
       for (; t < t_end && ok; ++t, ++it) {
-        const uint32_t buf = it & 1u;
-        ok = mbar_wait(&acce[buf], ((it >> 1) & 1u) ^ 1u);
+        const uint32_t buf = it % HALO_ACC;
+        ok = mbar_wait(&acce[buf], ((it / HALO_ACC) & 1u) ^ 1u);
         if (!ok) break;
         ok = mbar_wait(&afull[st], sph);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tacc = tmem_base + buf * uint32_t(BN);
         const uint32_t a_lo = dA_lo0 + st * uint32_t(HALO_BYTES >> 4);
-        auto taps = [&](auto SLICES) {
-          uint32_t acc = 0;
+        uint32_t acc = 0;
 #pragma unroll
-          for (int tap = 0; tap < 9; ++tap) {
-            if (tap >= ntaps) break;
+        for (int tap = 0; tap < 9; ++tap) {
+          if (tap >= ntaps) break;
 #pragma unroll
-            for (int j = 0; j < int(SLICES); ++j) {
-              umma_f16_lohi(tacc, a_lo + tap_off[tap] + uint32_t(j * 2), dA_hi,
-                            dB_lo0 + uint32_t(tap) * uint32_t(HALO_TAP_BYTES >> 4) + uint32_t(j) * stepB, dB_hi, idesc, acc);
-              acc = 1;
-            }
+          for (int j = 0; j < SLICES; ++j) {
+            umma_f16_lohi(tacc, a_lo + tap_off[tap] + uint32_t(j * 2), dA_hi,
+                          dB_lo0 + uint32_t(tap) * uint32_t(HALO_TAP_BYTES >> 4) + uint32_t(j) * stepB, dB_hi, idesc, acc);
+            acc = 1;
           }
-        };
-        if (slices == 4) taps(std::integral_constant<int, 4>{});
-        else if (slices == 3) taps(std::integral_constant<int, 3>{});
-        else if (slices == 2) taps(std::integral_constant<int, 2>{});
-        else taps(std::integral_constant<int, 1>{});
+        }
         umma_commit(&aempty[st]);
         umma_commit(&accf[buf]);
         if (++st == uint32_t(HALO_STAGES)) { st = 0; sph ^= 1u; }
@@ -184,46 +183,51 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (!ok) report_expired(p.status, WAIT_HALO_MMA, t, 0);
     }
   } else {
-    // Eight warps: warp w reads tensor-memory lanes 32 * (w % 4) (the rows of its quarter of the
-    // tile) and takes columns 32 * half .. + 32.  With one warp per scheduler there is nothing to
+    // Warp w reads tensor-memory lanes 32 * (w % 4) (the rows of its quarter of the tile), a lane one row: 32 columns of
+    // it where all eight warps share a tile, else all of it.  With one warp per scheduler there is nothing to
     // hide an instruction's latency behind, so the epilogue is spread as wide as the tile allows.
     const int q = warp & 3;
-    const int half = (warp - 2) >> 2;
+    const int grp = (warp - 2) / GW, half0 = TURNS ? 0 : (warp - 2) >> 2;
     float* tile = epi_tile + (warp - 2) * (32 * EPI_PITCH);
     const int sub_row = lane >> 3;
     const int sub_col = (lane & 7) * 4;
-    uint32_t it = 0;
+    const bool chief = threadIdx.x == 64u + 32u * uint32_t(GW * grp);    // issues its group's stores
+    auto group_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(32 * GW) : "memory"); };
+    uint32_t it = uint32_t(grp);
     bool dead = false;      // a wait ran out: keep the named-barrier count, touch nothing else
-    // the bias of this warp's 32 output channels does not depend on the tile (rows are padded to 8 with zeros)
-    float4 bias4[8];
+    const int halves = TURNS ? min((p.N + 31) / 32, 2) : 1;          // of this warp's column halves, those with output channels
+    // the bias of this warp's output channels does not depend on the tile (rows are padded to 8 with zeros)
+    float4 bias4[8 * H];
 #pragma unroll
-    for (int g = 0; g < 8; ++g) {
-      const int n = half * 32 + 4 * g;
+    for (int g = 0; g < 8 * H; ++g) {
+      const int n = half0 * 32 + 4 * g;
       bias4[g] = (MODE == EPI_FPROP && p.bias != nullptr && n < p.N) ? __ldg(reinterpret_cast<const float4*>(p.bias + n))
                                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    int tw = tw_begin - 1, th = th_begin, tn = tn_begin;
-    // delta: what f' is evaluated on, this lane's pixel and 32 columns, asked for one tile ahead: an accumulator is
+    int tw = tw_begin, th = th_begin, tn = tn_begin;
+    auto next_tile = [&] { if (!plain && ++tw == p.g.tiles_w) { tw = 0; if (++th == p.g.tiles_h) { th = 0; ++tn; } } };
+    if (grp == 1) next_tile();
+    // delta: what f' is evaluated on, this lane's pixel and columns, asked for one tile of the group ahead: an accumulator is
     // usually complete when these warps reach it, and the round trip would be theirs alone
-    uint4 av[4], av_next[4];
-    auto load_aux = [&](int t, uint4 (&v)[4]) {
+    constexpr int kAux = MODE == EPI_DGRAD ? 4 * H : 1;
+    uint4 av[kAux], av_next[kAux];
+    auto load_aux = [&](int t, uint4 (&v)[kAux]) {
       const int img = t / tiles_per_image, r = t - img * tiles_per_image, rh = r / p.g.tiles_w;
       const int trow = q * 32 + lane;
       const size_t pix = (size_t(img) * p.g.H + rh * 16 + (trow >> 3)) * p.g.W + (r - rh * p.g.tiles_w) * 8 + (trow & 7);
-      const __nv_bfloat16* src = p.aux + pix * p.ld_aux + half * 32;
+      const __nv_bfloat16* src = p.aux + pix * p.ld_aux + half0 * 32;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        v[u] = (p.act != ACT_NONE && half * 32 + 8 * u < p.ld_aux) ? *reinterpret_cast<const uint4*>(src + 8 * u) : make_uint4(0u, 0u, 0u, 0u);
+      for (int u = 0; u < kAux; ++u)
+        v[u] = (p.act != ACT_NONE && half0 * 32 + 8 * u < p.ld_aux) ? *reinterpret_cast<const uint4*>(src + 8 * u) : make_uint4(0u, 0u, 0u, 0u);
     };
-    if (MODE == EPI_DGRAD && t_begin < t_end) load_aux(t_begin, av_next);
-    for (int t = t_begin; t < t_end; ++t, ++it) {
-      const uint32_t buf = it & 1u;
+    if (MODE == EPI_DGRAD && t_begin + grp < t_end) load_aux(t_begin + grp, av_next);
+    for (int t = t_begin + grp; t < t_end; t += NGRP, it += NGRP) {
+      const uint32_t buf = it % HALO_ACC;
       if constexpr (MODE == EPI_DGRAD) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) av[u] = av_next[u];
-        if (t + 1 < t_end) load_aux(t + 1, av_next);
+        for (int u = 0; u < kAux; ++u) av[u] = av_next[u];
+        if (t + NGRP < t_end) load_aux(t + NGRP, av_next);
       }
-      if (!plain && ++tw == p.g.tiles_w) { tw = 0; if (++th == p.g.tiles_h) { th = 0; ++tn; } }
       TileMap tm;
       tm.m0 = t * GEMM_BM;            // (plain geometry)
       tm.n0 = 0;
@@ -231,17 +235,19 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       tm.pw0 = tw * 8;
       tm.ph0 = th * 16;
       tm.pn0 = tn;
+#pragma unroll
+      for (int k = 0; k < NGRP; ++k) next_tile();
       if (!dead) {
-        bool ok = mbar_wait(&accf[buf], (it >> 1) & 1u);
+        bool ok = mbar_wait(&accf[buf], (it / HALO_ACC) & 1u);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) {
           if (lane == 0) report_expired(p.status, WAIT_HALO_EPILOGUE, t, -1);
           dead = true;
         }
       }
-      if (dead && MODE == EPI_DGRAD_UNPOOL) break;      // the other epilogues have CTA-wide barriers
+      if (dead && MODE == EPI_DGRAD_UNPOOL) break;      // the other epilogues have barriers of the group
       tc_fence_after();
-      const uint32_t tacc = tmem_base + buf * uint32_t(BN);
+      const uint32_t tacc = tmem_base + buf * uint32_t(BN) + (uint32_t(q * 32) << 16);
       if constexpr (MODE != EPI_DGRAD_UNPOOL) {
         // A lane keeps its accumulator row (one pixel), adds the bias and applies f (forward) or multiplies by
         // f' (delta), and writes the 64 bf16 channels as one 128-byte swizzled row of a shared-memory tile that a
@@ -249,28 +255,32 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // arithmetic per element, and the global writes are whole lines.  (Delta through transposition
         // tiles and 8-byte accesses: 418 us for 64 channels at 224 x 224, batch 64; this form 314, 428 without the look-ahead.)
         const int trow = q * 32 + lane;
-        const uint32_t so = smem_u32(sO) + buf * uint32_t(HALO_OUT_BYTES) + uint32_t(trow) * 128u;
+        const uint32_t stage = smem_u32(sO) + (TURNS ? uint32_t(grp) : buf) * uint32_t(HALO_OUT_BYTES);
+        const uint32_t so = stage + uint32_t(trow) * 128u;
         const uint32_t swz = uint32_t(trow & 7);
         uint32_t packed[16];
-        const bool live = !dead && half * 32 < p.N;       // (at most 32 channels: the second half has none)
-        if (!dead) {
+        auto compute = [&](int h) {                     // h: which of this warp's column halves
           uint32_t r[32];
-          if (live) {
-            tmem_ld_32x32(tacc + (uint32_t(q * 32) << 16) + uint32_t(half * 32), r);
-            tmem_ld_wait();
+          tmem_ld_32x32(tacc + uint32_t((half0 + h) * 32), r);
+          tmem_ld_wait();
+          if (h == halves - 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce[buf]);
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&acce[buf]);
 #pragma unroll
           for (int g = 0; g < 8; ++g) {
-            if (!live) break;
-            const int n = half * 32 + 4 * g;
+            const int n = (half0 + h) * 32 + 4 * g;
             float v[4] = {__uint_as_float(r[4 * g]), __uint_as_float(r[4 * g + 1]), __uint_as_float(r[4 * g + 2]), __uint_as_float(r[4 * g + 3])};
+            uint32_t a01 = 0u, a23 = 0u;
             if constexpr (MODE == EPI_FPROP) {
-              v[0] += bias4[g].x; v[1] += bias4[g].y; v[2] += bias4[g].z; v[3] += bias4[g].w;
+              const float4 b = bias4[h * 8 + g];
+              v[0] += b.x; v[1] += b.y; v[2] += b.z; v[3] += b.w;
+            } else {
+              const uint4 a = av[h * 4 + (g >> 1)];
+              a01 = (g & 1) ? a.z : a.x;
+              a23 = (g & 1) ? a.w : a.y;
             }
-            const uint32_t a01 = (g & 1) ? av[g >> 1].z : av[g >> 1].x, a23 = (g & 1) ? av[g >> 1].w : av[g >> 1].y;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               if (n + e >= p.N) v[e] = 0.f;
@@ -283,22 +293,38 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             packed[2 * g] = pack_bf16x2(v[0], v[1]);
             packed[2 * g + 1] = pack_bf16x2(v[2], v[3]);
           }
-        }
-        // the staging tile of two tiles ago must have been read by its store
-        if (threadIdx.x == 64) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (live) {
+        };
+        auto put = [&](int h) {
 #pragma unroll
           for (int u = 0; u < 4; ++u)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(so + ((uint32_t(half * 4 + u) ^ swz) << 4)), "r"(packed[4 * u]),
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(so + ((uint32_t((half0 + h) * 4 + u) ^ swz) << 4)), "r"(packed[4 * u]),
                          "r"(packed[4 * u + 1]), "r"(packed[4 * u + 2]), "r"(packed[4 * u + 3])
                          : "memory");
+        };
+        if (!TURNS && !dead) compute(0);
+        // the staging tile must have been read by its last store -- the group's last, or that of two tiles ago -- and by the
+        // threads that pooled it
+        if (chief) {
+          if (TURNS) tma_store_wait_read0();
+          else       asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         }
+        group_sync();
+        if (TURNS && !dead) {
+#pragma unroll
+          for (int h = 0; h < H; ++h) {
+            if (h >= halves) break;
+            compute(h);
+            put(h);
+          }
+        }
+        if (!TURNS && !dead) put(0);
         if (MODE == EPI_FPROP && p.pool_out_idx != nullptr) {
-          // 2x2 max pool of the staged tile: a thread takes one of its 32 windows and eight channels
-          asm volatile("bar.sync 1, 256;" ::: "memory");
-          const int e = int(threadIdx.x) - 64, pp = e >> 3, cg = e & 7;
-          if (!dead && cg * 8 < p.ld_out) {
+          // 2x2 max pool of the staged tile: a thread takes eight channels of one of its 32 windows, or of two
+          group_sync();
+#pragma unroll
+          for (int k2 = 0; k2 < H; ++k2) {
+            const int e = ((int(threadIdx.x) - 64) & (32 * GW - 1)) + k2 * (32 * GW), pp = e >> 3, cg = e & 7;
+            if (dead || cg * 8 >= p.ld_out) continue;
             const int pw = pp & 3, ph = pp >> 2;
             float best[8];
             uint32_t idx[2] = {0u, 0u};
@@ -307,7 +333,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               const uint32_t tr = uint32_t((2 * ph + (k >> 1)) * 8 + 2 * pw + (k & 1));
               uint32_t w[4];
               asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
-                           : "r"(smem_u32(sO) + buf * uint32_t(HALO_OUT_BYTES) + tr * 128u + ((uint32_t(cg) ^ (tr & 7u)) << 4)));
+                           : "r"(stage + tr * 128u + ((uint32_t(cg) ^ (tr & 7u)) << 4)));
 #pragma unroll
               for (int j = 0; j < 4; ++j) pool_step(w[j], k, best + 4 * (j >> 1), idx[j >> 1], 2 * (j & 1));
             }
@@ -319,45 +345,47 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           continue;
         }
         fence_proxy_async_smem();
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (threadIdx.x == 64 && !dead) {
+        group_sync();
+        if (chief && !dead) {
           if (plain) {
-            tma_store_2d_addr(&tmO, smem_u32(sO) + buf * uint32_t(HALO_OUT_BYTES), 0, tm.m0);
+            tma_store_2d_addr(&tmO, stage, 0, tm.m0);
           } else {
             asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
                              reinterpret_cast<uint64_t>(&tmO)),
-                         "r"(smem_u32(sO) + buf * uint32_t(HALO_OUT_BYTES)), "r"(0), "r"(tm.pw0), "r"(tm.ph0), "r"(tm.pn0)
+                         "r"(stage), "r"(0), "r"(tm.pw0), "r"(tm.ph0), "r"(tm.pn0)
                          : "memory");
           }
           tma_store_commit();
         }
         continue;
       }
-      {
-        const int c = half;
+#pragma unroll 1
+      for (int h = 0; h < halves; ++h) {
+        const int c = half0 + h;
         uint32_t r[32];
         __syncwarp();
-        tmem_ld_32x32(tacc + (uint32_t(q * 32) << 16) + uint32_t(c * 32), r);
+        tmem_ld_32x32(tacc + uint32_t(c * 32), r);
         tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acce[buf]);
+        if (h == halves - 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acce[buf]);
+        }
 #pragma unroll
         for (int g = 0; g < 8; ++g)
           *reinterpret_cast<uint4*>(tile + lane * EPI_PITCH + g * 4) = make_uint4(r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
         __syncwarp();
-        const int n = c * 32 + sub_col;
-        epilogue_rows8<MODE>(p, tm, tile, q, sub_row, sub_col, n);
+        epilogue_rows8<MODE>(p, tm, tile, q, sub_row, sub_col, c * 32 + sub_col);
       }
     }
+    if (MODE != EPI_DGRAD_UNPOOL && chief) tma_store_wait_read0();   // shared memory must outlive the stores' reads
   }
-  if (MODE != EPI_DGRAD_UNPOOL && threadIdx.x == 64) tma_store_wait_read0();   // shared memory must outlive the stores' reads
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 2 * BN);
-    if (lane == 0) tmem_note_freed(TK_HALO, 2 * BN);
+    tmem_dealloc(tmem_base, HALO_ACC * BN);
+    if (lane == 0) tmem_note_freed(TK_HALO, HALO_ACC * BN);
   }
 }
 
@@ -387,7 +415,7 @@ constexpr int HALOG_PART_FLOATS = HALOG_GROUPS * GEMM_BM * 64;  // partial sums 
 template <int kInstance = 0>   // (a template only so that the header may be included by several translation units)
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD, const ConvGeom g,
-                   const int tiles_total, const int co0, const int cols, float* __restrict__ partial, int* __restrict__ status) {
+                   const int tiles_total, const int co0, float* __restrict__ partial, int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + HALOG_STAGES * HALOG_STAGE_BYTES);
@@ -448,7 +476,7 @@ conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = idesc_with_cols(make_idesc_bf16(GEMM_BM, 64, true, true), min(64, (cols + 15) & ~15));
+      constexpr uint32_t idesc = make_idesc_bf16(GEMM_BM, 64, true, true);      // (fewer columns for narrow layers gain nothing: the MMAs wait for A)
       // tap groups: first tap of the group as a halo row offset, and the distance to its partner
       const uint32_t first_row[HALOG_GROUPS] = {0u, 2u, uint32_t(HALO_W + 1), uint32_t(2 * HALO_W), uint32_t(2 * HALO_W + 2)};
       const uint32_t lbo[HALOG_GROUPS] = {128u, uint32_t((HALO_W - 2) * 128), 128u, 128u, 0u};

@@ -460,10 +460,12 @@ static cudaError_t configure_pair() {
   X(true, true, EPI_WGRAD_UPDATE)
 
 // ---- halo-tile convolution (3x3, at most 64 channels on both sides) ------------------------------
-#define LP_FOR_EACH_HALO_VARIANT(X) \
-  X(false, EPI_FPROP)               \
-  X(true, EPI_DGRAD)                \
-  X(true, EPI_DGRAD_UNPOOL)
+#define LP_FOR_EACH_HALO_FORM(X, B, M) \
+  X(B, M, 1, false) X(B, M, 2, false) X(B, M, 3, false) X(B, M, 4, false) X(B, M, 1, true) X(B, M, 2, true) X(B, M, 3, true) X(B, M, 4, true)
+#define LP_FOR_EACH_HALO_VARIANT(X)          \
+  LP_FOR_EACH_HALO_FORM(X, false, EPI_FPROP) \
+  LP_FOR_EACH_HALO_FORM(X, true, EPI_DGRAD)  \
+  LP_FOR_EACH_HALO_FORM(X, true, EPI_DGRAD_UNPOOL)
 
 cudaError_t conv_halo_launch(int which, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmO,
                              const GemmArgs& args, cudaStream_t st) {
@@ -472,9 +474,11 @@ cudaError_t conv_halo_launch(int which, const CUtensorMap& tmA, const CUtensorMa
                                                : args.g.tiles_w * args.g.tiles_h * (args.M / (args.g.H * args.g.W));
   const int grid = std::min(tiles, sm_count());
   note_form(args.g.kind == GEOM_PLAIN ? "halo plain" : "halo", 64);
-#define LP_TRYH(B, M)                                                                                          \
-  if (b_mn == B && args.mode == M)                                                                             \
-    return launch_chained(conv_halo_kernel<B, M>, grid, HALO_THREADS, HALO_SMEM_BYTES, st, 1, tmA, tmB, tmO, args, tiles);
+  // tiles in turn where a tile's MMAs are few: at most 32 output channels, or a single tap
+  const bool turns = args.N <= 32 || args.g.kind == GEOM_PLAIN;
+#define LP_TRYH(B, M, S, T)                                                                                    \
+  if (b_mn == B && args.mode == M && args.g.last_slices == S && turns == T)                                    \
+    return launch_chained(conv_halo_kernel<B, M, S, T>, grid, HALO_THREADS, HALO_SMEM_BYTES, st, 1, tmA, tmB, tmO, args, tiles);
   LP_FOR_EACH_HALO_VARIANT(LP_TRYH)
 #undef LP_TRYH
   return cudaErrorInvalidValue;
@@ -506,8 +510,7 @@ cudaError_t conv_halo_g_launch(const CUtensorMap& tmX, const CUtensorMap& tmD, c
   upd.n_ctas = grid;
   for (int co0 = 0; co0 < upd.n_out; co0 += 64) {      // one pass per 64 output channels; the stream orders the reuse of `partial`
     note_form("halo G", 64);
-    cudaError_t e = launch_chained(conv_halo_g_kernel<0>, grid, GEMM_THREADS, HALOG_SMEM_BYTES, st, 1, tmX, tmD, g, tiles, co0,
-                                   std::min(64, upd.n_out - co0), partial, status);
+    cudaError_t e = launch_chained(conv_halo_g_kernel<0>, grid, GEMM_THREADS, HALOG_SMEM_BYTES, st, 1, tmX, tmD, g, tiles, co0, partial, status);
     if (e != cudaSuccess) return e;
     upd.co0 = co0;
     e = launch_chained(conv_halo_g_update_kernel<0>, HALOG_PART_FLOATS / 32, 256, 0, st, 1, upd);
@@ -523,8 +526,8 @@ cudaError_t gemm_configure() {
     return e;
   if ((e = cudaFuncSetAttribute(conv_halo_g_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, HALOG_SMEM_BYTES)) != cudaSuccess)
     return e;
-#define LP_CFGH(B, M)                                                                                          \
-  if ((e = cudaFuncSetAttribute(conv_halo_kernel<B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
+#define LP_CFGH(B, M, S, T)                                                                                    \
+  if ((e = cudaFuncSetAttribute(conv_halo_kernel<B, M, S, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
                                 HALO_SMEM_BYTES)) != cudaSuccess)                                              \
     return e;
   LP_FOR_EACH_HALO_VARIANT(LP_CFGH)
