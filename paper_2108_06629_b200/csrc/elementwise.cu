@@ -543,13 +543,17 @@ cudaError_t launch_maxpool2(const __nv_bfloat16* a, __nv_bfloat16* pooled, unsig
 // block of a 64-column group (a counter that it leaves at zero) adds the chunks in a fixed order and applies the update.
 // Device time with cold caches, before (two-byte loads, a second launch for the chunk sums) and now: 802 816 x 128
 // 109 + 6 -> 41 us, 3 211 264 x 64 210 + 46 -> 75 us (5.5 TB/s), 2048 x 8192 17 + 4 -> 12 us.
-constexpr int COLSUM_LANES = 32;
+// Narrow matrices: G8 threads of eight columns to a row, as few as cover it, and 256 / G8 row lanes (16 columns read by eight threads
+// a row left six of them idle: 1 605 632 x 16 31 -> 18 us, 802 816 x 32 20 -> 17).
+template <int G8>
 __global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* __restrict__ x, int rows, int ld, int n_cols, int chunk_rows,
                                                           float* __restrict__ partial, unsigned* __restrict__ counter,
                                                           const BiasUpdate u) {
-  __shared__ __align__(16) float part[COLSUM_LANES][64 + 4];
+  constexpr int LANES = 256 / G8;                                  // row lanes
+  constexpr int COLS = 8 * G8, PITCH = COLS + 4;
+  __shared__ __align__(16) float part[LANES * PITCH > 16 * 68 ? LANES * PITCH : 16 * 68];
   __shared__ bool last;
-  const int g = threadIdx.x & 7, lane = threadIdx.x >> 3;
+  const int g = threadIdx.x % G8, lane = threadIdx.x / G8;
   const int col0 = blockIdx.x * 64;
   const int c8 = col0 + g * 8;
   const int r0 = blockIdx.y * chunk_rows, r1 = min(rows, r0 + chunk_rows);
@@ -566,30 +570,34 @@ __global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* _
         acc[2 * j + 1] += __uint_as_float(w[j] & 0xFFFF0000u);
       }
     };
-    for (; r + 3 * COLSUM_LANES < r1; r += 4 * COLSUM_LANES) {
+    for (; r + 3 * LANES < r1; r += 4 * LANES) {
       uint4 v[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const uint4*>(src + (long long)(r + k * COLSUM_LANES) * ld);
+      for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const uint4*>(src + (long long)(r + k * LANES) * ld);
 #pragma unroll
       for (int k = 0; k < 4; ++k) add(v[k]);
     }
-    for (; r < r1; r += COLSUM_LANES) add(*reinterpret_cast<const uint4*>(src + (long long)r * ld));
+    for (; r < r1; r += LANES) add(*reinterpret_cast<const uint4*>(src + (long long)r * ld));
   }
 #pragma unroll
-  for (int j = 0; j < 8; ++j) part[lane][g * 8 + j] = acc[j];
+  for (int j = 0; j < 8; ++j) part[lane * PITCH + g * 8 + j] = acc[j];
   __syncthreads();
   launch_next();
-  const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;          // four threads a column, eight row lanes each
+  constexpr int PER = 256 / COLS;                                  // threads a column, each with its share of the row lanes
+  const int tx = threadIdx.x % COLS, ty = threadIdx.x / COLS;
   float s = 0.f;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) s += part[ty * 8 + k][tx];
+  for (int k = 0; k < LANES / PER; ++k) s += part[(ty * (LANES / PER) + k) * PITCH + tx];
   __syncthreads();
-  part[ty][tx] = s;
+  part[ty * PITCH + tx] = s;
   __syncthreads();
   const int n_chunks = gridDim.y;
   float* mine = partial + (long long)blockIdx.x * n_chunks * 64;   // [chunk][64]
   if (ty == 0) {
-    __stcg(mine + blockIdx.y * 64 + tx, part[0][tx] + part[1][tx] + part[2][tx] + part[3][tx]);
+    float t = part[tx];
+#pragma unroll
+    for (int k = 1; k < PER; ++k) t += part[k * PITCH + tx];
+    __stcg(mine + blockIdx.y * 64 + tx, t);
     __threadfence();
   }
   __syncthreads();
@@ -606,13 +614,13 @@ __global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* _
     t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
   }
   __syncthreads();
-  *reinterpret_cast<float4*>(&part[l16][q]) = t;
+  *reinterpret_cast<float4*>(&part[l16 * 68 + q]) = t;
   __syncthreads();
   const int col = col0 + threadIdx.x;
   if (threadIdx.x < 64 && col < n_cols) {
     float grad = 0.f;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) grad += part[k][threadIdx.x];
+    for (int k = 0; k < 16; ++k) grad += part[k * 68 + threadIdx.x];
     u.db[col] = grad;
     float m = grad;
     if (u.mb != nullptr) {
@@ -628,7 +636,8 @@ cudaError_t launch_colsum_bias(const __nv_bfloat16* x, int rows, int ld, int n_c
                                const BiasUpdate& u, cudaStream_t stream) {
   const int chunk = colsum_chunk_rows(rows, n_cols);
   dim3 grid((n_cols + 63) / 64, (rows + chunk - 1) / chunk);
-  return launch_chained(colsum_bias_kernel, grid, 256, 0, stream, 1, x, rows, ld, n_cols, chunk, partial, counter, u);
+  auto* kernel = ld <= 8 ? colsum_bias_kernel<1> : ld <= 16 ? colsum_bias_kernel<2> : ld <= 32 ? colsum_bias_kernel<4> : colsum_bias_kernel<8>;
+  return launch_chained(kernel, grid, 256, 0, stream, 1, x, rows, ld, n_cols, chunk, partial, counter, u);
 }
 }  // namespace lp
 
