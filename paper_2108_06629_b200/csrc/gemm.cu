@@ -163,9 +163,11 @@ int gemm_pick_splits(int M, int N, int K, int bn) {
   // 392 k-blocks, one CTA streaming 6.4 MB of weights each): 145 us unsplit, 95 / 74 / 89 us at
   // 2 / 4 / 8 splits.
   const long long tiles = (long long)((M + GEMM_BM - 1) / GEMM_BM) * ((N + bn - 1) / bn);
-  // Fewer tiles with longer contractions take more splits: about one CTA per SM, never fewer than 64 k-blocks per
-  // split (a single 10-column tile over 100352 inputs, the classifier behind an unpooled 28 x 28 x 128 image: 24 splits).
-  const int automatic = (tiles <= 48 && num_kb >= 256) ? int(std::max<long long>(1, std::min<long long>(std::min<long long>(kSMs / tiles, num_kb / 64), 64))) : 1;
+  // Fewer tiles with longer contractions take more splits: about one CTA per SM, never fewer than 16 k-blocks per
+  // split (a single 10-column tile over 100352 inputs, the classifier behind an unpooled 28 x 28 x 128 image: 24 splits
+  // added by the last CTA of the tile 37 us, 98 added by a launch on all SMs 15; 64 x 300 x 24576 40 -> 15; at
+  // least 32 k-blocks a split, or two CTAs per SM, are no better).
+  const int automatic = (tiles <= 48 && num_kb >= 256) ? int(std::max<long long>(1, std::min<long long>(kSMs / tiles, num_kb / 16))) : 1;
   int s = g_force_splits > 0 ? g_force_splits : automatic;
   s = std::max(1, std::min(s, num_kb));
   const int per = (num_kb + s - 1) / s;
@@ -180,7 +182,7 @@ int gemm_pick_splits(int M, int N, int K, int bn) {
 //   (32 x 256 x 256, one each: 4.5; undivided 5.6) -- or two per SM if each keeps 16 k-blocks (1000^3 on 128 tiles:
 //   undivided 11.0, halves 11.9; 64 x 4096 x 4096 on 64 tiles 14.7 in quarters, 16.6 in halves, undivided 27.6);
 // * eight for a handful of tiles with a long contraction (128 x 512 x 4096: 8.1, in quarters 9.8, undivided 24.9).
-int gemm_pick_cluster(int M, int N, int K, int* bn) {
+int gemm_pick_cluster(int M, int N, int K, int* bn, bool can_split) {
   if (g_force_bn != 0 || g_force_stages != 0 || g_force_splits != 0 || g_force_persistent >= 0) return 0;
   const long long rows = (M + GEMM_BM - 1) / GEMM_BM;
   const int width = rows * ((N + 63) / 64) <= sm_count() ? 64 : 128;
@@ -192,7 +194,7 @@ int gemm_pick_cluster(int M, int N, int K, int* bn) {
   const int c = (num_kb >= 64 && tiles * 8 <= sm_count()) ? 8 : fits(4) ? 4 : fits(2) ? 2 : 0;
   // (one tile over a hundred thousand terms: the split through global memory, which a layer has and lp_gemm_bf16 has not,
   // spreads it wider than a cluster can)
-  if (c == 0 || gemm_pick_splits(M, N, K, width) > 2 * c) return 0;
+  if (c == 0 || (can_split && gemm_pick_splits(M, N, K, width) > 2 * c)) return 0;
   *bn = width;
   return c;
 }
@@ -231,8 +233,7 @@ void gemm_box_dims(int which, int bn, uint32_t boxA[2], uint32_t boxB[2]) {
 }
 
 
-// Which contractions exist in a form split over k: forward and delta of a layer (the last CTA of a tile adds), and G of a
-// convolution (a launch of its own adds).
+// Which contractions exist in a form split over k: forward and delta of a layer, and G of a convolution.
 template <int BN, bool A_MN, int MODE>
 constexpr bool kHasSplit = A_MN ? BN <= 128 : MODE != EPI_STORE_F32;
 
@@ -289,14 +290,11 @@ static cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, Ge
   if constexpr (kHasSplit<BN, A_MN, MODE>) {
     if (a.splits > 1) {
       const cudaError_t e = a.persistent ? LP_LAUNCH(true, true) : LP_LAUNCH(true, false);
-      if constexpr (A_MN) {
-        if (e != cudaSuccess) return e;
-        constexpr int blocks = GEMM_BM * (BN / 4) / 256;      // per tile with one lane
-        const int tiles = tiles_m * tiles_n;
-        if (a.splits >= 16) return launch_chained(gemm_split_finish_kernel<BN, MODE, 8>, tiles * blocks * 8, 256, 0, st, 1, a, tiles_m, tiles_n);
-        return launch_chained(gemm_split_finish_kernel<BN, MODE, 1>, tiles * blocks, 256, 0, st, 1, a, tiles_m, tiles_n);
-      }
-      return e;
+      if (e != cudaSuccess) return e;
+      constexpr int blocks = GEMM_BM * (BN / 4) / 256;      // per tile with one lane
+      const int tiles = tiles_m * tiles_n;
+      if (a.splits >= 16) return launch_chained(gemm_split_finish_kernel<BN, MODE, 8>, tiles * blocks * 8, 256, 0, st, 1, a, tiles_m, tiles_n);
+      return launch_chained(gemm_split_finish_kernel<BN, MODE, 1>, tiles * blocks, 256, 0, st, 1, a, tiles_m, tiles_n);
     }
   }
   return a.persistent ? LP_LAUNCH(false, true) : LP_LAUNCH(false, false);
@@ -647,7 +645,7 @@ int gemm_standalone(int which, int M, int N, int K, const void* A, int lda, cons
   int rc = gemm_device_setup(&status_dev);
   if (rc != LP_OK) return rc;
   int bn = gemm_pick_bn(which, M, N, K);
-  const int cluster = gemm_is_pair(bn) ? 0 : gemm_pick_cluster(M, N, K, &bn);
+  const int cluster = gemm_is_pair(bn) ? 0 : gemm_pick_cluster(M, N, K, &bn, false);
   uint32_t boxA[2], boxB[2];
   gemm_box_dims(which, bn, boxA, boxB);
   CUtensorMap tmA, tmB;

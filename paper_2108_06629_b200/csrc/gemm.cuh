@@ -108,14 +108,11 @@ struct GemmArgs {
   // the (first) maximum of every window, and the activation itself goes nowhere.  Needs pixel boxes at most 16
   // wide, so that a window lies inside the 32 rows of one epilogue warp.
   unsigned char* pool_out_idx;
-  // split-K (splits > 1): blockIdx.z owns k-blocks [z*kb_per_split, (z+1)*kb_per_split); every CTA
-  // writes its fp32 partial tile to `partial`, the last CTA of a tile to arrive (tile_counter)
-  // adds the partials in split order -- a fixed order, so results do not depend on timing --
-  // and runs the epilogue.  In the G contraction (A_MN), which has many splits, the sum and the epilogue are a
-  // launch of their own on all SMs (gemm_split_finish_kernel).
+  // split-K (splits > 1): a work item owns k-blocks [z*kb_per_split, (z+1)*kb_per_split) of a tile and
+  // writes its fp32 partial tile to `partial`; a second launch on all SMs (gemm_split_finish_kernel) adds the partials in
+  // a fixed order, so results do not depend on timing, and runs the epilogue.
   int splits, kb_per_split;
   float* partial;           // [tiles][splits][128][BN]
-  unsigned* tile_counter;   // [tiles], zero between launches (not in the G contraction)
   int cluster;              // 2, 4 or 8: one tile per cluster of that many CTAs, which divide the contraction (gemmc.cuh); 0: other forms
   ConvGeom g;
   int persistent;           // CTAs loop over tiles (grid sized to the machine) instead of one tile each
@@ -1073,51 +1070,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           epilogue_rows8<MODE>(p, tm, tile, q, sub_row, sub_col, n);
         }
       }
-      if constexpr (split && !A_MN) {
-        // all four epilogue warps have written their part of the partial tile: publish it, and
-        // let the last CTA of this tile reduce the partials in split order
-        volatile uint32_t* is_last = tmem_slot + 1;
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (threadIdx.x == 64) {
-          __threadfence();
-          const unsigned prev = atomicAdd(p.tile_counter + tc.tile_id, 1u);
-          const bool last = (prev == unsigned(p.splits) - 1u);
-          if (last) p.tile_counter[tc.tile_id] = 0u;          // ready for the next launch
-          *is_last = last ? 1u : 0u;
-          __threadfence();
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (*is_last != 0u) {
-          const float* base = p.partial + size_t(tc.tile_id) * p.splits * (size_t(GEMM_BM) * BN);
-          const size_t zstride = size_t(GEMM_BM) * BN;
-#pragma unroll 1
-          for (int c = 0; c < BN / 32; ++c) {
-            const int n = tm.n0 + c * 32 + sub_col;
-            // eight independent rows per lane: their loads are issued together for every split,
-            // the additions keep split order
-            float4 acc[8];
-#pragma unroll
-            for (int i8 = 0; i8 < 8; ++i8)
-              acc[i8] = __ldcg(reinterpret_cast<const float4*>(base + size_t(q * 32 + i8 * 4 + sub_row) * BN + c * 32 + sub_col));
-            for (int z = 1; z < p.splits; ++z) {
-              float4 tt[8];
-#pragma unroll
-              for (int i8 = 0; i8 < 8; ++i8)
-                tt[i8] = __ldcg(reinterpret_cast<const float4*>(base + z * zstride + size_t(q * 32 + i8 * 4 + sub_row) * BN + c * 32 + sub_col));
-#pragma unroll
-              for (int i8 = 0; i8 < 8; ++i8) {
-                acc[i8].x += tt[i8].x; acc[i8].y += tt[i8].y; acc[i8].z += tt[i8].z; acc[i8].w += tt[i8].w;
-              }
-            }
-#pragma unroll
-            for (int i8 = 0; i8 < 8; ++i8) {
-              const int row = tile_row(p, tm, q * 32 + i8 * 4 + sub_row);
-              if (row >= 0) epilogue_store4<MODE>(p, row, n, tm.nlim, acc[i8]);
-            }
-          }
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");     // is_last is rewritten by the next tile
-      }
     }
     if constexpr (kUpdTmaOk) {
       if (pending) {                       // (thread 64 only) shared memory must outlive the last stores' reads
@@ -1135,7 +1087,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   }
 }
 
-// Second launch of a split G contraction: adds the partial tiles and runs the epilogue.  A thread owns four
+// Second launch of a split contraction: adds the partial tiles and runs the epilogue.  A thread owns four
 // consecutive columns of a tile row; with LANES > 1 (many splits of few tiles) LANES threads share them, lane j
 // adding splits j, j + LANES, ... in order and the lane sums following in order.  Reads splits x tile from L2 once.
 template <int BN, int MODE, int LANES>

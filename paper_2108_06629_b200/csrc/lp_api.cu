@@ -88,7 +88,7 @@ struct Layer {
   float* part_g = nullptr;
   bool pool_fused = false;           // the forward epilogue pools (no a_full)
   Res rAfull;
-  Res rPartF, rPartD;               // split-K partial tiles and arrival counters of the forward / delta contraction
+  Res rPartF, rPartD;               // split-K partial tiles of the forward / delta contraction
   // device memory (all inside the workspace)
   float *W = nullptr, *mW = nullptr, *b = nullptr, *mb = nullptr, *dW = nullptr, *db = nullptr, *bring = nullptr;
   __nv_bfloat16 *ring = nullptr, *X = nullptr, *Z = nullptr, *delta = nullptr;
@@ -98,7 +98,6 @@ struct Layer {
   int cl_f = 0, cl_d = 0;                       // CTAs of a cluster that share a tile of the forward / delta contraction
   int split_f = 1, split_d = 1;                 // split-K factors of the forward / delta contractions
   float *part_f = nullptr, *part_d = nullptr;   // fp32 partial tiles [tiles][splits][128][BN]
-  unsigned *cnt_f = nullptr, *cnt_d = nullptr;  // per-tile arrival counters
   std::vector<CUtensorMap> tm_f_A, tm_f_B, tm_d_A, tm_d_B, tm_g_A, tm_g_B;
   // 3x3 layers with at most 64 channels on both sides and images tiled by 8 x 16 pixels: the
   // activation / delta box is fetched once per tile with its halo (see conv_halo.cuh)
@@ -361,12 +360,10 @@ static size_t carve(lp_ctx* c, char* base) {
     if (y.split_f > 1) {
       const size_t t = tiles_of(B, y.n_out, y.bn_f);
       y.part_f = reinterpret_cast<float*>(take(t * y.split_f * GEMM_BM * y.bn_f * 4));
-      y.cnt_f = reinterpret_cast<unsigned*>(take(t * 4));
     }
     if (y.split_d > 1 && l > 0) {
       const size_t t = tiles_of(B, y.n_in, y.bn_d);
       y.part_d = reinterpret_cast<float*>(take(t * y.split_d * GEMM_BM * y.bn_d * 4));
-      y.cnt_d = reinterpret_cast<unsigned*>(take(t * 4));
     }
     if (y.halo_g) {
       y.part_g = reinterpret_cast<float*>(take(size_t(conv_halo_g_max_ctas()) * HALOG_PART_FLOATS * 4));
@@ -396,8 +393,8 @@ static void pick_fc_tiles(Layer* y, int B, bool allow_pair) {
   // 289 / 280, 3072 357 / 378, 4096 565 / 623; batch 64, 2048 218 / 156, 3072 341 / 291, 4096 520 / 529.  So the line, at
   // 2048 x 2048, is on the safe side of where clusters begin to cost, which lies between 2560 and 4096 with the batch.
   const bool chain_bound = (long long)y->n_in * y->n_out <= (1ll << 22);
-  y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f) : 0;
-  y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d) : 0;
+  y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f, true) : 0;
+  y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d, true) : 0;
   y->split_f = gemm_is_pair(y->bn_f) || y->cl_f > 0 ? 1 : gemm_pick_splits(B, y->n_out, y->n_in, y->bn_f);
   y->split_d = gemm_is_pair(y->bn_d) || y->cl_d > 0 ? 1 : gemm_pick_splits(B, y->n_in, y->n_out, y->bn_d);
 }
@@ -495,7 +492,11 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       const int tiles = ((y.n_out + GEMM_BM - 1) / GEMM_BM) * y.taps * ((y.ld_in + y.bn_g - 1) / y.bn_g);
       const int num_kb = y.out_rows / GEMM_BK;
       const int s_opt = int(std::lround(std::sqrt(double(num_kb) * (y.bn_g <= 64 ? 0.6 : 0.3))));
-      y.split_g = std::max(1, std::min(std::min(2 * kSMs / std::max(tiles, 1), s_opt), y.patch ? kSMs : 64));
+      // A patch layer is a single tile or two, so its splits are all the SMs it gets: one CTA on each, of at least 32 k-blocks
+      // (the 5x5 patch layer of the sample network, 43 -> 148 splits, 66 -> 45 us; two CTAs on each: 88 -> 98 us at 16
+      // channels of 224 x 224, batch 32).
+      y.split_g = y.patch ? std::min(kSMs / std::max(tiles, 1), num_kb / 32) : std::min(std::min(2 * kSMs / std::max(tiles, 1), s_opt), 64);
+      y.split_g = std::max(1, y.split_g);
       const int per = (num_kb + y.split_g - 1) / y.split_g;
       y.split_g = (num_kb + per - 1) / per;
     } else {
@@ -875,9 +876,9 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
       a.ld_out2 = y.ld_out;
     }
   }
-  a.splits = y.split_f; a.partial = y.part_f; a.tile_counter = y.cnt_f;
+  a.splits = y.split_f; a.partial = y.part_f;
   a.cluster = y.cl_f;
-  ++c->launches;
+  c->launches += y.split_f > 1 ? 2 : 1;
   TimedScope ts(c, LP_TASK_FORWARD, st, l);
   if (y.lean_f) {
     a.g.last_slices = last_slices(y.n_in);      // (plain geometry otherwise)
@@ -952,9 +953,9 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
   a.status = c->status;
   a.tmem_policy = c->tmem_policy;
   a.phase = c->trace_done ? c->status + 8 : nullptr;
-  a.splits = y.split_d; a.partial = y.part_d; a.tile_counter = y.cnt_d;
+  a.splits = y.split_d; a.partial = y.part_d;
   a.cluster = y.cl_d;
-  ++c->launches;
+  c->launches += y.split_d > 1 ? 2 : 1;
   TimedScope ts(c, LP_TASK_DELTA, st, l);
   if (y.halo_d) {
     a.g = halo_geom(y, 1);
