@@ -406,7 +406,9 @@ def test_tasks_sm_pair_persistent_g_update():
         lpb.lp_set_tuning(0, 0, 0)
 
 
-@pytest.mark.parametrize("rows, n_out", [(513, 8), (545, 72), (1000, 130), (2049, 64), (70000, 10), (4133, 1000)])
+@pytest.mark.parametrize("rows, n_out", [(513, 8), (545, 72), (1000, 130), (2049, 64), (70000, 10), (4133, 1000),
+                                         # one, two and four threads a row, and the first width of eight
+                                         (70001, 8), (5000, 16), (90000, 24), (4097, 32), (2050, 40)])
 def test_tasks_bias_gradient_of_many_rows(rows, n_out):
     """Column sums over chunks of rows (ragged chunks, columns past a 64-column group, one chunk and many) and the bias
     update, twice in a row, against float64: fp32 sums of `rows` bf16 values, |error| <= sqrt(rows) ulps of the rms sum."""
@@ -481,3 +483,27 @@ def test_tasks_two_halo_tiles_by_the_automatic_rule(monkeypatch):
     layers = [I.conv(3, 72, 80, 120), I.conv(72, 136, 80, 120), I.conv(136, 72, 80, 120, pool=2), I.fc(72 * 40 * 60, 10, "none")]
     run_teacher_forced(layers, 8, 2, None, 0.05, 0.0, 1)
     assert _wide_layers(forms, "forward") == [1] and _wide_layers(forms, "delta") == [2], forms
+
+
+# narrow: channel counts on both sides of each number of 16-channel slices and of the line between warps that take tiles in turn and
+# warps that share them; one tile per CTA, an odd number of tiles, more than a round; pooled, un-pooling, patch-matrix first layer
+@pytest.mark.parametrize("H, W, B, chans, pools", [
+    (16, 8, 16, [8, 16, 24, 32], [0, 0, 0, 0]), (32, 16, 2, [40, 8, 56, 16], [0, 0, 0, 0]), (16, 24, 5, [32, 64, 40, 24], [0, 0, 0, 0]),
+    (32, 32, 40, [16, 32, 48, 8], [0, 2, 0, 0]), (48, 40, 16, [24, 24, 64], [0, 0, 2])])
+def test_tasks_halo_tiles_of_narrow_layers(H, W, B, chans, pools):
+    from paper_2108_06629_b200 import inputs as I
+    layers, c = [], 3
+    for n, pool in zip(chans, pools):
+        layers.append(I.conv(c, n, H, W, pool=pool))
+        c = n
+        if pool:
+            H, W = H // 2, W // 2
+    layers.append(I.fc(c * H * W, 10, "none"))
+    run_teacher_forced(layers, B, 2, None, 0.05, 0.9, 1)
+
+
+@pytest.mark.parametrize("n_in, n_out, batch", [(17000, 10, 5), (16390, 130, 3), (20000, 300, 130)])
+def test_tasks_long_contractions_split_over_all_sms(n_in, n_out, batch):
+    """One to six tiles of 256 k-blocks and more, the last split shorter than the others: sum and epilogue in a second launch."""
+    from paper_2108_06629_b200 import inputs as I
+    run_teacher_forced([I.fc(24, n_in), I.fc(n_in, n_out, "gelu"), I.fc(n_out, 6, "none")], batch, 2, None, 0.01, 0.0, 1)
