@@ -110,8 +110,8 @@ cudaError_t gemm_configure();   // opt in to large dynamic shared memory; call o
 void gemm_set_tuning(int bn, int stages, int splits);   // 0 = automatic
 int gemm_pick_splits(int M, int N, int K, int bn);
 // CTAs of a cluster that share one tile's contraction (GemmArgs::cluster) and, where that is not 0, the tile width
-// (can_split: the caller has scratch for a contraction split through global memory, which may then be the better one)
-int gemm_pick_cluster(int M, int N, int K, int* bn, bool can_split);
+// (layer: the epilogue is that of a layer, and there is scratch for a contraction split through global memory, which may be the better one)
+int gemm_pick_cluster(int M, int N, int K, int* bn, bool layer);
 
 // ---- planner.cpp ------------------------------------------------------------
 struct PlanResult {

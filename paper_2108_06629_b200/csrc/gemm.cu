@@ -175,26 +175,38 @@ int gemm_pick_splits(int M, int N, int K, int bn) {
 }
 
 // Outputs of few tiles: one tile per cluster, the contraction divided over its CTAs (gemmc.cuh).  Sets the tile width and
-// returns the cluster size, or 0 where another form is the better one.  Rule, each side measured alone on the GPU (us):
+// returns the cluster size (1: undivided, in that kernel's form), or 0 where another form is the better one.  Rule, each side
+// measured on calls that follow one another in a stream (us):
 // * 64-column tiles while they fit one CTA on every SM (100 x 777 x 1003 6.1 against 7.3 with 128 columns, 700^3 6.9 / 7.9,
 //   512 x 2048 x 2048 12.7 / 13.3; beyond that 128: 512 x 4096 x 4096 24.5 / 25.7);
-// * four CTAs to a tile, else two, while that is at most one CTA per SM -- a few k-blocks each are enough
-//   (32 x 256 x 256, one each: 4.5; undivided 5.6) -- or two per SM if each keeps 16 k-blocks (1000^3 on 128 tiles:
-//   undivided 11.0, halves 11.9; 64 x 4096 x 4096 on 64 tiles 14.7 in quarters, 16.6 in halves, undivided 27.6);
-// * eight for a handful of tiles with a long contraction (128 x 512 x 4096: 8.1, in quarters 9.8, undivided 24.9).
-int gemm_pick_cluster(int M, int N, int K, int* bn, bool can_split) {
+// * up to four k-blocks of such a tile undivided: a barrier and a pass through distributed shared memory cost what
+//   they save (128 x 256 x 256 one CTA a tile 4.6, two 4.9, four 4.8; 128 x 256 x 128 4.1, two 4.6) -- but not in a layer, whose
+//   epilogue gains by the division (16 steps of the ragged GELU MLP 620, undivided 640);
+// * else eight CTAs to a tile for a handful of tiles (128 x 64 x 1500 5.6, in quarters 6.2; 128 x 800 x 3000 on 13 tiles 7.5 / 8.3, but
+//   x 784 6.1 / 5.7), four, or two, while that is at most one CTA per SM (128 x 2048 x 784 four 6.1, two 6.6, undivided 7.8);
+// * undivided where the tiles leave no room for that, up to 64 k-blocks (1000 x 800 x 784 7.9, two 8.3, 128-column tiles
+//   13.5; x 1500 10.9 / 10.3 / 14.1; x 3000 18.9 / 20.7);
+// * beyond, two CTAs per SM if each keeps 16 k-blocks (64 x 4096 x 4096 on 64 tiles: 14.7 in quarters, 16.6 in halves,
+//   undivided 27.6).
+int gemm_pick_cluster(int M, int N, int K, int* bn, bool layer) {
   if (g_force_bn != 0 || g_force_stages != 0 || g_force_splits != 0 || g_force_persistent >= 0) return 0;
   const long long rows = (M + GEMM_BM - 1) / GEMM_BM;
   const int width = rows * ((N + 63) / 64) <= sm_count() ? 64 : 128;
   const long long tiles = rows * ((N + width - 1) / width);
   const int num_kb = (K + GEMM_BK - 1) / GEMM_BK;
-  auto fits = [&](int c) {
-    return num_kb >= c && (tiles * c <= sm_count() || (tiles * c <= 2 * sm_count() && num_kb >= 16 * c));
-  };
-  const int c = (num_kb >= 64 && tiles * 8 <= sm_count()) ? 8 : fits(4) ? 4 : fits(2) ? 2 : 0;
+  auto one_each = [&](int c) { return num_kb >= c && tiles * c <= sm_count(); };
+  auto two_each = [&](int c) { return tiles * c <= 2 * sm_count() && num_kb >= 16 * c; };
+  int c = 0;
+  if (width == 64 && num_kb <= 4 && !layer) c = 1;
+  else if ((num_kb >= 16 && tiles <= 8) || (num_kb >= 40 && one_each(8))) c = 8;
+  else if (one_each(4)) c = 4;
+  else if (one_each(2)) c = 2;
+  else if (width == 64 && num_kb <= 64) c = 1;
+  else if (two_each(4)) c = 4;
+  else if (two_each(2)) c = 2;
   // (one tile over a hundred thousand terms: the split through global memory, which a layer has and lp_gemm_bf16 has not,
   // spreads it wider than a cluster can)
-  if (c == 0 || (can_split && gemm_pick_splits(M, N, K, width) > 2 * c)) return 0;
+  if (c == 0 || (layer && gemm_pick_splits(M, N, K, width) > 2 * c)) return 0;
   *bn = width;
   return c;
 }
@@ -338,7 +350,8 @@ static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB
   if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
   const int tiles_m = (a.M + GEMM_BM - 1) / GEMM_BM, tiles_n = (a.N - a.n_begin + BN - 1) / BN;
   note_form("cluster", BN, a.cluster);
-  return launch_chained(gemmc_kernel<BN, A_MN, B_MN, MODE>, dim3(a.cluster, tiles_m * tiles_n), GEMM_THREADS, gemmc_smem_bytes(BN), st, a.cluster,
+  if (a.cluster == 1 && BN != 64) return cudaErrorInvalidValue;
+  return launch_chained(a.cluster == 1 ? gemmc_kernel<64, A_MN, B_MN, MODE, true> : gemmc_kernel<BN, A_MN, B_MN, MODE, false>, dim3(a.cluster, tiles_m * tiles_n), GEMM_THREADS, gemmc_smem_bytes(BN), st, a.cluster,
                         tmA, tmB, a, tiles_m);
 }
 #define LP_FOR_EACH_CLUSTER_VARIANT(X, BN) \
@@ -541,8 +554,10 @@ cudaError_t gemm_configure() {
   LP_FOR_EACH_PAIR_VARIANT(LP_CFGP)
 #undef LP_CFGP
 #define LP_CFGC(BN, A, B, M)                                                                                   \
-  if ((e = cudaFuncSetAttribute(gemmc_kernel<BN, A, B, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
-                                gemmc_smem_bytes(BN))) != cudaSuccess)                                         \
+  if ((e = cudaFuncSetAttribute(gemmc_kernel<BN, A, B, M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                gemmc_smem_bytes(BN))) != cudaSuccess ||                                       \
+      (BN == 64 && (e = cudaFuncSetAttribute(gemmc_kernel<64, A, B, M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                             gemmc_smem_bytes(64))) != cudaSuccess))                           \
     return e;
   LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 64)
   LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 128)

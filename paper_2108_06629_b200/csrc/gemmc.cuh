@@ -7,7 +7,8 @@
 // tiles of ITS share of the elements through distributed shared memory, in rank order -- a fixed order, so results
 // do not depend on timing -- and runs the epilogue on them.  The chain of k-blocks and the epilogue both
 // shrink by C, nothing goes through global memory (the split-K form of gemm.cuh writes and re-reads its partial tiles there and
-// leaves the whole sum and epilogue to the last CTA).
+// leaves the sum and the epilogue to a second launch).  A cluster of one is the same without the sum: 64-column tiles and all
+// six warps in the epilogue (32 x 256 x 10 5.1 -> 3.1 us, 1000 x 900 x 1000 13.5 -> 9.3 against the 128-column form of gemm.cuh).
 #pragma once
 #include "gemm2.cuh"
 
@@ -72,7 +73,8 @@ __device__ __forceinline__ void gemmc_reduce_store(const GemmArgs& p, const Tile
   }
 }
 
-template <int BN, bool A_MN, bool B_MN, int MODE>
+// ONE: a cluster of one (a kernel of its own: one more case in the switch at the end slowed the others, the ragged GELU MLP 627 -> 637 us)
+template <int BN, bool A_MN, bool B_MN, int MODE, bool ONE>
 __global__ void __launch_bounds__(GEMM_THREADS, 2)
 gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs p, const int tiles_m) {
   static_assert(MODE != EPI_WGRAD_UPDATE, "the update has tiles enough");
@@ -88,7 +90,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  const int C = p.cluster;
+  const int C = ONE ? 1 : p.cluster;
   TileMap tm;
   tm.m0 = (int(blockIdx.y) % tiles_m) * GEMM_BM;
   tm.n0 = p.n_begin + (int(blockIdx.y) / tiles_m) * BN;
@@ -224,6 +226,10 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     if (lane == 0) tmem_note_freed(TK_GEMM, BN);
   }
   const uint32_t part = smem_u32(smem);
+  if constexpr (ONE) {
+    gemmc_reduce_store<BN, MODE, 1>(p, tm, part, rank);
+    return;
+  }
   switch (C) {
     case 2: gemmc_reduce_store<BN, MODE, 2>(p, tm, part, rank); break;
     case 4: gemmc_reduce_store<BN, MODE, 4>(p, tm, part, rank); break;

@@ -222,3 +222,22 @@ def test_kernels_of_a_stream_see_what_the_one_before_wrote(B, n, classes):
     graph.replay()
     torch.cuda.synchronize()
     assert all(torch.equal(p, q) for p, q in zip(want, got))
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_undivided_contraction_in_the_cluster_form(which):
+    """A cluster of one: one to four k-blocks with ragged ends, one element, ragged tiles, the most tiles, and long contractions
+    of tiles that fill the SMs by themselves."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    for i, (M, N, K) in enumerate([(1, 1, 1), (33, 70, 10), (129, 65, 250), (513, 1000, 256), (128, 9400, 60), (800, 1300, 700), (1000, 1000, 2100)]):
+        A, B = _operands(which, M, N, K, 3000 + 100 * which + i)
+        ldc = (N + 3) // 4 * 4
+        Cd = torch.full((M, ldc), 7.0, device="cuda")
+        lpb.lp_gemm_bf16(which, M, N, K, A.cuda(), A.shape[1], B.cuda(), B.shape[1], Cd, ldc)
+        assert lpb.lp_debug_last_contraction() == "cluster 64 x1", (M, N, K)
+        torch.cuda.synchronize()
+        got = Cd.cpu().numpy()
+        assert rel_l2(got[:, :N], _reference(which, M, N, K, A, B)) < 1e-6 + 2e-7 * np.sqrt(K), (which, M, N, K)
+        assert np.all(got[:, N:] == 0.0)
+    assert lpb.lp_gemm_status() == (lpb.LP_OK, 0)
