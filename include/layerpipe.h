@@ -135,10 +135,8 @@ int lp_workspace_size(const lp_layer* layers, int n_layers, int n_stages, const 
  * is smaller than eight (LP_STREAM_TRIPLES in the environment limits each kind further).
  * Kernel selection: a handle uses one kind of tensor-memory allocation -- a fully connected network
  * whose layers are mostly wide (batch, inputs and outputs all >= 1024) runs every contraction on SM
- * pairs (tcgen05 cta_group::2), every other network runs single-CTA kernels only.  LP_CONV_PAIR=1
- * in the environment also puts wide convolution layers on SM pairs: a measurement mode, not for
- * long runs (networks that alternate the two kinds on the same SMs have stalled in tcgen05.alloc
- * after some 10^6 pair CTAs).  LP_CONV_WIDE_ITEMS=n in the environment lets the two-tile convolution
+ * pairs (tcgen05 cta_group::2), every other network runs single-CTA kernels only (networks that alternate the two
+ * kinds on the same SMs have stalled in tcgen05.alloc after some 10^6 pair CTAs).  LP_CONV_WIDE_ITEMS=n in the environment lets the two-tile convolution
  * kernel of more than 64 channels start at n items a launch instead of 592 (verification).  Two handles of different kinds should not run concurrently on one GPU.
  */
 int lp_create(lp_handle* out, const lp_layer* layers, int n_layers, int n_stages,

@@ -212,8 +212,8 @@ int gemm_pick_cluster(int M, int N, int K, int* bn, bool layer) {
 }
 
 int gemm_pick_bn(int which, int M, int N, int K, bool allow_pair) {
-  if (g_force_bn == 64 || g_force_bn == 128 || g_force_bn == 256 || g_force_bn == GEMM_BN_PAIR) return g_force_bn;
-  if (g_force_bn == GEMM_BN_PAIR224) return which == 2 ? GEMM_BN_PAIR : GEMM_BN_PAIR224;
+  if (g_force_bn == 64 || g_force_bn == 128 || g_force_bn == 256) return g_force_bn;
+  if (allow_pair && gemm_is_pair(g_force_bn)) return which == 2 ? GEMM_BN_PAIR : g_force_bn;
   if (N <= 64) return 64;
   // tensor-bound shapes: 256 x 256 tiles on SM pairs (code GEMM_BN_PAIR)
   if (allow_pair && M >= 1024 && N >= 1024 && K >= 1024) {
@@ -368,26 +368,23 @@ static cudaError_t launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, G
   a.splits = 1;
   if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
   static const UpdMaps no_maps{};
-  a.upd_tma = (MODE == EPI_WGRAD_UPDATE && um != nullptr && a.g.kind == GEOM_PLAIN) ? 1 : 0;
+  a.upd_tma = (MODE == EPI_WGRAD_UPDATE && um != nullptr) ? 1 : 0;
   if (!a.upd_tma) um = &no_maps;
   const int stage_bytes = 32 * 1024;
   const int num_kb = (a.K + GEMM_BK - 1) / GEMM_BK;
   // 3 x 32 KiB: two CTAs per SM, one's epilogue under the other's main loop; 6 where a CTA has its SM to itself anyway,
   // the launch having no more tiles than there are SM pairs (1024 x 4096 x 4096: 37.2 -> 29.1 us)
   const long long all_tiles = (long long)((a.M + 255) / 256) * ((a.N - a.n_begin + BN2 - 1) / BN2);
-  const bool alone = a.tmem_policy == TMEM_PAIR_ALONE || all_tiles <= std::max(1, sm_count() / 2);
+  const bool alone = all_tiles <= std::max(1, sm_count() / 2);
   int s = g_force_stages > 0 ? g_force_stages : (alone ? 6 : 3);
   s = std::max(2, std::min(std::min(s, GEMM_MAX_STAGES), std::max(num_kb + (a.upd_tma ? GEMM2_BN / 64 : 0), 2)));
   const size_t tail = 1024 + 256 + (a.upd_tma ? 1024 + UPD_RING_BYTES : 0);   // alignment slack, barriers, bf16 staging tile
   while (s > 2 && size_t(s) * stage_bytes + tail > 227 * 1024) --s;
   a.num_stages = s;
   cudaLaunchConfig_t cfg = {};
-  // (convolution geometry: M is a whole number of 128-pixel boxes, and an even one -- the caller checks)
   cfg.gridDim = dim3(2 * ((a.M + 255) / 256), (a.N - a.n_begin + BN2 - 1) / BN2, 1);
   cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
   cfg.dynamicSmemBytes = size_t(s) * stage_bytes + tail;
-  if (a.tmem_policy == TMEM_PAIR_ALONE)      // (also when a short contraction takes fewer stages)
-    cfg.dynamicSmemBytes = std::max<size_t>(cfg.dynamicSmemBytes, size_t(6) * stage_bytes + tail);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -419,17 +416,16 @@ static cudaError_t launch_pair(const CUtensorMap& tmA, const CUtensorMap& tmB, G
       return cudaLaunchKernelEx(&cfg, gemm2_tcgen05_kernel<A_MN, B_MN, MODE, true>, tmA, tmB, *um, a);
     }
   }
-  if constexpr (MODE == EPI_STORE_F32 || (!A_MN && (MODE == EPI_FPROP || MODE == EPI_DGRAD || MODE == EPI_DGRAD_UNPOOL))) {
+  if constexpr (MODE == EPI_STORE_F32 || (!A_MN && (MODE == EPI_FPROP || MODE == EPI_DGRAD))) {
     // A pair CTA that has its SM to itself walks the tiles with two accumulators (see gemm2q.cuh)
     const int tiles_m = (a.M + 255) / 256, tiles_n = (a.N - a.n_begin + BN2 - 1) / BN2;
     const int pairs = std::max(1, sm_count() / 2);
     // also for the delta contraction of wide fully connected layers (MN-major B: 211 -> 206 us on 2048 x 8192 x 8192
     // in a burst, 252 -> 246 us in a 300-step run; the forward contraction measures the same either way)
-    const bool long_delta = (MODE == EPI_DGRAD || MODE == EPI_DGRAD_UNPOOL) && a.g.kind == GEOM_PLAIN &&
-                            tiles_m * tiles_n >= 2 * pairs && num_kb >= 32;
+    const bool long_delta = MODE == EPI_DGRAD && tiles_m * tiles_n >= 2 * pairs && num_kb >= 32;
     // and for plain fp32 results of at least two tiles per SM pair (4096 x 4096 x 1024: 39.3 -> 35.7 us, 4096^3: 105 -> 100 us)
-    const bool many_stores = MODE == EPI_STORE_F32 && a.g.kind == GEOM_PLAIN && tiles_m * tiles_n >= 2 * pairs;
-    if ((a.tmem_policy == TMEM_PAIR_ALONE || (g_force_persistent == 1 && MODE != EPI_STORE_F32) || long_delta || many_stores) && a.starve_kb == 0 && g_force_persistent != 0 &&
+    const bool many_stores = MODE == EPI_STORE_F32 && tiles_m * tiles_n >= 2 * pairs;
+    if (((g_force_persistent == 1 && MODE != EPI_STORE_F32) || long_delta || many_stores) && a.starve_kb == 0 && g_force_persistent != 0 &&
         g_force_stages == 0) {
       cfg.gridDim = dim3(2 * std::min(tiles_m * tiles_n, pairs), 1, 1);
       cfg.blockDim = dim3(GEMM2Q_THREADS, 1, 1);
@@ -465,7 +461,6 @@ static cudaError_t configure_pair() {
   X(false, false, EPI_FPROP)          \
   X(false, false, EPI_STORE_F32)      \
   X(false, true, EPI_DGRAD)           \
-  X(false, true, EPI_DGRAD_UNPOOL)    \
   X(false, true, EPI_STORE_F32)       \
   X(true, true, EPI_STORE_F32)        \
   X(true, true, EPI_WGRAD_UPDATE)
@@ -574,8 +569,9 @@ cudaError_t gemm_configure() {
 cudaError_t gemm_launch(int which, int bn, const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmArgs& args,
                         cudaStream_t st, const UpdMaps* um) {
   const bool a_mn = (which == 2), b_mn = (which != 0);
+  if (gemm_is_pair(bn) && args.g.kind != GEOM_PLAIN) return cudaErrorInvalidValue;
   if (bn == GEMM_BN_PAIR224) {
-    if (a_mn || args.g.kind != GEOM_PLAIN) return cudaErrorInvalidValue;
+    if (a_mn) return cudaErrorInvalidValue;
 #define LP_TRYP224(A, B, M) \
   if (!A && b_mn == B && args.mode == M) return launch_pair<A, B, M, 224>(tmA, tmB, args, st, nullptr);
     LP_FOR_EACH_PAIR_VARIANT(LP_TRYP224)
@@ -583,7 +579,6 @@ cudaError_t gemm_launch(int which, int bn, const CUtensorMap& tmA, const CUtenso
     return cudaErrorInvalidValue;
   }
   if (bn == GEMM_BN_PAIR) {
-    if (args.g.kind == GEOM_PIX_K) return cudaErrorInvalidValue;
 #define LP_TRYP(A, B, M) \
   if (a_mn == A && b_mn == B && args.mode == M) return launch_pair<A, B, M>(tmA, tmB, args, st, um);
     LP_FOR_EACH_PAIR_VARIANT(LP_TRYP)

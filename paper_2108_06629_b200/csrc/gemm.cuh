@@ -36,10 +36,7 @@ constexpr int GEMM_MAX_STAGES = 8;
 // run side by side by one handle: where they alternated on the same SMs a pair CTA was found, about once
 // in 10^6, waiting in tcgen05.alloc for ever on an otherwise idle GPU (every other CTA of its launch
 // had its columns, no bounded wait had expired); handles with one kind only never showed it.  The
-// handle picks the kind (lp_api.cu, shape_layers).  TMEM_PAIR_ALONE is the measurement mode in which
-// a convolutional network runs its wide layers on pairs all the same: a pair CTA then takes 181 - 193
-// KiB of shared memory, so that no single-CTA kernel's allocation shares its SM.
-enum { TMEM_DEFAULT = 0, TMEM_PAIR_ALONE = 1 };
+// handle picks the kind (lp_api.cu, shape_layers), and a network with a convolution runs single-CTA kernels only.
 
 enum { EPI_STORE_F32 = 0, EPI_FPROP = 1, EPI_DGRAD = 2, EPI_WGRAD_UPDATE = 3, EPI_DGRAD_UNPOOL = 4 };
 enum { ACT_NONE = 0, ACT_RELU = 1, ACT_GELU = 2 };
@@ -125,7 +122,6 @@ struct GemmArgs {
   float *bb, *bmb, *bdb, *bbring;   // bias master, momentum (may be null), gradient, destination ring slot
   int* status;              // status block (STATUS_WORDS): the first bounded wait that expires writes it
   long long wait_limit;     // SM cycles after which a wait on a barrier gives up (0 at the call = the default, about 2 s)
-  int tmem_policy;          // host side only, see TMEM_* below
   int* phase;               // diagnosis of a stall (LP_TRACE_TASKS): eight counters of CTAs past each phase of the pair kernel, or null
   int starve_kb;            // verification of the bounded waits only: the TMA producer skips the last starve_kb k-blocks of
                             // every tile, so the MMA issuer's wait for them must run out (plain GEMM, one tile per CTA)

@@ -1,10 +1,8 @@
-// Persistent SM-pair kernel for the forward (Eqs. 1-2) and delta (Eqs. 3-4) contractions: the form the
-// pair kernel takes when a pair CTA has its SM to itself (TMEM_PAIR_ALONE, networks that mix pair and
-// single-CTA kernels).  Alone on the SM, a one-tile CTA has nothing that hides its epilogue; here one
-// CTA pair per SM pair walks the 256 x 256 tiles pair_id, pair_id + pairs, ... with the accumulator
-// double-buffered in tensor memory (2 x 256 columns = all 512, which is why it must be alone), so the
-// epilogue of tile i (activation / f' multiply / un-pooling, bf16 stores) runs under the main loop
-// of tile i + 1:
+// Persistent SM-pair kernel for long delta contractions (Eqs. 3-4) and plain fp32 results of at least two
+// tiles per SM pair (launch_pair in gemm.cu has the rules).  One CTA pair per SM pair walks the 256 x BN2
+// tiles pair_id, pair_id + pairs, ... with the accumulator double-buffered in tensor memory
+// (2 x 256 columns = all 512, so a CTA has its SM to itself), and the epilogue of tile i
+// (activation / f' multiply, stores) runs under the main loop of tile i + 1:
 //   warp 0     operand producer (TMA, ring of S stages of 32 KiB, runs on across tile boundaries)
 //   warp 1     MMA issuer (leader CTA)
 //   warps 2-5  epilogue of both CTAs, each on its own 128 rows
@@ -45,7 +43,6 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   const int num_kb = (p.K + GEMM_BK - 1) / GEMM_BK;
   const int total = tiles_m * tiles_n;
   const int pair_id = int(blockIdx.x >> 1), pairs = int(gridDim.x >> 1);
-  const bool pix = (p.g.kind == GEOM_PIX_M);
 
   // this CTA's part of tile t
   auto tile_map = [&](int t) {
@@ -55,13 +52,6 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     tm.n0 = p.n_begin + tni * BN2;
     tm.nlim = p.N;
     tm.pn0 = tm.ph0 = tm.pw0 = 0;
-    if (pix) {
-      const int bx = tmi * 2 + int(rank);
-      const int tw = bx % p.g.tiles_w, th = (bx / p.g.tiles_w) % p.g.tiles_h, tn = bx / (p.g.tiles_w * p.g.tiles_h);
-      tm.pw0 = tw << p.g.lw;
-      tm.ph0 = th << p.g.lh;
-      tm.pn0 = tn * (GEMM_BM >> (p.g.lw + p.g.lh));
-    }
     return tm;
   };
 
@@ -102,7 +92,7 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       for (; t < total && ok; t += pairs) {
         const TileMap tm = tile_map(t);
         const int nb0 = tm.n0 + int(rank) * (BN2 / 2);        // the half of B this CTA stages
-        int k0 = 0, c_tap = 0, c_chunk = 0;
+        int k0 = 0;
         for (kb = 0; kb < num_kb; ++kb, k0 += GEMM_BK) {
           ok = mbar_wait_addr(empty0 + 8u * s, ph ^ 1u, p.wait_limit);
           if (!ok) break;
@@ -110,32 +100,17 @@ gemm2q_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
           const uint32_t sb = sa + GEMM_A_BYTES;
           const uint32_t fb = map_to_cta(full0 + 8u * s, 0);          // the leader's barrier
           if (rank == 0) mbar_arrive_expect_tx_addr(full0 + 8u * s, 2u * kLoadBytes);
-          if (pix) {
-            // (stride-1 layers: the tap's shift is the whole coordinate arithmetic)
-            const int r = c_tap / p.g.S, sft = c_tap % p.g.S;
-            const int sh = p.g.flip ? p.g.pad - r : r - p.g.pad;
-            const int sw = p.g.flip ? p.g.pad - sft : sft - p.g.pad;
-            tma2_load_4d_addr(sa, &tmA, fb, c_chunk * 64, tm.pw0 + sw, tm.ph0 + sh, tm.pn0);
-            if (B_MN) {   // delta: B[k = (tap, co)][n = ci]
+          if (A_MN) {
 #pragma unroll
-              for (int c = 0; c < 2; ++c) tma2_load_2d_addr(sb + c * 8192, &tmB, fb, c_tap * p.g.tap_pitch + nb0 + c * 64, c_chunk * 64);
-            } else {      // forward: B[n = co][k = (tap, ci)]
-              tma2_load_2d_addr(sb, &tmB, fb, c_tap * p.g.tap_pitch + c_chunk * 64, nb0);
-            }
-            if (++c_chunk == p.g.chunks_per_tap) { c_chunk = 0; ++c_tap; }
+            for (int c = 0; c < 2; ++c) tma2_load_2d_addr(sa + c * 8192, &tmA, fb, tm.m0 + c * 64, k0);
           } else {
-            if (A_MN) {
+            tma2_load_2d_addr(sa, &tmA, fb, k0, tm.m0);
+          }
+          if (B_MN) {
 #pragma unroll
-              for (int c = 0; c < 2; ++c) tma2_load_2d_addr(sa + c * 8192, &tmA, fb, tm.m0 + c * 64, k0);
-            } else {
-              tma2_load_2d_addr(sa, &tmA, fb, k0, tm.m0);
-            }
-            if (B_MN) {
-#pragma unroll
-              for (int c = 0; c < 2; ++c) tma2_load_2d_addr(sb + c * 8192, &tmB, fb, nb0 + c * 64, k0);
-            } else {
-              tma2_load_2d_addr(sb, &tmB, fb, k0, nb0);
-            }
+            for (int c = 0; c < 2; ++c) tma2_load_2d_addr(sb + c * 8192, &tmB, fb, nb0 + c * 64, k0);
+          } else {
+            tma2_load_2d_addr(sb, &tmB, fb, k0, nb0);
           }
           ++issued;
           if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }

@@ -138,7 +138,6 @@ struct lp_ctx {
   int n_stages = 0;
   int stages_used = 0;
   int n_chain = 1, n_g = 1;     // P chain streams (minibatch n on n % P), Q G streams (layer l on l % Q; none under fused-B)
-  int tmem_policy = 0;          // TMEM_*: how pair and single-CTA kernels keep out of each other's tensor memory
   int classes = 0, ld_cls = 0;
   // shared buffers
   float* zL = nullptr;          // [kDeltaSlots][B][ld_cls] fp32
@@ -447,17 +446,6 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
       y.bn_f = y.n_out <= 64 ? 64 : 128;
       y.bn_d = y.ld_in <= 64 ? 64 : 128;
       y.bn_g = y.ld_in <= 64 ? 64 : 128;
-      // Wide layers (at least 256 channels on both sides) on an even number of pixel boxes:
-      // 256-pixel x 256-column tiles on SM pairs.  Measured on the VGG-16 layers at batch 64,
-      // pair against single CTA: 512 -> 512 at 28^2 forward 180 / 245 us, delta 189 / 253 us;
-      // 256 -> 256 at 56^2 216 / 240 and 230 / 249 us; 512 -> 512 at 14^2 66 / 79 and 67 / 84 us;
-      // 128 -> 256 forward (18 k-blocks) is slower as a pair (149 / 131 us) and stays single.
-      // Off by default: a convolutional network always has single-CTA kernels too, and the two kinds of
-      // tensor-memory allocation do not mix (see the end of this function).  LP_CONV_PAIR=1 in the
-      // environment turns the pair tiles on, as persistent CTA pairs that have their SMs to themselves
-      // (gemm2q.cuh; VGG-16 step 7.75 ms against 8.38 ms) -- for measurements and the kernels' parity
-      // tests, not for long runs.
-      const bool even_boxes = ((y.in_rows / GEMM_BM) % 2) == 0;
       // 128 x 256 single-CTA tiles where gemm_pick_bn's rule for them holds (a long contraction, enough tiles for
       // one persistent CTA on every SM): a third less operand traffic per multiply-accumulate than 128 x 128
       const long long row_tiles = y.in_rows / GEMM_BM;
@@ -465,9 +453,6 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
         if (y.n_out >= 256 && y.taps * y.ld_in >= 1024 && row_tiles * ((y.n_out + 255) / 256) >= 2 * kSMs) y.bn_f = 256;
         if (l > 0 && y.ld_in >= 256 && y.taps * y.n_out >= 1024 && row_tiles * ((y.ld_in + 255) / 256) >= 2 * kSMs) y.bn_d = 256;
       }
-      const bool conv_pair = getenv("LP_CONV_PAIR") != nullptr;
-      if (conv_pair && !y.gen && even_boxes && y.n_out >= 256 && y.ld_in >= 256) y.bn_f = GEMM_BN_PAIR;
-      if (conv_pair && !y.gen && even_boxes && l > 0 && y.ld_in >= 256 && y.n_out >= 256) y.bn_d = GEMM_BN_PAIR;
       y.split_f = y.split_d = 1;
       const bool tiles_8x16 = !y.gen && (y.imW % 8 == 0) && (y.imH % 16 == 0);
       y.halo_f = !y.patch && tiles_8x16 && y.ld_in <= 64 && y.n_out <= 64;
@@ -512,7 +497,8 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
   // CTAs, with a pair CTA waiting in tcgen05.alloc for ever on an otherwise idle GPU; handles of one
   // kind only never did.  So a fully connected network whose layers are mostly wide runs EVERY
   // contraction on SM pairs (the narrow classifier too: a 256-column tile that is mostly padding
-  // costs microseconds), and every other network runs none there.
+  // costs microseconds), and every other network runs none there, whatever tile lp_set_tuning asks for: a network with
+  // convolutions always has single-CTA kernels too.
   const int B = c->cfg.batch;
   bool any_conv = false;
   int fc_pair = 0;
@@ -521,24 +507,20 @@ static void shape_layers(lp_ctx* c, const lp_layer* layers, int n, const std::ve
     any_conv = any_conv || y.conv;
     if (!y.conv && (gemm_is_pair(y.bn_f) || (l > 0 && gemm_is_pair(y.bn_d)) || gemm_is_pair(y.bn_g))) ++fc_pair;
   }
-  const bool conv_pair = getenv("LP_CONV_PAIR") != nullptr;     // measurement aid, see the convolution branch above
-  if (!conv_pair) {
-    const bool pure_pair = !any_conv && fc_pair * 2 >= n;
-    for (int l = 0; l < n; ++l) {
-      Layer& y = c->L[l];
-      if (y.conv) continue;
-      if (pure_pair) {
-        if (!gemm_is_pair(y.bn_f)) y.bn_f = GEMM_BN_PAIR;
-        if (!gemm_is_pair(y.bn_d)) y.bn_d = GEMM_BN_PAIR;
-        if (!gemm_is_pair(y.bn_g)) y.bn_g = GEMM_BN_PAIR;
-        y.split_f = y.split_d = 1;
-        y.cl_f = y.cl_d = 0;
-      } else if (fc_pair > 0) {
-        pick_fc_tiles(&y, B, false);
-      }
+  const bool pure_pair = !any_conv && fc_pair * 2 >= n;
+  for (int l = 0; l < n; ++l) {
+    Layer& y = c->L[l];
+    if (y.conv) continue;
+    if (pure_pair) {
+      if (!gemm_is_pair(y.bn_f)) y.bn_f = GEMM_BN_PAIR;
+      if (!gemm_is_pair(y.bn_d)) y.bn_d = GEMM_BN_PAIR;
+      if (!gemm_is_pair(y.bn_g)) y.bn_g = GEMM_BN_PAIR;
+      y.split_f = y.split_d = 1;
+      y.cl_f = y.cl_d = 0;
+    } else if (fc_pair > 0) {
+      pick_fc_tiles(&y, B, false);
     }
   }
-  c->tmem_policy = conv_pair ? TMEM_PAIR_ALONE : TMEM_DEFAULT;
   c->classes = layers[n - 1].out;
   c->ld_cls = pad8(c->classes);
 }
@@ -690,7 +672,7 @@ static int build_tensor_maps(lp_ctx* c) {
       }
       for (int s = 0; s < y.slots; ++s) {
         if ((rc = make_tmap_bf16_2d(&y.tm_f_B[s], y.ring + s * y.w_elems, y.w_ld, y.n_out, y.w_ld, 64,
-                                    y.bn_f == GEMM_BN_PAIR ? 128 : y.bn_f, &err)) != LP_OK)   // a pair CTA stages half of the 256 columns
+                                    y.bn_f, &err)) != LP_OK)
           return fail(c, rc, err);
         if ((rc = make_tmap_bf16_2d(&y.tm_d_B[s], y.ring + s * y.w_elems, y.w_ld, y.n_out, y.w_ld, 64, 64, &err)) != LP_OK)
           return fail(c, rc, err);
@@ -852,7 +834,6 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
   a.act = y.d.act;
   a.bias = y.d.has_bias ? y.bring + size_t(ring_slot) * y.ld_out : nullptr;
   a.status = c->status;
-  a.tmem_policy = c->tmem_policy;
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   if (last) {
     a.out = nullptr;
@@ -951,7 +932,6 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
     }
   }
   a.status = c->status;
-  a.tmem_policy = c->tmem_policy;
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   a.splits = y.split_d; a.partial = y.part_d;
   a.cluster = y.cl_d;
@@ -1013,7 +993,6 @@ static cudaError_t launch_G(lp_ctx* c, int l, long long n, cudaStream_t st) {
   if (!y.conv || y.patch) a.N = y.n_in;
   a.ld_out = y.w_ld;
   a.status = c->status;
-  a.tmem_policy = c->tmem_policy;
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   if (y.conv && !y.patch) a.g = conv_geom(y, GEOM_PIX_K, y.box64, 0, 0, (y.ld_in + y.bn_g - 1) / y.bn_g);
   if (y.split_g > 1) {

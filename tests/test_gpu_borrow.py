@@ -106,13 +106,14 @@ def test_split_delta_fc_persistent_pair_kernel():
     _split_delta_case(layers, 2048, 3, {1: (1, 1), 2: (1, 2)})
 
 
-def test_split_delta_convolution_single_cta_and_pair_tiles(conv_pair_tiles):
+@pytest.mark.parametrize("tile_n", [0, 512])
+def test_split_delta_convolution(tile_n):
+    """128-wide single-CTA tiles, 384 input channels = 3 tiles, also where SM-pair tiles are asked for."""
     from paper_2108_06629_b200 import inputs as I
     layers = I.vgg(8, [384, 384, 384], [10])
-    # batch 6: three 128-pixel boxes (odd) -> single-CTA 128-wide tiles, 384 input channels = 3 tiles
-    _split_delta_case(layers, 6, 3, {1: (1, 2), 2: (2, 1)}, expect_cols=[0, 128, 256, 0])
-    # batch 8: four boxes -> 256-pixel x 256-column pair tiles, 384 channels = 2 tiles
-    _split_delta_case(layers, 8, 3, {1: (1, 1), 2: (1, 3)}, expect_cols=[0, 256, 256, 0])
+    # an odd number of 128-pixel boxes, and an even one
+    _split_delta_case(layers, 6, 3, {1: (1, 2), 2: (2, 1)}, tile_n=tile_n, expect_cols=[0, 128, 256, 0])
+    _split_delta_case(layers, 8, 3, {1: (1, 2), 2: (2, 1)}, tile_n=tile_n, expect_cols=[0, 128, 256, 0])
 
 
 def test_narrow_split_k_and_halo_layers_keep_one_piece():
