@@ -110,8 +110,9 @@ cudaError_t gemm_configure();   // opt in to large dynamic shared memory; call o
 void gemm_set_tuning(int bn, int stages, int splits);   // 0 = automatic
 int gemm_pick_splits(int M, int N, int K, int bn);
 // CTAs of a cluster that share one tile's contraction (GemmArgs::cluster) and, where that is not 0, the tile width
-// (layer: the epilogue is that of a layer, and there is scratch for a contraction split through global memory, which may be the better one)
-int gemm_pick_cluster(int M, int N, int K, int* bn, bool layer);
+// (layer: the epilogue is that of a layer, and there is scratch for a contraction split through global memory, which may be the better one);
+// *segs: accumulators of each of them (GemmArgs::segs)
+int gemm_pick_cluster(int M, int N, int K, int* bn, int* segs, bool layer);
 
 // ---- planner.cpp ------------------------------------------------------------
 struct PlanResult {

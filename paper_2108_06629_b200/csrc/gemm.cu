@@ -188,7 +188,13 @@ int gemm_pick_splits(int M, int N, int K, int bn) {
 //   13.5; x 1500 10.9 / 10.3 / 14.1; x 3000 18.9 / 20.7);
 // * beyond, two CTAs per SM if each keeps 16 k-blocks (64 x 4096 x 4096 on 64 tiles: 14.7 in quarters, 16.6 in halves,
 //   undivided 27.6).
-int gemm_pick_cluster(int M, int N, int K, int* bn, bool layer) {
+//
+// No sum is longer than in the divided form that the shape would otherwise take (the error of a chain grows with its length): one
+// CTA where four or two could share the tile has four or two accumulators, and halves have two where quarters could share it.  Relative
+// error against 64 bits and time, one sum / in parts / divided: 64 x 64 x 256 2.3e-7 3.5 us / 7.7e-8 3.8 / 7.7e-8 4.3;
+// 300 x 1000 x 256 2.3e-7 4.2 / 1.2e-7 4.3 / 1.2e-7 5.7; 1000 x 1000 x 2100 2.2e-6 13.9 / 1.0e-6 13.9 / 1.0e-6 16.9.
+int gemm_pick_cluster(int M, int N, int K, int* bn, int* segs, bool layer) {
+  *segs = 1;
   if (g_force_bn != 0 || g_force_stages != 0 || g_force_splits != 0 || g_force_persistent >= 0) return 0;
   const long long rows = (M + GEMM_BM - 1) / GEMM_BM;
   const int width = rows * ((N + 63) / 64) <= sm_count() ? 64 : 128;
@@ -197,12 +203,11 @@ int gemm_pick_cluster(int M, int N, int K, int* bn, bool layer) {
   auto one_each = [&](int c) { return num_kb >= c && tiles * c <= sm_count(); };
   auto two_each = [&](int c) { return tiles * c <= 2 * sm_count() && num_kb >= 16 * c; };
   int c = 0;
-  if (width == 64 && num_kb <= 4 && !layer) c = 1;
+  if (width == 64 && num_kb <= 4 && !layer) c = 1, *segs = one_each(4) ? 4 : one_each(2) ? 2 : 1;
   else if ((num_kb >= 16 && tiles <= 8) || (num_kb >= 40 && one_each(8))) c = 8;
   else if (one_each(4)) c = 4;
-  else if (one_each(2)) c = 2;
-  else if (width == 64 && num_kb <= 64) c = 1;
-  else if (two_each(4)) c = 4;
+  else if (one_each(2)) c = 2, *segs = two_each(4) ? 2 : 1;
+  else if (width == 64 && num_kb <= 64) c = 1, *segs = two_each(2) ? 2 : 1;
   else if (two_each(2)) c = 2;
   // (one tile over a hundred thousand terms: the split through global memory, which a layer has and lp_gemm_bf16 has not,
   // spreads it wider than a cluster can)
@@ -350,9 +355,14 @@ static cudaError_t launch_cluster(const CUtensorMap& tmA, const CUtensorMap& tmB
   if (a.wait_limit <= 0) a.wait_limit = LP_WAIT_LIMIT_CYCLES;
   const int tiles_m = (a.M + GEMM_BM - 1) / GEMM_BM, tiles_n = (a.N - a.n_begin + BN - 1) / BN;
   note_form("cluster", BN, a.cluster);
-  if (a.cluster == 1 && BN != 64) return cudaErrorInvalidValue;
-  return launch_chained(a.cluster == 1 ? gemmc_kernel<64, A_MN, B_MN, MODE, true> : gemmc_kernel<BN, A_MN, B_MN, MODE, false>, dim3(a.cluster, tiles_m * tiles_n), GEMM_THREADS, gemmc_smem_bytes(BN), st, a.cluster,
-                        tmA, tmB, a, tiles_m);
+  auto* kernel = gemmc_kernel<BN, A_MN, B_MN, MODE, false, 1>;
+  if constexpr (BN == 64) {
+    if (a.cluster == 1) kernel = a.segs == 4 ? gemmc_kernel<64, A_MN, B_MN, MODE, true, 4> : a.segs == 2 ? gemmc_kernel<64, A_MN, B_MN, MODE, true, 2> : gemmc_kernel<64, A_MN, B_MN, MODE, true, 1>;
+    else if (a.segs == 2) kernel = gemmc_kernel<64, A_MN, B_MN, MODE, false, 2>;
+  } else if (a.cluster == 1 || a.segs != 1) {
+    return cudaErrorInvalidValue;
+  }
+  return launch_chained(kernel, dim3(a.cluster, tiles_m * tiles_n), GEMM_THREADS, gemmc_smem_bytes(BN), st, a.cluster, tmA, tmB, a, tiles_m);
 }
 #define LP_FOR_EACH_CLUSTER_VARIANT(X, BN) \
   X(BN, false, false, EPI_FPROP)           \
@@ -548,14 +558,18 @@ cudaError_t gemm_configure() {
   if ((e = configure_pair<A, B, M>()) != cudaSuccess) return e;
   LP_FOR_EACH_PAIR_VARIANT(LP_CFGP)
 #undef LP_CFGP
-#define LP_CFGC(BN, A, B, M)                                                                                   \
-  if ((e = cudaFuncSetAttribute(gemmc_kernel<BN, A, B, M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                gemmc_smem_bytes(BN))) != cudaSuccess ||                                       \
-      (BN == 64 && (e = cudaFuncSetAttribute(gemmc_kernel<64, A, B, M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                             gemmc_smem_bytes(64))) != cudaSuccess))                           \
+#define LP_CFGC(BN, A, B, M, ONE, SEGS)                                                                        \
+  if ((e = cudaFuncSetAttribute(gemmc_kernel<BN, A, B, M, ONE, SEGS>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                gemmc_smem_bytes(BN))) != cudaSuccess)                                         \
     return e;
-  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 64)
-  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC, 128)
+#define LP_CFGC64(BN, A, B, M)                                                                                 \
+  LP_CFGC(BN, A, B, M, false, 1) LP_CFGC(BN, A, B, M, false, 2)                                                \
+  LP_CFGC(BN, A, B, M, true, 1) LP_CFGC(BN, A, B, M, true, 2) LP_CFGC(BN, A, B, M, true, 4)
+#define LP_CFGC128(BN, A, B, M) LP_CFGC(BN, A, B, M, false, 1)
+  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC64, 64)
+  LP_FOR_EACH_CLUSTER_VARIANT(LP_CFGC128, 128)
+#undef LP_CFGC128
+#undef LP_CFGC64
 #undef LP_CFGC
 #define LP_CFG(BN, A, B, M) \
   if ((e = configure_one<BN, A, B, M>()) != cudaSuccess) return e;
@@ -655,7 +669,8 @@ int gemm_standalone(int which, int M, int N, int K, const void* A, int lda, cons
   int rc = gemm_device_setup(&status_dev);
   if (rc != LP_OK) return rc;
   int bn = gemm_pick_bn(which, M, N, K);
-  const int cluster = gemm_is_pair(bn) ? 0 : gemm_pick_cluster(M, N, K, &bn, false);
+  int segs = 1;
+  const int cluster = gemm_is_pair(bn) ? 0 : gemm_pick_cluster(M, N, K, &bn, &segs, false);
   uint32_t boxA[2], boxB[2];
   gemm_box_dims(which, bn, boxA, boxB);
   CUtensorMap tmA, tmB;
@@ -676,6 +691,7 @@ int gemm_standalone(int which, int M, int N, int K, const void* A, int lda, cons
   a.wait_limit = wait_limit;
   a.starve_kb = starve_kb;
   a.cluster = cluster;
+  a.segs = segs;
   cudaError_t e = gemm_launch(which, bn, tmA, tmB, a, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) { set_global_error(std::string("lp_gemm_bf16 launch: ") + cudaGetErrorString(e)); return LP_ERR_CUDA; }
   return LP_OK;

@@ -111,6 +111,7 @@ struct GemmArgs {
   int splits, kb_per_split;
   float* partial;           // [tiles][splits][128][BN]
   int cluster;              // 1, 2, 4 or 8: one tile per cluster of that many CTAs, which divide the contraction (gemmc.cuh); 0: other forms
+  int segs;                 // (with cluster > 0) accumulators of a CTA: parts of its k-blocks that are summed apart; 1, or 2 or 4 with 64-column tiles
   ConvGeom g;
   int persistent;           // CTAs loop over tiles (grid sized to the machine) instead of one tile each
   int l2_ahead;             // plain GEMM: k-blocks of the B operand to pull into L2 ahead of the pipeline (0 = off)

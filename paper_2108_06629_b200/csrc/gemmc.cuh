@@ -9,6 +9,10 @@
 // shrink by C, nothing goes through global memory (the split-K form of gemm.cuh writes and re-reads its partial tiles there and
 // leaves the sum and the epilogue to a second launch).  A cluster of one is the same without the sum: 64-column tiles and all
 // six warps in the epilogue (32 x 256 x 10 5.1 -> 3.1 us, 1000 x 900 x 1000 13.5 -> 9.3 against the 128-column form of gemm.cuh).
+//
+// SEGS: consecutive parts of a CTA's k-blocks with an accumulator of their own, which the epilogue adds in order.  The tensor
+// core truncates the running sum once per 16 terms, so the error grows with the length of a chain; SEGS keeps the chains as short as
+// a division over more CTAs has them where fewer CTAs are the faster ones.
 #pragma once
 #include "gemm2.cuh"
 
@@ -74,7 +78,7 @@ __device__ __forceinline__ void gemmc_reduce_store(const GemmArgs& p, const Tile
 }
 
 // ONE: a cluster of one (a kernel of its own: one more case in the switch at the end slowed the others, the ragged GELU MLP 627 -> 637 us)
-template <int BN, bool A_MN, bool B_MN, int MODE, bool ONE>
+template <int BN, bool A_MN, bool B_MN, int MODE, bool ONE, int SEGS>
 __global__ void __launch_bounds__(GEMM_THREADS, 2)
 gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs p, const int tiles_m) {
   static_assert(MODE != EPI_WGRAD_UPDATE, "the update has tiles enough");
@@ -99,7 +103,7 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   const int kb_total = (p.K + GEMM_BK - 1) / GEMM_BK;
   const int kb_each = kb_total / C, kb_more = kb_total % C;       // the first kb_more ranks take one more
   const int kb0 = int(rank) * kb_each + min(int(rank), kb_more);
-  const int num_kb = kb_each + (int(rank) < kb_more ? 1 : 0);     // (at least one: gemm_pick_cluster)
+  const int num_kb = kb_each + (int(rank) < kb_more ? 1 : 0);     // (at least one a part: gemm_pick_cluster)
 
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmA);
@@ -113,8 +117,8 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   }
   if (warp == 1) {
     if (lane == 0) tmem_note_enter(TK_GEMM);
-    tmem_alloc(tmem_slot, BN);
-    if (lane == 0) tmem_note_got(TK_GEMM, BN);
+    tmem_alloc(tmem_slot, BN * SEGS);
+    if (lane == 0) tmem_note_got(TK_GEMM, BN * SEGS);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -165,21 +169,27 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                                : make_smem_desc(smem_u32(smem) + GEMM_A_BYTES, 16, 1024);
       const uint32_t dA_hi = uint32_t(dA >> 32), dB_hi = uint32_t(dB >> 32);
       constexpr uint32_t stepA = (A_MN ? 2048 : 32) >> 4, stepB = (B_MN ? 2048 : 32) >> 4;
-      uint32_t s = 0, ph = 0, acc = 0;
+      uint32_t s = 0, ph = 0;
       bool ok = true;
       int kb = 0;
-      for (; kb < num_kb; ++kb) {
-        ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t off = s * uint32_t(SM::STAGE_BYTES >> 4);
+#pragma unroll 1
+      for (int g = 0; g < SEGS && ok; ++g) {
+        const uint32_t tacc = tmem_base + uint32_t(g * BN);
+        const int end = SEGS == 1 ? num_kb : kb + num_kb / SEGS + (g < num_kb % SEGS ? 1 : 0);    // (the first parts take one more)
+        uint32_t acc = 0;
+        for (; kb < end; ++kb) {
+          ok = mbar_wait_addr(full0 + 8u * s, ph, p.wait_limit);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t off = s * uint32_t(SM::STAGE_BYTES >> 4);
 #pragma unroll
-        for (int j = 0; j < GEMM_BK / 16; ++j) {
-          umma_f16_lohi(tmem_base, uint32_t(dA) + off + j * stepA, dA_hi, uint32_t(dB) + off + j * stepB, dB_hi, idesc, acc);
-          acc = 1;
+          for (int j = 0; j < GEMM_BK / 16; ++j) {
+            umma_f16_lohi(tacc, uint32_t(dA) + off + j * stepA, dA_hi, uint32_t(dB) + off + j * stepB, dB_hi, idesc, acc);
+            acc = 1;
+          }
+          umma_commit_addr(empty0 + 8u * s);
+          if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
         }
-        umma_commit_addr(empty0 + 8u * s);
-        if (++s == uint32_t(S)) { s = 0; ph ^= 1u; }
       }
       umma_commit(acc_bar);
       if (!ok) report_expired(p.status, WAIT_CLUSTER_MMA, int(blockIdx.y), kb);
@@ -212,6 +222,14 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         tmem_ld_32x32(tmem_base + (uint32_t(q * 32) << 16) + uint32_t(c * 32), r);
         tmem_ld_wait();
 #pragma unroll
+        for (int s = 1; s < SEGS; ++s) {
+          uint32_t t[32];
+          tmem_ld_32x32(tmem_base + (uint32_t(q * 32) << 16) + uint32_t(s * BN + c * 32), t);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(t[i]));
+        }
+#pragma unroll
         for (int g = 0; g < 8; ++g)
           *reinterpret_cast<uint4*>(row + c * 32 + g * 4) = make_uint4(r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
       }
@@ -222,8 +240,8 @@ gemmc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   cluster_sync_all();                     // every partial tile of the cluster is in shared memory
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, BN);
-    if (lane == 0) tmem_note_freed(TK_GEMM, BN);
+    tmem_dealloc(tmem_base, BN * SEGS);
+    if (lane == 0) tmem_note_freed(TK_GEMM, BN * SEGS);
   }
   const uint32_t part = smem_u32(smem);
   if constexpr (ONE) {

@@ -96,6 +96,7 @@ struct Layer {
   int z_slots = 0;
   int bn_f = 128, bn_d = 128, bn_g = 128;
   int cl_f = 0, cl_d = 0;                       // CTAs of a cluster that share a tile of the forward / delta contraction
+  int seg_f = 1, seg_d = 1;                     // and accumulators of each of them
   int split_f = 1, split_d = 1;                 // split-K factors of the forward / delta contractions
   float *part_f = nullptr, *part_d = nullptr;   // fp32 partial tiles [tiles][splits][128][BN]
   std::vector<CUtensorMap> tm_f_A, tm_f_B, tm_d_A, tm_d_B, tm_g_A, tm_g_B;
@@ -392,8 +393,8 @@ static void pick_fc_tiles(Layer* y, int B, bool allow_pair) {
   // 289 / 280, 3072 357 / 378, 4096 565 / 623; batch 64, 2048 218 / 156, 3072 341 / 291, 4096 520 / 529.  So the line, at
   // 2048 x 2048, is on the safe side of where clusters begin to cost, which lies between 2560 and 4096 with the batch.
   const bool chain_bound = (long long)y->n_in * y->n_out <= (1ll << 22);
-  y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f, true) : 0;
-  y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d, true) : 0;
+  y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f, &y->seg_f, true) : 0;
+  y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d, &y->seg_d, true) : 0;
   y->split_f = gemm_is_pair(y->bn_f) || y->cl_f > 0 ? 1 : gemm_pick_splits(B, y->n_out, y->n_in, y->bn_f);
   y->split_d = gemm_is_pair(y->bn_d) || y->cl_d > 0 ? 1 : gemm_pick_splits(B, y->n_in, y->n_out, y->bn_d);
 }
@@ -858,7 +859,7 @@ static cudaError_t launch_forward(lp_ctx* c, int l, long long n, int ring_slot, 
     }
   }
   a.splits = y.split_f; a.partial = y.part_f;
-  a.cluster = y.cl_f;
+  a.cluster = y.cl_f; a.segs = y.seg_f;
   c->launches += y.split_f > 1 ? 2 : 1;
   TimedScope ts(c, LP_TASK_FORWARD, st, l);
   if (y.lean_f) {
@@ -934,7 +935,7 @@ static cudaError_t launch_delta(lp_ctx* c, int l, long long n, int ring_slot, cu
   a.status = c->status;
   a.phase = c->trace_done ? c->status + 8 : nullptr;
   a.splits = y.split_d; a.partial = y.part_d;
-  a.cluster = y.cl_d;
+  a.cluster = y.cl_d; a.segs = y.seg_d;
   c->launches += y.split_d > 1 ? 2 : 1;
   TimedScope ts(c, LP_TASK_DELTA, st, l);
   if (y.halo_d) {

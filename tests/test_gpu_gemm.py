@@ -150,6 +150,52 @@ def test_contraction_divided_over_a_cluster(which):
     assert {"cluster 64 x2", "cluster 64 x4", "cluster 64 x8", "cluster 128 x2"} <= forms, forms
 
 
+def _sum_of_parts(which, M, N, A, B, ldc, k0, k1, parts):
+    """The product over [k0, k1) as undivided contractions of consecutive k-blocks, added in order: parts[0] of them (the first ones
+    a k-block longer), each made in turn of parts[1] of them, ..."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    if not parts:
+        C = torch.zeros((M, ldc), device="cuda")
+        a = A[k0:k1] if which == 2 else A[:, k0:k1]
+        b = B[:, k0:k1] if which == 0 else B[k0:k1]
+        lpb.lp_set_tuning(64, 0, 1)                  # (64-column tiles, one CTA each)
+        try:
+            lpb.lp_gemm_bf16(which, M, N, k1 - k0, a, A.shape[1], b, B.shape[1], C, ldc)
+        finally:
+            lpb.lp_set_tuning(0, 0, 0)
+        assert lpb.lp_debug_last_contraction().startswith("single 64")
+        return C
+    kb, total = (k1 - k0 + 63) // 64, None
+    for r in range(parts[0]):
+        end = min(k1, k0 + 64 * (kb // parts[0] + (r < kb % parts[0])))
+        C = _sum_of_parts(which, M, N, A, B, ldc, k0, end, parts[1:])
+        total = C if total is None else total + C
+        k0 = end
+    return total
+
+
+# CTAs of a cluster, accumulators of a CTA: one to four k-blocks on tiles that leave room for four CTAs, for two and for one; 75 and more
+# tiles on both sides of 32 k-blocks; 74 tiles (halves) on both sides of 64.
+@pytest.mark.parametrize("M, N, K, parts", [
+    (64, 64, 256, (1, 4)), (33, 70, 250, (1, 4)), (128, 2368, 200, (1, 4)), (128, 2369, 200, (1, 2)), (129, 65, 130, (1, 2)), (1, 1, 128, (1, 2)),
+    (300, 1000, 256, (1, 2)), (513, 1000, 256, (1, 1)), (65, 130, 40, (1, 1)), (1000, 1000, 2100, (1, 2)), (128, 4800, 1980, (1, 1)),
+    (128, 6000, 4096, (1, 2)), (64, 4736, 4096, (2, 2)), (100, 4730, 4290, (2, 2)), (64, 4736, 4030, (2, 1))])
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_sums_of_a_contraction_are_no_longer_than_its_parts(which, M, N, K, parts):
+    """The accumulator is truncated once per 16 terms, so its error grows with the length of a sum: bit for bit the sums of
+    the parts, added in order."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    A, B = (t.cuda() for t in _operands(which, M, N, K, 5000 + which))
+    ldc = (N + 3) // 4 * 4
+    Cd = torch.full((M, ldc), 7.0, device="cuda")
+    lpb.lp_gemm_bf16(which, M, N, K, A, A.shape[1], B, B.shape[1], Cd, ldc)
+    assert lpb.lp_debug_last_contraction() == "cluster 64 x%d" % parts[0]
+    assert torch.equal(Cd, _sum_of_parts(which, M, N, A, B, ldc, 0, K, parts))
+    assert lpb.lp_gemm_status() == (lpb.LP_OK, 0)
+
+
 # Plain fp32 results on SM pairs: at least two tiles a pair (persistent, 256 and 224 columns, MN-major A in the G form), and no
 # more tiles than pairs (six stages), with ragged last rows, columns and k-blocks.
 @pytest.mark.parametrize("which, M, N, K, form", [

@@ -506,6 +506,15 @@ def test_tasks_halo_tiles_of_narrow_layers(H, W, B, chans, pools):
     run_teacher_forced(layers, B, 2, None, 0.05, 0.9, 1)
 
 
+@pytest.mark.parametrize("wide, narrow, form", [(4160, 832, "cluster 64 x2"), (2112, 1664, "cluster 64 x1")])
+def test_tasks_two_accumulators_a_cta(wide, narrow, form, monkeypatch):
+    """Forward and delta of 39 tiles over 65 k-blocks (halves) and of 78 tiles over 33 (one CTA a tile): two accumulators each."""
+    from paper_2108_06629_b200 import inputs as I
+    forms = _forms(monkeypatch)
+    run_teacher_forced(I.mlp([wide, narrow, wide, 10], "gelu"), 300, 2, None, 0.01, 0.9, 1)
+    assert forms["forward", 0] == {form} and forms["delta", 1] == {form}, forms
+
+
 @pytest.mark.parametrize("n_in, n_out, batch", [(17000, 10, 5), (16390, 130, 3), (20000, 300, 130)])
 def test_tasks_long_contractions_split_over_all_sms(n_in, n_out, batch):
     """One to six tiles of 256 k-blocks and more, the last split shorter than the others: sum and epilogue in a second launch."""
