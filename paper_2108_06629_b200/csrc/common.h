@@ -111,8 +111,9 @@ void gemm_set_tuning(int bn, int stages, int splits);   // 0 = automatic
 int gemm_pick_splits(int M, int N, int K, int bn);
 // CTAs of a cluster that share one tile's contraction (GemmArgs::cluster) and, where that is not 0, the tile width
 // (layer: the epilogue is that of a layer, and there is scratch for a contraction split through global memory, which may be the better one);
-// *segs: accumulators of each of them (GemmArgs::segs)
-int gemm_pick_cluster(int M, int N, int K, int* bn, int* segs, bool layer);
+// sectors: the rows of both operands start on 32-byte sectors, and the launch has the GPU to itself; *segs: accumulators of
+// each of them (GemmArgs::segs)
+int gemm_pick_cluster(int M, int N, int K, int* bn, int* segs, bool layer, bool sectors);
 
 // ---- planner.cpp ------------------------------------------------------------
 struct PlanResult {

@@ -184,16 +184,22 @@ int gemm_pick_splits(int M, int N, int K, int bn) {
 //   epilogue gains by the division (16 steps of the ragged GELU MLP 620, undivided 640);
 // * else eight CTAs to a tile for a handful of tiles (128 x 64 x 1500 5.6, in quarters 6.2; 128 x 800 x 3000 on 13 tiles 7.5 / 8.3, but
 //   x 784 6.1 / 5.7), four, or two, while that is at most one CTA per SM (128 x 2048 x 784 four 6.1, two 6.6, undivided 7.8);
-// * undivided where the tiles leave no room for that, up to 64 k-blocks (1000 x 800 x 784 7.9, two 8.3, 128-column tiles
-//   13.5; x 1500 10.9 / 10.3 / 14.1; x 3000 18.9 / 20.7);
-// * beyond, two CTAs per SM if each keeps 16 k-blocks (64 x 4096 x 4096 on 64 tiles: 14.7 in quarters, 16.6 in halves,
-//   undivided 27.6).
+// * two CTAs per SM if each keeps 16 k-blocks: quarters on up to 68 tiles -- 71 found room at once, clusters of four
+//   leaving some SMs out, and 72 take two rounds (64 x 2560 x 4096 9.7, in halves 12.4; x 4352 10.3 / 12.8; x 4608 17.3 / 12.8;
+//   64 x 2560 x 8192 14.7 / 20.8; 384 x 1024 x 4096 11.0 / 12.8) -- and halves on up to 148 (128 x 4800 x 2048 9.8, undivided 12.1;
+//   1000 x 1024 x 4096 15.3 / 21.0), where the rows of both operands start on 32-byte sectors.  Else a row of a box touches five sectors
+//   instead of four, the kernel is bound by what L2 delivers, and fewer CTAs are as good or better (1000 x 800 x 3000 halves 19.9,
+//   undivided 17.5, but x 3024 15.6 / 17.1; 1000 x 1000 x 2100 15.7 / 13.6; 384 x 1024 x 4100 quarters 16.1, halves 14.4; the largest the
+//   other way is 64 x 2512 x 4100, delta, 12.1 / 13.0).  Not in a layer either, which shares the SMs with its neighbours' kernels (16
+//   steps of six layers 2048 wide, batch 512, 2490 us undivided, 2910 in halves; 4096 - 1024 at batch 384 2120 in halves, 2160 in quarters);
+// * undivided up to 64 k-blocks where the tiles leave no room for more (1000 x 800 x 784 7.9, two 8.3, 128-column tiles 13.5);
+// * beyond 64 k-blocks in halves, two CTAs per SM, all the same.
 //
 // No sum is longer than in the divided form that the shape would otherwise take (the error of a chain grows with its length): one
 // CTA where four or two could share the tile has four or two accumulators, and halves have two where quarters could share it.  Relative
 // error against 64 bits and time, one sum / in parts / divided: 64 x 64 x 256 2.3e-7 3.5 us / 7.7e-8 3.8 / 7.7e-8 4.3;
 // 300 x 1000 x 256 2.3e-7 4.2 / 1.2e-7 4.3 / 1.2e-7 5.7; 1000 x 1000 x 2100 2.2e-6 13.9 / 1.0e-6 13.9 / 1.0e-6 16.9.
-int gemm_pick_cluster(int M, int N, int K, int* bn, int* segs, bool layer) {
+int gemm_pick_cluster(int M, int N, int K, int* bn, int* segs, bool layer, bool sectors) {
   *segs = 1;
   if (g_force_bn != 0 || g_force_stages != 0 || g_force_splits != 0 || g_force_persistent >= 0) return 0;
   const long long rows = (M + GEMM_BM - 1) / GEMM_BM;
@@ -205,8 +211,9 @@ int gemm_pick_cluster(int M, int N, int K, int* bn, int* segs, bool layer) {
   int c = 0;
   if (width == 64 && num_kb <= 4 && !layer) c = 1, *segs = one_each(4) ? 4 : one_each(2) ? 2 : 1;
   else if ((num_kb >= 16 && tiles <= 8) || (num_kb >= 40 && one_each(8))) c = 8;
-  else if (one_each(4)) c = 4;
+  else if (one_each(4) || (sectors && two_each(4) && tiles * 4 <= 2 * sm_count() - 24)) c = 4;
   else if (one_each(2)) c = 2, *segs = two_each(4) ? 2 : 1;
+  else if (sectors && two_each(2)) c = 2;
   else if (width == 64 && num_kb <= 64) c = 1, *segs = two_each(2) ? 2 : 1;
   else if (two_each(2)) c = 2;
   // (one tile over a hundred thousand terms: the split through global memory, which a layer has and lp_gemm_bf16 has not,
@@ -670,7 +677,8 @@ int gemm_standalone(int which, int M, int N, int K, const void* A, int lda, cons
   if (rc != LP_OK) return rc;
   int bn = gemm_pick_bn(which, M, N, K);
   int segs = 1;
-  const int cluster = gemm_is_pair(bn) ? 0 : gemm_pick_cluster(M, N, K, &bn, &segs, false);
+  const bool sectors = lda % 16 == 0 && ldb % 16 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 31) == 0;
+  const int cluster = gemm_is_pair(bn) ? 0 : gemm_pick_cluster(M, N, K, &bn, &segs, false, sectors);
   uint32_t boxA[2], boxB[2];
   gemm_box_dims(which, bn, boxA, boxB);
   CUtensorMap tmA, tmB;

@@ -393,8 +393,8 @@ static void pick_fc_tiles(Layer* y, int B, bool allow_pair) {
   // 289 / 280, 3072 357 / 378, 4096 565 / 623; batch 64, 2048 218 / 156, 3072 341 / 291, 4096 520 / 529.  So the line, at
   // 2048 x 2048, is on the safe side of where clusters begin to cost, which lies between 2560 and 4096 with the batch.
   const bool chain_bound = (long long)y->n_in * y->n_out <= (1ll << 22);
-  y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f, &y->seg_f, true) : 0;
-  y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d, &y->seg_d, true) : 0;
+  y->cl_f = chain_bound && !gemm_is_pair(y->bn_f) ? gemm_pick_cluster(B, y->n_out, y->n_in, &y->bn_f, &y->seg_f, true, false) : 0;
+  y->cl_d = chain_bound && !gemm_is_pair(y->bn_d) ? gemm_pick_cluster(B, y->n_in, y->n_out, &y->bn_d, &y->seg_d, true, false) : 0;
   y->split_f = gemm_is_pair(y->bn_f) || y->cl_f > 0 ? 1 : gemm_pick_splits(B, y->n_out, y->n_in, y->bn_f);
   y->split_d = gemm_is_pair(y->bn_d) || y->cl_d > 0 ? 1 : gemm_pick_splits(B, y->n_in, y->n_out, y->bn_d);
 }

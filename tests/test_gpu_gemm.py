@@ -180,7 +180,7 @@ def _sum_of_parts(which, M, N, A, B, ldc, k0, k1, parts):
 @pytest.mark.parametrize("M, N, K, parts", [
     (64, 64, 256, (1, 4)), (33, 70, 250, (1, 4)), (128, 2368, 200, (1, 4)), (128, 2369, 200, (1, 2)), (129, 65, 130, (1, 2)), (1, 1, 128, (1, 2)),
     (300, 1000, 256, (1, 2)), (513, 1000, 256, (1, 1)), (65, 130, 40, (1, 1)), (1000, 1000, 2100, (1, 2)), (128, 4800, 1980, (1, 1)),
-    (128, 6000, 4096, (1, 2)), (64, 4736, 4096, (2, 2)), (100, 4730, 4290, (2, 2)), (64, 4736, 4030, (2, 1))])
+    (120, 6008, 4040, (1, 2)), (64, 4736, 4096, (2, 2)), (100, 4730, 4290, (2, 2)), (64, 4736, 4030, (2, 1))])
 @pytest.mark.parametrize("which", [0, 1, 2])
 def test_sums_of_a_contraction_are_no_longer_than_its_parts(which, M, N, K, parts):
     """The accumulator is truncated once per 16 terms, so its error grows with the length of a sum: bit for bit the sums of
@@ -188,6 +188,28 @@ def test_sums_of_a_contraction_are_no_longer_than_its_parts(which, M, N, K, part
     import torch
     from paper_2108_06629_b200 import binding as lpb
     A, B = (t.cuda() for t in _operands(which, M, N, K, 5000 + which))
+    ldc = (N + 3) // 4 * 4
+    Cd = torch.full((M, ldc), 7.0, device="cuda")
+    lpb.lp_gemm_bf16(which, M, N, K, A, A.shape[1], B, B.shape[1], Cd, ldc)
+    assert lpb.lp_debug_last_contraction() == "cluster 64 x%d" % parts[0]
+    assert torch.equal(Cd, _sum_of_parts(which, M, N, A, B, ldc, 0, K, parts))
+    assert lpb.lp_gemm_status() == (lpb.LP_OK, 0)
+
+
+# Two CTAs an SM: one and several rows of tiles, the most tiles of quarters and the fewest and most of halves, k-blocks on the line and an odd
+# number of them; and the same where a row, or the matrix, does not start on a sector (shift: elements).
+@pytest.mark.parametrize("M, N, K, shift, parts", [
+    (64, 4096, 4096, 0, (4,)), (256, 2048, 4096, 0, (4,)), (384, 1024, 4096, 0, (4,)), (112, 2448, 4144, 0, (4,)), (64, 4352, 4096, 0, (4,)),
+    (64, 4736, 4096, 0, (2, 2)), (64, 2416, 4032, 0, (2,)), (64, 4752, 2048, 0, (2,)), (1008, 1152, 2064, 0, (2,)), (1008, 1152, 1984, 0, (1,)),
+    (120, 2504, 4104, 0, (2, 2)), (120, 6008, 2056, 0, (1, 2)), (64, 4096, 4096, 8, (2, 2)), (1008, 1152, 2064, 8, (1, 2))])
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_long_contraction_is_divided_over_two_ctas_an_sm(which, M, N, K, shift, parts):
+    """The form, and bit for bit the sums of its parts."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    A, B = (t.cuda() for t in _operands(which, M, N, K, 4000 + which))
+    if shift:
+        B = torch.nn.functional.pad(B.reshape(-1), (shift, 0))[shift:].view(B.shape)
     ldc = (N + 3) // 4 * 4
     Cd = torch.full((M, ldc), 7.0, device="cuda")
     lpb.lp_gemm_bf16(which, M, N, K, A, A.shape[1], B, B.shape[1], Cd, ldc)
