@@ -506,6 +506,46 @@ def test_tasks_halo_tiles_of_narrow_layers(H, W, B, chans, pools):
     run_teacher_forced(layers, B, 2, None, 0.05, 0.9, 1)
 
 
+# 32, 128, 256 and 200 k-blocks of 64 pixels; 27 or 75 columns, one and two tiles
+@pytest.mark.parametrize("hw, batch, n_out, net, splits", [(16, 8, 16, "3x3", 4), (16, 32, 16, "3x3", 9), (16, 64, 136, "3x3", 12), (40, 8, 24, "3x3", 11),
+                                                           (32, 32, 32, "5x5", 6)])
+def test_tasks_patch_layer_gradient_is_the_sum_of_its_splits(hw, batch, n_out, net, splits):
+    """G of a patch-matrix first layer on small images: sqrt(0.6 k-blocks) splits (0.3 for more than 64 columns), which bound the length of its
+    sums; bit for bit the undivided contractions of the splits, added in order."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    from paper_2108_06629_b200 import inputs as I
+    R, stride, pad = (3, 1, 1) if net == "3x3" else (5, 2, 2)
+    ho = hw // stride
+    conv = I.conv(3, n_out, hw, hw) if net == "3x3" else I.conv(3, n_out, hw, hw, R=R, S=R, stride=stride, pad=pad)
+    layers = [conv, I.fc(n_out * ho * ho, 4, "none")]
+    W0, b0 = I.initial_weights(layers, 0)
+    tr = lpb.Trainer(layers, batch, 1, lr=0.1, momentum=0.0, flags=lpb.LP_CAPTURE_GRADS, W0=W0, b0=b0)
+    g = torch.Generator().manual_seed(hw)
+    x = torch.randn(batch, hw, hw, 3, generator=g).bfloat16()
+    d = torch.randn(batch, ho, ho, n_out, generator=g).bfloat16()
+    tr.debug_write("input", 0, 0, x.float().numpy())
+    tr.debug_write("delta", 0, 0, d.float().numpy())
+    tr.debug_run_task("G", 0, 0)
+    got = torch.from_numpy(tr.debug_read("grad_w", 0, 0)).reshape(n_out, -1)
+    tr.close()
+    cols = torch.nn.functional.unfold(x.float().permute(0, 3, 1, 2), R, padding=pad, stride=stride)     # [batch][channel, tap][pixel]
+    cols = cols.reshape(batch, 3, R * R, ho * ho).permute(0, 3, 2, 1).reshape(batch * ho * ho, -1)
+    pad8 = lambda m: torch.nn.functional.pad(m, (0, -m.shape[1] % 8)).bfloat16().cuda()             # noqa: E731
+    A, X = pad8(d.float().reshape(-1, n_out)), pad8(cols)
+    K, N = len(X), R * R * 3
+    per, total = -(-(K // 64) // splits) * 64, 0.0
+    lpb.lp_set_tuning(64, 0, 1)
+    try:
+        for k in range(0, K, per):
+            part = torch.zeros(n_out, (N + 3) // 4 * 4, device="cuda")
+            lpb.lp_gemm_bf16(2, n_out, N, min(per, K - k), A[k:], A.shape[1], X[k:], X.shape[1], part, part.shape[1])
+            total = total + part
+    finally:
+        lpb.lp_set_tuning(0, 0, 0)
+    assert torch.equal(got, total[:, :N].cpu())
+
+
 @pytest.mark.parametrize("wide, narrow, form", [(4160, 832, "cluster 64 x2"), (2112, 1664, "cluster 64 x1")])
 def test_tasks_two_accumulators_a_cta(wide, narrow, form, monkeypatch):
     """Forward and delta of 39 tiles over 65 k-blocks (halves) and of 78 tiles over 33 (one CTA a tile): two accumulators each."""
