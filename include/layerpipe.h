@@ -336,7 +336,8 @@ int lp_debug_gemm_starved(int M, int N, int K, const void* A_dev, int lda, const
  * caller has the logits and the labels and room for the outputs, but nothing to pass as
  * the per-row scratch the kernel needs.
  *
- * Computes exactly what the loss task of lp_step computes:
+ * Computes exactly what the loss task of lp_step computes (bit for bit where the pitches are a trainer's: classes
+ * rounded up to a multiple of 8):
  *   delta_dev[r][c] = bf16( (softmax(logits_dev[r])[c] - [c == labels_dev[r]]) / batch )
  *   *loss_dev       = mean over rows of -log softmax(logits_dev[r])[labels_dev[r]]
  * logits_dev: device fp32 [batch][ld_logits]; labels_dev: device int32 [batch], values in

@@ -237,20 +237,41 @@ __device__ __forceinline__ float row_reduce(float v, float* sh, bool is_max) {
   return r;
 }
 
-// Mean of B row losses by the block: thread t adds rows t, t + THREADS, ... in that order, then a tree over the threads.
+// Mean of B row losses by the block, in one order whatever the block's size, so that a trainer's loss and the static call's are the
+// same bits: sum t of XENT_SUMS takes rows t, t + XENT_SUMS, ... in that order, 32 neighbouring sums are added as a tree, the 32 results in order.
+constexpr int XENT_SUMS = 1024;
 template <int THREADS>
 __device__ __forceinline__ void row_loss_mean(const float* row_loss, float* loss_out, int B, float* sh) {
-  float acc = 0.f;
+  constexpr int PER = XENT_SUMS / THREADS;            // sums of a thread
+  if (PER > 1 && B <= THREADS) {                      // (the other sums are empty: the same bits)
+    const float sum = row_reduce<THREADS>(int(threadIdx.x) < B ? __ldcg(row_loss + threadIdx.x) : 0.f, sh, false);
+    if (threadIdx.x == 0) *loss_out = sum * (1.0f / float(B));
+    return;
+  }
+  float acc[PER] = {};
 #pragma unroll 8
-  for (int i = threadIdx.x; i < B; i += THREADS) acc += __ldcg(row_loss + i);
-  acc = row_reduce<THREADS>(acc, sh, false);
-  if (threadIdx.x == 0) *loss_out = acc * (1.0f / float(B));
+  for (int i = threadIdx.x; i < B; i += XENT_SUMS)
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+      if (PER == 1 || i + k * THREADS < B) acc[k] += __ldcg(row_loss + i + k * THREADS);
+#pragma unroll
+  for (int k = 0; k < PER; ++k) acc[k] = row_reduce<32>(acc[k], nullptr, false);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < PER; ++k)
+    if ((threadIdx.x & 31) == 0) sh[k * (THREADS / 32) + int(threadIdx.x >> 5)] = acc[k];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float sum = sh[0];
+#pragma unroll
+    for (int i = 1; i < XENT_SUMS / 32; ++i) sum += sh[i];
+    *loss_out = sum * (1.0f / float(B));
+  }
 }
-constexpr int XENT_MEAN_THREADS = 1024;
-__global__ void __launch_bounds__(XENT_MEAN_THREADS) softmax_xent_mean_kernel(const float* row_loss, float* loss_out, int B) {
-  __shared__ float sh[XENT_MEAN_THREADS / 32];
+__global__ void __launch_bounds__(XENT_SUMS) softmax_xent_mean_kernel(const float* row_loss, float* loss_out, int B) {
+  __shared__ float sh[XENT_SUMS / 32];
   launch_wait();
-  row_loss_mean<XENT_MEAN_THREADS>(row_loss, loss_out, B, sh);
+  row_loss_mean<XENT_SUMS>(row_loss, loss_out, B, sh);
 }
 
 // N = classes that a thread keeps in registers; what lies beyond TPR * N goes in several sweeps over memory
@@ -259,7 +280,7 @@ __global__ void __launch_bounds__(XENT_THREADS, 4)
 softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict__ labels, __nv_bfloat16* __restrict__ delta, int ldd,
                     float* __restrict__ row_loss, unsigned* __restrict__ ticket, float* __restrict__ loss_out, int B, int C, int* __restrict__ status) {
   constexpr int ROWS = XENT_THREADS / TPR;            // rows of a block
-  __shared__ float sh[XENT_THREADS / 32];
+  __shared__ float sh[XENT_SUMS / 32];
   __shared__ bool last;
   const int t = int(threadIdx.x) % TPR;
   const float invB = 1.0f / float(B);
@@ -374,7 +395,7 @@ cudaError_t launch_softmax_xent(const float* zL, int ldz, const int* labels, __n
 #undef LP_XENT_VEC
 #undef LP_XENT
   if (e != cudaSuccess || ticket != nullptr || grid == 1) return e;
-  return launch_chained(softmax_xent_mean_kernel, 1, XENT_MEAN_THREADS, 0, stream, 1, static_cast<const float*>(row_loss), loss_out, B);
+  return launch_chained(softmax_xent_mean_kernel, 1, XENT_SUMS, 0, stream, 1, static_cast<const float*>(row_loss), loss_out, B);
 }
 
 // ---------------------------------------------------------------------------

@@ -137,6 +137,29 @@ def test_static_loss_at_the_edges_of_its_row_forms(B, C, ld):
     assert abs(float(loss) - ref_loss) <= 2e-6 * max(1.0, abs(ref_loss))
 
 
+@pytest.mark.parametrize("B, C", [(1, 10), (64, 10), (300, 10), (3000, 10), (1025, 100), (2049, 1000), (700, 1100), (16384, 33)])
+def test_static_loss_is_the_loss_task_bit_for_bit(B, C):
+    """The same logits through a trainer's loss task and through the static call: one block, a few, more rows than sums."""
+    import torch
+    from paper_2108_06629_b200 import binding as lpb
+    from paper_2108_06629_b200 import inputs as I
+    g = torch.Generator().manual_seed(B + C)
+    z = torch.zeros(B, (C + 7) // 8 * 8)
+    z[:, :C] = 3.0 * torch.randn(B, C, generator=g)
+    y = torch.randint(0, C, (B,), generator=g, dtype=torch.int32)
+    layers = [I.fc(8, C, "none")]
+    W0, b0 = I.initial_weights(layers, 0)
+    tr = lpb.Trainer(layers, B, 1, W0=W0, b0=b0)
+    tr.debug_write("labels", 0, 0, y.float().numpy())
+    tr.debug_write("logits", 0, 0, z[:, :C].numpy())
+    tr.debug_run_task("loss", 0, 0)
+    delta, loss = torch.zeros(B, z.shape[1], dtype=torch.bfloat16, device="cuda"), torch.zeros(1, device="cuda")
+    assert lpb.lp_softmax_xent_static(z.cuda(), y.cuda(), delta, loss, C) == lpb.LP_OK
+    assert np.array_equal(tr.debug_read("delta", 0, 0), delta[:, :C].float().cpu().numpy())
+    assert float(tr.debug_read("loss", 0, 0)[0]) == float(loss)
+    tr.close()
+
+
 def test_static_loss_after_calls_that_overlapped():
     """Two calls that overlap on the shared scratch may give wrong losses and leave its counter anywhere; the header
     promises that ordered calls after them are right again.  16 pairs of calls of many blocks, numbers unequal, run on
