@@ -1097,9 +1097,9 @@ __global__ void __launch_bounds__(256) gemm_split_finish_kernel(const GemmArgs p
   const int j = int(threadIdx.x) / GROUPS, e = int(threadIdx.x) % GROUPS;
   const int g = (int(blockIdx.x) % BLOCKS) * GROUPS + e;
   const int r = g / (BN / 4), c = (g % (BN / 4)) * 4;
+  launch_wait();
   if (tc.tm.m0 + (int(blockIdx.x) % BLOCKS) * GROUPS / (BN / 4) >= p.M) return;     // the block's first row
   const float* src = p.partial + (size_t(tile) * p.splits * GEMM_BM + r) * BN + c;
-  launch_wait();
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
   for (int z = j; z < p.splits; z += LANES) {
