@@ -43,7 +43,8 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
   cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
-// Holds until the kernel before this one in the stream has completed (returns at once in a launch without the attribute).
+// Holds until the kernel before this one in the stream has completed (returns at once in a launch without the attribute).  What that
+// kernel writes changes while this one runs: no __restrict__ on parameters and no read-only loads, which the compiler may move in front.
 __device__ __forceinline__ void launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The next kernel of the stream may start its blocks once every block of this one has said so or has ended.  Said by the
 // kernels of short chains only (cluster contractions, loss, column sums), once a block has asked for its last operands.  Blocks that

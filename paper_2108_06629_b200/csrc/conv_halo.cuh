@@ -201,7 +201,7 @@ conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
     for (int g = 0; g < 8 * H; ++g) {
       const int n = half0 * 32 + 4 * g;
-      bias4[g] = (MODE == EPI_FPROP && p.bias != nullptr && n < p.N) ? __ldg(reinterpret_cast<const float4*>(p.bias + n))
+      bias4[g] = (MODE == EPI_FPROP && p.bias != nullptr && n < p.N) ? *reinterpret_cast<const float4*>(p.bias + n)
                                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     int tw = tw_begin, th = th_begin, tn = tn_begin;
@@ -415,7 +415,7 @@ constexpr int HALOG_PART_FLOATS = HALOG_GROUPS * GEMM_BM * 64;  // partial sums 
 template <int kInstance = 0>   // (a template only so that the header may be included by several translation units)
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 conv_halo_g_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD, const ConvGeom g,
-                   const int tiles_total, const int co0, float* __restrict__ partial, int* __restrict__ status) {
+                   const int tiles_total, const int co0, float* partial, int* status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + HALOG_STAGES * HALOG_STAGE_BYTES);

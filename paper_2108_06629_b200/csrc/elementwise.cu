@@ -20,9 +20,9 @@ cudaError_t launch_trace_mark(unsigned* flag, unsigned value, cudaStream_t strea
 // ---------------------------------------------------------------------------
 // a^0 = RN_bf16(batch) into the first layer's activation-stash slot; labels are copied
 // into the library's label ring so that the caller may reuse its buffers.
-__global__ void cast_stash_kernel(const void* __restrict__ batch, int input_is_bf16,
-                                  const int* __restrict__ labels, __nv_bfloat16* __restrict__ x0,
-                                  int* __restrict__ labels_copy, int rows, int B, int n_in, int ld) {
+__global__ void cast_stash_kernel(const void* batch, int input_is_bf16,
+                                  const int* labels, __nv_bfloat16* x0,
+                                  int* labels_copy, int rows, int B, int n_in, int ld) {
   launch_wait();
   const long long groups_per_row = ld / 8;
   const long long total = (long long)rows * groups_per_row;
@@ -79,9 +79,9 @@ cudaError_t launch_cast_stash(const void* batch, int input_is_bf16, const int* l
 // One thread per output pixel; C is a template parameter so that the 9*C gathered values stay in
 // registers and the column arithmetic folds at compile time.
 template <int C>
-__global__ void cast_patch3x3_kernel(const void* __restrict__ batch, int input_is_bf16,
-                                     const int* __restrict__ labels, __nv_bfloat16* __restrict__ x0,
-                                     int* __restrict__ labels_copy, int B, int H, int W) {
+__global__ void cast_patch3x3_kernel(const void* batch, int input_is_bf16,
+                                     const int* labels, __nv_bfloat16* x0,
+                                     int* labels_copy, int B, int H, int W) {
   constexpr int LD = (9 * C + 7) / 8 * 8;
   launch_wait();
   const int total = B * H * W;
@@ -151,8 +151,8 @@ constexpr int PATCH_PIX = 64;
 constexpr int PATCH_COLS_MAX = 128;
 inline int patch_span(int S, int stride) { return (PATCH_PIX - 1) * stride + S; }     // input pixels of one staged row
 __global__ void __launch_bounds__(256)
-cast_patch_general_kernel(const void* __restrict__ batch, int input_is_bf16, const int* __restrict__ labels,
-                          __nv_bfloat16* __restrict__ x0, int* __restrict__ labels_copy, int B, int H, int W, int C, int R, int S,
+cast_patch_general_kernel(const void* batch, int input_is_bf16, const int* labels,
+                          __nv_bfloat16* x0, int* labels_copy, int B, int H, int W, int C, int R, int S,
                           int stride, int pad, int Ho, int Wo, int ld, int span, int segs) {
   extern __shared__ __nv_bfloat16 rows[];                      // [R][span][C]
   __shared__ short col_off[PATCH_COLS_MAX];                    // column -> offset in `rows` for output pixel 0, -1: padding column
@@ -277,8 +277,8 @@ __global__ void __launch_bounds__(XENT_SUMS) softmax_xent_mean_kernel(const floa
 // N = classes that a thread keeps in registers; what lies beyond TPR * N goes in several sweeps over memory
 template <int TPR, int VEC, int N>
 __global__ void __launch_bounds__(XENT_THREADS, 4)
-softmax_xent_kernel(const float* __restrict__ zL, int ldz, const int* __restrict__ labels, __nv_bfloat16* __restrict__ delta, int ldd,
-                    float* __restrict__ row_loss, unsigned* __restrict__ ticket, float* __restrict__ loss_out, int B, int C, int* __restrict__ status) {
+softmax_xent_kernel(const float* zL, int ldz, const int* labels, __nv_bfloat16* delta, int ldd,
+                    float* row_loss, unsigned* ticket, float* loss_out, int B, int C, int* status) {
   constexpr int ROWS = XENT_THREADS / TPR;            // rows of a block
   __shared__ float sh[XENT_SUMS / 32];
   __shared__ bool last;
@@ -511,8 +511,8 @@ cudaError_t launch_round_to_bf16(const float* src, __nv_bfloat16* dst, long long
 namespace lp {
 // ---------------------------------------------------------------------------
 // 2x2 stride-2 max pool, NHWC, 8 channels (16 bytes) per thread.
-__global__ void maxpool2_kernel(const __nv_bfloat16* __restrict__ a, __nv_bfloat16* __restrict__ pooled,
-                                unsigned char* __restrict__ idx, int B, int H, int W, int C) {
+__global__ void maxpool2_kernel(const __nv_bfloat16* a, __nv_bfloat16* pooled,
+                                unsigned char* idx, int B, int H, int W, int C) {
   const int Hp = H / 2, Wp = W / 2, cg = C / 8;
   const long long total = (long long)B * Hp * Wp * cg;
   launch_wait();
@@ -567,8 +567,8 @@ cudaError_t launch_maxpool2(const __nv_bfloat16* a, __nv_bfloat16* pooled, unsig
 // Narrow matrices: G8 threads of eight columns to a row, as few as cover it, and 256 / G8 row lanes (16 columns read by eight threads
 // a row left six of them idle: 1 605 632 x 16 31 -> 18 us, 802 816 x 32 20 -> 17).
 template <int G8>
-__global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* __restrict__ x, int rows, int ld, int n_cols, int chunk_rows,
-                                                          float* __restrict__ partial, unsigned* __restrict__ counter,
+__global__ void __launch_bounds__(256) colsum_bias_kernel(const __nv_bfloat16* x, int rows, int ld, int n_cols, int chunk_rows,
+                                                          float* partial, unsigned* counter,
                                                           const BiasUpdate u) {
   constexpr int LANES = 256 / G8;                                  // row lanes
   constexpr int COLS = 8 * G8, PITCH = COLS + 4;

@@ -176,7 +176,7 @@ __device__ __forceinline__ int tile_row(const GemmArgs& p, const TileMap& t, int
 // Bias of four consecutive output columns (zero where there is none).
 __device__ __forceinline__ void load_bias4(const GemmArgs& p, int n, int N, float b[4]) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) b[j] = (p.bias != nullptr && n + j < N) ? __ldg(p.bias + n + j) : 0.f;
+  for (int j = 0; j < 4; ++j) b[j] = (p.bias != nullptr && n + j < N) ? p.bias[n + j] : 0.f;
 }
 // Forward epilogue for columns n..n+3 of one row: z = acc + b; z^L / stored z; a = f(z).
 __device__ __forceinline__ void fprop_store4(const GemmArgs& p, int row, int n, int N, const float acc[4], const float b[4]) {

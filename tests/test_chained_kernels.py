@@ -48,3 +48,16 @@ def test_every_block_waits_before_it_leaves_or_lets_the_next_kernel_start(name):
     before = body[:body.index("launch_wait()")]
     before = re.sub(r"\[[&=]?\]\s*(\([^)]*\))?\s*\{[^{}]*\}", "", before)       # (a lambda's return is not the kernel's)
     assert "return" not in before and "launch_next()" not in before
+
+
+@pytest.mark.parametrize("name", WAITING)
+def test_nothing_lets_a_load_move_in_front_of_the_wait(name):
+    """What the kernel before writes is no constant of the kernel that reads it: no restricted parameters, ..."""
+    assert "__restrict__" not in KERNELS[name][0]
+
+
+def test_no_read_only_loads():
+    """... and no loads from the read-only path, in the kernels or in what they share."""
+    for f in os.listdir(CSRC):
+        if f.endswith((".cu", ".cuh", ".h")):
+            assert not re.search(r"__ldg\s*\(|ld\.global\.nc", open(os.path.join(CSRC, f)).read()), f
