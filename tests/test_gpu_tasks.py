@@ -177,7 +177,7 @@ def test_tasks_unfused_update_path():
 
 def test_tasks_split_k_forward_and_delta():
     """Forced split-K (3 and 8 splits, more splits than k-blocks in some layers): partial tiles
-    reduced in split order by the last CTA of each tile."""
+    added in split order by a second launch."""
     from paper_2108_06629_b200 import binding as lpb
     from paper_2108_06629_b200 import inputs as I
     layers = I.mlp([520, 328, 200, 75], "gelu")
@@ -187,6 +187,23 @@ def test_tasks_split_k_forward_and_delta():
             run_teacher_forced(layers, 72, 3, [2, 1, 0], 0.05, 0.9, 4)
         finally:
             lpb.lp_set_tuning(0, 0, 0)
+
+
+def test_tasks_sixteen_and_more_splits(monkeypatch):
+    """Forced split-K of 18 and 19 splits, which eight threads a group of columns add: forward on 128- and 64-column tiles, delta, and the
+    un-pooling delta of a fully connected layer behind a pool."""
+    from paper_2108_06629_b200 import binding as lpb
+    from paper_2108_06629_b200 import inputs as I
+    forms = _forms(monkeypatch)
+    lpb.lp_set_tuning(0, 0, 20)
+    try:
+        run_teacher_forced(I.mlp([520, 1160, 1100, 10], "gelu"), 72, 3, [2, 1, 0], 0.05, 0.9, 2)
+        assert forms["forward", 1] == {"single split 128"} and forms["forward", 2] == {"single split 64"} and forms["delta", 1] == {"single split 128"}, forms
+        forms.clear()
+        run_teacher_forced(I.vgg(16, [16, "P"], [1100, 10]), 8, 2, None, 0.05, 0.0, 2)
+        assert forms["delta", 1] == {"single split 128"} and forms["forward", 2] == {"single split 64"}, forms
+    finally:
+        lpb.lp_set_tuning(0, 0, 0)
 
 
 def test_tasks_persistent_tile_loop():
@@ -328,9 +345,9 @@ def test_tasks_convolutional_network_runs_no_sm_pair_kernel(code, monkeypatch):
 
 
 def test_tasks_single_image_224_patch_layer_and_automatic_split_k():
-    """One 224 x 224 RGB image: the patch-matrix first layer (forward through the halo pipeline, G as
-    one tile split 148 ways over 50 k pixel rows) and a fully connected layer with 3136 k-blocks and
-    a single tile, which takes the automatic four-way split-K."""
+    """One 224 x 224 RGB image, and two: the patch-matrix first layer (forward through the halo pipeline, G as
+    one tile whose 50 k or 100 k pixel rows are split) and a fully connected layer with 3136 k-blocks and
+    a single tile, which takes the automatic split-K over all SMs."""
     from paper_2108_06629_b200 import inputs as I
     layers = I.vgg(224, [16, "P"], [10])
     run_teacher_forced(layers, 1, 2, None, 0.05, 0.9, 3)
@@ -555,8 +572,12 @@ def test_tasks_two_accumulators_a_cta(wide, narrow, form, monkeypatch):
     assert forms["forward", 0] == {form} and forms["delta", 1] == {form}, forms
 
 
-@pytest.mark.parametrize("n_in, n_out, batch", [(17000, 10, 5), (16390, 130, 3), (20000, 300, 130)])
-def test_tasks_long_contractions_split_over_all_sms(n_in, n_out, batch):
-    """One to six tiles of 256 k-blocks and more, the last split shorter than the others: sum and epilogue in a second launch."""
+@pytest.mark.parametrize("n_in, n_out, batch, form", [(17500, 10, 5, "single split 64"), (17410, 130, 3, "single split 128"),
+                                                      (100352, 10, 2, "single split 64"), (20000, 300, 130, "single split 128"), (17000, 10, 5, "cluster 64 x8")])
+def test_tasks_long_contractions_split_over_all_sms(n_in, n_out, batch, form, monkeypatch):
+    """One to six tiles of 273 k-blocks and more, the last split shorter than the others: sum and epilogue in a second launch.  At 266 k-blocks
+    eight CTAs of a cluster still do it."""
     from paper_2108_06629_b200 import inputs as I
+    forms = _forms(monkeypatch)
     run_teacher_forced([I.fc(24, n_in), I.fc(n_in, n_out, "gelu"), I.fc(n_out, 6, "none")], batch, 2, None, 0.01, 0.0, 1)
+    assert forms["forward", 1] == {form}, forms
