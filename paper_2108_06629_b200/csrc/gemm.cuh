@@ -59,7 +59,7 @@ struct ConvGeom {
   int S, pad;            // filter width (tap = r*S + s) and padding
   int flip;              // 0: forward / G (input pixel = output pixel * stride + tap - pad); 1: delta
   int chunks_per_tap;    // PIX_M: 64-channel chunks of the A tensor per tap
-  int last_slices;       // halo-tile kernels: slices of 16 channels that the last of them holds
+  int last_slices;       // conv_halo_kernel only, which has one chunk: slices of 16 channels that exist.  The others multiply whole chunks.
   int tap_pitch;         // elements between taps inside a row of the weight matrix (padded Cin)
   int n_per_tap;         // PIX_K: column tiles per tap
   // General filters and strides.  stride: the convolution's stride (forward and G fetch the input

@@ -777,7 +777,7 @@ struct TimedScope {
 
 // ---------------------------------------------------------------------------
 // the kernels of one minibatch
-// slices of 16 that the last 64 of `channels` hold
+// slices of 16 that at most 64 channels hold
 static int last_slices(int channels) { return ((channels - 1) % 64) / 16 + 1; }
 static ConvGeom conv_geom(const Layer& y, int kind, const PixBox& bx, int flip, int chunks_per_tap, int n_per_tap) {
   ConvGeom g{};
@@ -790,7 +790,6 @@ static ConvGeom conv_geom(const Layer& y, int kind, const PixBox& bx, int flip, 
   g.S = y.cS; g.pad = y.cpad;
   g.flip = flip;
   g.chunks_per_tap = chunks_per_tap;
-  g.last_slices = last_slices(flip ? y.n_out : y.n_in);
   g.tap_pitch = y.ld_in;
   g.n_per_tap = n_per_tap;
   g.stride = y.cstride;
